@@ -244,20 +244,18 @@ mem_status mem_phase_rotate(int64_t n_vis, const double *u, const double *v, dou
  * not a peak. */
 mem_status mem_beam_fit(const float *psf_host, int32_t n, double dx, double dy, double *out4);
 
-/* Tensor-core tiling.  fwd_kernel selects the forward kernel:
- *   MEM_FWD_STREAM    the split image operand streams through shared memory
- *                     for every 64-visibility tile, in column blocks of
- *                     fwd_cols (a multiple of 32 dividing N, at most 256);
- *                     fwd_stages 3 or 4;
- *   MEM_FWD_RESIDENT  (N <= 256) each CTA keeps a 128-row slice of the split
- *                     image operand in shared memory and only the phase
- *                     tables stream; fwd_cols is N; fwd_stages 4 to 6 (as
- *                     shared memory allows).
- * adj_stages: adjoint pipeline depth, 2 or 3.  The two forward kernels round
- * differently (the resident one sums 128-row slices in FP64 and issues the
- * small correction products before the main ones); both meet the form's
- * tolerances; at a solve's final image the resident order halves the chi^2
- * error. */
+/* Tensor-core tiling.  fwd_kernel selects where the forward's image operand
+ * lives (FP16X3: the image folded about its centre, whose mirror pixels share
+ * their products; BF16X3: the image):
+ *   MEM_FWD_STREAM    it streams through shared memory for every tile of
+ *                     visibilities, in column blocks of fwd_cols (a multiple
+ *                     of 32 dividing N, at most 256); fwd_stages 3 or 4;
+ *   MEM_FWD_RESIDENT  (N <= 256) each CTA keeps it in shared memory (at N = 256
+ *                     half of it) and only the phase tables stream; fwd_cols
+ *                     is N; fwd_stages 4 to 6 (as shared memory allows).
+ * adj_stages: adjoint pipeline depth, 2 or 3.  The choices round differently
+ * (for N <= 128 the resident one issues the small correction products before
+ * the main ones); all meet the form's tolerances. */
 typedef enum { MEM_FWD_STREAM = 0, MEM_FWD_RESIDENT = 1 } mem_fwd_kernel;
 
 typedef struct {
@@ -285,7 +283,7 @@ mem_status mem_set_tiling(mem_ctx *ctx, const mem_tiling_t *tiling);
 /* The tiling in use.  The direct forms report the defaults, which they do
  * not use.  Defaults (before mem_autotune or a cached choice): for N <= 128
  * MEM_FWD_RESIDENT with the deepest pipeline that fits (mem_autotune keeps
- * the resident kernel there: it is the more accurate one, see above), for
+ * the resident form there: it is the more accurate one, see above), for
  * N >= 256 MEM_FWD_STREAM with 256 columns and 4 stages; adjoint 3 stages. */
 mem_status mem_tiling(const mem_ctx *ctx, mem_tiling_t *out);
 

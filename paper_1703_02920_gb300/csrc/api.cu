@@ -55,8 +55,8 @@ struct mem_ctx {
     float* beam = nullptr;
     int64_t* doff = nullptr;
 
-    // work lists: visibility tiles for the direct forms (128) and the
-    // tensor-core form (TC_TILE)
+    // work lists: visibility tiles of VIS_TILE and (BF16X3) of TC_TILE, and the
+    // adjoint's units
     std::vector<VisTile> tiles_h, tiles_tc_h;
     std::vector<int> tile_off_h, tile_off_tc_h;
     VisTile *tiles = nullptr, *tiles_tc = nullptr;
@@ -76,7 +76,7 @@ struct mem_ctx {
     float* bf32 = nullptr;
     double* bf64 = nullptr;
     uint16_t* planes = nullptr;
-    float* cmean = nullptr;  // column means of the centred tensor-core operand
+    float* cmean = nullptr;  // means of the centred tensor-core operand
     float* cscale = nullptr;                    // FP16X3 operand scales per channel
     double* col_psum = nullptr;                 // column-mean partial sums
     float* col_pmax = nullptr;
@@ -111,11 +111,11 @@ struct mem_ctx {
         int64_t n_pro = 0, n_iter = 0, n_probe = 0;  // kernel launches per part
     } g_solve;
 
-    // tensor-core tiling (autotuned): forward kernel (MEM_FWD_STREAM: image
-    // operand streamed per tile, column block fwd_bn; MEM_FWD_RESIDENT: image
-    // slice resident in shared memory, N <= 256), pipeline depths
+    // tensor-core tiling (autotuned): forward operand (MEM_FWD_STREAM: streamed
+    // per tile in column blocks of fwd_bn; MEM_FWD_RESIDENT: resident in shared
+    // memory, N <= 256), pipeline depths
     int fwd_kernel = MEM_FWD_STREAM, fwd_bn = 0, fwd_stages = 4, adj_stages = 3;
-    double2* vpart = nullptr;  // resident kernel: slice partials [slice][Z]
+    float4* vpart = nullptr;  // resident forward: partial sums, two per visibility (BF16X3: double2 per slice)
 
     // gridded forward (the paper's FFT + bilinear approximation): row
     // spectra and 2-D half spectra for `grid_pad`
@@ -363,7 +363,7 @@ mem_status after_launch(mem_ctx* c, const char* what) {
 mem_status ensure_buffers(mem_ctx* c) {
     const size_t NN = (size_t)c->N * c->N;
     TRY(dalloc(c, &c->chi_part, (size_t)4 * std::max(std::max(c->n_tiles, c->n_tiles_tc), 1)));
-    TRY(dalloc(c, &c->ent_part, (size_t)c->n_images * prep_blocks(c->N)));
+    TRY(dalloc(c, &c->ent_part, (size_t)c->n_images * std::max(prep_blocks(c->N), tc_ent_blocks(c->N))));
     TRY(dalloc(c, &c->scal, (size_t)3 + 3 * c->n_images));
     if (!c->img_tmp) {  // holds the scalar reduction's completion counter, which starts at zero
         TRY(dalloc(c, &c->img_tmp, (size_t)scalars_tmp_doubles(c->n_images)));
@@ -390,8 +390,8 @@ mem_status ensure_buffers(mem_ctx* c) {
         TRY(dalloc(c, &c->ymax_part, (size_t)256));
         const int BLK = tca_blk(c->N);
         TRY(dalloc(c, &c->partial, std::max<size_t>(c->units_h.size(), 1) * BLK * BLK));
-        if (c->N <= 256)
-            TRY(dalloc(c, &c->vpart, (size_t)(c->N / fwd_rs_ks(c->N)) * std::max<int64_t>(c->Z, 1)));
+        if (c->fwd_kernel == MEM_FWD_RESIDENT && (c->prec == MEM_PREC_BF16X3 || fold_combines(c->N)))
+            TRY(dalloc(c, &c->vpart, (size_t)2 * std::max<int64_t>(c->Z, 1)));
     }
     int ks = 1;
     if (!is_tc(c->prec)) ks = adj_direct_splits(c->dd(), c->num_sms);
@@ -404,16 +404,12 @@ mem_status ensure_buffers(mem_ctx* c) {
     return MEM_OK;
 }
 
-int bformat(int prec) {
-    return prec == MEM_PREC_FP64_DIRECT   ? BF_F64
-           : prec == MEM_PREC_FP32_DIRECT ? BF_F32
-           : prec == MEM_PREC_FP16X3      ? BF_F16X3
-                                          : BF_BF16X3;
-}
-void* bbuf(mem_ctx* c) {
-    return c->prec == MEM_PREC_FP64_DIRECT ? (void*)c->bf64
-           : c->prec == MEM_PREC_FP32_DIRECT ? (void*)c->bf32 : (void*)c->planes;
-}
+void* bbuf(mem_ctx* c) { return c->prec == MEM_PREC_FP64_DIRECT ? (void*)c->bf64 : (void*)c->bf32; }
+
+// tile list that the form's forward ran over (4 chi^2 partials per tile)
+const int* fwd_tile_off(const mem_ctx* c) { return c->prec == MEM_PREC_BF16X3 ? c->tile_off_tc : c->tile_off; }
+
+int ent_blocks(const mem_ctx* c) { return is_tc(c->prec) ? tc_ent_blocks(c->N) : prep_blocks(c->N); }
 
 // prep + forward for one image source.  mode: FwdMode.  defer_scalars: the
 // objective's scalar reduction is left to a later launch (the gradient's).
@@ -426,36 +422,49 @@ mem_status run_forward(mem_ctx* c, const ImgSrc& src, int mode, bool entropy, vo
     // (zeroed by the column-mean kernel)
     float* ymax = (tc && f16 && mode == FWD_RESID) ? c->ymax : nullptr;
     if (tc) {
-        KTimer t(c, "colmean");
-        launch_colmean(d, src, c->cmean, c->cscale, c->col_psum, c->col_pmax, c->col_count, ymax, c->st);
-        c->launches++;
-    }
-    {
-        KTimer t(c, "prep");
-        launch_prep(d, src, bformat(c->prec), bbuf(c), entropy ? c->ent_part : nullptr, tc ? c->cmean : nullptr,
-                    c->cscale, c->st);
-    }
-    c->launches++;
-    TRY(after_launch(c, "prep kernel"));
-    if (tc && c->fwd_kernel == MEM_FWD_RESIDENT) {
-        KTimer t(c, "fwd_rs");
-        launch_fwd_rs(d, f16, c->tiles_tc, c->n_tiles_tc, c->planes, c->cmean, c->cscale, mode, (float2*)yout,
-                      c->chi_part, ymax, c->vpart, c->Z, c->num_sms, c->spin, c->dstatus, c->st);
-        if (c->n_tiles_tc > 0) c->launches++;  // + the slice combination
-    } else if (tc) {
-        KTimer t(c, "fwd_tc");
-        launch_fwd_tc(d, f16, c->tiles_tc, c->n_tiles_tc, c->planes, c->cmean, c->cscale, mode, (float2*)yout,
-                      c->chi_part, ymax, c->num_sms, c->spin, c->dstatus, c->st);
+        {
+            KTimer t(c, "colmean");
+            launch_colmean(d, src, f16, c->cmean, c->cscale, c->col_psum, c->col_pmax, c->col_count, ymax,
+                           entropy ? c->ent_part : nullptr, c->st);
+        }
+        {
+            KTimer t(c, "prep");
+            if (f16) launch_fold(d, src, c->planes, c->cmean, c->cscale, c->st);
+            else launch_planes(d, src, c->planes, c->cmean, c->st);
+        }
+        c->launches += 2;
+        TRY(after_launch(c, "operand kernels"));
+        const bool resident = c->fwd_kernel == MEM_FWD_RESIDENT;
+        KTimer t(c, resident ? "fwd_rs" : "fwd_tc");
+        if (f16) {
+            c->launches += launch_fwd_fold(d, resident, c->tiles, c->n_tiles, c->planes, c->cmean, c->cscale, mode,
+                                           (float2*)yout, c->chi_part, ymax, c->vpart, c->Z, c->num_sms, c->spin,
+                                           c->dstatus, c->st);
+        } else if (resident) {
+            launch_fwd_rs(d, c->tiles_tc, c->n_tiles_tc, c->planes, c->cmean, mode, (float2*)yout, c->chi_part,
+                          (double2*)c->vpart, c->Z, c->num_sms, c->spin, c->dstatus, c->st);
+            if (c->n_tiles_tc > 0) c->launches += 2;  // and the slice combination
+        } else {
+            launch_fwd_tc(d, c->tiles_tc, c->n_tiles_tc, c->planes, c->cmean, mode, (float2*)yout, c->chi_part,
+                          c->num_sms, c->spin, c->dstatus, c->st);
+            if (c->n_tiles_tc > 0) c->launches++;
+        }
     } else {
-        KTimer t(c, c->prec == MEM_PREC_FP64_DIRECT ? "fwd_direct_f64" : "fwd_direct_f32");
-        launch_fwd_direct(d, c->prec == MEM_PREC_FP64_DIRECT, c->tiles, c->n_tiles, bbuf(c), mode, yout,
-                          c->chi_part, c->st);
+        const int f64 = c->prec == MEM_PREC_FP64_DIRECT;
+        {
+            KTimer t(c, "prep");
+            launch_prep(d, src, f64 ? BF_F64 : BF_F32, bbuf(c), entropy ? c->ent_part : nullptr, c->st);
+        }
+        c->launches++;
+        TRY(after_launch(c, "prep kernel"));
+        KTimer t(c, f64 ? "fwd_direct_f64" : "fwd_direct_f32");
+        launch_fwd_direct(d, f64, c->tiles, c->n_tiles, bbuf(c), mode, yout, c->chi_part, c->st);
+        if (c->n_tiles > 0) c->launches++;
     }
-    if ((tc ? c->n_tiles_tc : c->n_tiles) > 0) c->launches++;
     TRY(after_launch(c, "forward kernel"));
     if (mode != FWD_VIS && !defer_scalars) {
         KTimer t(c, "scalars");
-        launch_scalars(d, tc ? c->tile_off_tc : c->tile_off, c->chi_part, c->ent_part, entropy ? 1 : 0,
+        launch_scalars(d, fwd_tile_off(c), c->chi_part, c->ent_part, entropy ? 1 : 0, ent_blocks(c),
                        c->scal, c->img_tmp, c->st);
         c->launches++;
         TRY(after_launch(c, "scalar reduction"));
@@ -515,10 +524,11 @@ mem_status run_objgrad(mem_ctx* c, const ImgSrc& src, int projected, float* out3
     if (fused) {
         KTimer t(c, "adj_reduce_grad");
         ScalarArgs sc;
-        sc.tile_off = c->tile_off_tc;
+        sc.tile_off = fwd_tile_off(c);
         sc.chi_part = c->chi_part;
         sc.ent_part = c->ent_part;
         sc.with_entropy = 1;
+        sc.n_ent = ent_blocks(c);
         sc.scal = c->scal;
         sc.img_tmp = c->img_tmp;
         launch_adj_tc_reduce_grad(c->dd(), src, c->cb_off, c->partial, c->prec == MEM_PREC_FP16X3 ? c->ymax : nullptr,
@@ -624,8 +634,8 @@ void msk::set_global_error(const char* msg) { g_last_error = msg ? msg : ""; }
 namespace {
 
 // ---------------------------------------------------------------------------
-// Autotuner.  Candidates: forward image column block BN in {128, 256} (N >=
-// 256; the operand planes are laid out per BN) and pipeline depth {3, 4};
+// Autotuner.  Candidates: forward column block BN in {128, 256} (N >= 256; the
+// operand planes are laid out per BN) and pipeline depth {3, 4};
 // adjoint pipeline depth {2, 3}.  Each candidate is timed with per-kernel
 // CUDA events over a few full objective + gradient evaluations of the
 // context's own data; the fastest is kept and recorded in a cache file
@@ -636,7 +646,7 @@ std::string tune_key(const mem_ctx* c) {
     int zb = 0;
     while (((int64_t)1 << (zb + 1)) <= std::max<int64_t>(c->Z, 1)) ++zb;
     char buf[256];
-    std::snprintf(buf, sizeof buf, "%s|N=%d|z=%d|C=%d|prec=%d", c->gpu_name.c_str(), c->N, zb, c->C, c->prec);
+    std::snprintf(buf, sizeof buf, "%s|N=%d|z=%d|C=%d|prec=%d|folded", c->gpu_name.c_str(), c->N, zb, c->C, c->prec);
     std::string k = buf;
     for (char& ch : k)
         if (ch == ' ') ch = '_';
@@ -650,17 +660,31 @@ std::string tune_path() {
     return std::string(h ? h : ".") + "/.cache/libmemsynth_tune.txt";
 }
 
+// shared memory of the form's forward kernel
+int fwd_smem_bytes(const mem_ctx* c, int kernel, int cols, int stages) {
+    if (c->prec != MEM_PREC_BF16X3) return fold_smem_bytes(c->N, cols, stages, kernel == MEM_FWD_RESIDENT);
+    return kernel == MEM_FWD_RESIDENT ? fwd_rs_smem_bytes(c->N, stages) : fwd_tc_smem_bytes(c->N, cols, stages);
+}
+
+// Deepest resident pipeline that fits.
+int resident_stages(const mem_ctx* c) {
+    int s = 6;
+    while (s > 4 && fwd_smem_bytes(c, MEM_FWD_RESIDENT, c->N, s) > 227 * 1024) --s;
+    return s;
+}
+
 bool tune_valid(const mem_ctx* c, const mem_tiling_t& t) {
     if (!(t.adj_stages == 2 || t.adj_stages == 3) || adj_tc_smem_bytes(c->N, t.adj_stages) > 227 * 1024)
         return false;
     if (t.fwd_kernel == MEM_FWD_RESIDENT)
-        return c->N <= 256 && t.fwd_stages >= 4 && t.fwd_stages <= fwd_rs_max_stages(c->N);
+        return c->N <= 256 && t.fwd_stages >= 4 && t.fwd_stages <= 6 &&
+               fwd_smem_bytes(c, MEM_FWD_RESIDENT, c->N, t.fwd_stages) <= 227 * 1024;
     if (t.fwd_kernel != MEM_FWD_STREAM) return false;
     // the epilogue reduces 32-column pairs of 16-column chunks
     const int bn = t.fwd_cols;
     if (bn < 32 || bn > 256 || c->N % bn != 0 || bn % 32 != 0) return false;
     if (!(t.fwd_stages == 3 || t.fwd_stages == 4)) return false;
-    return fwd_tc_smem_bytes(c->N, bn, t.fwd_stages) <= 227 * 1024;
+    return fwd_smem_bytes(c, MEM_FWD_STREAM, bn, t.fwd_stages) <= 227 * 1024;
 }
 
 mem_tiling_t tiling_of(const mem_ctx* c) {
@@ -679,23 +703,26 @@ void apply_tiling(mem_ctx* c, const mem_tiling_t& t) {
     c->adj_stages = t.adj_stages;
 }
 
-// N <= 128: the resident kernel (one row slice, no duplicated work; its
-// corrections-first order halves the chi^2 error at a solve's final image);
-// N >= 256: the streaming kernel (about 1.7x faster than two resident slices).
+// N <= 128: the resident form (the operand fits; its corrections-first order is
+// the more accurate one at a solve's final image); N >= 256: the streaming form
+// (at 256 x 256 with 999,600 visibilities 0.22 ms against 0.25 ms for FP16X3
+// with one resident part per CTA and the pass that adds the parts; BF16X3 0.49
+// against 1.05 ms for two resident slices).
 void default_tiling(mem_ctx* c) {
     mem_tiling_t t;
     if (c->N <= 128) {
         t.fwd_kernel = MEM_FWD_RESIDENT;
         t.fwd_cols = c->N;
-        t.fwd_stages = fwd_rs_max_stages(c->N);
+        t.fwd_stages = resident_stages(c);
     } else {
         t.fwd_kernel = MEM_FWD_STREAM;
         t.fwd_cols = tc_bn(c->N);
         t.fwd_stages = 4;
     }
     t.adj_stages = 3;
-    // very large N: the epilogue's column-mean copies leave room for 3 stages
-    if (t.fwd_kernel == MEM_FWD_STREAM && fwd_tc_smem_bytes(c->N, t.fwd_cols, 4) > 227 * 1024) t.fwd_stages = 3;
+    // BF16X3 at very large N: the epilogue's column-mean copies leave room for 3 stages
+    if (t.fwd_kernel == MEM_FWD_STREAM && fwd_smem_bytes(c, MEM_FWD_STREAM, t.fwd_cols, 4) > 227 * 1024)
+        t.fwd_stages = 3;
     apply_tiling(c, t);
 }
 
@@ -986,7 +1013,7 @@ mem_status mem_autotune(mem_ctx* c, const float* image_dev, int32_t reps, mem_ti
     for (const mem_tiling_t& t : fwd) {
         apply_tiling(c, t);
         double ms = 0;
-        // the resident kernel's slice combination is part of its cost
+        // the resident form's combination of the parts is part of its cost
         if ((st = time_kernels({"fwd_tc", "fwd_rs"}, &ms)) != MEM_OK) break;
         if (ms < best_f) {
             best_f = ms;
@@ -1023,7 +1050,7 @@ mem_status mem_set_tiling(mem_ctx* c, const mem_tiling_t* t) {
         return fail(c, MEM_EINVAL,
                     "tiling: streaming kernel needs a column block dividing N (32..256, multiple of 32) and 3|4 "
                     "stages; resident kernel N <= 256 and 4..%d stages; adjoint 2|3 stages",
-                    c->N <= 256 ? fwd_rs_max_stages(c->N) : 0);
+                    c->N <= 256 ? resident_stages(c) : 0);
     TRY(mem_sync(c));
     apply_tiling(c, x);
     drop_graphs(c);
@@ -1331,7 +1358,7 @@ mem_status mem_create(const mem_config* cfg, const double* u, const double* v, c
     launch_phase_prep(Z, c->u, c->v, c->dx, c->dy, c->pa, c->pb, c->st);
     c->launches++;
 
-    build_tiles(c, 128, c->tiles_h, c->tile_off_h);
+    build_tiles(c, VIS_TILE, c->tiles_h, c->tile_off_h);
     build_tiles(c, TC_TILE, c->tiles_tc_h, c->tile_off_tc_h);
     c->n_tiles = (int)c->tiles_h.size();
     c->n_tiles_tc = (int)c->tiles_tc_h.size();

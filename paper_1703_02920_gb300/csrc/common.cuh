@@ -95,6 +95,37 @@ __device__ __forceinline__ cf2 cis_neg(uint64_t p) {
     return {c * r, -s * r};
 }
 
+// High 32 bits of the phase k p for 0 <= k < 2^31: all that an FP32 angle needs.
+__device__ __forceinline__ uint32_t phase_hi(uint32_t k, uint64_t p) {
+    return __umulhi(k, (uint32_t)p) + k * (uint32_t)(p >> 32);
+}
+
+// e^{-2 pi i t / 2^32} to FP32 rounding (t: the high word of a phase; the rest
+// is below 2^-32 turns).  The nearest quarter turn is taken out in integers, so
+// the angle y is at most pi/4 and good to 2^-24 of itself; sin y and cos y are
+// their Taylor polynomials (truncation below 2^-25 there).  Half as long again
+// as cis_neg, whose SFU approximations are only good to about 2^-22: used where
+// one value feeds many products.
+__device__ __forceinline__ cf2 cis_neg_accurate(uint32_t t) {
+    t += 1u << 29;
+    const float y = (float)(int32_t)((t << 2) ^ 0x80000000u) * (6.283185307179586f / 17179869184.0f);
+    const float y2 = y * y;
+    float sn = fmaf(y2, 2.7557319e-6f, -1.9841270e-4f);
+    sn = fmaf(sn, y2, 8.3333333e-3f);
+    sn = fmaf(sn, y2, -1.6666667e-1f);
+    sn = fmaf(sn * y2, y, y);
+    float cs = fmaf(y2, -2.7557319e-7f, 2.4801587e-5f);
+    cs = fmaf(cs, y2, -1.3888889e-3f);
+    cs = fmaf(cs, y2, 4.1666667e-2f);
+    cs = fmaf(cs, y2, -0.5f);
+    cs = fmaf(cs, y2, 1.0f);
+    // exp(-i (q pi/2 + y)) = (-i)^q (cs - i sn), q the top two bits
+    const bool odd = t & 0x40000000u;
+    const uint32_t neg = t & 0x80000000u;
+    const float x = odd ? -sn : cs, z = odd ? cs : sn;
+    return {__uint_as_float(__float_as_uint(x) ^ neg), __uint_as_float(__float_as_uint(z) ^ neg ^ 0x80000000u)};
+}
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
@@ -118,6 +149,18 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     return ok != 0;
 }
 
+// Non-blocking test of a phase (acquire).
+__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
@@ -131,21 +174,33 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t by
 // Bounded wait: gives up after `limit` polls or when another role of the CTA
 // has already given up (*abort != 0); on give-up sets the device status and
 // the CTA's abort flag.  Returns true when the phase completed.  sleep_ns > 0
-// backs off between polls (for long waits, so that waiting warps leave the
-// issue slots to working ones); the poll bound is then limit / 16.
+// backs off between polls (so that waiting warps leave the issue slots to
+// working ones); the poll bound is then limit / 16.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64_t limit,
                                           volatile int* abort, int* status, unsigned sleep_ns = 0) {
-    uint64_t it = 0;
-    const uint64_t lim = sleep_ns ? (limit >> 4 ? limit >> 4 : 1) : limit;
-    while (!mbar_try_wait(bar, parity)) {
-        if (++it >= lim || *abort) {
-            *abort = 1;
-            atomicOr(status, DEV_TIMEOUT);
-            return false;
-        }
+    if (mbar_try_wait(bar, parity)) return true;
+    const uint64_t lim64 = sleep_ns ? (limit >> 4 ? limit >> 4 : 1) : limit;
+    const uint32_t lim = lim64 < 0xffffffffull ? (uint32_t)lim64 : 0xffffffffu;
+    uint32_t it = 1;  // the try above was the first poll
+    while (it < lim && !*abort) {
         if (sleep_ns) __nanosleep(sleep_ns);
+        if (mbar_try_wait(bar, parity)) return true;
+        ++it;
     }
-    return true;
+    *abort = 1;
+    atomicOr(status, DEV_TIMEOUT);
+    return false;
+}
+
+// The same with non-blocking polls, for waits off the hot path (a try_wait
+// sleeps between its own tests, so that a poll can last microseconds).
+__device__ __forceinline__ bool mbar_poll(uint64_t* bar, uint32_t parity, uint64_t limit, volatile int* abort,
+                                          int* status) {
+    for (uint64_t it = 0; it < limit && !*abort; ++it)
+        if (mbar_test_wait(bar, parity)) return true;
+    *abort = 1;
+    atomicOr(status, DEV_TIMEOUT);
+    return false;
 }
 
 // Bound for the end-of-kernel waits on the CTA's own in-flight tensor-core
@@ -171,6 +226,18 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 // Make generic-proxy shared-memory writes visible to the async proxy (tensor core).
 __device__ __forceinline__ void fence_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+
+// Registers per thread of the calling warpgroup (four warps, all of them
+// call).  The shares of a block's warpgroups must not exceed the registers
+// that it was launched with.
+template <int REGS>
+__device__ __forceinline__ void regs_inc() {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS));
+}
+template <int REGS>
+__device__ __forceinline__ void regs_dec() {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS));
 }
 
 // ---------------------------------------------------------------------------
@@ -275,6 +342,64 @@ __device__ __forceinline__ void umma6_stage_elect(uint32_t dt, uint32_t ah, uint
         "r"(ah), "r"(al), "r"(bh), "r"(bl), "r"(hia), "r"(hib), "r"(ka), "r"(kb), "r"(idesc), "r"(acc), "r"(1u));
 }
 
+// The MMAs of one folded-forward stage (two K steps of 16) in one block, whole-warp
+// form (elect.sync picks the issuing lane, as in umma_f16_elect): the
+// correction products lo x hi, and hi x lo followed by the main product
+// hi x hi, which share their A tile through the collector buffer.  The
+// corrections come first: the accumulation then holds fewer roundings at full
+// magnitude.  Each descriptor is assembled from its low word (start address
+// field already moved to the stage's slot; ka / kb move it to the second K
+// step) and the high word it shares with its operand's other planes.
+// acc = 0 starts a fresh accumulation with the first MMA.
+__device__ __forceinline__ void umma6_fold_elect(uint32_t dt, uint32_t ah, uint32_t al, uint32_t bh, uint32_t bl,
+                                                  uint32_t hia, uint32_t hib, uint32_t ka, uint32_t kb,
+                                                  uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n .reg .pred p, one, e;\n .reg .b64 d0, d1, d2, d3, d4, d5, d6, d7;\n .reg .b32 t0, t1, t2, t3;\n"
+        " setp.ne.b32 p, %10, 0;\n setp.ne.b32 one, %11, 0;\n"
+        " elect.sync _|e, 0xffffffff;\n"
+        " mov.b64 d0, {%1, %5};\n mov.b64 d1, {%2, %5};\n mov.b64 d2, {%3, %6};\n mov.b64 d3, {%4, %6};\n"
+        " add.u32 t0, %1, %7;\n add.u32 t1, %2, %7;\n add.u32 t2, %3, %8;\n add.u32 t3, %4, %8;\n"
+        " mov.b64 d4, {t0, %5};\n mov.b64 d5, {t1, %5};\n mov.b64 d6, {t2, %6};\n mov.b64 d7, {t3, %6};\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], d1, d2, %9, p;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], d5, d6, %9, one;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%0], d0, d3, %9, one;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%0], d0, d2, %9, one;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%0], d4, d7, %9, one;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%0], d4, d6, %9, one;\n}\n" ::"r"(dt),
+        "r"(ah), "r"(al), "r"(bh), "r"(bl), "r"(hia), "r"(hib), "r"(ka), "r"(kb), "r"(idesc), "r"(acc), "r"(1u));
+}
+
+// The stage's four correction products only, and its two main products only
+// (for an accumulation that issues all of its corrections first).
+__device__ __forceinline__ void umma_corrections_elect(uint32_t dt, uint32_t ah, uint32_t al, uint32_t bh,
+                                                       uint32_t bl, uint32_t hia, uint32_t hib, uint32_t ka,
+                                                       uint32_t kb, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n .reg .pred p, one, e;\n .reg .b64 d0, d1, d2, d3, d4, d5, d6, d7;\n .reg .b32 t0, t1, t2, t3;\n"
+        " setp.ne.b32 p, %10, 0;\n setp.ne.b32 one, %11, 0;\n"
+        " elect.sync _|e, 0xffffffff;\n"
+        " mov.b64 d0, {%1, %5};\n mov.b64 d1, {%2, %5};\n mov.b64 d2, {%3, %6};\n mov.b64 d3, {%4, %6};\n"
+        " add.u32 t0, %1, %7;\n add.u32 t1, %2, %7;\n add.u32 t2, %3, %8;\n add.u32 t3, %4, %8;\n"
+        " mov.b64 d4, {t0, %5};\n mov.b64 d5, {t1, %5};\n mov.b64 d6, {t2, %6};\n mov.b64 d7, {t3, %6};\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], d1, d2, %9, p;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], d5, d6, %9, one;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], d0, d3, %9, one;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], d4, d7, %9, one;\n}\n" ::"r"(dt),
+        "r"(ah), "r"(al), "r"(bh), "r"(bl), "r"(hia), "r"(hib), "r"(ka), "r"(kb), "r"(idesc), "r"(acc), "r"(1u));
+}
+__device__ __forceinline__ void umma_main_elect(uint32_t dt, uint32_t ah, uint32_t bh, uint32_t hia, uint32_t hib,
+                                                uint32_t ka, uint32_t kb, uint32_t idesc) {
+    asm volatile(
+        "{\n .reg .pred one, e;\n .reg .b64 d0, d2, d4, d6;\n .reg .b32 t0, t2;\n"
+        " setp.ne.b32 one, %8, 0;\n elect.sync _|e, 0xffffffff;\n"
+        " mov.b64 d0, {%1, %3};\n mov.b64 d2, {%2, %4};\n"
+        " add.u32 t0, %1, %5;\n add.u32 t2, %2, %6;\n mov.b64 d4, {t0, %3};\n mov.b64 d6, {t2, %4};\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], d0, d2, %7, one;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], d4, d6, %7, one;\n}\n" ::"r"(dt),
+        "r"(ah), "r"(bh), "r"(hia), "r"(hib), "r"(ka), "r"(kb), "r"(idesc), "r"(1u));
+}
+
 // 32 lanes x 16 consecutive 32-bit columns; thread i of the warp gets lane
 // (warp's lane quarter base + i).
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
@@ -286,10 +411,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
           "=r"(r[14]), "=r"(r[15])
         : "r"(taddr));
 }
-__device__ __forceinline__ void tmem_ld_wait() {
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
 // Wait for outstanding TMEM loads and tie the given destination registers to
 // the wait, so that no use of them can be scheduled before it.
 __device__ __forceinline__ void tmem_ld_wait(uint32_t* r) {
@@ -319,10 +440,6 @@ __host__ __device__ constexpr uint32_t idesc_f16kind(int M, int N, int a_mn_majo
     return (1u << 4) | ((uint32_t)bf16 << 7) | ((uint32_t)bf16 << 10) | ((uint32_t)a_mn_major << 15) |
            ((uint32_t)b_mn_major << 16) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, int a_mn_major, int b_mn_major) {
-    return idesc_f16kind(M, N, a_mn_major, b_mn_major, 1);
-}
-
 // Split x into f16 hi + lo with x ~= hi + lo (|x - hi - lo| <~ 2^-22 |x| in the
 // normal range; callers scale operands so that they stay in range).
 __device__ __forceinline__ void split_f16x2(float a, float b, uint32_t& hi, uint32_t& lo) {
@@ -359,8 +476,8 @@ __device__ __forceinline__ void split16x2(float a, float b, uint32_t& hi, uint32
 
 // ---------------------------------------------------------------------------
 // Packed FP32x2 forms (sm_100 and later) of the table arithmetic above.
-// Results are bit-identical to cmul / split16x2: every component sees the
-// same roundings in the same order, two lanes per instruction.
+// Every component sees the roundings of cmul / split16x2 in the same order,
+// two lanes per instruction.
 // ---------------------------------------------------------------------------
 
 // Eight rotation factors w_0..w_7 in planar pairs: x[p] = (Re w_2p, Re w_2p+1),
@@ -392,6 +509,28 @@ __device__ __forceinline__ void rotate8(cf2 base, const Rot8& w, float2 (&re)[4]
     }
 }
 
+// The factors exp(-2 pi i q p / 2^64), q = 0..7, and step8 = that of q = 8:
+// the powers of two to FP32 rounding, the others by one product each.
+__device__ __forceinline__ Rot8 rot8_steps(uint64_t p, cf2& step8) {
+    cf2 w[8];
+    w[0] = {1.f, 0.f};
+    w[1] = cis_neg_accurate((uint32_t)(p >> 32));
+    w[2] = cis_neg_accurate((uint32_t)((2 * p) >> 32));
+    w[4] = cis_neg_accurate((uint32_t)((4 * p) >> 32));
+    step8 = cis_neg_accurate((uint32_t)((8 * p) >> 32));
+    w[3] = cmul(w[2], w[1]);
+    w[5] = cmul(w[4], w[1]);
+    w[6] = cmul(w[4], w[2]);
+    w[7] = cmul(step8, cf2{w[1].x, -w[1].y});
+    Rot8 r;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        r.x[q] = make_float2(w[2 * q].x, w[2 * q + 1].x);
+        r.y[q] = make_float2(w[2 * q].y, w[2 * q + 1].y);
+    }
+    return r;
+}
+
 // split16x2 of the pair v = (a, b): the residual a - hi, b - hi in one
 // packed subtraction.
 template <bool F16>
@@ -399,13 +538,13 @@ __device__ __forceinline__ void split16x2p(float2 v, uint32_t& hi, uint32_t& lo)
     if (F16) {
         const __half2 h = __float22half2_rn(v);
         const float2 hf = __half22float2(h);
-        const __half2 l = __float22half2_rn(__fadd2_rn(v, make_float2(-hf.x, -hf.y)));
+        const __half2 l = __float22half2_rn(__ffma2_rn(hf, make_float2(-1.f, -1.f), v));
         hi = *reinterpret_cast<const uint32_t*>(&h);
         lo = *reinterpret_cast<const uint32_t*>(&l);
     } else {
         const __nv_bfloat162 h = __float22bfloat162_rn(v);
         const float2 hf = __bfloat1622float2(h);
-        const __nv_bfloat162 l = __float22bfloat162_rn(__fadd2_rn(v, make_float2(-hf.x, -hf.y)));
+        const __nv_bfloat162 l = __float22bfloat162_rn(__ffma2_rn(hf, make_float2(-1.f, -1.f), v));
         hi = *reinterpret_cast<const uint32_t*>(&h);
         lo = *reinterpret_cast<const uint32_t*>(&l);
     }
@@ -426,6 +565,19 @@ __device__ __forceinline__ void table8_split(cf2 base, const Rot8& w, uint4& rh,
     split16x2p<F16>(im[1], ih.y, il.y);
     split16x2p<F16>(im[2], ih.z, il.z);
     split16x2p<F16>(im[3], ih.w, il.w);
+}
+
+// Eight real table entries p Re w_q + r Im w_q (q = 0..7; p and r hold their
+// value twice) split into the two 16-byte operand rows of one 8-element group.
+template <bool F16>
+__device__ __forceinline__ void table8_real(float2 p, float2 r, const Rot8& w, uint4& h, uint4& l) {
+    float2 v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = __ffma2_rn(p, w.x[q], __fmul2_rn(r, w.y[q]));
+    split16x2p<F16>(v[0], h.x, l.x);
+    split16x2p<F16>(v[1], h.y, l.y);
+    split16x2p<F16>(v[2], h.z, l.z);
+    split16x2p<F16>(v[3], h.w, l.w);
 }
 
 }  // namespace msk

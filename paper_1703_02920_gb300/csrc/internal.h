@@ -9,8 +9,8 @@ namespace msk {
 // Device status word bits (the host maps them to mem_status).
 enum : int { DEV_OK = 0, DEV_TIMEOUT = 1, DEV_BADARG = 2 };
 
-// Consecutive visibilities of one channel (the forward kernels' unit: 128 for
-// the direct forms, TC_TILE for the tensor-core form).
+// Consecutive visibilities of one channel (the forward kernels' unit: at most
+// VIS_TILE, or TC_TILE).
 struct VisTile {
     int32_t chan;
     int32_t count;
@@ -62,7 +62,7 @@ struct ImgSrc {
     int diff;             // operand is max(I + alpha d, G) - I, entropy as a difference
 };
 
-enum BFormat { BF_F32 = 0, BF_F64 = 1, BF_BF16X3 = 2, BF_F16X3 = 3 };
+enum BFormat { BF_F32 = 0, BF_F64 = 1 };
 // FWD_VIS: write V.  FWD_RESID: write y = w (V - V^o), chi^2 partials.
 // FWD_CHI: chi^2 partials only.  FWD_CURV: 1/2 w |V|^2 partials.
 // FWD_DCHI: chi^2 change for an operand that is an image difference delta,
@@ -70,11 +70,17 @@ enum BFormat { BF_F32 = 0, BF_F64 = 1, BF_BF16X3 = 2, BF_F16X3 = 3 };
 //   image read from the y buffer.
 enum FwdMode { FWD_VIS = 0, FWD_RESID = 1, FWD_CHI = 2, FWD_CURV = 3, FWD_DCHI = 4 };
 
-// Forward tensor-core tiling: 64 visibilities per tile, image column block
-// width BN and image rows per pipeline stage.
-constexpr int TC_BK = 32;
+// Visibilities per tile of the direct and the folded forward (VIS_TILE) and of
+// the BF16X3 forward (TC_TILE), operand rows per tensor-core pipeline stage,
+// and default column block.
+constexpr int VIS_TILE = 128;
 constexpr int TC_TILE = 64;
+constexpr int TC_BK = 32;
 __host__ __device__ inline int tc_bn(int N) { return N < 256 ? N : 256; }
+constexpr int MEAN_L = 16;  // folded columns l that share the operand's means
+// First column (P) of folded column l within a part: groups of eight P columns
+// followed by the eight Q columns of the same l (Q = P + 8).
+__host__ __device__ inline int fold_col(int l) { return 16 * (l / 8) + l % 8; }
 // Adjoint tensor-core tiling: output block side and visibilities per stage.
 constexpr int TCA_BK = 16;
 inline int tca_blk(int N) { return N < 256 ? N : 256; }
@@ -86,21 +92,28 @@ void set_global_error(const char* msg);
 void launch_phase_prep(int64_t Z, const double* u, const double* v, double dx, double dy,
                        uint64_t* pa, uint64_t* pb, cudaStream_t st);
 
-// B_c = A_c * img(c) for every channel in the requested format; entropy
-// partials S_i per (image, block) when ent_part != nullptr.  The tensor-core
-// formats hold B - c_m (c_m the column mean from launch_colmean); F16X3 also
-// scales each channel by cscale[c] (a power of two, from launch_colmean).
-void launch_prep(const DevData& d, const ImgSrc& src, int fmt, void* bout, double* ent_part,
-                 const float* cmean, const float* cscale, cudaStream_t st);
-// Column means of B_c per channel into cmean[C][N] and the channel's FP16X3
-// operand scale into cscale[C] (from the bound max_m (max_n |B| + |c_m|)).
-// psum (double) and pmax (float) hold colmean_tmp_count(N, C) entries each;
-// count holds C completion counters, zero between calls (each call leaves
-// them zero).  ymax_clear (nullable) is set to zero.
-void launch_colmean(const DevData& d, const ImgSrc& src, float* cmean, float* cscale, double* psum, float* pmax,
-                    unsigned* count, float* ymax_clear, cudaStream_t st);
+// B_c = A_c * img(c) for every channel (direct forms); entropy partials S_i
+// per (image, block of 256 pixels) when ent_part != nullptr.
+void launch_prep(const DevData& d, const ImgSrc& src, int fmt, void* bout, double* ent_part, cudaStream_t st);
+// Tensor-core forms: the means that centre the operand.  fold = 0 (BF16X3): of
+// every column of B_c, cmean[C][N].  fold = 1 (FP16X3): of the folded operand
+// over all rows j and MEAN_L neighbouring l, (P, Q) pairs
+// cmean[C][2 parts][N/2/MEAN_L][2], and the channel's operand scale cscale[C]
+// (a power of two, from a bound on the folded operand).  psum (double) and pmax
+// (float) hold colmean_tmp_count(N, C) entries each; count holds C completion
+// counters, zero between calls (each call leaves them zero).  ymax_clear
+// (nullable) is set to zero.  ent_part (nullable): tc_ent_blocks(N) entropy
+// partials per image.
+void launch_colmean(const DevData& d, const ImgSrc& src, int fold, float* cmean, float* cscale, double* psum,
+                    float* pmax, unsigned* count, float* ymax_clear, double* ent_part, cudaStream_t st);
 int colmean_tmp_count(int N, int C);
-__host__ __device__ inline int colmean_blocks(int N) { return (N + 31) / 32; }
+constexpr int COL_RB = 16;  // row blocks of the column sums
+__host__ __device__ inline int tc_ent_blocks(int N) { return (N + 31) / 32 * COL_RB; }
+// The centred operand split into 16-bit hi and lo planes in the forward
+// kernel's chunk layout: FP16X3 (folded, scaled by cscale) and BF16X3.
+void launch_fold(const DevData& d, const ImgSrc& src, void* planes, const float* cmean, const float* cscale,
+                 cudaStream_t st);
+void launch_planes(const DevData& d, const ImgSrc& src, void* planes, const float* cmean, cudaStream_t st);
 // max |component| of n floats into ymax[0]; the FP16X3 adjoint scales y by
 // pow2_scale_for(ymax[0]).  The forward writes the same maximum of the y it
 // produces (RESID mode) when given ymax (zeroed before).
@@ -115,13 +128,30 @@ void launch_adj_direct(const DevData& d, int fp64, const void* y, double* gsum, 
 int adj_direct_splits(const DevData& d, int num_sms);
 
 // Tensor-core forms.
+// FP16X3 forward on the folded image: operand streamed (any N) or resident (N <=
+// 256).  For fold_combines(N) the resident form splits every tile over two
+// CTAs, whose partial sums (vpart, two float4 per visibility) a second kernel
+// adds.  Planes scaled by cscale[c].  ymax (nullable, RESID mode): max
+// |component| of the weighted residual written to yout is combined into ymax[0]
+// (which the caller zeroes).  Returns the number of kernels launched.
+int fold_smem_bytes(int N, int BN, int stages, int resident);
+bool fold_combines(int N);
+int launch_fwd_fold(const DevData& d, int resident, const VisTile* tiles, int n_tiles, const void* planes,
+                    const float* cmean, const float* cscale, int mode, float2* yout, double* chi_part, float* ymax,
+                    float4* vpart, int64_t z_total, int num_sms, uint64_t spin, int* status, cudaStream_t st);
+// BF16X3 forward, streamed operand (TC_TILE tiles).
 int fwd_tc_smem_bytes(int N, int BN, int stages);
-// Resident-operand forward (N <= 256): the image rows are cut into slices of
-// fwd_rs_ks(N); each CTA keeps one slice of the operand planes in shared
-// memory; slice partials (FP64, [slice][visibility]) are combined by a second
-// kernel that also applies the forward mode.
+void launch_fwd_tc(const DevData& d, const VisTile* tiles, int n_tiles, const void* planes, const float* cmean,
+                   int mode, float2* yout, double* chi_part, int grid, uint64_t spin, int* status, cudaStream_t st);
+// BF16X3 forward, resident operand (N <= 256): the image rows are cut into
+// slices of fwd_rs_ks(N); each CTA keeps one slice of the operand planes in
+// shared memory; slice partials (FP64, [slice][visibility]) are combined by a
+// second kernel that also applies the forward mode.
 __host__ __device__ inline int fwd_rs_ks(int N) { return N < 128 ? N : 128; }
 int fwd_rs_smem_bytes(int N, int stages);
+void launch_fwd_rs(const DevData& d, const VisTile* tiles, int n_tiles, const void* planes, const float* cmean,
+                   int mode, float2* yout, double* chi_part, double2* vpart, int64_t z_total, int num_sms,
+                   uint64_t spin, int* status, cudaStream_t st);
 // The paper's gridded forward: the 2-D real-to-complex transform of every
 // channel's A_c * I zero-padded to M x M (image centred), as this library's
 // own FFT kernels (rows into R[C][M/2+1][N], columns into F[C][M][M/2+1]),
@@ -136,17 +166,6 @@ void launch_dirty_y(const DevData& d, const double* wsum, int what, int64_t z_to
                     cudaStream_t st);
 void launch_dirty_out(const DevData& d, const double* gsum, int ks, float* out, cudaStream_t st);
 void launch_grid_interp(const DevData& d, int M, const float2* F, int64_t z_total, float2* vis, cudaStream_t st);
-int fwd_rs_max_stages(int N);
-void launch_fwd_rs(const DevData& d, int f16, const VisTile* tiles, int n_tiles, const void* planes,
-                   const float* cmean, const float* cscale, int mode, float2* yout, double* chi_part,
-                   float* ymax, double2* vpart, int64_t z_total, int num_sms, uint64_t spin, int* status,
-                   cudaStream_t st);
-// f16 = 1: FP16X3 operands (planes scaled by cscale[c]); 0: BF16X3.
-// ymax (nullable, RESID mode): max |component| of the weighted residual
-// written to yout is combined into ymax[0] (which the caller zeroes).
-void launch_fwd_tc(const DevData& d, int f16, const VisTile* tiles, int n_tiles, const void* planes,
-                   const float* cmean, const float* cscale, int mode, float2* yout, double* chi_part,
-                   float* ymax, int grid, uint64_t spin, int* status, cudaStream_t st);
 int adj_tc_smem_bytes(int N, int stages);
 // units sorted by CTA: CTA b runs units [cta_unit_off[b], cta_unit_off[b+1]).
 // f16 = 1: FP16X3 with y scaled by pow2_scale_for(ymax[0]) (partials carry the scale).
@@ -172,6 +191,7 @@ struct ScalarArgs {
     const double* chi_part = nullptr;
     const double* ent_part = nullptr;
     int with_entropy = 0;
+    int n_ent = 0;  // entropy partials per image
     double* scal = nullptr;
     double* img_tmp = nullptr;
 };
@@ -186,10 +206,11 @@ void launch_adj_tc_reduce_grad(const DevData& d, const ImgSrc& src, const int* c
 void launch_finalize(const DevData& d, const ImgSrc& src, const double* gsum, int ks, int projected,
                      float* out32, double* full64, double* proj64, cudaStream_t st);
 
-// chi_part holds 4 partials per visibility tile (one per 32 visibilities).
+// chi_part holds 4 partials per visibility tile (one per 32 visibilities),
+// ent_part n_ent entropy partials per image.
 // Per-image chi^2 / S / Phi into scal[3 + 3 i ...] and totals into scal[0..2].
 void launch_scalars(const DevData& d, const int* tile_off, const double* chi_part,
-                    const double* ent_part, int with_entropy, double* scal, double* img_tmp,
+                    const double* ent_part, int with_entropy, int n_ent, double* scal, double* img_tmp,
                     cudaStream_t st);
 int scalars_tmp_doubles(int n_images);
 

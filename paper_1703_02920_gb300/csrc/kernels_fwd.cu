@@ -1,7 +1,10 @@
-// Tensor-core forward operator (Eq. 1 on the pixel grid) with the fused
-// per-visibility reduction, residual, weight and chi^2 partials.
+// Tensor-core forward operator of the BF16X3 form (Eq. 1 on the pixel grid),
+// operand streamed, with the fused per-visibility reduction, residual, weight
+// and chi^2 partials.  (FP16X3 contracts the folded image, kernels_fold.cu.
+// BF16X3 does not: its 8 + 8-bit splits leave errors up to 3e-5 of the residual
+// at a good model, so that other products change its results by as much.)
 //
-//   T = Ey B^T  (tcgen05.mma kind::f16, 3-term FP16 or BF16 split, FP32 accumulation)
+//   T = Ey B^T  (tcgen05.mma kind::f16, 3-term BF16 split, FP32 accumulation)
 //   V_k = sum_m Ex[k,m] T[k,m]
 //
 // The image operand is centred column by column, B'[n][m] = B[n][m] - c_m
@@ -69,15 +72,12 @@ struct F2Shared {
     int abort;
 };
 
-// F16: FP16X3 operands (the image planes are scaled by cscale[channel], a
-// power of two undone in the epilogue); otherwise BF16X3.
 // F2_STAGES: depth of the shared-memory pipeline (autotuned).
-template <bool F16, int F2_STAGES>
+template <int F2_STAGES>
 __global__ void __launch_bounds__(F2_THREADS, 1)
     k_fwd_tc(DevData d, const VisTile* __restrict__ tiles, int n_tiles,
              const uint16_t* __restrict__ planes, const float* __restrict__ cmean,
-             const float* __restrict__ cscale, int mode, float2* __restrict__ yout,
-             double* __restrict__ chi_part, unsigned* __restrict__ ymax_bits, uint64_t spin, int* status) {
+             int mode, float2* __restrict__ yout, double* __restrict__ chi_part, uint64_t spin, int* status) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ F2Shared S;
     const int N = d.N, c0 = N / 2;
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(F2_THREADS, 1)
         // is made warp-uniform), and one elected lane issues the MMAs and
         // commits.
         {
-            const uint32_t idesc = idesc_f16kind(128, BN, 0, 0, F16 ? 0 : 1);
+            const uint32_t idesc = idesc_f16kind(128, BN, 0, 0, 1);
             const uint32_t sbase = smem_u32(smem);
             const uint32_t lboB = (uint32_t)(BN / 8) * 128;
             // Operand descriptors of slot 0; another slot or K step only moves
@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(F2_THREADS, 1)
                     if (valid) {
                         const int n0 = ks * TC_BK + g * 8;
                         base = (ks % PHASE_REFRESH) ? cmul(base, step_bk) : cis_neg(phase_mul(n0 - c0, pb));
-                        table8_split<F16>(base, w, rh, rl, ih, il);
+                        table8_split<false>(base, w, rh, rl, ih, il);
                     }
                     ok = __all_sync(0xffffffffu, mbar_wait(&S.empty[s], ((sc / F2_STAGES) & 1) ^ 1, spin,
                                                            abort, status, 64));
@@ -323,8 +323,6 @@ __global__ void __launch_bounds__(F2_THREADS, 1)
                 const float D = (sh != 0.f) ? snb / sh : (float)N;
                 scomp = comp ? sh * D : ch * D;
             }
-            const float osc = F16 ? cscale[tl.chan] : 1.f;  // operand scale (power of two)
-            scomp *= osc;
             float s0 = 0.f, s1 = 0.f, c0s = 0.f, c1s = 0.f;  // compensated sums
             for (int u = 0; u < n_mb * n_seg; ++u, ++it) {
                 const int mb = u / n_seg;
@@ -393,16 +391,14 @@ __global__ void __launch_bounds__(F2_THREADS, 1)
             if (!ok) break;
             if (t + (int)gridDim.x < n_tiles) load_phases(tl_next);
             // lane < 16: (sum ReEx ReT, sum ImEx ReT); lane >= 16: (sum ReEx ImT, sum ImEx ImT),
-            // each a compensated (hi, lo) pair, unscaled exactly (a power of two).
+            // each a compensated (hi, lo) pair.
             // The tail runs in FP32 pair arithmetic: the residual V - V° is an
             // exact pair difference, and chi^2 per visibility needs only FP32
             // relative accuracy (the partials are summed in FP64).
-            const float inv = 1.f / osc;
-            const float p0h = s0 * inv, p0l = c0s * inv, p1h = s1 * inv, p1l = c1s * inv;
+            const float p0h = s0, p0l = c0s, p1h = s1, p1l = c1s;
             const float q0h = __shfl_xor_sync(0xffffffffu, p0h, 16), q0l = __shfl_xor_sync(0xffffffffu, p0l, 16);
             const float q1h = __shfl_xor_sync(0xffffffffu, p1h, 16), q1l = __shfl_xor_sync(0xffffffffu, p1l, 16);
             float chi = 0.f;
-            float ym = 0.f;  // max |component| of the weighted residual (RESID mode)
             if (valid && comp == 0) {
                 const float2 vre = df_add(p0h, p0l, -q1h, -q1l);  // ReEx ReT - ImEx ImT
                 const float2 vim = df_add(q0h, q0l, p1h, p1l);    // ReEx ImT + ImEx ReT
@@ -426,15 +422,8 @@ __global__ void __launch_bounds__(F2_THREADS, 1)
                     if (mode == FWD_RESID) {
                         const float2 yv = make_float2(w * rr, w * ri);
                         yout[j] = yv;
-                        ym = fmaxf(fabsf(yv.x), fabsf(yv.y));
                     }
                 }
-            }
-            if (mode == FWD_RESID && ymax_bits) {
-                // order-independent maximum (non-negative floats order as their bits)
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) ym = fmaxf(ym, __shfl_down_sync(0xffffffffu, ym, o));
-                if (lane == 0) atomicMax(ymax_bits, __float_as_uint(ym));
             }
             if (mode != FWD_VIS) {
                 // one partial per warp (16 visibilities), summed later in a fixed order
@@ -458,31 +447,23 @@ __global__ void __launch_bounds__(F2_THREADS, 1)
 // stage ring + the epilogue warps' column-mean copies (4 x N floats) + alignment
 int fwd_tc_smem_bytes(int N, int BN, int stages) { return stages * f2_stage_bytes(BN) + 16 * N + 1024; }
 
-template <bool F16, int STAGES>
+template <int STAGES>
 static void launch_fwd_variant(const DevData& d, const VisTile* tiles, int n_tiles, const void* planes,
-                               const float* cmean, const float* cscale, int mode, float2* yout,
-                               double* chi_part, unsigned* ymax_bits, int grid, uint64_t spin, int* status,
-                               cudaStream_t st) {
+                               const float* cmean, int mode, float2* yout, double* chi_part, int grid,
+                               uint64_t spin, int* status, cudaStream_t st) {
     const int smem = fwd_tc_smem_bytes(d.N, d.fwd_bn, STAGES);
-    cudaFuncSetAttribute(k_fwd_tc<F16, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    k_fwd_tc<F16, STAGES><<<grid, F2_THREADS, smem, st>>>(d, tiles, n_tiles, (const uint16_t*)planes, cmean,
-                                                          cscale, mode, yout, chi_part, ymax_bits, spin, status);
+    cudaFuncSetAttribute(k_fwd_tc<STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    k_fwd_tc<STAGES><<<grid, F2_THREADS, smem, st>>>(d, tiles, n_tiles, (const uint16_t*)planes, cmean, mode, yout,
+                                                     chi_part, spin, status);
 }
 
-void launch_fwd_tc(const DevData& d, int f16, const VisTile* tiles, int n_tiles, const void* planes,
-                   const float* cmean, const float* cscale, int mode, float2* yout, double* chi_part,
-                   float* ymax, int grid, uint64_t spin, int* status, cudaStream_t st) {
-    unsigned* ymax_bits = (unsigned*)ymax;
+void launch_fwd_tc(const DevData& d, const VisTile* tiles, int n_tiles, const void* planes, const float* cmean,
+                   int mode, float2* yout, double* chi_part, int grid, uint64_t spin, int* status,
+                   cudaStream_t st) {
     if (n_tiles <= 0) return;
     if (grid > n_tiles) grid = n_tiles;
-    const bool s3 = d.fwd_stages == 3;
-    if (f16) {
-        if (s3) launch_fwd_variant<true, 3>(d, tiles, n_tiles, planes, cmean, cscale, mode, yout, chi_part, ymax_bits, grid, spin, status, st);
-        else launch_fwd_variant<true, 4>(d, tiles, n_tiles, planes, cmean, cscale, mode, yout, chi_part, ymax_bits, grid, spin, status, st);
-    } else {
-        if (s3) launch_fwd_variant<false, 3>(d, tiles, n_tiles, planes, cmean, cscale, mode, yout, chi_part, ymax_bits, grid, spin, status, st);
-        else launch_fwd_variant<false, 4>(d, tiles, n_tiles, planes, cmean, cscale, mode, yout, chi_part, ymax_bits, grid, spin, status, st);
-    }
+    if (d.fwd_stages == 3) launch_fwd_variant<3>(d, tiles, n_tiles, planes, cmean, mode, yout, chi_part, grid, spin, status, st);
+    else launch_fwd_variant<4>(d, tiles, n_tiles, planes, cmean, mode, yout, chi_part, grid, spin, status, st);
 }
 
 }  // namespace msk

@@ -1,5 +1,5 @@
-// Tensor-core forward operator (Eq. 1 on the pixel grid) for images of side
-// N <= 256, with the image operand resident in shared memory.
+// Tensor-core forward operator of the BF16X3 form (Eq. 1 on the pixel grid) for
+// images of side N <= 256, with the image operand resident in shared memory.
 //
 //   T_s = Ey[:, rows of slice s] B'[rows of slice s, :]^T   (tcgen05.mma kind::f16)
 //   V_k = sum_s sum_m Ex[k,m] T_s[k,m]  (+ c_m S_k from slice 0)
@@ -61,11 +61,10 @@ struct RsShared {
     int abort;
 };
 
-// F16: FP16X3 operands (planes scaled by cscale[channel]); else BF16X3.
-template <bool F16, int STAGES>
+template <int STAGES>
 __global__ void __launch_bounds__(RS_THREADS, 1)
     k_fwd_rs(DevData d, const VisTile* __restrict__ tiles, int n_tiles, const uint16_t* __restrict__ planes,
-             const float* __restrict__ cmean, const float* __restrict__ cscale, double2* __restrict__ vpart,
+             const float* __restrict__ cmean, double2* __restrict__ vpart,
              int64_t z_total, uint64_t spin, int* status) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ RsShared S;
@@ -111,7 +110,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
     if (warp == 4) {
         // ------------------------------------------ MMA + resident operand
         if (lane == 0) {
-            const uint32_t idesc = idesc_f16kind(128, N, 0, 0, F16 ? 0 : 1);
+            const uint32_t idesc = idesc_f16kind(128, N, 0, 0, 1);
             const uint32_t abase = smem_u32(sA), bbase = smem_u32(sB);
             const uint32_t lboB = (uint32_t)(N / 8) * 128;
             const uint32_t lo_off = (uint32_t)N * TC_BK * 2;  // lo plane within a chunk
@@ -205,7 +204,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
                     uint4 rh = {0, 0, 0, 0}, rl = {0, 0, 0, 0}, ih = {0, 0, 0, 0}, il = {0, 0, 0, 0};
                     if (valid) {
                         const int n0 = slice * KS + ks * TC_BK + g * 8;
-                        table8_split<F16>(cis_neg(phase_mul(n0 - c0, pb)), w, rh, rl, ih, il);
+                        table8_split<false>(cis_neg(phase_mul(n0 - c0, pb)), w, rh, rl, ih, il);
                     }
                     ok = __all_sync(0xffffffffu, mbar_wait(&S.empty[s], ((sc / STAGES) & 1) ^ 1, spin, abort,
                                                            status, 64));
@@ -252,8 +251,6 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
                 const float D = (sh != 0.f) ? snb / sh : (float)N;
                 scomp = comp ? sh * D : ch * D;
             }
-            const float osc = F16 ? cscale[tl.chan] : 1.f;  // operand scale (power of two)
-            scomp *= osc;
             const float* cm = cmean + (int64_t)tl.chan * N;
             float s0 = 0.f, s1 = 0.f, c0s = 0.f, c1s = 0.f;  // compensated sums
             const int b = it & 1;
@@ -307,8 +304,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
             __syncwarp();
             if (lane == 0) mbar_arrive(&S.tempty[b]);
             // lane < 16: (sum ReEx ReT, sum ImEx ReT); lane >= 16: (sum ReEx ImT, sum ImEx ImT)
-            const double inv = 1.0 / (double)osc;
-            const double p0 = ((double)s0 + (double)c0s) * inv, p1 = ((double)s1 + (double)c1s) * inv;
+            const double p0 = (double)s0 + (double)c0s, p1 = (double)s1 + (double)c1s;
             const double q0 = __shfl_xor_sync(0xffffffffu, p0, 16);
             const double q1 = __shfl_xor_sync(0xffffffffu, p1, 16);
             if (valid && comp == 0) vpart[(int64_t)slice * z_total + j] = make_double2(p0 - q1, q0 + p1);
@@ -329,13 +325,11 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
 // visibilities, the layout the scalar reduction reads (4 per tile).
 __global__ void __launch_bounds__(64) k_fwd_combine(DevData d, const VisTile* __restrict__ tiles,
                                                     const double2* __restrict__ vpart, int n_slices,
-                                                    int64_t z_total, int mode, float2* yout, double* chi_part,
-                                                    unsigned* ymax_bits) {
+                                                    int64_t z_total, int mode, float2* yout, double* chi_part) {
     const int t = blockIdx.x;
     const VisTile tl = tiles[t];
     const int jv = threadIdx.x;
     double chi = 0.0;
-    float ym = 0.f;  // max |component| of the weighted residual (RESID mode)
     if (jv < tl.count) {
         const int64_t j = tl.start + jv;
         double Vre = 0.0, Vim = 0.0;
@@ -360,15 +354,8 @@ __global__ void __launch_bounds__(64) k_fwd_combine(DevData d, const VisTile* __
             if (mode == FWD_RESID) {
                 const float2 yv = make_float2((float)(w * rr), (float)(w * ri));
                 yout[j] = yv;
-                ym = fmaxf(fabsf(yv.x), fabsf(yv.y));
             }
         }
-    }
-    if (mode == FWD_RESID && ymax_bits) {
-        // order-independent maximum (non-negative floats order as their bits)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ym = fmaxf(ym, __shfl_down_sync(0xffffffffu, ym, o));
-        if ((jv & 31) == 0) atomicMax(ymax_bits, __float_as_uint(ym));
     }
     if (mode != FWD_VIS) {
 #pragma unroll
@@ -377,49 +364,32 @@ __global__ void __launch_bounds__(64) k_fwd_combine(DevData d, const VisTile* __
     }
 }
 
-template <bool F16, int STAGES>
+template <int STAGES>
 void launch_rs_variant(const DevData& d, const VisTile* tiles, int n_tiles, const void* planes, const float* cmean,
-                       const float* cscale, double2* vpart, int64_t z_total, int grid, uint64_t spin, int* status,
-                       cudaStream_t st) {
+                       double2* vpart, int64_t z_total, int grid, uint64_t spin, int* status, cudaStream_t st) {
     const int smem = fwd_rs_smem_bytes(d.N, STAGES);
-    cudaFuncSetAttribute(k_fwd_rs<F16, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    k_fwd_rs<F16, STAGES><<<grid, RS_THREADS, smem, st>>>(d, tiles, n_tiles, (const uint16_t*)planes, cmean,
-                                                          cscale, vpart, z_total, spin, status);
+    cudaFuncSetAttribute(k_fwd_rs<STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    k_fwd_rs<STAGES><<<grid, RS_THREADS, smem, st>>>(d, tiles, n_tiles, (const uint16_t*)planes, cmean, vpart,
+                                                     z_total, spin, status);
 }
 
 }  // namespace
 
 int fwd_rs_smem_bytes(int N, int stages) { return fwd_rs_ks(N) * N * 4 + stages * RS_ABYTES + 1024; }
 
-int fwd_rs_max_stages(int N) {
-    int s = RS_MAX_STAGES;
-    while (s > 2 && fwd_rs_smem_bytes(N, s) > 227 * 1024) --s;
-    return s;
-}
-
-void launch_fwd_rs(const DevData& d, int f16, const VisTile* tiles, int n_tiles, const void* planes,
-                   const float* cmean, const float* cscale, int mode, float2* yout, double* chi_part,
-                   float* ymax, double2* vpart, int64_t z_total, int num_sms, uint64_t spin, int* status,
-                   cudaStream_t st) {
+void launch_fwd_rs(const DevData& d, const VisTile* tiles, int n_tiles, const void* planes, const float* cmean,
+                   int mode, float2* yout, double* chi_part, double2* vpart, int64_t z_total, int num_sms,
+                   uint64_t spin, int* status, cudaStream_t st) {
     if (n_tiles <= 0) return;
     const int n_slices = d.N / fwd_rs_ks(d.N);
     // CTAs per slice: one per SM, at most one per tile
     const int per = std::max(1, std::min(num_sms / n_slices, n_tiles));
     const int grid = per * n_slices;
     const int stages = d.fwd_stages;
-#define MSK_RS(F, S) launch_rs_variant<F, S>(d, tiles, n_tiles, planes, cmean, cscale, vpart, z_total, grid, spin, status, st)
-    if (f16) {
-        if (stages <= 4) MSK_RS(true, 4);
-        else if (stages == 5) MSK_RS(true, 5);
-        else MSK_RS(true, 6);
-    } else {
-        if (stages <= 4) MSK_RS(false, 4);
-        else if (stages == 5) MSK_RS(false, 5);
-        else MSK_RS(false, 6);
-    }
-#undef MSK_RS
-    k_fwd_combine<<<n_tiles, 64, 0, st>>>(d, tiles, vpart, n_slices, z_total, mode, yout, chi_part,
-                                          (unsigned*)ymax);
+    if (stages <= 4) launch_rs_variant<4>(d, tiles, n_tiles, planes, cmean, vpart, z_total, grid, spin, status, st);
+    else if (stages == 5) launch_rs_variant<5>(d, tiles, n_tiles, planes, cmean, vpart, z_total, grid, spin, status, st);
+    else launch_rs_variant<6>(d, tiles, n_tiles, planes, cmean, vpart, z_total, grid, spin, status, st);
+    k_fwd_combine<<<n_tiles, 64, 0, st>>>(d, tiles, vpart, n_slices, z_total, mode, yout, chi_part);
 }
 
 }  // namespace msk

@@ -53,34 +53,29 @@ __device__ __forceinline__ int image_of(const DevData& d, int c) { return d.shar
 
 
 // ---------------------------------------------------------------------------
-// a2: attenuation and operand preparation.  B_c = A_c * I.  The BF16x3 form
-// stores hi/lo planes pre-arranged in the tensor-core operand layout of the
-// forward kernel: per channel, chunks (m-block mb, n-stage ks) of BN x BK
-// elements, K-major interleaved 8x8 core matrices, hi plane then lo plane.
+// a2, tensor-core forms: attenuation, centring and splitting of the forward's
+// operand.  FP16X3 folds it first (the fold is defined in kernels_fold.cu).
+//
+// Two kernels.  k_colsum forms the column sums of B = A I over the lower and
+// the upper half of the rows, from which the means follow, and for FP16X3 the
+// channel's operand scale.  k_fold (FP16X3) or k_planes (BF16X3) writes the
+// centred, split planes.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int64_t tc_plane_index(int n, int m, int N, int BN) {
-    int nk = N / TC_BK;
-    int mb = m / BN, r = m % BN, ks = n / TC_BK, k = n % TC_BK;
-    int64_t chunk = (int64_t)mb * nk + ks;
-    int64_t chunk_elems = (int64_t)2 * BN * TC_BK;  // hi + lo
-    int64_t off = ((int64_t)(k / 8) * (BN / 8) + r / 8) * 64 + (r % 8) * 8 + (k % 8);
-    return chunk * chunk_elems + off;  // in bf16 elements; lo at + BN*BK
-}
 
-// Column means c_m = (1/N) sum_n B[n][m] per channel (the operand of the
-// tensor-core forward is centred column by column, see k_fwd_tc), in two
-// stages with a fixed summation order.  Stage 1: block (column block of 32,
-// row block rb of N/COL_RB rows, channel) -> partial sums and max |B| per
-// column.  Stage 2, run by the channel's last stage-1 block to finish (a
-// completion counter per channel, which that block resets): c_m, then the
-// bound max_n |B[n][m] - c_m| <= max|B| + |c_m| maximised over the channel,
-// and from it the channel's power-of-two FP16X3 operand scale.
-constexpr int COL_RB = 16;
-
+// Column sums in two stages with a fixed summation order.  Stage 1: block
+// (column block of 32, row block rb of N/COL_RB rows, channel) -> partial sums
+// and max |B| per column (row blocks below COL_RB/2 lie in the lower half).
+// Stage 2, run by the channel's last stage-1 block to finish (a completion
+// counter per channel, which that block resets): for BF16X3 the column means
+// c_m; for FP16X3 the folded operand's means over the rows and MEAN_L
+// neighbouring columns l, then the bound max |B'| <= 2 (max|B| of the column and
+// of its mirror) + |cm| maximised over the channel, and from it the channel's
+// power-of-two FP16X3 operand scale.
+template <bool FOLD>
 __global__ void __launch_bounds__(256) k_colsum(DevData d, ImgSrc src, double* __restrict__ psum,
                                                 float* __restrict__ pmax, unsigned* __restrict__ count,
                                                 float* __restrict__ cmean, float* __restrict__ cscale,
-                                                float* __restrict__ ymax_clear) {
+                                                float* __restrict__ ymax_clear, double* __restrict__ ent_part) {
     __shared__ double sh[8][33];
     __shared__ float shm[8][33];
     __shared__ bool last;
@@ -94,17 +89,34 @@ __global__ void __launch_bounds__(256) k_colsum(DevData d, ImgSrc src, double* _
     // the FP16X3 residual maximum of the forward that follows starts at zero
     if (ymax_clear && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) *ymax_clear = 0.f;
     const int n0 = (int)((int64_t)N * rb / COL_RB), n1 = (int)((int64_t)N * (rb + 1) / COL_RB);
-    double acc = 0.0;
+    // the entropy partial of an image is formed by its first channel only
+    // (the others would repeat it in the shared-image mode)
+    const bool ent = ent_part && !(d.shared && c != 0);
+    double acc = 0.0, e = 0.0;
     float amax = 0.f;
     if (m < N) {
         for (int n = n0 + rg; n < n1; n += 8) {
             const int64_t p = (int64_t)n * N + m;
             double x = img_value(src, i, p, NN);
-            if (src.diff) x -= src.f64[(int64_t)i * NN + p];
+            if (src.diff) {
+                // line-search probe as a difference from the base image I: the
+                // operand is delta = max(I + alpha d, G) - I, the entropy term
+                // the change of sum x log(x/G)
+                const double x0 = src.f64[(int64_t)i * NN + p];
+                if (ent) e += x * log(x / src.G) - x0 * log(x0 / src.G);
+                x -= x0;
+            } else if (ent) {
+                e += x * log(x / src.G);
+            }
             const double b = (double)d.beam[(int64_t)c * NN + p] * x;
             acc += b;
             amax = fmaxf(amax, (float)fabs(b));
         }
+    }
+    if (ent) {  // uniform over the block
+        const double s = block_sum<256>(e, &sh[0][0]);
+        if (threadIdx.x == 0)
+            ent_part[(int64_t)i * gridDim.x * gridDim.y + (int64_t)rb * gridDim.x + blockIdx.x] = -s;
     }
     sh[rg][lane] = acc;
     shm[rg][lane] = amax;
@@ -126,18 +138,50 @@ __global__ void __launch_bounds__(256) k_colsum(DevData d, ImgSrc src, double* _
     if (!last) return;
     __threadfence();
     // stage 2: the partials of channel c in row-block order (read through L2)
-    float bound = 0.f;
-    for (int mm = threadIdx.x; mm < N; mm += blockDim.x) {
-        double t = 0.0;
-        float mx = 0.f;
+    if (!FOLD) {
+        for (int mm = threadIdx.x; mm < N; mm += blockDim.x) {
+            double t = 0.0;
 #pragma unroll
-        for (int r = 0; r < COL_RB; ++r) {
-            t += __ldcg(psum + ((int64_t)c * COL_RB + r) * N + mm);
-            mx = fmaxf(mx, __ldcg(pmax + ((int64_t)c * COL_RB + r) * N + mm));
+            for (int r = 0; r < COL_RB; ++r) t += __ldcg(psum + ((int64_t)c * COL_RB + r) * N + mm);
+            cmean[(int64_t)c * N + mm] = (float)(t / N);
         }
-        const float cm = (float)(t / N);
-        cmean[(int64_t)c * N + mm] = cm;
-        bound = fmaxf(bound, mx + fabsf(cm));
+        if (threadIdx.x == 0) count[c] = 0;  // ready for the next evaluation
+        return;
+    }
+    // one thread per mirror pair of columns
+    float bound = 0.f;
+    const double inv = 2.0 / ((double)N * MEAN_L);
+    for (int l = threadIdx.x; l < N / 2; l += blockDim.x) {
+        double lo[2] = {0.0, 0.0}, up[2] = {0.0, 0.0};  // [column, mirror]: lower and upper rows
+        float mx[2] = {0.f, 0.f};
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int mm = h ? N / 2 - 1 - l : N / 2 + l;
+#pragma unroll
+            for (int r = 0; r < COL_RB; ++r) {
+                const double q = __ldcg(psum + ((int64_t)c * COL_RB + r) * N + mm);
+                if (r < COL_RB / 2) lo[h] += q;
+                else up[h] += q;
+                mx[h] = fmaxf(mx[h], __ldcg(pmax + ((int64_t)c * COL_RB + r) * N + mm));
+            }
+        }
+        // MEAN_L consecutive lanes hold one group (N/2 is a multiple of 32)
+        auto group_mean = [&](double x) {
+#pragma unroll
+            for (int o = MEAN_L / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            return (float)(x * inv);
+        };
+        const float ss = group_mean(up[0] + lo[0] + up[1] + lo[1]);
+        const float sa = group_mean(up[0] + lo[0] - up[1] - lo[1]);
+        const float as = group_mean(up[0] - lo[0] + up[1] - lo[1]);
+        const float aa = group_mean(up[0] - lo[0] - up[1] + lo[1]);
+        if (l % MEAN_L == 0) {
+            float2* cm = (float2*)cmean + (int64_t)c * (N / MEAN_L) + l / MEAN_L;
+            cm[0] = make_float2(ss, sa);
+            cm[N / 2 / MEAN_L] = make_float2(as, aa);
+        }
+        const float cmax = fmaxf(fmaxf(fabsf(ss), fabsf(sa)), fmaxf(fabsf(as), fabsf(aa)));
+        bound = fmaxf(bound, 2.f * (mx[0] + mx[1]) + cmax);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) bound = fmaxf(bound, __shfl_down_sync(0xffffffffu, bound, o));
@@ -151,13 +195,107 @@ __global__ void __launch_bounds__(256) k_colsum(DevData d, ImgSrc src, double* _
     }
 }
 
-void launch_colmean(const DevData& d, const ImgSrc& src, float* cmean, float* cscale, double* psum, float* pmax,
-                    unsigned* count, float* ymax_clear, cudaStream_t st) {
-    k_colsum<<<dim3(colmean_blocks(d.N), COL_RB, d.C), 256, 0, st>>>(d, src, psum, pmax, count, cmean, cscale,
-                                                                    ymax_clear);
+void launch_colmean(const DevData& d, const ImgSrc& src, int fold, float* cmean, float* cscale, double* psum,
+                    float* pmax, unsigned* count, float* ymax_clear, double* ent_part, cudaStream_t st) {
+    const dim3 grid((d.N + 31) / 32, COL_RB, d.C);
+    if (fold)
+        k_colsum<true><<<grid, 256, 0, st>>>(d, src, psum, pmax, count, cmean, cscale, ymax_clear, ent_part);
+    else
+        k_colsum<false><<<grid, 256, 0, st>>>(d, src, psum, pmax, count, cmean, cscale, ymax_clear, ent_part);
 }
 
 int colmean_tmp_count(int N, int C) { return COL_RB * N * C; }
+
+// One block folds 8 rows j by 32 columns l: thread (warp: j, lane: l) reads the
+// four mirror pixels (coalesced along the row, two of the reads reversed),
+// forms the four sums and splits them into a shared-memory tile whose 16-byte
+// rows (8 consecutive j of one column) are then stored, four whole core
+// matrices per column type.  Chunk layout of the planes: chunk (column block
+// mb, part, row stage ks) of BN columns x TC_BK rows, K-major interleaved 8 x 8
+// core matrices, hi plane then lo plane.
+__global__ void __launch_bounds__(256) k_fold(DevData d, ImgSrc src, uint16_t* __restrict__ planes,
+                                              const float* __restrict__ cmean, const float* __restrict__ cscale) {
+    __shared__ __align__(16) uint16_t sp[4][2][32][8];  // column type, hi / lo, l, j
+    const int N = d.N, M = N / 2, BN = d.fwd_bn, nk = M / TC_BK;
+    const int64_t NN = (int64_t)N * N;
+    const int c = blockIdx.z;
+    const int i = image_of(d, c);
+    const int jl = threadIdx.x >> 5, ll = threadIdx.x & 31;
+    const int j0 = blockIdx.y * 8, l0 = blockIdx.x * 32;
+    const int j = j0 + jl, l = l0 + ll;
+    const float* A = d.beam + (int64_t)c * NN;
+    auto pixel = [&](int n, int m) {
+        const int64_t p = (int64_t)n * N + m;
+        double x = img_value(src, i, p, NN);
+        if (src.diff) x -= src.f64[(int64_t)i * NN + p];
+        return (double)A[p] * x;
+    };
+    const double pp = pixel(M + j, M + l), pm = pixel(M + j, M - 1 - l);
+    const double mp = pixel(M - 1 - j, M + l), mm = pixel(M - 1 - j, M - 1 - l);
+    const double sp0 = pp + mp, sp1 = pm + mm, sm0 = pp - mp, sm1 = pm - mm;  // over the rows
+    const double f[4] = {sp0 + sp1, sp0 - sp1, sm0 + sm1, sm0 - sm1};        // ss, sa, as, aa
+    const float2* cm = (const float2*)cmean + (int64_t)c * (N / MEAN_L) + l / MEAN_L;
+    const float2 cs = cm[0], cy = cm[N / 2 / MEAN_L];
+    const float mean[4] = {cs.x, cs.y, cy.x, cy.y};
+    const double sc = (double)cscale[c];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float v = (float)((f[k] - (double)mean[k]) * sc);
+        uint32_t hi, lo;
+        split_f16x2(v, 0.f, hi, lo);
+        sp[k][0][ll][jl] = (uint16_t)hi;
+        sp[k][1][ll][jl] = (uint16_t)lo;
+    }
+    __syncthreads();
+    // thread -> one 16-byte row: column type, plane, l
+    const int k = threadIdx.x >> 6, pl = (threadIdx.x >> 5) & 1;
+    const int col = fold_col(l0 + ll) + (k & 1) * 8;
+    const int mb = col / BN, r = col % BN, ks = j0 / TC_BK, kk = j0 % TC_BK;
+    const int64_t chunk = (int64_t)(2 * mb + (k >> 1)) * nk + ks;
+    uint16_t* dst = planes + (int64_t)c * 2 * NN + chunk * 2 * BN * TC_BK + (int64_t)pl * BN * TC_BK +
+                    ((int64_t)(kk / 8) * (BN / 8) + r / 8) * 64 + (r % 8) * 8;
+    *(uint4*)dst = *(const uint4*)sp[k][pl][ll];
+}
+
+void launch_fold(const DevData& d, const ImgSrc& src, void* planes, const float* cmean, const float* cscale,
+                 cudaStream_t st) {
+    k_fold<<<dim3(d.N / 64, d.N / 16, d.C), 256, 0, st>>>(d, src, (uint16_t*)planes, cmean, cscale);
+}
+
+// BF16X3: B - c_m as hi / lo planes, per channel chunks (m-block mb, n-stage
+// ks) of BN x BK elements, K-major interleaved 8x8 core matrices, hi plane then
+// lo plane.
+__device__ __forceinline__ int64_t tc_plane_index(int n, int m, int N, int BN) {
+    int nk = N / TC_BK;
+    int mb = m / BN, r = m % BN, ks = n / TC_BK, k = n % TC_BK;
+    int64_t chunk = (int64_t)mb * nk + ks;
+    int64_t chunk_elems = (int64_t)2 * BN * TC_BK;  // hi + lo
+    int64_t off = ((int64_t)(k / 8) * (BN / 8) + r / 8) * 64 + (r % 8) * 8 + (k % 8);
+    return chunk * chunk_elems + off;  // in bf16 elements; lo at + BN*BK
+}
+
+__global__ void __launch_bounds__(256) k_planes(DevData d, ImgSrc src, __nv_bfloat16* __restrict__ planes,
+                                                const float* __restrict__ cmean) {
+    const int N = d.N, BN = d.fwd_bn;
+    const int64_t NN = (int64_t)N * N;
+    const int c = blockIdx.y;
+    const int i = image_of(d, c);
+    const int64_t p = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (p >= NN) return;
+    double x = img_value(src, i, p, NN);
+    if (src.diff) x -= src.f64[(int64_t)i * NN + p];
+    const int n = (int)(p / N), m = (int)(p % N);
+    const double b = (double)d.beam[(int64_t)c * NN + p] * x;
+    const float bf = (float)(b - (double)cmean[(int64_t)c * N + m]);
+    const __nv_bfloat16 hi = __float2bfloat16_rn(bf);
+    __nv_bfloat16* base = planes + (int64_t)c * 2 * NN + tc_plane_index(n, m, N, BN);
+    base[0] = hi;
+    base[(int64_t)BN * TC_BK] = __float2bfloat16_rn(bf - __bfloat162float(hi));
+}
+
+void launch_planes(const DevData& d, const ImgSrc& src, void* planes, const float* cmean, cudaStream_t st) {
+    k_planes<<<dim3(prep_blocks(d.N), d.C), 256, 0, st>>>(d, src, (__nv_bfloat16*)planes, cmean);
+}
 
 // max |y| over n floats: 256 block maxima, then one block forms the scale.
 __global__ void __launch_bounds__(256) k_absmax_part(int64_t n, const float* __restrict__ y,
@@ -189,59 +327,28 @@ void launch_absmax(int64_t n, const float* y, float* part, float* ymax, cudaStre
     k_absmax_final<<<1, 32, 0, st>>>(part, ymax);
 }
 
-__global__ void __launch_bounds__(256) k_prep(DevData d, ImgSrc src, int fmt, void* bout,
-                                              double* ent_part, const float* __restrict__ cmean,
-                                              const float* __restrict__ cscale) {
+// a2, direct forms: B_c = A_c I in the form's precision.
+template <typename T>
+__global__ void __launch_bounds__(256) k_prep(DevData d, ImgSrc src, T* __restrict__ bout, double* ent_part) {
     __shared__ double sh[8];
     const int N = d.N;
     const int64_t NN = (int64_t)N * N;
     const int c = blockIdx.y;
     const int i = image_of(d, c);
     const int64_t p = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    // the entropy partial of an image is formed by its first channel only
-    // (the others would repeat it in the shared-image mode)
-    const bool ent = ent_part && !(d.shared && c != 0);
+    const bool ent = ent_part && !(d.shared && c != 0);  // as in k_colsum
     double e = 0.0;
     if (p < NN) {
         double x = img_value(src, i, p, NN);
         double xb = x;
         if (src.diff) {
-            // line-search probe as a difference from the base image I: the
-            // operand is delta = max(I + alpha d, G) - I, the entropy term the
-            // change of sum x log(x/G)
             const double x0 = src.f64[(int64_t)i * NN + p];
             xb = x - x0;
             if (ent) e = x * log(x / src.G) - x0 * log(x0 / src.G);
         } else if (ent) {
             e = x * log(x / src.G);
         }
-        double b = (double)d.beam[(int64_t)c * NN + p] * xb;
-        if (fmt == BF_F32) {
-            ((float*)bout)[(int64_t)c * NN + p] = (float)b;
-        } else if (fmt == BF_F64) {
-            ((double*)bout)[(int64_t)c * NN + p] = b;
-        } else {
-            int n = (int)(p / N), m = (int)(p % N);
-            int BN = d.fwd_bn;
-            const double cb = b - (cmean ? (double)cmean[(int64_t)c * N + m] : 0.0);
-            const int64_t q = tc_plane_index(n, m, N, BN);
-            if (fmt == BF_BF16X3) {
-                const float bf = (float)cb;
-                __nv_bfloat16 hi = __float2bfloat16_rn(bf);
-                __nv_bfloat16 lo = __float2bfloat16_rn(bf - __bfloat162float(hi));
-                __nv_bfloat16* base = (__nv_bfloat16*)bout + (int64_t)c * 2 * NN;
-                base[q] = hi;
-                base[q + (int64_t)BN * TC_BK] = lo;
-            } else {
-                const float sc = cscale[c];
-                const float bf = (float)(cb * (double)sc);
-                __half hi = __float2half_rn(bf);
-                __half lo = __float2half_rn(bf - __half2float(hi));
-                __half* base = (__half*)bout + (int64_t)c * 2 * NN;
-                base[q] = hi;
-                base[q + (int64_t)BN * TC_BK] = lo;
-            }
-        }
+        bout[(int64_t)c * NN + p] = (T)((double)d.beam[(int64_t)c * NN + p] * xb);
     }
     if (ent) {  // uniform over the block (one channel per block row)
         double s = block_sum<256>(e, sh);
@@ -249,11 +356,10 @@ __global__ void __launch_bounds__(256) k_prep(DevData d, ImgSrc src, int fmt, vo
     }
 }
 
-
-void launch_prep(const DevData& d, const ImgSrc& src, int fmt, void* bout, double* ent_part,
-                 const float* cmean, const float* cscale, cudaStream_t st) {
+void launch_prep(const DevData& d, const ImgSrc& src, int fmt, void* bout, double* ent_part, cudaStream_t st) {
     dim3 grid(prep_blocks(d.N), d.C);
-    k_prep<<<grid, 256, 0, st>>>(d, src, fmt, bout, ent_part, cmean, cscale);
+    if (fmt == BF_F64) k_prep<double><<<grid, 256, 0, st>>>(d, src, (double*)bout, ent_part);
+    else k_prep<float><<<grid, 256, 0, st>>>(d, src, (float*)bout, ent_part);
 }
 
 // ---------------------------------------------------------------------------
@@ -480,12 +586,12 @@ __global__ void __launch_bounds__(256) k_scalars(DevData d, const int* __restric
 }
 
 void launch_scalars(const DevData& d, const int* tile_off, const double* chi_part,
-                    const double* ent_part, int with_entropy, double* scal, double* img_tmp,
+                    const double* ent_part, int with_entropy, int n_ent, double* scal, double* img_tmp,
                     cudaStream_t st) {
     double* part = scalars_part(img_tmp, d.n_images);
     unsigned* counter = scalars_counter(img_tmp, d.n_images);
     k_scalars<<<dim3(d.n_images, SCAL_SPLIT), 256, 0, st>>>(d, tile_off, chi_part, ent_part, with_entropy,
-                                                             prep_blocks(d.N), part, img_tmp, scal, counter);
+                                                             n_ent, part, img_tmp, scal, counter);
 }
 
 int scalars_tmp_doubles(int n_images) { return 3 * n_images + 2 * SCAL_SPLIT * n_images + 1; }

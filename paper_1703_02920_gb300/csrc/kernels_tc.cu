@@ -538,7 +538,7 @@ __global__ void __launch_bounds__(256) k_adj_tc_reduce_grad(DevData d, ImgSrc sr
     const int64_t NN = (int64_t)N * N;
     const int n_scal = sc.scal ? SCAL_SPLIT : 0;
     if ((int)blockIdx.x < n_scal) {
-        scalars_block(d, sc.tile_off, sc.chi_part, sc.ent_part, sc.with_entropy, prep_blocks(N),
+        scalars_block(d, sc.tile_off, sc.chi_part, sc.ent_part, sc.with_entropy, sc.n_ent,
                       scalars_part(sc.img_tmp, d.n_images), sc.img_tmp, sc.scal,
                       scalars_counter(sc.img_tmp, d.n_images), blockIdx.y, blockIdx.x);
         return;
