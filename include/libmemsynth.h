@@ -284,7 +284,8 @@ mem_status mem_set_tiling(mem_ctx *ctx, const mem_tiling_t *tiling);
  * not use.  Defaults (before mem_autotune or a cached choice): for N <= 128
  * MEM_FWD_RESIDENT with the deepest pipeline that fits (mem_autotune keeps
  * the resident form there: it is the more accurate one, see above), for
- * N >= 256 MEM_FWD_STREAM with 256 columns and 4 stages; adjoint 3 stages. */
+ * N >= 256 MEM_FWD_STREAM with 256 columns and 4 stages; adjoint 3 stages,
+ * FP16X3 with N >= 256 2 (of 32 visibilities each; 16 with 3). */
 mem_status mem_tiling(const mem_ctx *ctx, mem_tiling_t *out);
 
 /* CUDA graphs (default on): every repeated launch sequence (objective +

@@ -288,7 +288,7 @@ void build_tiles(const mem_ctx* c, int size, std::vector<VisTile>& tiles, std::v
 }
 
 // Split-K work of the tensor-core adjoint: the (channel, output block)
-// segments' 16-visibility stages concatenated and cut into one contiguous run
+// segments' TCA_BK-visibility stages concatenated and cut into one contiguous run
 // per CTA; every (CTA, segment) overlap is a unit with its own partial.
 void build_units(mem_ctx* c) {
     const int BLK = tca_blk(c->N), nbx = c->N / BLK, nb = nbx * nbx;
@@ -486,15 +486,19 @@ mem_status run_adjoint(mem_ctx* c, int* ks_out, bool ymax_ready = false, bool re
         }
         if (c->adj_ctas > 0) {
             KTimer t(c, "adj_tc");
-            launch_adj_tc(d, f16, c->units, c->cta_off, c->adj_ctas, c->y32, c->ymax, c->partial, c->spin,
-                          c->dstatus, c->st);
+            if (f16)
+                launch_adj_fold(d, c->units, c->cta_off, c->adj_ctas, c->y32, c->ymax, c->partial, c->spin, c->dstatus,
+                                c->st);
+            else
+                launch_adj_tc(d, c->units, c->cta_off, c->adj_ctas, c->y32, c->partial, c->spin, c->dstatus, c->st);
             c->launches++;
             TRY(after_launch(c, "adjoint kernel"));
         }
         *ks_out = 1;
         if (!reduce) return MEM_OK;
         KTimer t(c, "adj_tc_reduce");
-        launch_adj_tc_reduce(d, c->units, c->cb_off, c->partial, f16 ? c->ymax : nullptr, c->gsum, c->st);
+        if (f16) launch_adj_fold_reduce(d, c->cb_off, c->partial, c->ymax, c->gsum, c->st);
+        else launch_adj_tc_reduce(d, c->cb_off, c->partial, c->gsum, c->st);
         c->launches++;
         TRY(after_launch(c, "adjoint reduction"));
         *ks_out = 1;
@@ -531,8 +535,12 @@ mem_status run_objgrad(mem_ctx* c, const ImgSrc& src, int projected, float* out3
         sc.n_ent = ent_blocks(c);
         sc.scal = c->scal;
         sc.img_tmp = c->img_tmp;
-        launch_adj_tc_reduce_grad(c->dd(), src, c->cb_off, c->partial, c->prec == MEM_PREC_FP16X3 ? c->ymax : nullptr,
-                                  projected, out32, full64, proj64, sc, c->st);
+        if (c->prec == MEM_PREC_FP16X3)
+            launch_adj_fold_reduce_grad(c->dd(), src, c->cb_off, c->partial, c->ymax, projected, out32, full64, proj64,
+                                        sc, c->st);
+        else
+            launch_adj_tc_reduce_grad(c->dd(), src, c->cb_off, c->partial, projected, out32, full64, proj64, sc,
+                                      c->st);
     } else {
         KTimer t(c, "finalize");
         launch_finalize(c->dd(), src, c->gsum, ks, projected, out32, full64, proj64, c->st);
@@ -666,6 +674,10 @@ int fwd_smem_bytes(const mem_ctx* c, int kernel, int cols, int stages) {
     return kernel == MEM_FWD_RESIDENT ? fwd_rs_smem_bytes(c->N, stages) : fwd_tc_smem_bytes(c->N, cols, stages);
 }
 
+int adj_smem_bytes(const mem_ctx* c, int stages) {
+    return c->prec != MEM_PREC_BF16X3 ? adj_fold_smem_bytes(c->N, stages) : adj_tc_smem_bytes(c->N, stages);
+}
+
 // Deepest resident pipeline that fits.
 int resident_stages(const mem_ctx* c) {
     int s = 6;
@@ -674,7 +686,7 @@ int resident_stages(const mem_ctx* c) {
 }
 
 bool tune_valid(const mem_ctx* c, const mem_tiling_t& t) {
-    if (!(t.adj_stages == 2 || t.adj_stages == 3) || adj_tc_smem_bytes(c->N, t.adj_stages) > 227 * 1024)
+    if (!(t.adj_stages == 2 || t.adj_stages == 3) || adj_smem_bytes(c, t.adj_stages) > 227 * 1024)
         return false;
     if (t.fwd_kernel == MEM_FWD_RESIDENT)
         return c->N <= 256 && t.fwd_stages >= 4 && t.fwd_stages <= 6 &&
@@ -719,7 +731,9 @@ void default_tiling(mem_ctx* c) {
         t.fwd_cols = tc_bn(c->N);
         t.fwd_stages = 4;
     }
-    t.adj_stages = 3;
+    // FP16X3, N >= 256: two stages of 32 visibilities (three hold 16 each): at
+    // 256 x 256 with 999,600 visibilities 0.22 ms against 0.28 ms
+    t.adj_stages = c->prec != MEM_PREC_BF16X3 && c->N >= 256 ? 2 : 3;
     // BF16X3 at very large N: the epilogue's column-mean copies leave room for 3 stages
     if (t.fwd_kernel == MEM_FWD_STREAM && fwd_smem_bytes(c, MEM_FWD_STREAM, t.fwd_cols, 4) > 227 * 1024)
         t.fwd_stages = 3;

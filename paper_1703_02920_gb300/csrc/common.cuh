@@ -567,17 +567,86 @@ __device__ __forceinline__ void table8_split(cf2 base, const Rot8& w, uint4& rh,
     split16x2p<F16>(im[3], ih.w, il.w);
 }
 
-// Eight real table entries p Re w_q + r Im w_q (q = 0..7; p and r hold their
-// value twice) split into the two 16-byte operand rows of one 8-element group.
-template <bool F16>
-__device__ __forceinline__ void table8_real(float2 p, float2 r, const Rot8& w, uint4& h, uint4& l) {
-    float2 v[4];
+// ---------------------------------------------------------------------------
+// Table entries about a group's centre.  The eight entries of a group lie at
+// +-(k + 1/2) steps, k = 0..3, from its centre: with s_k = exp(-2 pi i (k + 1/2) p)
+// and the centre's factor e, entry 4 + k is e s_k and entry 3 - k is e conj(s_k),
+// which share their products e c_k: 1.5 operations per value where a rotation
+// of each takes 2.
+// ---------------------------------------------------------------------------
+
+// hi = rn(x), lo = rn(x - hi) of the pair (a, b) in FP16.  x - hi is one
+// mixed-precision FMA (exact), without a conversion of hi back to FP32.
+__device__ __forceinline__ void split_pair_f16(float a, float b, uint32_t& hi, uint32_t& lo) {
+    asm("{\n .reg .b16 h0, h1, m1;\n .reg .f32 la, lb;\n mov.b16 m1, 0xBC00;\n cvt.rn.f16x2.f32 %0, %3, %2;\n"
+        " mov.b32 {h0, h1}, %0;\n fma.rn.f32.f16 la, h0, m1, %2;\n fma.rn.f32.f16 lb, h1, m1, %3;\n"
+        " cvt.rn.f16x2.f32 %1, lb, la;\n}\n"
+        : "=&r"(hi), "=r"(lo)
+        : "f"(a), "f"(b));
+}
+
+// The half steps s_0..s_3 and the step over a group, exp(-2 pi i 8 p): both
+// ends of the chain to FP32 rounding, the others by one to three products.
+struct HalfSteps {
+    cf2 s[4], s8;
+};
+__device__ __forceinline__ HalfSteps half_steps(uint64_t p) {
+    HalfSteps h;
+    h.s[0] = cis_neg_accurate((uint32_t)((int32_t)(uint32_t)(p >> 32) >> 1));
+    const cf2 w = cmul(h.s[0], h.s[0]);
+    h.s[1] = cmul(h.s[0], w);
+    h.s[2] = cmul(h.s[1], w);
+    h.s[3] = cmul(h.s[2], w);
+    h.s8 = cis_neg_accurate((uint32_t)((8 * p) >> 32));
+    return h;
+}
+
+// Eight real entries: entry 4 + k is A Re s_k + B Im s_k, entry 3 - k has B's
+// sign turned (A and B hold their value twice; k = 0, 1 and 2, 3 packed, ni =
+// -Im s), split into the two 16-byte operand rows of the group.
+struct HalfPairs {
+    float2 re[2], im[2], ni[2];
+};
+__device__ __forceinline__ HalfPairs half_pairs(const HalfSteps& h) {
+    HalfPairs r;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) v[q] = __ffma2_rn(p, w.x[q], __fmul2_rn(r, w.y[q]));
-    split16x2p<F16>(v[0], h.x, l.x);
-    split16x2p<F16>(v[1], h.y, l.y);
-    split16x2p<F16>(v[2], h.z, l.z);
-    split16x2p<F16>(v[3], h.w, l.w);
+    for (int p = 0; p < 2; ++p) {
+        r.re[p] = make_float2(h.s[2 * p].x, h.s[2 * p + 1].x);
+        r.im[p] = make_float2(h.s[2 * p].y, h.s[2 * p + 1].y);
+        r.ni[p] = make_float2(-h.s[2 * p].y, -h.s[2 * p + 1].y);
+    }
+    return r;
+}
+__device__ __forceinline__ void table8_real(float2 A, float2 B, const HalfPairs& w, uint4& h, uint4& l) {
+    const float2 p0 = __fmul2_rn(A, w.re[0]), p1 = __fmul2_rn(A, w.re[1]);
+    const float2 u0 = __ffma2_rn(B, w.im[0], p0), u1 = __ffma2_rn(B, w.im[1], p1);
+    const float2 d0 = __ffma2_rn(B, w.ni[0], p0), d1 = __ffma2_rn(B, w.ni[1], p1);
+    split_pair_f16(d1.y, d1.x, h.x, l.x);
+    split_pair_f16(d0.y, d0.x, h.y, l.y);
+    split_pair_f16(u0.x, u0.y, h.z, l.z);
+    split_pair_f16(u1.x, u1.y, h.w, l.w);
+}
+
+// Eight complex entries e s_k, e conj(s_k), split into four operand rows.
+__device__ __forceinline__ void table8_complex(cf2 e, const HalfSteps& w, uint4& rh, uint4& rl, uint4& ih,
+                                               uint4& il) {
+    float ru[4], rd[4], iu[4], id[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float p = e.x * w.s[k].x, q = e.y * w.s[k].x;
+        ru[k] = fmaf(-e.y, w.s[k].y, p);
+        rd[k] = fmaf(e.y, w.s[k].y, p);
+        iu[k] = fmaf(e.x, w.s[k].y, q);
+        id[k] = fmaf(-e.x, w.s[k].y, q);
+    }
+    split_pair_f16(rd[3], rd[2], rh.x, rl.x);
+    split_pair_f16(rd[1], rd[0], rh.y, rl.y);
+    split_pair_f16(ru[0], ru[1], rh.z, rl.z);
+    split_pair_f16(ru[2], ru[3], rh.w, rl.w);
+    split_pair_f16(id[3], id[2], ih.x, il.x);
+    split_pair_f16(id[1], id[0], ih.y, il.y);
+    split_pair_f16(iu[0], iu[1], ih.z, il.z);
+    split_pair_f16(iu[2], iu[3], ih.w, il.w);
 }
 
 }  // namespace msk

@@ -21,7 +21,7 @@ struct VisTile {
 // over a visibility range.
 struct AdjUnit {
     int32_t chan;
-    int32_t block;   // output block index (row-major over N/BLK x N/BLK)
+    int32_t block;   // output block index (row-major over N/BLK x N/BLK; FP16X3: row blocks of mirror pairs)
     int64_t start;   // first visibility (global index)
     int64_t count;
 };
@@ -81,7 +81,8 @@ constexpr int MEAN_L = 16;  // folded columns l that share the operand's means
 // First column (P) of folded column l within a part: groups of eight P columns
 // followed by the eight Q columns of the same l (Q = P + 8).
 __host__ __device__ inline int fold_col(int l) { return 16 * (l / 8) + l % 8; }
-// Adjoint tensor-core tiling: output block side and visibilities per stage.
+// Adjoint tensor-core tiling: output block side, and the multiple of
+// visibilities at which units are cut.
 constexpr int TCA_BK = 16;
 inline int tca_blk(int N) { return N < 256 ? N : 256; }
 
@@ -166,12 +167,24 @@ void launch_dirty_y(const DevData& d, const double* wsum, int what, int64_t z_to
                     cudaStream_t st);
 void launch_dirty_out(const DevData& d, const double* gsum, int ks, float* out, cudaStream_t st);
 void launch_grid_interp(const DevData& d, int M, const float2* F, int64_t z_total, float2* vis, cudaStream_t st);
+// Adjoint: units sorted by CTA: CTA b runs units [cta_unit_off[b],
+// cta_unit_off[b+1]) into partials of BLK x BLK floats each, which the reductions
+// below sum in unit order per (channel, block).
+//
+// FP16X3, folded: y scaled by pow2_scale_for(ymax[0]) (the partials carry the
+// scale); a unit's output block is its two D blocks.
+int adj_fold_smem_bytes(int N, int stages);
+void launch_adj_fold(const DevData& d, const AdjUnit* units, const int* cta_unit_off, int n_ctas, const float2* y,
+                     const float* ymax, float* partial, uint64_t spin, int* status, cudaStream_t st);
+// into gsum[C][N*N], without the beam factor
+void launch_adj_fold_reduce(const DevData& d, const int* cb_unit_off, const float* partial, const float* ymax,
+                            double* gsum, cudaStream_t st);
+// BF16X3.
 int adj_tc_smem_bytes(int N, int stages);
-// units sorted by CTA: CTA b runs units [cta_unit_off[b], cta_unit_off[b+1]).
-// f16 = 1: FP16X3 with y scaled by pow2_scale_for(ymax[0]) (partials carry the scale).
-void launch_adj_tc(const DevData& d, int f16, const AdjUnit* units, const int* cta_unit_off, int n_ctas,
-                   const float2* y, const float* ymax, float* partial, uint64_t spin, int* status,
-                   cudaStream_t st);
+void launch_adj_tc(const DevData& d, const AdjUnit* units, const int* cta_unit_off, int n_ctas, const float2* y,
+                   float* partial, uint64_t spin, int* status, cudaStream_t st);
+void launch_adj_tc_reduce(const DevData& d, const int* cb_unit_off, const float* partial, double* gsum,
+                          cudaStream_t st);
 // Variant reading u, v (FP64, wavelengths) instead of the prepared phase
 // increments: the caller passes d.u, d.v, d.dx, d.dy; d.pa / d.pb are unused.
 void launch_adj_tc_uv(const DevData& d, const AdjUnit* units, const int* cta_unit_off, int n_ctas,
@@ -180,10 +193,6 @@ void launch_adj_tc_uv(const DevData& d, const AdjUnit* units, const int* cta_uni
 // compensated FP32 two-sum).
 void launch_adj_tc_reduce_out(int N, const int* cb_unit_off, const float* partial, const float* beam,
                               float* out, cudaStream_t st);
-// Sum unit partials per channel (unit order) into gsum[C][N*N].
-// ymax (nullable, FP16X3): partials are divided by pow2_scale_for(ymax[0]).
-void launch_adj_tc_reduce(const DevData& d, const AdjUnit* units, const int* unit_off_by_chan_blk,
-                          const float* partial, const float* ymax, double* gsum, cudaStream_t st);
 // Inputs of the objective's scalar reduction (launch_scalars) when it runs
 // inside another launch; scal == nullptr: not run.
 struct ScalarArgs {
@@ -198,9 +207,12 @@ struct ScalarArgs {
 // Unit-partial sum plus gradient assembly in one launch, for images of one
 // channel each (not the shared-image mode); with sc.scal set, the same launch
 // also forms the objective scalars (as launch_scalars).
+void launch_adj_fold_reduce_grad(const DevData& d, const ImgSrc& src, const int* cb_unit_off, const float* partial,
+                                 const float* ymax, int projected, float* out32, double* full64, double* proj64,
+                                 const ScalarArgs& sc, cudaStream_t st);
 void launch_adj_tc_reduce_grad(const DevData& d, const ImgSrc& src, const int* cb_unit_off, const float* partial,
-                               const float* ymax, int projected, float* out32, double* full64, double* proj64,
-                               const ScalarArgs& sc, cudaStream_t st);
+                               int projected, float* out32, double* full64, double* proj64, const ScalarArgs& sc,
+                               cudaStream_t st);
 
 // grad_i = sum_{c in image i} A_c * sum_k gsum[k][c] + lambda (1 + log(I/G)); optional projection.
 void launch_finalize(const DevData& d, const ImgSrc& src, const double* gsum, int ks, int projected,

@@ -486,17 +486,18 @@ __global__ void __launch_bounds__(FW_THREADS, 1)
         for (int t = t_begin; t < t_end && ok; t += t_step) {
             const uint64_t pb = pb_next;
             if (t + t_step < t_end) load_tile(t + t_step);
-            const uint64_t hb = (uint64_t)((int64_t)pb >> 1);  // half the row step: (j + 1/2) b = (2 j + 1) hb
-            cf2 step8;
-            const Rot8 w = rot8_steps(pb, step8);
+            const HalfSteps hs = half_steps(pb);
+            const HalfPairs w = half_pairs(hs);
+            const cf2 step8 = hs.s8;
             const cf2 step64 = cis_neg_accurate((uint32_t)((2 * TC_BK * pb) >> 32));  // over two stages
             for (int mb = 0, ks0 = 0, part = RES == RES_PART ? my_part : 0; mb < n_mb && ok;) {
-                // Phase factor x + i y of this group's first stage of the
-                // accumulation, held as (x, q) with q = y in the sine part and
+                // Phase factor x + i y at the centre of the first 8 rows of this
+                // group's first stage of the accumulation (row j0 + 3.5, so
+                // (j + 1/2) b = (j0 + 4) b there), held as (x, q) with q = y in the sine part and
                 // -y in the cosine part (products of conjugates), so that
                 //   Re(base w) = x Re w + q Im w,  Im(base w) = q Re w + x Im w.
                 const int k0 = (int)((sc ^ grp) & 1);
-                cf2 base0 = cis_neg_accurate(phase_hi(2 * (ks0 + k0) * TC_BK + 1, hb));
+                cf2 base0 = cis_neg_accurate(phase_hi((ks0 + k0) * TC_BK + 4, pb));
                 const float sgn = part ? 1.f : -1.f;
                 base0.y *= sgn;
                 const cf2 s64 = {step64.x, step64.y * sgn};
@@ -514,7 +515,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1)
 #pragma unroll
                         for (int g = 0; g < 4; ++g) {
                             uint4 h, l;
-                            table8_real<true>(sine ? y : x, sine ? x : y, w, h, l);
+                            table8_real(sine ? y : x, sine ? x : y, w, h, l);
                             *(uint4*)(A + g * 2048) = h;
                             *(uint4*)(A + F2_APLANE + g * 2048) = l;
                             if (g < 3) {  // the next 8 rows' factor

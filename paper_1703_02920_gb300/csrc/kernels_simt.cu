@@ -581,7 +581,7 @@ __global__ void __launch_bounds__(256) k_scalars(DevData d, const int* __restric
                                                  const double* __restrict__ ent_part, int with_entropy,
                                                  int n_ent_blocks, double* part, double* img_tmp, double* scal,
                                                  unsigned* counter) {
-    scalars_block(d, tile_off, chi_part, ent_part, with_entropy, n_ent_blocks, part, img_tmp, scal, counter,
+    scalars_block<256>(d, tile_off, chi_part, ent_part, with_entropy, n_ent_blocks, part, img_tmp, scal, counter,
                   blockIdx.x, blockIdx.y);
 }
 

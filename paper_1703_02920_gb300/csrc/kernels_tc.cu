@@ -1,5 +1,8 @@
-// Tensor-core (tcgen05) adjoint of the measurement operator (the forward
-// operator is in kernels_fwd.cu).
+// Tensor-core (tcgen05) adjoint of the BF16X3 form (its forward is in
+// kernels_fwd.cu and kernels_fwd_rs.cu).  Both take the same table entries, so
+// that the computed pair stays adjoint to itself: with the folded adjoint of
+// FP16X3 (kernels_adj_fold.cu) beside the unfolded forward, a converged 64 x 64
+// solve stops at Phi* + 3.6e-6 instead of Phi* + 2.8e-6.
 //
 // On the regular pixel grid the phase of Eq. (1) separates,
 //   exp(-2 pi i (u x_m + v y_n)) = Ex[k,m] Ey[k,n],
@@ -9,7 +12,7 @@
 //   G[n,m] = sum_k Re(Ey)[k,n] Re(P)[k,m] + Im(Ey)[k,n] Im(P)[k,m],
 //   P[k,m] = y_k conj(Ex[k,m]),  y = w r.
 // Both contractions run on the 5th-generation tensor cores (tcgen05.mma,
-// kind::f16, accumulators in TMEM) in a 3-term FP16 or BF16 split: x = hi + lo,
+// kind::f16, accumulators in TMEM) in a 3-term BF16 split: x = hi + lo,
 // a b ~= a_hi b_hi + a_hi b_lo + a_lo b_hi, FP32 accumulation.  The phase
 // tables are never stored: producer warps generate each tile in shared
 // memory from the exact fixed-point phases (one SFU sincos per 8 entries,
@@ -129,14 +132,11 @@ struct AdjShared {
 
 // FROM_UV: phase increments reduced from u, v inside the producers instead of
 // read from the prepared arrays.
-// F16: FP16X3 operands with y scaled by pow2_scale_for(ymax[0]) (a power of
-// two, undone when the partials are summed); otherwise BF16X3.
 // ADJ_STAGES: depth of the shared-memory pipeline (autotuned).
-template <bool FROM_UV, bool F16, int ADJ_STAGES>
+template <bool FROM_UV, int ADJ_STAGES>
 __global__ void __launch_bounds__(ADJ_THREADS, 1)
     k_adj_tc(DevData d, const AdjUnit* __restrict__ units, const int* __restrict__ cta_unit_off,
-             const float2* __restrict__ y, const float* __restrict__ ymax, float* __restrict__ partial,
-             uint64_t spin, int* status) {
+             const float2* __restrict__ y, float* __restrict__ partial, uint64_t spin, int* status) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ AdjShared S;
     const int N = d.N, c0 = N / 2;
@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(ADJ_THREADS, 1)
         // The whole warp runs the issue loop, converged (every wait's outcome is
         // made warp-uniform), and one elected lane issues the MMAs and commits.
         {
-            const uint32_t idesc = idesc_f16kind(128, BLK, 1, 1, F16 ? 0 : 1);
+            const uint32_t idesc = idesc_f16kind(128, BLK, 1, 1, 1);
             const uint32_t sbase = smem_u32(smem);
             const uint32_t lboA = (uint32_t)(R / 8) * 128, lboB = (uint32_t)(BLK / 8) * 128;
             // Operand descriptors of slot 0; another slot or row block only
@@ -245,7 +245,6 @@ __global__ void __launch_bounds__(ADJ_THREADS, 1)
         const int jj = lane & 15;           // visibility within the stage
         const int ngA = R / 8, ngB = BLK / 8;
         const int wi_end = min(wi_start + wi_cap, (ey_side ? ngA : ngB) / 2);
-        const float ysc = F16 ? pow2_scale_for(ymax[0]) : 1.f;
         uint32_t sc = 0, dr = 0;  // stages produced; accumulator drains (warps 0-3)
         bool ok = true;
         for (int u = u0; u < u1 && ok; ++u) {
@@ -277,7 +276,7 @@ __global__ void __launch_bounds__(ADJ_THREADS, 1)
             for (int ks = seg0; ks < seg1; ++ks, ++sc) {
                 const int s = sc % ADJ_STAGES;
                 const uint64_t pa = na, pb = nb;
-                const cf2 yv = {ny.x * ysc, ny.y * ysc};
+                const cf2 yv = {ny.x, ny.y};
                 const bool valid = (int64_t)ks * TCA_BK + jj < un.count;
                 fetch(ks + 1, na, nb, ny);
                 // rotation steps exp(-i 2 pi q c), q = 0..7, by powers of one SFU
@@ -315,14 +314,14 @@ __global__ void __launch_bounds__(ADJ_THREADS, 1)
                             cf2 z[8];
 #pragma unroll
                             for (int q = 0; q < 8; ++q) z[q] = cmul(base, st[q]);
-                            split16x2<F16>(z[0].x, z[1].x, rh.x, rl.x);
-                            split16x2<F16>(z[2].x, z[3].x, rh.y, rl.y);
-                            split16x2<F16>(z[4].x, z[5].x, rh.z, rl.z);
-                            split16x2<F16>(z[6].x, z[7].x, rh.w, rl.w);
-                            split16x2<F16>(z[0].y, z[1].y, ih.x, il.x);
-                            split16x2<F16>(z[2].y, z[3].y, ih.y, il.y);
-                            split16x2<F16>(z[4].y, z[5].y, ih.z, il.z);
-                            split16x2<F16>(z[6].y, z[7].y, ih.w, il.w);
+                            split_bf16x2(z[0].x, z[1].x, rh.x, rl.x);
+                            split_bf16x2(z[2].x, z[3].x, rh.y, rl.y);
+                            split_bf16x2(z[4].x, z[5].x, rh.z, rl.z);
+                            split_bf16x2(z[6].x, z[7].x, rh.w, rl.w);
+                            split_bf16x2(z[0].y, z[1].y, ih.x, il.x);
+                            split_bf16x2(z[2].y, z[3].y, ih.y, il.y);
+                            split_bf16x2(z[4].y, z[5].y, ih.z, il.z);
+                            split_bf16x2(z[6].y, z[7].y, ih.w, il.w);
                         }
                         dst = A + ((jj >> 3) * ngA + g) * 128 + (jj & 7) * 16;
                         plane = a_plane;
@@ -336,14 +335,14 @@ __global__ void __launch_bounds__(ADJ_THREADS, 1)
                             cf2 z[8];
 #pragma unroll
                             for (int q = 0; q < 8; ++q) z[q] = cmul(base, cf2{st[q].x, -st[q].y});
-                            split16x2<F16>(z[0].x, z[1].x, rh.x, rl.x);
-                            split16x2<F16>(z[2].x, z[3].x, rh.y, rl.y);
-                            split16x2<F16>(z[4].x, z[5].x, rh.z, rl.z);
-                            split16x2<F16>(z[6].x, z[7].x, rh.w, rl.w);
-                            split16x2<F16>(z[0].y, z[1].y, ih.x, il.x);
-                            split16x2<F16>(z[2].y, z[3].y, ih.y, il.y);
-                            split16x2<F16>(z[4].y, z[5].y, ih.z, il.z);
-                            split16x2<F16>(z[6].y, z[7].y, ih.w, il.w);
+                            split_bf16x2(z[0].x, z[1].x, rh.x, rl.x);
+                            split_bf16x2(z[2].x, z[3].x, rh.y, rl.y);
+                            split_bf16x2(z[4].x, z[5].x, rh.z, rl.z);
+                            split_bf16x2(z[6].x, z[7].x, rh.w, rl.w);
+                            split_bf16x2(z[0].y, z[1].y, ih.x, il.x);
+                            split_bf16x2(z[2].y, z[3].y, ih.y, il.y);
+                            split_bf16x2(z[4].y, z[5].y, ih.z, il.z);
+                            split_bf16x2(z[6].y, z[7].y, ih.w, il.w);
                         }
                         dst = B + ((jj >> 3) * ngB + g) * 128 + (jj & 7) * 16;
                         plane = b_plane;
@@ -381,35 +380,25 @@ __global__ void __launch_bounds__(ADJ_THREADS, 1)
     }
 }
 
-template <bool FROM_UV, bool F16, int STAGES>
+template <bool FROM_UV, int STAGES>
 static void launch_adj_variant(const DevData& d, const AdjUnit* units, const int* cta_unit_off, int n_ctas,
-                               const float2* y, const float* ymax, float* partial, uint64_t spin,
-                               int* status, cudaStream_t st) {
+                               const float2* y, float* partial, uint64_t spin, int* status, cudaStream_t st) {
     const int smem = adj_tc_smem_bytes(d.N, STAGES);
-    cudaFuncSetAttribute(k_adj_tc<FROM_UV, F16, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    k_adj_tc<FROM_UV, F16, STAGES><<<n_ctas, ADJ_THREADS, smem, st>>>(d, units, cta_unit_off, y, ymax,
-                                                                      partial, spin, status);
+    cudaFuncSetAttribute(k_adj_tc<FROM_UV, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    k_adj_tc<FROM_UV, STAGES><<<n_ctas, ADJ_THREADS, smem, st>>>(d, units, cta_unit_off, y, partial, spin, status);
 }
 
-void launch_adj_tc(const DevData& d, int f16, const AdjUnit* units, const int* cta_unit_off, int n_ctas,
-                   const float2* y, const float* ymax, float* partial, uint64_t spin, int* status,
-                   cudaStream_t st) {
+void launch_adj_tc(const DevData& d, const AdjUnit* units, const int* cta_unit_off, int n_ctas, const float2* y,
+                   float* partial, uint64_t spin, int* status, cudaStream_t st) {
     if (n_ctas <= 0) return;
-    const bool s2 = d.adj_stages == 2;
-    if (f16) {
-        if (s2) launch_adj_variant<false, true, 2>(d, units, cta_unit_off, n_ctas, y, ymax, partial, spin, status, st);
-        else launch_adj_variant<false, true, 3>(d, units, cta_unit_off, n_ctas, y, ymax, partial, spin, status, st);
-    } else {
-        if (s2) launch_adj_variant<false, false, 2>(d, units, cta_unit_off, n_ctas, y, ymax, partial, spin, status, st);
-        else launch_adj_variant<false, false, 3>(d, units, cta_unit_off, n_ctas, y, ymax, partial, spin, status, st);
-    }
+    if (d.adj_stages == 2) launch_adj_variant<false, 2>(d, units, cta_unit_off, n_ctas, y, partial, spin, status, st);
+    else launch_adj_variant<false, 3>(d, units, cta_unit_off, n_ctas, y, partial, spin, status, st);
 }
 
 void launch_adj_tc_uv(const DevData& d, const AdjUnit* units, const int* cta_unit_off, int n_ctas,
                       const float2* y, float* partial, uint64_t spin, int* status, cudaStream_t st) {
     if (n_ctas <= 0) return;
-    launch_adj_variant<true, false, ADJ_MAX_STAGES>(d, units, cta_unit_off, n_ctas, y, nullptr, partial, spin,
-                                                    status, st);
+    launch_adj_variant<true, ADJ_MAX_STAGES>(d, units, cta_unit_off, n_ctas, y, partial, spin, status, st);
 }
 
 // Single channel: out[p] = A[p] * (unit partials summed in unit order,
@@ -480,7 +469,6 @@ __device__ __forceinline__ float unit_sum_combine(float s, float comp, int el, i
 
 __global__ void __launch_bounds__(256) k_adj_tc_reduce(DevData d, const int* __restrict__ cb_unit_off,
                                                        const float* __restrict__ partial,
-                                                       const float* __restrict__ ymax,
                                                        double* __restrict__ gsum) {
     __shared__ float sh[4][RED_ELEMS][2];
     const int N = d.N;
@@ -503,16 +491,14 @@ __global__ void __launch_bounds__(256) k_adj_tc_reduce(DevData d, const int* __r
     int nl, ml;
     adj_partial_rc(loc, BLK, nl, ml);
     const int64_t p = (int64_t)((blk / nbx) * BLK + nl) * N + (blk % nbx) * BLK + ml;
-    const double inv = ymax ? 1.0 / (double)pow2_scale_for(ymax[0]) : 1.0;
-    gsum[(int64_t)c * NN + p] = (double)tot * inv;
+    gsum[(int64_t)c * NN + p] = (double)tot;
 }
 
-void launch_adj_tc_reduce(const DevData& d, const AdjUnit* units, const int* cb_unit_off,
-                          const float* partial, const float* ymax, double* gsum, cudaStream_t st) {
-    (void)units;
+void launch_adj_tc_reduce(const DevData& d, const int* cb_unit_off, const float* partial, double* gsum,
+                          cudaStream_t st) {
     const int64_t NN = (int64_t)d.N * d.N;
     dim3 grid((unsigned)((NN + RED_ELEMS - 1) / RED_ELEMS), d.C);
-    k_adj_tc_reduce<<<grid, 256, 0, st>>>(d, cb_unit_off, partial, ymax, gsum);
+    k_adj_tc_reduce<<<grid, 256, 0, st>>>(d, cb_unit_off, partial, gsum);
 }
 
 // The unit-partial sum of k_adj_tc_reduce followed directly by the gradient
@@ -529,8 +515,7 @@ void launch_adj_tc_reduce(const DevData& d, const AdjUnit* units, const int* cb_
 // of its own.
 __global__ void __launch_bounds__(256) k_adj_tc_reduce_grad(DevData d, ImgSrc src,
                                                             const int* __restrict__ cb_unit_off,
-                                                            const float* __restrict__ partial,
-                                                            const float* __restrict__ ymax, int projected,
+                                                            const float* __restrict__ partial, int projected,
                                                             float* out32, double* full64, double* proj64,
                                                             ScalarArgs sc) {
     __shared__ float sh[4][RED_ELEMS][2];
@@ -538,7 +523,7 @@ __global__ void __launch_bounds__(256) k_adj_tc_reduce_grad(DevData d, ImgSrc sr
     const int64_t NN = (int64_t)N * N;
     const int n_scal = sc.scal ? SCAL_SPLIT : 0;
     if ((int)blockIdx.x < n_scal) {
-        scalars_block(d, sc.tile_off, sc.chi_part, sc.ent_part, sc.with_entropy, sc.n_ent,
+        scalars_block<256>(d, sc.tile_off, sc.chi_part, sc.ent_part, sc.with_entropy, sc.n_ent,
                       scalars_part(sc.img_tmp, d.n_images), sc.img_tmp, sc.scal,
                       scalars_counter(sc.img_tmp, d.n_images), blockIdx.y, blockIdx.x);
         return;
@@ -560,8 +545,7 @@ __global__ void __launch_bounds__(256) k_adj_tc_reduce_grad(DevData d, ImgSrc sr
     int nl, ml;
     adj_partial_rc(loc, BLK, nl, ml);
     const int64_t p = (int64_t)((blk / nbx) * BLK + nl) * N + (blk % nbx) * BLK + ml;
-    const double inv = ymax ? 1.0 / (double)pow2_scale_for(ymax[0]) : 1.0;
-    const double gchi = (double)tot * inv;
+    const double gchi = (double)tot;
     double gr = (double)d.beam[(int64_t)c * NN + p] * gchi;
     const double x = img_value(src, c, p, NN);
     if (d.lambda != 0.0) gr += d.lambda * (1.0 + log(x / d.G));
@@ -572,12 +556,12 @@ __global__ void __launch_bounds__(256) k_adj_tc_reduce_grad(DevData d, ImgSrc sr
 }
 
 void launch_adj_tc_reduce_grad(const DevData& d, const ImgSrc& src, const int* cb_unit_off, const float* partial,
-                               const float* ymax, int projected, float* out32, double* full64, double* proj64,
+                               int projected, float* out32, double* full64, double* proj64,
                                const ScalarArgs& sc, cudaStream_t st) {
     const int64_t NN = (int64_t)d.N * d.N;
     const unsigned gb = (unsigned)((NN + RED_ELEMS - 1) / RED_ELEMS);
     dim3 grid(gb + (sc.scal ? SCAL_SPLIT : 0), d.C);
-    k_adj_tc_reduce_grad<<<grid, 256, 0, st>>>(d, src, cb_unit_off, partial, ymax, projected, out32, full64,
+    k_adj_tc_reduce_grad<<<grid, 256, 0, st>>>(d, src, cb_unit_off, partial, projected, out32, full64,
                                                 proj64, sc);
 }
 

@@ -44,27 +44,28 @@ __device__ __host__ inline unsigned* scalars_counter(double* img_tmp, int n_imag
     return (unsigned*)(scalars_part(img_tmp, n_images) + 2 * SCAL_SPLIT * n_images);
 }
 
-// Every thread of the block calls this (block-wide barriers inside).
+// Every thread of the block (THREADS) calls this (block-wide barriers inside).
+template <int THREADS>
 __device__ __forceinline__ void scalars_block(const DevData& d, const int* __restrict__ tile_off,
                                               const double* __restrict__ chi_part,
                                               const double* __restrict__ ent_part, int with_entropy,
                                               int n_ent_blocks, double* part, double* img_tmp, double* scal,
                                               unsigned* counter, int i, int q) {
-    __shared__ double sh[8];
+    __shared__ double sh[THREADS / 32];
     __shared__ bool last;
     int c_lo = d.shared ? 0 : i, c_hi = d.shared ? d.C : i + 1;
     const int64_t t0 = 4LL * tile_off[c_lo], t1 = 4LL * tile_off[c_hi];  // channels are contiguous
     const int64_t len = t1 - t0;
     const int64_t a = t0 + len * q / SCAL_SPLIT, b = t0 + len * (q + 1) / SCAL_SPLIT;
     double x = 0.0;
-    for (int64_t t = a + threadIdx.x; t < b; t += 256) x += chi_part[t];
-    const double chi = block_sum<256>(x, sh);
+    for (int64_t t = a + threadIdx.x; t < b; t += THREADS) x += chi_part[t];
+    const double chi = block_sum<THREADS>(x, sh);
     double S = 0.0;
     if (with_entropy) {
         const int e0 = (int)((int64_t)n_ent_blocks * q / SCAL_SPLIT), e1 = (int)((int64_t)n_ent_blocks * (q + 1) / SCAL_SPLIT);
         double y = 0.0;
-        for (int e = e0 + threadIdx.x; e < e1; e += 256) y += ent_part[(int64_t)i * n_ent_blocks + e];
-        S = block_sum<256>(y, sh);
+        for (int e = e0 + threadIdx.x; e < e1; e += THREADS) y += ent_part[(int64_t)i * n_ent_blocks + e];
+        S = block_sum<THREADS>(y, sh);
     }
     if (threadIdx.x == 0) {
         part[((int64_t)i * SCAL_SPLIT + q) * 2] = chi;
