@@ -77,9 +77,8 @@ struct mem_ctx {
     double* bf64 = nullptr;
     uint16_t* planes = nullptr;
     float* cmean = nullptr;  // means of the centred tensor-core operand
-    float* cscale = nullptr;                    // FP16X3 operand scales per channel
+    float4* cmean4 = nullptr;                   // FP16X3: means and inverse scale per strip
     double* col_psum = nullptr;                 // column-mean partial sums
-    float* col_pmax = nullptr;
     unsigned* col_count = nullptr;              // column-mean completion counters (zero between calls)
     float *ymax = nullptr, *ymax_part = nullptr;  // FP16X3: max |y| (adjoint operand scale), partials
     float* partial = nullptr;  // adjoint unit partials (FP32, one BLK x BLK block each)
@@ -152,6 +151,7 @@ struct mem_ctx {
         d.n_images = n_images;
         d.shared = shared;
         d.G = G;
+        d.ginv = 1.0 / G;
         d.lambda = lambda;
         d.pa = pa;
         d.pb = pb;
@@ -363,7 +363,7 @@ mem_status after_launch(mem_ctx* c, const char* what) {
 mem_status ensure_buffers(mem_ctx* c) {
     const size_t NN = (size_t)c->N * c->N;
     TRY(dalloc(c, &c->chi_part, (size_t)4 * std::max(std::max(c->n_tiles, c->n_tiles_tc), 1)));
-    TRY(dalloc(c, &c->ent_part, (size_t)c->n_images * std::max(prep_blocks(c->N), tc_ent_blocks(c->N))));
+    TRY(dalloc(c, &c->ent_part, (size_t)c->n_images * std::max(prep_blocks(c->N), std::max(tc_ent_blocks(c->N), fold_ent_blocks(c->N)))));
     TRY(dalloc(c, &c->scal, (size_t)3 + 3 * c->n_images));
     if (!c->img_tmp) {  // holds the scalar reduction's completion counter, which starts at zero
         TRY(dalloc(c, &c->img_tmp, (size_t)scalars_tmp_doubles(c->n_images)));
@@ -378,14 +378,16 @@ mem_status ensure_buffers(mem_ctx* c) {
         TRY(dalloc(c, &c->bf32, (size_t)c->C * NN));
     } else {
         TRY(dalloc(c, &c->planes, (size_t)2 * c->C * NN));
-        TRY(dalloc(c, &c->cmean, (size_t)c->C * c->N));
-        if (!c->col_count) {
-            TRY(dalloc(c, &c->col_count, (size_t)c->C));
-            CK(cudaMemsetAsync(c->col_count, 0, (size_t)c->C * sizeof(unsigned), c->st), "column-mean counters");
+        if (c->prec == MEM_PREC_FP16X3) {
+            TRY(dalloc(c, &c->cmean4, (size_t)c->C * c->N / MEAN_L));
+        } else {
+            TRY(dalloc(c, &c->cmean, (size_t)c->C * c->N));
+            if (!c->col_count) {
+                TRY(dalloc(c, &c->col_count, (size_t)c->C));
+                CK(cudaMemsetAsync(c->col_count, 0, (size_t)c->C * sizeof(unsigned), c->st), "column-mean counters");
+            }
+            TRY(dalloc(c, &c->col_psum, (size_t)colmean_tmp_count(c->N, c->C)));
         }
-        TRY(dalloc(c, &c->col_psum, (size_t)colmean_tmp_count(c->N, c->C)));
-        TRY(dalloc(c, &c->col_pmax, (size_t)colmean_tmp_count(c->N, c->C)));
-        TRY(dalloc(c, &c->cscale, (size_t)c->C));
         TRY(dalloc(c, &c->ymax, (size_t)1));
         TRY(dalloc(c, &c->ymax_part, (size_t)256));
         const int BLK = tca_blk(c->N);
@@ -409,7 +411,10 @@ void* bbuf(mem_ctx* c) { return c->prec == MEM_PREC_FP64_DIRECT ? (void*)c->bf64
 // tile list that the form's forward ran over (4 chi^2 partials per tile)
 const int* fwd_tile_off(const mem_ctx* c) { return c->prec == MEM_PREC_BF16X3 ? c->tile_off_tc : c->tile_off; }
 
-int ent_blocks(const mem_ctx* c) { return is_tc(c->prec) ? tc_ent_blocks(c->N) : prep_blocks(c->N); }
+int ent_blocks(const mem_ctx* c) {
+    return c->prec == MEM_PREC_FP16X3   ? fold_ent_blocks(c->N)
+           : c->prec == MEM_PREC_BF16X3 ? tc_ent_blocks(c->N) : prep_blocks(c->N);
+}
 
 // prep + forward for one image source.  mode: FwdMode.  defer_scalars: the
 // objective's scalar reduction is left to a later launch (the gradient's).
@@ -419,26 +424,29 @@ mem_status run_forward(mem_ctx* c, const ImgSrc& src, int mode, bool entropy, vo
     const bool tc = is_tc(c->prec);
     const int f16 = c->prec == MEM_PREC_FP16X3;
     // FP16X3: the weighted residual's maximum for the adjoint's operand scale
-    // (zeroed by the column-mean kernel)
+    // (zeroed by the operand preparation)
     float* ymax = (tc && f16 && mode == FWD_RESID) ? c->ymax : nullptr;
     if (tc) {
-        {
-            KTimer t(c, "colmean");
-            launch_colmean(d, src, f16, c->cmean, c->cscale, c->col_psum, c->col_pmax, c->col_count, ymax,
-                           entropy ? c->ent_part : nullptr, c->st);
-        }
-        {
+        double* ent = entropy ? c->ent_part : nullptr;
+        if (f16) {
             KTimer t(c, "prep");
-            if (f16) launch_fold(d, src, c->planes, c->cmean, c->cscale, c->st);
-            else launch_planes(d, src, c->planes, c->cmean, c->st);
+            launch_prep_fold(d, src, c->planes, c->cmean4, ymax, ent, c->st);
+            c->launches++;
+        } else {
+            {
+                KTimer t(c, "colmean");
+                launch_colmean(d, src, c->cmean, c->col_psum, c->col_count, ent, c->st);
+            }
+            KTimer t(c, "prep");
+            launch_planes(d, src, c->planes, c->cmean, c->st);
+            c->launches += 2;
         }
-        c->launches += 2;
         TRY(after_launch(c, "operand kernels"));
         const bool resident = c->fwd_kernel == MEM_FWD_RESIDENT;
         KTimer t(c, resident ? "fwd_rs" : "fwd_tc");
         if (f16) {
-            c->launches += launch_fwd_fold(d, resident, c->tiles, c->n_tiles, c->planes, c->cmean, c->cscale, mode,
-                                           (float2*)yout, c->chi_part, ymax, c->vpart, c->Z, c->num_sms, c->spin,
+            c->launches += launch_fwd_fold(d, resident, c->tiles, c->n_tiles, c->planes, c->cmean4, mode, (float2*)yout,
+                                           c->chi_part, ymax, c->vpart, c->Z, c->num_sms, c->spin,
                                            c->dstatus, c->st);
         } else if (resident) {
             launch_fwd_rs(d, c->tiles_tc, c->n_tiles_tc, c->planes, c->cmean, mode, (float2*)yout, c->chi_part,
@@ -543,7 +551,7 @@ mem_status run_objgrad(mem_ctx* c, const ImgSrc& src, int projected, float* out3
                                       c->st);
     } else {
         KTimer t(c, "finalize");
-        launch_finalize(c->dd(), src, c->gsum, ks, projected, out32, full64, proj64, c->st);
+        launch_finalize(c->dd(), src, is_tc(c->prec), c->gsum, ks, projected, out32, full64, proj64, c->st);
     }
     c->launches++;
     return after_launch(c, "gradient assembly");
@@ -1460,7 +1468,7 @@ mem_status mem_adjoint(mem_ctx* c, const float* y_dev, float* img_dev) {
     // the assembly reads pixel values only for the entropy term and projection;
     // give it the output buffer as a harmless source (lambda = 0, no projection)
     src.f32 = img_dev;
-    launch_finalize(d, src, c->gsum, ks, 0, img_dev, nullptr, nullptr, c->st);
+    launch_finalize(d, src, is_tc(c->prec), c->gsum, ks, 0, img_dev, nullptr, nullptr, c->st);
     c->launches++;
     return after_launch(c, "adjoint assembly");
 }

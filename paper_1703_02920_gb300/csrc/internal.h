@@ -32,7 +32,7 @@ struct DevData {
     int C;
     int n_images;
     int shared;          // 1: one image for all channels
-    double G;
+    double G, ginv;      // ginv = 1 / G
     double lambda;
     const uint64_t* pa;  // frac(u dx) as 64-bit fixed-point turns
     const uint64_t* pb;  // frac(v dy)
@@ -77,7 +77,7 @@ constexpr int VIS_TILE = 128;
 constexpr int TC_TILE = 64;
 constexpr int TC_BK = 32;
 __host__ __device__ inline int tc_bn(int N) { return N < 256 ? N : 256; }
-constexpr int MEAN_L = 16;  // folded columns l that share the operand's means
+constexpr int MEAN_L = 16;  // folded columns l that share the operand's means and scale
 // First column (P) of folded column l within a part: groups of eight P columns
 // followed by the eight Q columns of the same l (Q = P + 8).
 __host__ __device__ inline int fold_col(int l) { return 16 * (l / 8) + l % 8; }
@@ -96,25 +96,27 @@ void launch_phase_prep(int64_t Z, const double* u, const double* v, double dx, d
 // B_c = A_c * img(c) for every channel (direct forms); entropy partials S_i
 // per (image, block of 256 pixels) when ent_part != nullptr.
 void launch_prep(const DevData& d, const ImgSrc& src, int fmt, void* bout, double* ent_part, cudaStream_t st);
-// Tensor-core forms: the means that centre the operand.  fold = 0 (BF16X3): of
-// every column of B_c, cmean[C][N].  fold = 1 (FP16X3): of the folded operand
-// over all rows j and MEAN_L neighbouring l, (P, Q) pairs
-// cmean[C][2 parts][N/2/MEAN_L][2], and the channel's operand scale cscale[C]
-// (a power of two, from a bound on the folded operand).  psum (double) and pmax
-// (float) hold colmean_tmp_count(N, C) entries each; count holds C completion
-// counters, zero between calls (each call leaves them zero).  ymax_clear
-// (nullable) is set to zero.  ent_part (nullable): tc_ent_blocks(N) entropy
-// partials per image.
-void launch_colmean(const DevData& d, const ImgSrc& src, int fold, float* cmean, float* cscale, double* psum,
-                    float* pmax, unsigned* count, float* ymax_clear, double* ent_part, cudaStream_t st);
+// BF16X3: means of every column of B_c into cmean[C][N].  psum holds
+// colmean_tmp_count(N, C) entries; count holds C completion counters, zero
+// between calls (each call leaves them zero).  ent_part (nullable):
+// tc_ent_blocks(N) entropy partials per image.
+void launch_colmean(const DevData& d, const ImgSrc& src, float* cmean, double* psum, unsigned* count,
+                    double* ent_part, cudaStream_t st);
 int colmean_tmp_count(int N, int C);
 constexpr int COL_RB = 16;  // row blocks of the column sums
 __host__ __device__ inline int tc_ent_blocks(int N) { return (N + 31) / 32 * COL_RB; }
-// The centred operand split into 16-bit hi and lo planes in the forward
-// kernel's chunk layout: FP16X3 (folded, scaled by cscale) and BF16X3.
-void launch_fold(const DevData& d, const ImgSrc& src, void* planes, const float* cmean, const float* cscale,
-                 cudaStream_t st);
+// BF16X3: the centred operand split into 16-bit hi and lo planes in the
+// forward kernel's chunk layout.
 void launch_planes(const DevData& d, const ImgSrc& src, void* planes, const float* cmean, cudaStream_t st);
+// FP16X3: the folded operand, centred and scaled per strip of MEAN_L columns l,
+// split into planes; cmean[C][2 parts][N/2/MEAN_L] holds (P mean, Q mean, 1 /
+// scale).  ymax_clear (nullable) is set to zero.  ent_part (nullable):
+// fold_ent_blocks(N) entropy partials per image.
+void launch_prep_fold(const DevData& d, const ImgSrc& src, void* planes, float4* cmean, float* ymax_clear,
+                      double* ent_part, cudaStream_t st);
+// pixels per entropy partial of launch_prep_fold, partials per image
+__host__ __device__ inline int fold_ent_pixels(int N) { return N <= 256 ? 256 : 1024; }
+__host__ __device__ inline int fold_ent_blocks(int N) { return (N * N + fold_ent_pixels(N) - 1) / fold_ent_pixels(N); }
 // max |component| of n floats into ymax[0]; the FP16X3 adjoint scales y by
 // pow2_scale_for(ymax[0]).  The forward writes the same maximum of the y it
 // produces (RESID mode) when given ymax (zeroed before).
@@ -132,13 +134,13 @@ int adj_direct_splits(const DevData& d, int num_sms);
 // FP16X3 forward on the folded image: operand streamed (any N) or resident (N <=
 // 256).  For fold_combines(N) the resident form splits every tile over two
 // CTAs, whose partial sums (vpart, two float4 per visibility) a second kernel
-// adds.  Planes scaled by cscale[c].  ymax (nullable, RESID mode): max
+// adds.  planes and cmean from launch_prep_fold.  ymax (nullable, RESID mode): max
 // |component| of the weighted residual written to yout is combined into ymax[0]
 // (which the caller zeroes).  Returns the number of kernels launched.
 int fold_smem_bytes(int N, int BN, int stages, int resident);
 bool fold_combines(int N);
 int launch_fwd_fold(const DevData& d, int resident, const VisTile* tiles, int n_tiles, const void* planes,
-                    const float* cmean, const float* cscale, int mode, float2* yout, double* chi_part, float* ymax,
+                    const float4* cmean, int mode, float2* yout, double* chi_part, float* ymax,
                     float4* vpart, int64_t z_total, int num_sms, uint64_t spin, int* status, cudaStream_t st);
 // BF16X3 forward, streamed operand (TC_TILE tiles).
 int fwd_tc_smem_bytes(int N, int BN, int stages);
@@ -215,7 +217,8 @@ void launch_adj_tc_reduce_grad(const DevData& d, const ImgSrc& src, const int* c
                                cudaStream_t st);
 
 // grad_i = sum_{c in image i} A_c * sum_k gsum[k][c] + lambda (1 + log(I/G)); optional projection.
-void launch_finalize(const DevData& d, const ImgSrc& src, const double* gsum, int ks, int projected,
+// fast_log: log_ratio instead of the library's logarithm (tensor-core forms).
+void launch_finalize(const DevData& d, const ImgSrc& src, int fast_log, const double* gsum, int ks, int projected,
                      float* out32, double* full64, double* proj64, cudaStream_t st);
 
 // chi_part holds 4 partials per visibility tile (one per 32 visibilities),

@@ -506,7 +506,7 @@ __global__ void __launch_bounds__(RedGeo<WIDE>::THREADS) k_adj_fold_reduce(DevDa
         } else {
             double gr = (double)d.beam[pix] * gchi;
             const double x = img_value(src, c, (int64_t)n * N + m, NN);
-            if (d.lambda != 0.0) gr += d.lambda * (1.0 + log(x / d.G));
+            if (d.lambda != 0.0) gr += d.lambda * (1.0 + log_ratio(x, d.G, d.ginv));
             const double gp = (x <= d.G && gr > 0.0) ? 0.0 : gr;
             if (a.full64) a.full64[pix] = gr;
             if (a.proj64) a.proj64[pix] = gp;

@@ -20,7 +20,7 @@
 // Tas) and the eight Q columns (multiplied by y_l: Tsa or Taa) of the same l.
 //
 // The operand is centred, B' = B - cm, with one mean cm per column type over
-// all rows j and MEAN_L neighbouring l, and T = sum_j t_j B'_j + cm S with the
+// all rows j and MEAN_L neighbouring l (a strip, which also has a scale), and T = sum_j t_j B'_j + cm S with the
 // closed forms
 //   sum_j c_j = sin(pi N b) / (2 sin(pi b)),  sum_j y_j = -sin^2(pi N b / 2) / sin(pi b).
 // For low spatial frequencies the uncentred partial sums grow monotonically
@@ -198,13 +198,13 @@ __device__ __forceinline__ void finish_warp(float chi, float ym, int mode, doubl
     }
 }
 
-// The image planes are scaled by cscale[channel], a power of two undone in the
-// epilogue.
+// The operand's strips of MEAN_L columns l are scaled by powers of two, undone in
+// the epilogue.
 // STAGES: depth of the shared-memory pipeline (autotuned).
 template <int STAGES, int RES>
 __global__ void __launch_bounds__(FW_THREADS, 1)
     k_fwd_fold(DevData d, const VisTile* __restrict__ tiles, int n_tiles, const uint16_t* __restrict__ planes,
-             const float* __restrict__ cmean, const float* __restrict__ cscale, int mode,
+             const float4* __restrict__ cmean, int mode,
              float2* __restrict__ yout, double* __restrict__ chi_part, unsigned* __restrict__ ymax_bits,
              float4* __restrict__ vpart, int64_t z_total, uint64_t spin, int* status) {
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -561,23 +561,20 @@ __global__ void __launch_bounds__(FW_THREADS, 1)
         bool ok = true;
         const int e_begin = RES == RES_PART ? t_begin + grp : t_begin, e_step = RES == RES_PART ? 2 : t_step;
         uint32_t ti = 0;  // tiles of this group
-        // the next tile's descriptor, phases and operand scale arrive while
-        // this tile's accumulators drain
+        // the next tile's descriptor and phases arrive while this tile's
+        // accumulators drain
         VisTile tl_next = {};
         uint64_t pa_next = 0, pb_next = 0;
-        float osc_next = 1.f;
         auto load_tile = [&](int t) {
             tl_next = tiles[t];
             const int64_t jn = tl_next.start + (jv < tl_next.count ? jv : 0);
             pa_next = d.pa[jn];
             pb_next = d.pb[jn];
-            osc_next = cscale[tl_next.chan];  // operand scale (power of two)
         };
         if (e_begin < t_end) load_tile(e_begin);
         for (int t = e_begin; t < t_end && ok; t += e_step, ++ti) {
             const VisTile tl = tl_next;
             const uint64_t pb = pb_next;
-            const float osc = osc_next;
             const uint64_t pa = pa_next, ha = (uint64_t)((int64_t)pa >> 1);
             if (t + e_step < t_end) load_tile(t + e_step);
             cf2 step8;  // chunk to chunk (recurrence below)
@@ -595,10 +592,9 @@ __global__ void __launch_bounds__(FW_THREADS, 1)
                 if (part == 0) scomp = (sh != 0.f) ? 0.5f * sn / sh : 0.5f * (float)N;
                 else scomp = (sh != 0.f) ? -sn * sn / sh : 0.f;
             }
-            scomp *= osc;
-            // (P mean, Q mean) per MEAN_L folded columns, and the sum of the
-            // step factors over them times S
-            const float2* cm_part = (const float2*)cmean + ((int64_t)tl.chan * 2 + part) * (N / 2 / MEAN_L);
+            // (P mean, Q mean, 1 / scale) per strip of MEAN_L folded columns, and
+            // the sum of the step factors over them times S
+            const float4* cm_part = cmean + ((int64_t)tl.chan * 2 + part) * (N / 2 / MEAN_L);
             cf2 wsum;
             {
                 const float2 x = __fadd2_rn(__fadd2_rn(wx8.x[0], wx8.x[1]), __fadd2_rn(wx8.x[2], wx8.x[3]));
@@ -614,10 +610,12 @@ __global__ void __launch_bounds__(FW_THREADS, 1)
                 // the phase factor exp(-2 pi i (l0 + 1/2) a) of the block's first l
                 const cf2 base_mb = cis_neg_accurate(phase_hi(mb * BN + 1, ha));
                 for (int seg = 0; seg < n_seg; ++seg, ++it) {
-                    // the mean's term cm S enters once per column: with the
-                    // block's first segment only.  Lane i holds the i-th group's means.
-                    float2 cm = {0.f, 0.f};
-                    if (seg == 0 && lane < BN / (2 * MEAN_L)) cm = __ldg(cm_part + mb * (BN / (2 * MEAN_L)) + lane);
+                    // Lane i holds the i-th strip's means and inverse scale; the
+                    // mean's term cm S enters once per column: with the block's
+                    // first segment only.
+                    float4 cm = {0.f, 0.f, 0.f, 0.f};
+                    if (lane < BN / (2 * MEAN_L)) cm = __ldg(cm_part + mb * (BN / (2 * MEAN_L)) + lane);
+                    if (seg != 0) cm.x = cm.y = 0.f;
                     ok = __all_sync(0xffffffffu, mbar_wait(&S.tfull[b], it & 1, spin, abort, status, 32));
                     if (!ok) break;
                     tc_fence_after();
@@ -654,11 +652,15 @@ __global__ void __launch_bounds__(FW_THREADS, 1)
                         const cf2 bw = cmul(base, wsum);
                         x0 = fmaf(__shfl_sync(0xffffffffu, cm.x, q / 2), bw.x, x0);
                         x1 = fmaf(__shfl_sync(0xffffffffu, cm.y, q / 2), bw.y, x1);
-                        reduce_chunk(base, 0, x0, x1);
+                        // (a power of two: exact)
+                        const float inv = __shfl_sync(0xffffffffu, cm.z, q / 2);
+                        cf2 bs = {base.x * inv, base.y * inv};
+                        reduce_chunk(bs, 0, x0, x1);
                         tmem_ld_wait(tv[1]);
                         load_chunk(q + 2 < nq ? q + 2 : 0, 0);  // (the last one is not used)
                         base = cmul(base, step8);
-                        reduce_chunk(base, 1, x0, x1);
+                        bs = {base.x * inv, base.y * inv};
+                        reduce_chunk(bs, 1, x0, x1);
                         tmem_ld_wait(tv[0]);
                     };
                     // chunk phase factors: step8 from chunk to chunk, step32 over
@@ -684,9 +686,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1)
                 }
             }
             if (!ok) break;
-            // unscaled exactly (a power of two)
-            const float inv = 1.f / osc;
-            const float4 sums = make_float4(s0 * inv, c0s * inv, s1 * inv, c1s * inv);
+            const float4 sums = make_float4(s0, c0s, s1, c1s);
             if (RES == RES_PART) {
                 if (jv < tl.count) vpart[(int64_t)part * z_total + tl.start + jv] = sums;
                 continue;
@@ -729,7 +729,7 @@ struct FwdArgs {
     const VisTile* tiles;
     int n_tiles;
     const uint16_t* planes;
-    const float *cmean, *cscale;
+    const float4* cmean;
     int mode;
     float2* yout;
     double* chi_part;
@@ -750,14 +750,14 @@ void launch_variant(const FwdArgs& a, int grid) {
         return cudaFuncGetAttributes(&at, k_fwd_fold<STAGES, RES>) == cudaSuccess && at.numRegs == FW_REGS;
     }();
     if (!regs_ok) {  // a launch with no threads leaves an error for the caller's check
-        k_fwd_fold<STAGES, RES><<<grid, 0, 0, a.st>>>(a.d, a.tiles, a.n_tiles, a.planes, a.cmean, a.cscale, a.mode,
+        k_fwd_fold<STAGES, RES><<<grid, 0, 0, a.st>>>(a.d, a.tiles, a.n_tiles, a.planes, a.cmean, a.mode,
                                                         a.yout, a.chi_part, a.ymax_bits, a.vpart, a.z_total, a.spin,
                                                         a.status);
         return;
     }
     cudaFuncSetAttribute(k_fwd_fold<STAGES, RES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     k_fwd_fold<STAGES, RES><<<grid, FW_THREADS, smem, a.st>>>(a.d, a.tiles, a.n_tiles, a.planes, a.cmean,
-                                                                 a.cscale, a.mode, a.yout, a.chi_part, a.ymax_bits,
+                                                                 a.mode, a.yout, a.chi_part, a.ymax_bits,
                                                                  a.vpart, a.z_total, a.spin, a.status);
 }
 
@@ -788,10 +788,10 @@ int fold_smem_bytes(int N, int BN, int stages, int resident) {
 bool fold_combines(int N) { return resident_kind(N) == RES_PART; }
 
 int launch_fwd_fold(const DevData& d, int resident, const VisTile* tiles, int n_tiles, const void* planes,
-                  const float* cmean, const float* cscale, int mode, float2* yout, double* chi_part, float* ymax,
+                    const float4* cmean, int mode, float2* yout, double* chi_part, float* ymax,
                   float4* vpart, int64_t z_total, int num_sms, uint64_t spin, int* status, cudaStream_t st) {
     if (n_tiles <= 0) return 0;
-    const FwdArgs a{d,      tiles,   n_tiles,         (const uint16_t*)planes, cmean, cscale, mode, yout,
+    const FwdArgs a{d,      tiles,   n_tiles,         (const uint16_t*)planes, cmean, mode, yout,
                     chi_part, (unsigned*)ymax, vpart, z_total, spin, status, st};
     const int res = resident ? resident_kind(d.N) : RES_STREAM;
     // one CTA per SM, at most one per tile (RES_PART: a pair of CTAs per tile)

@@ -8,6 +8,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "logratio.cuh"
 #include "reduce.cuh"
 
 namespace msk {
@@ -49,35 +50,21 @@ __device__ __forceinline__ double block_max(double x, double* sh) {
     return r;
 }
 
-__device__ __forceinline__ int image_of(const DevData& d, int c) { return d.shared ? 0 : c; }
-
-
 // ---------------------------------------------------------------------------
-// a2, tensor-core forms: attenuation, centring and splitting of the forward's
-// operand.  FP16X3 folds it first (the fold is defined in kernels_fold.cu).
-//
-// Two kernels.  k_colsum forms the column sums of B = A I over the lower and
-// the upper half of the rows, from which the means follow, and for FP16X3 the
-// channel's operand scale.  k_fold (FP16X3) or k_planes (BF16X3) writes the
-// centred, split planes.
+// a2, BF16X3: attenuation, centring and splitting of the forward's operand
+// (FP16X3: kernels_fold_prep.cu).
 // ---------------------------------------------------------------------------
 
-// Column sums in two stages with a fixed summation order.  Stage 1: block
-// (column block of 32, row block rb of N/COL_RB rows, channel) -> partial sums
-// and max |B| per column (row blocks below COL_RB/2 lie in the lower half).
-// Stage 2, run by the channel's last stage-1 block to finish (a completion
-// counter per channel, which that block resets): for BF16X3 the column means
-// c_m; for FP16X3 the folded operand's means over the rows and MEAN_L
-// neighbouring columns l, then the bound max |B'| <= 2 (max|B| of the column and
-// of its mirror) + |cm| maximised over the channel, and from it the channel's
-// power-of-two FP16X3 operand scale.
-template <bool FOLD>
+// Column means c_m = (1/N) sum_n B[n][m] per channel (the operand of the
+// tensor-core forward is centred column by column, see k_fwd_tc), in two
+// stages with a fixed summation order.  Stage 1: block (column block of 32,
+// row block rb of N/COL_RB rows, channel) -> partial sums per column.  Stage
+// 2, run by the channel's last stage-1 block to finish (a completion counter
+// per channel, which that block resets): c_m.
 __global__ void __launch_bounds__(256) k_colsum(DevData d, ImgSrc src, double* __restrict__ psum,
-                                                float* __restrict__ pmax, unsigned* __restrict__ count,
-                                                float* __restrict__ cmean, float* __restrict__ cscale,
-                                                float* __restrict__ ymax_clear, double* __restrict__ ent_part) {
+                                                unsigned* __restrict__ count, float* __restrict__ cmean,
+                                                double* __restrict__ ent_part) {
     __shared__ double sh[8][33];
-    __shared__ float shm[8][33];
     __shared__ bool last;
     const int N = d.N;
     const int64_t NN = (int64_t)N * N;
@@ -86,31 +73,18 @@ __global__ void __launch_bounds__(256) k_colsum(DevData d, ImgSrc src, double* _
     const int lane = threadIdx.x & 31;
     const int m = blockIdx.x * 32 + lane;
     const int rg = threadIdx.x >> 5;
-    // the FP16X3 residual maximum of the forward that follows starts at zero
-    if (ymax_clear && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) *ymax_clear = 0.f;
     const int n0 = (int)((int64_t)N * rb / COL_RB), n1 = (int)((int64_t)N * (rb + 1) / COL_RB);
     // the entropy partial of an image is formed by its first channel only
     // (the others would repeat it in the shared-image mode)
     const bool ent = ent_part && !(d.shared && c != 0);
     double acc = 0.0, e = 0.0;
-    float amax = 0.f;
     if (m < N) {
         for (int n = n0 + rg; n < n1; n += 8) {
             const int64_t p = (int64_t)n * N + m;
             double x = img_value(src, i, p, NN);
-            if (src.diff) {
-                // line-search probe as a difference from the base image I: the
-                // operand is delta = max(I + alpha d, G) - I, the entropy term
-                // the change of sum x log(x/G)
-                const double x0 = src.f64[(int64_t)i * NN + p];
-                if (ent) e += x * log(x / src.G) - x0 * log(x0 / src.G);
-                x -= x0;
-            } else if (ent) {
-                e += x * log(x / src.G);
-            }
-            const double b = (double)d.beam[(int64_t)c * NN + p] * x;
-            acc += b;
-            amax = fmaxf(amax, (float)fabs(b));
+            if (ent) e += entropy_term(d, src, x, (int64_t)i * NN + p);
+            if (src.diff) x -= src.f64[(int64_t)i * NN + p];
+            acc += (double)d.beam[(int64_t)c * NN + p] * x;
         }
     }
     if (ent) {  // uniform over the block
@@ -119,17 +93,11 @@ __global__ void __launch_bounds__(256) k_colsum(DevData d, ImgSrc src, double* _
             ent_part[(int64_t)i * gridDim.x * gridDim.y + (int64_t)rb * gridDim.x + blockIdx.x] = -s;
     }
     sh[rg][lane] = acc;
-    shm[rg][lane] = amax;
     __syncthreads();
     if (rg == 0 && m < N) {
         double t = 0.0;
-        float mx = 0.f;
-        for (int k = 0; k < 8; ++k) {
-            t += sh[k][lane];
-            mx = fmaxf(mx, shm[k][lane]);
-        }
+        for (int k = 0; k < 8; ++k) t += sh[k][lane];
         psum[((int64_t)c * COL_RB + rb) * N + m] = t;
-        pmax[((int64_t)c * COL_RB + rb) * N + m] = mx;
         __threadfence();  // each writer's partials visible device-wide before the count below
     }
     __syncthreads();
@@ -138,129 +106,21 @@ __global__ void __launch_bounds__(256) k_colsum(DevData d, ImgSrc src, double* _
     if (!last) return;
     __threadfence();
     // stage 2: the partials of channel c in row-block order (read through L2)
-    if (!FOLD) {
-        for (int mm = threadIdx.x; mm < N; mm += blockDim.x) {
-            double t = 0.0;
+    for (int mm = threadIdx.x; mm < N; mm += blockDim.x) {
+        double t = 0.0;
 #pragma unroll
-            for (int r = 0; r < COL_RB; ++r) t += __ldcg(psum + ((int64_t)c * COL_RB + r) * N + mm);
-            cmean[(int64_t)c * N + mm] = (float)(t / N);
-        }
-        if (threadIdx.x == 0) count[c] = 0;  // ready for the next evaluation
-        return;
+        for (int r = 0; r < COL_RB; ++r) t += __ldcg(psum + ((int64_t)c * COL_RB + r) * N + mm);
+        cmean[(int64_t)c * N + mm] = (float)(t / N);
     }
-    // one thread per mirror pair of columns
-    float bound = 0.f;
-    const double inv = 2.0 / ((double)N * MEAN_L);
-    for (int l = threadIdx.x; l < N / 2; l += blockDim.x) {
-        double lo[2] = {0.0, 0.0}, up[2] = {0.0, 0.0};  // [column, mirror]: lower and upper rows
-        float mx[2] = {0.f, 0.f};
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int mm = h ? N / 2 - 1 - l : N / 2 + l;
-#pragma unroll
-            for (int r = 0; r < COL_RB; ++r) {
-                const double q = __ldcg(psum + ((int64_t)c * COL_RB + r) * N + mm);
-                if (r < COL_RB / 2) lo[h] += q;
-                else up[h] += q;
-                mx[h] = fmaxf(mx[h], __ldcg(pmax + ((int64_t)c * COL_RB + r) * N + mm));
-            }
-        }
-        // MEAN_L consecutive lanes hold one group (N/2 is a multiple of 32)
-        auto group_mean = [&](double x) {
-#pragma unroll
-            for (int o = MEAN_L / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-            return (float)(x * inv);
-        };
-        const float ss = group_mean(up[0] + lo[0] + up[1] + lo[1]);
-        const float sa = group_mean(up[0] + lo[0] - up[1] - lo[1]);
-        const float as = group_mean(up[0] - lo[0] + up[1] - lo[1]);
-        const float aa = group_mean(up[0] - lo[0] - up[1] + lo[1]);
-        if (l % MEAN_L == 0) {
-            float2* cm = (float2*)cmean + (int64_t)c * (N / MEAN_L) + l / MEAN_L;
-            cm[0] = make_float2(ss, sa);
-            cm[N / 2 / MEAN_L] = make_float2(as, aa);
-        }
-        const float cmax = fmaxf(fmaxf(fabsf(ss), fabsf(sa)), fmaxf(fabsf(as), fabsf(aa)));
-        bound = fmaxf(bound, 2.f * (mx[0] + mx[1]) + cmax);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) bound = fmaxf(bound, __shfl_down_sync(0xffffffffu, bound, o));
-    if (lane == 0) shm[0][rg] = bound;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float mx = 0.f;
-        for (int k = 0; k < 8; ++k) mx = fmaxf(mx, shm[0][k]);
-        cscale[c] = pow2_scale_for(mx);
-        count[c] = 0;  // ready for the next evaluation
-    }
+    if (threadIdx.x == 0) count[c] = 0;  // ready for the next evaluation
 }
 
-void launch_colmean(const DevData& d, const ImgSrc& src, int fold, float* cmean, float* cscale, double* psum,
-                    float* pmax, unsigned* count, float* ymax_clear, double* ent_part, cudaStream_t st) {
-    const dim3 grid((d.N + 31) / 32, COL_RB, d.C);
-    if (fold)
-        k_colsum<true><<<grid, 256, 0, st>>>(d, src, psum, pmax, count, cmean, cscale, ymax_clear, ent_part);
-    else
-        k_colsum<false><<<grid, 256, 0, st>>>(d, src, psum, pmax, count, cmean, cscale, ymax_clear, ent_part);
+void launch_colmean(const DevData& d, const ImgSrc& src, float* cmean, double* psum, unsigned* count,
+                    double* ent_part, cudaStream_t st) {
+    k_colsum<<<dim3((d.N + 31) / 32, COL_RB, d.C), 256, 0, st>>>(d, src, psum, count, cmean, ent_part);
 }
 
 int colmean_tmp_count(int N, int C) { return COL_RB * N * C; }
-
-// One block folds 8 rows j by 32 columns l: thread (warp: j, lane: l) reads the
-// four mirror pixels (coalesced along the row, two of the reads reversed),
-// forms the four sums and splits them into a shared-memory tile whose 16-byte
-// rows (8 consecutive j of one column) are then stored, four whole core
-// matrices per column type.  Chunk layout of the planes: chunk (column block
-// mb, part, row stage ks) of BN columns x TC_BK rows, K-major interleaved 8 x 8
-// core matrices, hi plane then lo plane.
-__global__ void __launch_bounds__(256) k_fold(DevData d, ImgSrc src, uint16_t* __restrict__ planes,
-                                              const float* __restrict__ cmean, const float* __restrict__ cscale) {
-    __shared__ __align__(16) uint16_t sp[4][2][32][8];  // column type, hi / lo, l, j
-    const int N = d.N, M = N / 2, BN = d.fwd_bn, nk = M / TC_BK;
-    const int64_t NN = (int64_t)N * N;
-    const int c = blockIdx.z;
-    const int i = image_of(d, c);
-    const int jl = threadIdx.x >> 5, ll = threadIdx.x & 31;
-    const int j0 = blockIdx.y * 8, l0 = blockIdx.x * 32;
-    const int j = j0 + jl, l = l0 + ll;
-    const float* A = d.beam + (int64_t)c * NN;
-    auto pixel = [&](int n, int m) {
-        const int64_t p = (int64_t)n * N + m;
-        double x = img_value(src, i, p, NN);
-        if (src.diff) x -= src.f64[(int64_t)i * NN + p];
-        return (double)A[p] * x;
-    };
-    const double pp = pixel(M + j, M + l), pm = pixel(M + j, M - 1 - l);
-    const double mp = pixel(M - 1 - j, M + l), mm = pixel(M - 1 - j, M - 1 - l);
-    const double sp0 = pp + mp, sp1 = pm + mm, sm0 = pp - mp, sm1 = pm - mm;  // over the rows
-    const double f[4] = {sp0 + sp1, sp0 - sp1, sm0 + sm1, sm0 - sm1};        // ss, sa, as, aa
-    const float2* cm = (const float2*)cmean + (int64_t)c * (N / MEAN_L) + l / MEAN_L;
-    const float2 cs = cm[0], cy = cm[N / 2 / MEAN_L];
-    const float mean[4] = {cs.x, cs.y, cy.x, cy.y};
-    const double sc = (double)cscale[c];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const float v = (float)((f[k] - (double)mean[k]) * sc);
-        uint32_t hi, lo;
-        split_f16x2(v, 0.f, hi, lo);
-        sp[k][0][ll][jl] = (uint16_t)hi;
-        sp[k][1][ll][jl] = (uint16_t)lo;
-    }
-    __syncthreads();
-    // thread -> one 16-byte row: column type, plane, l
-    const int k = threadIdx.x >> 6, pl = (threadIdx.x >> 5) & 1;
-    const int col = fold_col(l0 + ll) + (k & 1) * 8;
-    const int mb = col / BN, r = col % BN, ks = j0 / TC_BK, kk = j0 % TC_BK;
-    const int64_t chunk = (int64_t)(2 * mb + (k >> 1)) * nk + ks;
-    uint16_t* dst = planes + (int64_t)c * 2 * NN + chunk * 2 * BN * TC_BK + (int64_t)pl * BN * TC_BK +
-                    ((int64_t)(kk / 8) * (BN / 8) + r / 8) * 64 + (r % 8) * 8;
-    *(uint4*)dst = *(const uint4*)sp[k][pl][ll];
-}
-
-void launch_fold(const DevData& d, const ImgSrc& src, void* planes, const float* cmean, const float* cscale,
-                 cudaStream_t st) {
-    k_fold<<<dim3(d.N / 64, d.N / 16, d.C), 256, 0, st>>>(d, src, (uint16_t*)planes, cmean, cscale);
-}
 
 // BF16X3: B - c_m as hi / lo planes, per channel chunks (m-block mb, n-stage
 // ks) of BN x BK elements, K-major interleaved 8x8 core matrices, hi plane then
@@ -542,6 +402,7 @@ void launch_adj_direct(const DevData& d, int fp64, const void* y, double* gsum, 
 // factor; Eq. chi2-multi for a shared image), plus lambda (1 + log(I/G))
 // (Eq. Sgradient), then the positive projection at the bound I = G.
 // ---------------------------------------------------------------------------
+template <bool FAST_LOG>
 __global__ void __launch_bounds__(256) k_finalize(DevData d, ImgSrc src,
                                                   const double* __restrict__ gsum, int ks,
                                                   int projected, float* out32, double* full64,
@@ -559,17 +420,18 @@ __global__ void __launch_bounds__(256) k_finalize(DevData d, ImgSrc src,
         g += (double)d.beam[(int64_t)c * NN + p] * s;
     }
     double x = img_value(src, i, p, NN);
-    if (d.lambda != 0.0) g += d.lambda * (1.0 + log(x / d.G));
+    if (d.lambda != 0.0) g += d.lambda * (1.0 + (FAST_LOG ? log_ratio(x, d.G, d.ginv) : log(x / d.G)));
     double gp = (x <= d.G && g > 0.0) ? 0.0 : g;
     if (full64) full64[(int64_t)i * NN + p] = g;
     if (proj64) proj64[(int64_t)i * NN + p] = gp;
     if (out32) out32[(int64_t)i * NN + p] = (float)(projected ? gp : g);
 }
 
-void launch_finalize(const DevData& d, const ImgSrc& src, const double* gsum, int ks, int projected,
+void launch_finalize(const DevData& d, const ImgSrc& src, int fast_log, const double* gsum, int ks, int projected,
                      float* out32, double* full64, double* proj64, cudaStream_t st) {
     dim3 grid(prep_blocks(d.N), d.n_images);
-    k_finalize<<<grid, 256, 0, st>>>(d, src, gsum, ks, projected, out32, full64, proj64);
+    if (fast_log) k_finalize<true><<<grid, 256, 0, st>>>(d, src, gsum, ks, projected, out32, full64, proj64);
+    else k_finalize<false><<<grid, 256, 0, st>>>(d, src, gsum, ks, projected, out32, full64, proj64);
 }
 
 // ---------------------------------------------------------------------------

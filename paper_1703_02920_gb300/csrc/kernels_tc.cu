@@ -548,7 +548,7 @@ __global__ void __launch_bounds__(256) k_adj_tc_reduce_grad(DevData d, ImgSrc sr
     const double gchi = (double)tot;
     double gr = (double)d.beam[(int64_t)c * NN + p] * gchi;
     const double x = img_value(src, c, p, NN);
-    if (d.lambda != 0.0) gr += d.lambda * (1.0 + log(x / d.G));
+    if (d.lambda != 0.0) gr += d.lambda * (1.0 + log_ratio(x, d.G, d.ginv));
     const double gp = (x <= d.G && gr > 0.0) ? 0.0 : gr;
     if (full64) full64[(int64_t)c * NN + p] = gr;
     if (proj64) proj64[(int64_t)c * NN + p] = gp;

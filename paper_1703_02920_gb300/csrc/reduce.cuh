@@ -7,6 +7,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "logratio.cuh"
 
 namespace msk {
 
@@ -26,6 +27,20 @@ __device__ __forceinline__ double block_sum(double x, double* sh) {
     }
     __syncthreads();
     return r;  // valid in thread 0
+}
+
+__device__ __forceinline__ int image_of(const DevData& d, int c) { return d.shared ? 0 : c; }
+
+// x log(x/G) of the pixel at flat index q (value x); for a line-search probe,
+// whose operand is the difference max(I + alpha d, G) - I, the change against
+// the base image.
+__device__ __forceinline__ double entropy_term(const DevData& d, const ImgSrc& src, double x, int64_t q) {
+    double e = x * log_ratio(x, d.G, d.ginv);
+    if (src.diff) {
+        const double x0 = src.f64[q];
+        e -= x0 * log_ratio(x0, d.G, d.ginv);
+    }
+    return e;
 }
 
 // ---------------------------------------------------------------------------
