@@ -73,7 +73,8 @@ typedef enum {
  * u x + v y are always reduced exactly (64-bit fixed-point turns obtained
  * from an FP64 reduction of u dx and v dy). */
 typedef enum {
-    MEM_PREC_FP64_DIRECT = 0,  /* one FP64 exponential per (visibility, pixel) pair */
+    MEM_PREC_FP64_DIRECT = 0,  /* direct sums, every product and sum in FP64 (row and column
+                                  phase factors, mirror pixels sharing them) */
     MEM_PREC_FP32_DIRECT = 1,  /* one FP32 (SFU) exponential per pair, FP64 partial sums */
     MEM_PREC_BF16X3 = 2,       /* separable phase tables generated on chip, tcgen05
                                   tensor-core contractions in 3-term split BF16 with FP32

@@ -13,7 +13,7 @@ CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libmemsynth.so")
 SOURCES = ["api.cu", "kernels_simt.cu", "kernels_tc.cu", "kernels_fwd.cu", "kernels_fwd_rs.cu",
-           "kernels_fold_prep.cu", "kernels_fold.cu", "kernels_adj_fold.cu", "noalloc.cu", "solver.cu",
+           "kernels_f64.cu", "kernels_fold_prep.cu", "kernels_fold.cu", "kernels_adj_fold.cu", "noalloc.cu", "solver.cu",
            "gridded.cu"]
 HEADERS = ["common.cuh", "internal.h", "logratio.cuh", "reduce.cuh", "solver.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

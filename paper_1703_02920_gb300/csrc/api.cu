@@ -75,6 +75,7 @@ struct mem_ctx {
     int gsum_ks = 0;
     float* bf32 = nullptr;
     double* bf64 = nullptr;
+    double2* wpart64 = nullptr;  // FP64 forward: sums per share of the work
     uint16_t* planes = nullptr;
     float* cmean = nullptr;  // means of the centred tensor-core operand
     float4* cmean4 = nullptr;                   // FP16X3: means and inverse scale per strip
@@ -359,6 +360,12 @@ mem_status after_launch(mem_ctx* c, const char* what) {
     return MEM_OK;
 }
 
+// Visibility shares of the adjoint in the forms whose sums go through gsum.
+int adj_splits(const mem_ctx* c) {
+    return c->prec == MEM_PREC_FP64_DIRECT ? f64_adj_splits(c->dd(), c->num_sms)
+                                           : adj_direct_splits(c->dd(), c->num_sms);
+}
+
 // Buffers needed by the current precision.
 mem_status ensure_buffers(mem_ctx* c) {
     const size_t NN = (size_t)c->N * c->N;
@@ -373,7 +380,9 @@ mem_status ensure_buffers(mem_ctx* c) {
     TRY(dalloc(c, &c->y32, (size_t)std::max<int64_t>(c->Z, 1)));
     if (c->prec == MEM_PREC_FP64_DIRECT) {
         TRY(dalloc(c, &c->y64, (size_t)std::max<int64_t>(c->Z, 1)));
-        TRY(dalloc(c, &c->bf64, (size_t)c->C * NN));
+        TRY(dalloc(c, &c->bf64, (size_t)c->C * f64_operand_doubles(c->N)));
+        const int shares = f64_shares(c->N, c->n_tiles, c->num_sms);
+        if (shares > 1) TRY(dalloc(c, &c->wpart64, (size_t)shares * std::max<int64_t>(c->Z, 1)));
     } else if (c->prec == MEM_PREC_FP32_DIRECT) {
         TRY(dalloc(c, &c->bf32, (size_t)c->C * NN));
     } else {
@@ -396,7 +405,7 @@ mem_status ensure_buffers(mem_ctx* c) {
             TRY(dalloc(c, &c->vpart, (size_t)2 * std::max<int64_t>(c->Z, 1)));
     }
     int ks = 1;
-    if (!is_tc(c->prec)) ks = adj_direct_splits(c->dd(), c->num_sms);
+    if (!is_tc(c->prec)) ks = adj_splits(c);
     if (ks > c->gsum_ks) {
         // grow: the old block stays allocated until destroy (rare)
         c->gsum = nullptr;
@@ -406,14 +415,13 @@ mem_status ensure_buffers(mem_ctx* c) {
     return MEM_OK;
 }
 
-void* bbuf(mem_ctx* c) { return c->prec == MEM_PREC_FP64_DIRECT ? (void*)c->bf64 : (void*)c->bf32; }
-
 // tile list that the form's forward ran over (4 chi^2 partials per tile)
 const int* fwd_tile_off(const mem_ctx* c) { return c->prec == MEM_PREC_BF16X3 ? c->tile_off_tc : c->tile_off; }
 
 int ent_blocks(const mem_ctx* c) {
     return c->prec == MEM_PREC_FP16X3   ? fold_ent_blocks(c->N)
-           : c->prec == MEM_PREC_BF16X3 ? tc_ent_blocks(c->N) : prep_blocks(c->N);
+           : c->prec == MEM_PREC_BF16X3 ? tc_ent_blocks(c->N)
+           : c->prec == MEM_PREC_FP64_DIRECT ? f64_ent_blocks(c->N) : prep_blocks(c->N);
 }
 
 // prep + forward for one image source.  mode: FwdMode.  defer_scalars: the
@@ -458,16 +466,23 @@ mem_status run_forward(mem_ctx* c, const ImgSrc& src, int mode, bool entropy, vo
             if (c->n_tiles_tc > 0) c->launches++;
         }
     } else {
-        const int f64 = c->prec == MEM_PREC_FP64_DIRECT;
+        const bool f64 = c->prec == MEM_PREC_FP64_DIRECT;
+        double* ent = entropy ? c->ent_part : nullptr;
         {
             KTimer t(c, "prep");
-            launch_prep(d, src, f64 ? BF_F64 : BF_F32, bbuf(c), entropy ? c->ent_part : nullptr, c->st);
+            if (f64) launch_prep_f64(d, src, c->bf64, ent, c->st);
+            else launch_prep(d, src, c->bf32, ent, c->st);
         }
         c->launches++;
         TRY(after_launch(c, "prep kernel"));
         KTimer t(c, f64 ? "fwd_direct_f64" : "fwd_direct_f32");
-        launch_fwd_direct(d, f64, c->tiles, c->n_tiles, bbuf(c), mode, yout, c->chi_part, c->st);
-        if (c->n_tiles > 0) c->launches++;
+        if (f64) {
+            c->launches += launch_fwd_f64(d, c->tiles, c->n_tiles, c->bf64, mode, (double2*)yout, c->chi_part,
+                                          c->wpart64, f64_shares(c->N, c->n_tiles, c->num_sms), c->Z, c->st);
+        } else {
+            launch_fwd_direct(d, c->tiles, c->n_tiles, c->bf32, mode, (float2*)yout, c->chi_part, c->st);
+            if (c->n_tiles > 0) c->launches++;
+        }
     }
     TRY(after_launch(c, "forward kernel"));
     if (mode != FWD_VIS && !defer_scalars) {
@@ -511,10 +526,10 @@ mem_status run_adjoint(mem_ctx* c, int* ks_out, bool ymax_ready = false, bool re
         TRY(after_launch(c, "adjoint reduction"));
         *ks_out = 1;
     } else {
-        int ks = adj_direct_splits(d, c->num_sms);
-        const void* y = c->prec == MEM_PREC_FP64_DIRECT ? (const void*)c->y64 : (const void*)c->y32;
+        int ks = adj_splits(c);
         KTimer t(c, c->prec == MEM_PREC_FP64_DIRECT ? "adj_direct_f64" : "adj_direct_f32");
-        launch_adj_direct(d, c->prec == MEM_PREC_FP64_DIRECT, y, c->gsum, ks, c->st);
+        if (c->prec == MEM_PREC_FP64_DIRECT) launch_adj_f64(d, c->y64, c->gsum, ks, c->st);
+        else launch_adj_direct(d, c->y32, c->gsum, ks, c->st);
         c->launches++;
         TRY(after_launch(c, "adjoint kernel"));
         *ks_out = ks;

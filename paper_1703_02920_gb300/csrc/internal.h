@@ -62,7 +62,6 @@ struct ImgSrc {
     int diff;             // operand is max(I + alpha d, G) - I, entropy as a difference
 };
 
-enum BFormat { BF_F32 = 0, BF_F64 = 1 };
 // FWD_VIS: write V.  FWD_RESID: write y = w (V - V^o), chi^2 partials.
 // FWD_CHI: chi^2 partials only.  FWD_CURV: 1/2 w |V|^2 partials.
 // FWD_DCHI: chi^2 change for an operand that is an image difference delta,
@@ -93,9 +92,9 @@ void set_global_error(const char* msg);
 void launch_phase_prep(int64_t Z, const double* u, const double* v, double dx, double dy,
                        uint64_t* pa, uint64_t* pb, cudaStream_t st);
 
-// B_c = A_c * img(c) for every channel (direct forms); entropy partials S_i
+// FP32 direct form: B_c = A_c * img(c) for every channel; entropy partials S_i
 // per (image, block of 256 pixels) when ent_part != nullptr.
-void launch_prep(const DevData& d, const ImgSrc& src, int fmt, void* bout, double* ent_part, cudaStream_t st);
+void launch_prep(const DevData& d, const ImgSrc& src, float* bout, double* ent_part, cudaStream_t st);
 // BF16X3: means of every column of B_c into cmean[C][N].  psum holds
 // colmean_tmp_count(N, C) entries; count holds C completion counters, zero
 // between calls (each call leaves them zero).  ent_part (nullable):
@@ -123,12 +122,24 @@ __host__ __device__ inline int fold_ent_blocks(int N) { return (N * N + fold_ent
 void launch_absmax(int64_t n, const float* y, float* part, float* ymax, cudaStream_t st);
 __host__ __device__ inline int prep_blocks(int N) { return (int)(((int64_t)N * N + 255) / 256); }
 
-void launch_fwd_direct(const DevData& d, int fp64, const VisTile* tiles, int n_tiles, const void* B,
-                       int mode, void* yout, double* chi_part, cudaStream_t st);
+void launch_fwd_direct(const DevData& d, const VisTile* tiles, int n_tiles, const float* B, int mode, float2* yout,
+                       double* chi_part, cudaStream_t st);
 // gsum: [ks][C][N*N] doubles, per-channel sums without the beam factor.
-void launch_adj_direct(const DevData& d, int fp64, const void* y, double* gsum, int ks,
-                       cudaStream_t st);
+void launch_adj_direct(const DevData& d, const float2* y, double* gsum, int ks, cudaStream_t st);
 int adj_direct_splits(const DevData& d, int num_sms);
+
+// FP64 form, folded (kernels_f64.cu).  Operand: f64_operand_doubles(N) per
+// channel; f64_ent_blocks(N) entropy partials per image.  The forward cuts a
+// tile's work into f64_shares(...) shares, whose sums (wpart[share][Z], needed
+// for more than one) a second kernel adds; returns the launches.
+int64_t f64_operand_doubles(int N);
+int f64_ent_blocks(int N);
+int f64_shares(int N, int n_tiles, int num_sms);
+int f64_adj_splits(const DevData& d, int num_sms);
+void launch_prep_f64(const DevData& d, const ImgSrc& src, double* B, double* ent_part, cudaStream_t st);
+int launch_fwd_f64(const DevData& d, const VisTile* tiles, int n_tiles, const double* B, int mode, double2* yout,
+                   double* chi_part, double2* wpart, int shares, int64_t z_total, cudaStream_t st);
+void launch_adj_f64(const DevData& d, const double2* y, double* gsum, int ks, cudaStream_t st);
 
 // Tensor-core forms.
 // FP16X3 forward on the folded image: operand streamed (any N) or resident (N <=

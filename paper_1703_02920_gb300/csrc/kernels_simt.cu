@@ -1,6 +1,6 @@
 // SIMT kernels of libmemsynth: per-visibility phase preparation, the
-// attenuation/operand preparation, the plain direct-sum operator pair in FP64
-// and FP32 (one exponential per visibility-pixel pair, the comparators of the
+// BF16X3 and FP32 operand preparation, the plain direct-sum operator pair in
+// FP32 (one exponential per visibility-pixel pair, the comparator of the
 // tensor-core form), gradient assembly with the entropy term and positivity
 // projection, ordered FP64 reductions and the CG vector updates.
 #include <cmath>
@@ -187,9 +187,8 @@ void launch_absmax(int64_t n, const float* y, float* part, float* ymax, cudaStre
     k_absmax_final<<<1, 32, 0, st>>>(part, ymax);
 }
 
-// a2, direct forms: B_c = A_c I in the form's precision.
-template <typename T>
-__global__ void __launch_bounds__(256) k_prep(DevData d, ImgSrc src, T* __restrict__ bout, double* ent_part) {
+// a2, FP32 direct form: B_c = A_c I.
+__global__ void __launch_bounds__(256) k_prep(DevData d, ImgSrc src, float* __restrict__ bout, double* ent_part) {
     __shared__ double sh[8];
     const int N = d.N;
     const int64_t NN = (int64_t)N * N;
@@ -208,7 +207,7 @@ __global__ void __launch_bounds__(256) k_prep(DevData d, ImgSrc src, T* __restri
         } else if (ent) {
             e = x * log(x / src.G);
         }
-        bout[(int64_t)c * NN + p] = (T)((double)d.beam[(int64_t)c * NN + p] * xb);
+        bout[(int64_t)c * NN + p] = (float)((double)d.beam[(int64_t)c * NN + p] * xb);
     }
     if (ent) {  // uniform over the block (one channel per block row)
         double s = block_sum<256>(e, sh);
@@ -216,10 +215,8 @@ __global__ void __launch_bounds__(256) k_prep(DevData d, ImgSrc src, T* __restri
     }
 }
 
-void launch_prep(const DevData& d, const ImgSrc& src, int fmt, void* bout, double* ent_part, cudaStream_t st) {
-    dim3 grid(prep_blocks(d.N), d.C);
-    if (fmt == BF_F64) k_prep<double><<<grid, 256, 0, st>>>(d, src, (double*)bout, ent_part);
-    else k_prep<float><<<grid, 256, 0, st>>>(d, src, (float*)bout, ent_part);
+void launch_prep(const DevData& d, const ImgSrc& src, float* bout, double* ent_part, cudaStream_t st) {
+    k_prep<<<dim3(prep_blocks(d.N), d.C), 256, 0, st>>>(d, src, bout, ent_part);
 }
 
 // ---------------------------------------------------------------------------
@@ -229,30 +226,22 @@ void launch_prep(const DevData& d, const ImgSrc& src, int fmt, void* bout, doubl
 // Fused epilogue (Algorithm 2 + the reduction of Algorithm 1): residual,
 // weight, chi^2 tile partial.
 // ---------------------------------------------------------------------------
-template <typename T>
-__device__ __forceinline__ void cis_minus(uint64_t p, T& c, T& s);
-template <>
-__device__ __forceinline__ void cis_minus<float>(uint64_t p, float& c, float& s) {
+__device__ __forceinline__ void cis_minus(uint64_t p, float& c, float& s) {
     __sincosf(phase_to_angle_f32(p), &s, &c);
 }
-template <>
-__device__ __forceinline__ void cis_minus<double>(uint64_t p, double& c, double& s) {
-    sincospi(2.0 * phase_to_turns_f64(p), &s, &c);
-}
 
-template <typename T>
 __global__ void __launch_bounds__(128) k_fwd_direct(DevData d, const VisTile* __restrict__ tiles,
-                                                    const T* __restrict__ B, int mode, void* yout,
+                                                    const float* __restrict__ B, int mode, float2* yout,
                                                     double* __restrict__ chi_part) {
     extern __shared__ __align__(16) unsigned char smraw[];
-    T* row = (T*)smraw;
+    float* row = (float*)smraw;
     const VisTile t = tiles[blockIdx.x];
     const int N = d.N, c0 = N / 2;
     const int64_t NN = (int64_t)N * N;
     const bool valid = (int)threadIdx.x < t.count;
     const int64_t j = t.start + (valid ? threadIdx.x : 0);
     const uint64_t a = d.pa[j], b = d.pb[j];
-    const T* Bc = B + (int64_t)t.chan * NN;
+    const float* Bc = B + (int64_t)t.chan * NN;
     double re = 0.0, im = 0.0;
     const uint64_t pstart = phase_mul(-c0, a);
     for (int n = 0; n < N; ++n) {
@@ -260,11 +249,11 @@ __global__ void __launch_bounds__(128) k_fwd_direct(DevData d, const VisTile* __
         for (int m = threadIdx.x; m < N; m += 128) row[m] = Bc[(int64_t)n * N + m];
         __syncthreads();
         uint64_t p = pstart + phase_mul(n - c0, b);
-        T rr = 0, ri = 0;
+        float rr = 0, ri = 0;
         for (int m = 0; m < N; ++m) {
-            T cs, sn;
-            cis_minus<T>(p, cs, sn);
-            T bv = row[m];
+            float cs, sn;
+            cis_minus(p, cs, sn);
+            float bv = row[m];
             rr += bv * cs;
             ri -= bv * sn;
             p += a;
@@ -275,21 +264,17 @@ __global__ void __launch_bounds__(128) k_fwd_direct(DevData d, const VisTile* __
     double chi = 0.0;
     if (valid) {
         if (mode == FWD_VIS) {
-            if (sizeof(T) == 8) ((double2*)yout)[j] = make_double2(re, im);
-            else ((float2*)yout)[j] = make_float2((float)re, (float)im);
+            yout[j] = make_float2((float)re, (float)im);
         } else if (mode == FWD_DCHI) {
-            double yr, yi;
-            if (sizeof(T) == 8) { double2 q = ((const double2*)yout)[j]; yr = q.x; yi = q.y; }
-            else { float2 q = ((const float2*)yout)[j]; yr = q.x; yi = q.y; }
-            chi = yr * re + yi * im + 0.5 * d.w[j] * (re * re + im * im);
+            const float2 q = yout[j];
+            chi = (double)q.x * re + (double)q.y * im + 0.5 * d.w[j] * (re * re + im * im);
         } else {
             double rr = re, ri = im;
             if (mode != FWD_CURV) { rr -= d.vo[j].x; ri -= d.vo[j].y; }
             double w = d.w[j];
             chi = 0.5 * w * (rr * rr + ri * ri);
             if (mode == FWD_RESID) {
-                if (sizeof(T) == 8) ((double2*)yout)[j] = make_double2(w * rr, w * ri);
-                else ((float2*)yout)[j] = make_float2((float)(w * rr), (float)(w * ri));
+                yout[j] = make_float2((float)(w * rr), (float)(w * ri));
             }
         }
     }
@@ -301,16 +286,10 @@ __global__ void __launch_bounds__(128) k_fwd_direct(DevData d, const VisTile* __
     }
 }
 
-void launch_fwd_direct(const DevData& d, int fp64, const VisTile* tiles, int n_tiles, const void* B,
-                       int mode, void* yout, double* chi_part, cudaStream_t st) {
+void launch_fwd_direct(const DevData& d, const VisTile* tiles, int n_tiles, const float* B, int mode, float2* yout,
+                       double* chi_part, cudaStream_t st) {
     if (n_tiles <= 0) return;
-    if (fp64) {
-        k_fwd_direct<double><<<n_tiles, 128, d.N * sizeof(double), st>>>(d, tiles, (const double*)B,
-                                                                        mode, yout, chi_part);
-    } else {
-        k_fwd_direct<float><<<n_tiles, 128, d.N * sizeof(float), st>>>(d, tiles, (const float*)B,
-                                                                      mode, yout, chi_part);
-    }
+    k_fwd_direct<<<n_tiles, 128, d.N * sizeof(float), st>>>(d, tiles, B, mode, yout, chi_part);
 }
 
 // ---------------------------------------------------------------------------
@@ -325,11 +304,10 @@ void launch_fwd_direct(const DevData& d, int fp64, const VisTile* tiles, int n_t
 constexpr int ADJ_PPT = 16;
 constexpr int ADJ_CHUNK = 256;
 
-template <typename T, typename T2>
-__global__ void __launch_bounds__(128) k_adj_direct(DevData d, const T2* __restrict__ y,
+__global__ void __launch_bounds__(128) k_adj_direct(DevData d, const float2* __restrict__ y,
                                                     double* __restrict__ gsum, int ks) {
     __shared__ uint64_t sa[ADJ_CHUNK], sb[ADJ_CHUNK];
-    __shared__ T syr[ADJ_CHUNK], syi[ADJ_CHUNK];
+    __shared__ float syr[ADJ_CHUNK], syi[ADJ_CHUNK];
     const int N = d.N, c0 = N / 2;
     const int64_t NN = (int64_t)N * N;
     const int c = blockIdx.y;
@@ -348,21 +326,21 @@ __global__ void __launch_bounds__(128) k_adj_direct(DevData d, const T2* __restr
         for (int q = threadIdx.x; q < cnt; q += 128) {
             sa[q] = d.pa[base + q];
             sb[q] = d.pb[base + q];
-            T2 yy = y[base + q];
+            float2 yy = y[base + q];
             syr[q] = yy.x;
             syi[q] = yy.y;
         }
         __syncthreads();
-        T part[ADJ_PPT];
+        float part[ADJ_PPT];
 #pragma unroll
         for (int q = 0; q < ADJ_PPT; ++q) part[q] = 0;
         for (int k = 0; k < cnt; ++k) {
             uint64_t p = phase_mul(m0 - c0, sa[k]) + phase_mul(n - c0, sb[k]);
-            T yr = syr[k], yi = syi[k];
+            float yr = syr[k], yi = syi[k];
 #pragma unroll
             for (int q = 0; q < ADJ_PPT; ++q) {
-                T cs, sn;
-                cis_minus<T>(p, cs, sn);
+                float cs, sn;
+                cis_minus(p, cs, sn);
                 // Re(y e^{+i theta}) = yr cos - yi sin
                 part[q] += yr * cs - yi * sn;
                 p += sa[k];
@@ -388,12 +366,10 @@ int adj_direct_splits(const DevData& d, int num_sms) {
     return ks;
 }
 
-void launch_adj_direct(const DevData& d, int fp64, const void* y, double* gsum, int ks,
-                       cudaStream_t st) {
+void launch_adj_direct(const DevData& d, const float2* y, double* gsum, int ks, cudaStream_t st) {
     int64_t NN = (int64_t)d.N * d.N;
     dim3 grid((unsigned)((NN / ADJ_PPT + 127) / 128), d.C, ks);
-    if (fp64) k_adj_direct<double, double2><<<grid, 128, 0, st>>>(d, (const double2*)y, gsum, ks);
-    else k_adj_direct<float, float2><<<grid, 128, 0, st>>>(d, (const float2*)y, gsum, ks);
+    k_adj_direct<<<grid, 128, 0, st>>>(d, y, gsum, ks);
 }
 
 // ---------------------------------------------------------------------------
