@@ -139,6 +139,7 @@ struct mem_ctx {
     // solver state
     double *I64 = nullptr, *d64 = nullptr, *g64 = nullptr, *gf64 = nullptr, *gp64 = nullptr;
     double *alpha = nullptr, *beta = nullptr, *dots = nullptr, *dpart = nullptr;
+    unsigned* dcount = nullptr;  // completion counters of the dot products, zero between launches
     int* mode = nullptr;
     CgImage* cg_st = nullptr;
     CgControl* cg_ctl = nullptr;
@@ -424,6 +425,24 @@ int ent_blocks(const mem_ctx* c) {
            : c->prec == MEM_PREC_FP64_DIRECT ? f64_ent_blocks(c->N) : prep_blocks(c->N);
 }
 
+// Inputs of the scalar reduction after the form's forward.
+ScalarArgs scalar_args(const mem_ctx* c, bool entropy) {
+    ScalarArgs sc;
+    sc.tile_off = fwd_tile_off(c);
+    sc.chi_part = c->chi_part;
+    sc.ent_part = c->ent_part;
+    sc.with_entropy = entropy;
+    sc.n_ent = ent_blocks(c);
+    const std::vector<int>& off = c->prec == MEM_PREC_BF16X3 ? c->tile_off_tc_h : c->tile_off_h;
+    int tiles = 0;  // most tiles of one image
+    for (int i = 0; i < c->C; ++i) tiles = std::max(tiles, off[i + 1] - off[i]);
+    if (c->shared) tiles = off[c->C];
+    sc.splits = scalar_splits(std::max<int64_t>(4ll * tiles, sc.n_ent));
+    sc.scal = c->scal;
+    sc.img_tmp = c->img_tmp;
+    return sc;
+}
+
 // prep + forward for one image source.  mode: FwdMode.  defer_scalars: the
 // objective's scalar reduction is left to a later launch (the gradient's).
 mem_status run_forward(mem_ctx* c, const ImgSrc& src, int mode, bool entropy, void* yout,
@@ -487,8 +506,7 @@ mem_status run_forward(mem_ctx* c, const ImgSrc& src, int mode, bool entropy, vo
     TRY(after_launch(c, "forward kernel"));
     if (mode != FWD_VIS && !defer_scalars) {
         KTimer t(c, "scalars");
-        launch_scalars(d, fwd_tile_off(c), c->chi_part, c->ent_part, entropy ? 1 : 0, ent_blocks(c),
-                       c->scal, c->img_tmp, c->st);
+        launch_scalars(d, scalar_args(c, entropy), c->st);
         c->launches++;
         TRY(after_launch(c, "scalar reduction"));
     }
@@ -550,14 +568,7 @@ mem_status run_objgrad(mem_ctx* c, const ImgSrc& src, int projected, float* out3
     TRY(run_adjoint(c, &ks, true, !fused));
     if (fused) {
         KTimer t(c, "adj_reduce_grad");
-        ScalarArgs sc;
-        sc.tile_off = fwd_tile_off(c);
-        sc.chi_part = c->chi_part;
-        sc.ent_part = c->ent_part;
-        sc.with_entropy = 1;
-        sc.n_ent = ent_blocks(c);
-        sc.scal = c->scal;
-        sc.img_tmp = c->img_tmp;
+        const ScalarArgs sc = scalar_args(c, true);
         if (c->prec == MEM_PREC_FP16X3)
             launch_adj_fold_reduce_grad(c->dd(), src, c->cb_off, c->partial, c->ymax, projected, out32, full64, proj64,
                                         sc, c->st);
@@ -810,24 +821,18 @@ mem_status solve_prologue(mem_ctx* c, unsigned long long h_outer) {
 // beta, direction (and its restart), slope, curvature, first trial step
 mem_status solve_iter_head(mem_ctx* c, unsigned long long h_inner) {
     const DevData d = c->dd();
-    const int NI = c->n_images;
     cudaStream_t st = c->st;
-    launch_dots(d, DOT_BETA, c->g64, c->gp64, nullptr, c->dpart, c->dots, st);
-    launch_cg_beta(NI, c->cg_st, c->cg_ctl, c->dots, c->beta, c->mode, st);
-    launch_cg_direction(d, c->I64, c->g64, c->beta, c->mode, c->d64, st);
-    launch_dots(d, DOT_SLOPE, c->gf64, c->d64, c->g64, c->dpart, c->dots, st);
-    launch_cg_slope(NI, c->cg_st, c->dots, c->beta, c->mode, st);
-    launch_cg_direction(d, c->I64, c->g64, c->beta, c->mode, c->d64, st);
-    launch_dots(d, DOT_SLOPE, c->gf64, c->d64, c->g64, c->dpart, c->dots, st);
-    launch_cg_slope2(NI, c->cg_st, c->cg_ctl, c->dots, c->mode, st);
-    c->launches += 11;
+    launch_cg_beta(d, c->g64, c->gp64, c->cg_st, c->cg_ctl, c->beta, c->mode, c->dpart, c->dcount, st);
+    for (bool again : {false, true})
+        launch_cg_direction(d, again, c->I64, c->g64, c->gf64, c->cg_st, c->cg_ctl, c->beta, c->mode, c->d64, c->dots,
+                            c->dpart, c->dcount, st);
+    c->launches += 3;
     TRY(after_launch(c, "search direction"));
     // quadratic model of chi^2 along d: curvature sum w |F(A d)|^2
     ImgSrc src{nullptr, c->d64, nullptr, nullptr, c->G, 0};
-    TRY(run_forward(c, src, FWD_CURV, false, nullptr));
-    launch_dots(d, DOT_MAX, c->I64, c->d64, nullptr, c->dpart, c->dots, st);
-    launch_ls_start(NI, c->cg_st, c->cg_ctl, c->scal, c->dots, c->alpha, c->dstatus, h_inner, st);
-    c->launches += 3;
+    TRY(run_forward(c, src, FWD_CURV, false, nullptr, true));
+    launch_scalars_ls(d, scalar_args(c, false), true, c->cg_st, c->cg_ctl, c->dots, c->alpha, c->dstatus, h_inner, st);
+    c->launches++;
     return after_launch(c, "line search start");
 }
 
@@ -837,25 +842,20 @@ mem_status solve_iter_head(mem_ctx* c, unsigned long long h_inner) {
 mem_status solve_probe(mem_ctx* c, unsigned long long h_inner) {
     ImgSrc src{nullptr, c->I64, c->d64, c->alpha, c->G, 1};
     void* ybuf = c->prec == MEM_PREC_FP64_DIRECT ? (void*)c->y64 : (void*)c->y32;
-    TRY(run_forward(c, src, FWD_DCHI, true, ybuf));
-    launch_ls_feed(c->n_images, c->cg_st, c->cg_ctl, c->scal, c->alpha, c->dstatus, h_inner, c->st);
+    TRY(run_forward(c, src, FWD_DCHI, true, ybuf, true));
+    launch_scalars_ls(c->dd(), scalar_args(c, true), false, c->cg_st, c->cg_ctl, c->dots, c->alpha, c->dstatus,
+                      h_inner, c->st);
     c->launches++;
     return after_launch(c, "line search");
 }
 
 // accepted step, new gradient, history row, loop condition
 mem_status solve_iter_tail(mem_ctx* c, unsigned long long h_outer) {
-    const DevData d = c->dd();
-    const int NI = c->n_images;
-    const size_t n = (size_t)NI * c->N * c->N;
-    cudaStream_t st = c->st;
-    launch_cg_finish(NI, c->cg_st, c->cg_ctl, c->alpha, st);
-    launch_cg_step(d, c->I64, c->d64, c->alpha, st);
-    c->launches += 2;
-    CK(cudaMemcpyAsync(c->gp64, c->g64, n * sizeof(double), cudaMemcpyDeviceToDevice, st), "copy g");
+    launch_cg_step(c->dd(), c->I64, c->d64, c->alpha, c->g64, c->gp64, c->st);
+    c->launches++;
     ImgSrc src{nullptr, c->I64, nullptr, nullptr, c->G, 0};
     TRY(run_objgrad(c, src, 1, nullptr, c->gf64, c->g64));
-    launch_cg_record(NI, c->cg_st, c->cg_ctl, c->scal, c->cg_hist, c->dstatus, h_outer, st);
+    launch_cg_record(c->n_images, c->cg_st, c->cg_ctl, c->scal, c->cg_hist, c->dstatus, h_outer, c->st);
     c->launches++;
     return after_launch(c, "iteration end");
 }
@@ -1541,7 +1541,11 @@ mem_status mem_solve(mem_ctx* c, float* image_dev_inout, int32_t n_iter, mem_sol
     TRY(dalloc(c, &c->beta, (size_t)NI));
     TRY(dalloc(c, &c->mode, (size_t)NI));
     TRY(dalloc(c, &c->dots, (size_t)2 * NI));
-    TRY(dalloc(c, &c->dpart, (size_t)2 * NI * prep_blocks(c->N)));
+    TRY(dalloc(c, &c->dpart, (size_t)4 * NI * prep_blocks(c->N)));
+    if (!c->dcount) {
+        TRY(dalloc(c, &c->dcount, (size_t)NI));
+        CK(cudaMemsetAsync(c->dcount, 0, NI * sizeof(unsigned), c->st), "counters");
+    }
     TRY(dalloc(c, &c->cg_st, (size_t)NI));
     TRY(dalloc(c, &c->cg_ctl, (size_t)1));
     const size_t hist_n = (size_t)NI * (n_iter + 1) * 6;

@@ -206,17 +206,23 @@ void launch_adj_tc_uv(const DevData& d, const AdjUnit* units, const int* cta_uni
 // compensated FP32 two-sum).
 void launch_adj_tc_reduce_out(int N, const int* cb_unit_off, const float* partial, const float* beam,
                               float* out, cudaStream_t st);
-// Inputs of the objective's scalar reduction (launch_scalars) when it runs
-// inside another launch; scal == nullptr: not run.
+// Inputs of the objective's scalar reduction, in a launch of its own or inside
+// another one (there scal == nullptr: not run).
 struct ScalarArgs {
     const int* tile_off = nullptr;
     const double* chi_part = nullptr;
     const double* ent_part = nullptr;
     int with_entropy = 0;
-    int n_ent = 0;  // entropy partials per image
+    int n_ent = 0;   // entropy partials per image
+    int splits = 1;  // blocks per image: scalar_splits
     double* scal = nullptr;
     double* img_tmp = nullptr;
 };
+// One block sums up to 4,096 partials of an image; beyond that SCAL_SPLIT do.
+// (256 threads read 4,096 partials in four rounds of four loads; the hand-over
+// between blocks costs as much as eight such rounds.)
+constexpr int SCAL_SPLIT = 32;
+inline int scalar_splits(int64_t partials) { return partials <= 4096 ? 1 : SCAL_SPLIT; }
 // Unit-partial sum plus gradient assembly in one launch, for images of one
 // channel each (not the shared-image mode); with sc.scal set, the same launch
 // also forms the objective scalars (as launch_scalars).
@@ -235,21 +241,14 @@ void launch_finalize(const DevData& d, const ImgSrc& src, int fast_log, const do
 // chi_part holds 4 partials per visibility tile (one per 32 visibilities),
 // ent_part n_ent entropy partials per image.
 // Per-image chi^2 / S / Phi into scal[3 + 3 i ...] and totals into scal[0..2].
-void launch_scalars(const DevData& d, const int* tile_off, const double* chi_part,
-                    const double* ent_part, int with_entropy, int n_ent, double* scal, double* img_tmp,
-                    cudaStream_t st);
+void launch_scalars(const DevData& d, const ScalarArgs& sc, cudaStream_t st);
 int scalars_tmp_doubles(int n_images);
 
-// Solver vector kernels (FP64, per image).
-void launch_dots(const DevData& d, int which, const double* a, const double* b, const double* c,
-                 double* part, double* out, cudaStream_t st);
-void launch_cg_direction(const DevData& d, const double* I, const double* g, const double* beta,
-                         const int* mode, double* dir, cudaStream_t st);
-void launch_cg_step(const DevData& d, double* I, const double* dir, const double* alpha,
-                    cudaStream_t st);
+// Solver vector kernel (FP64, per image).
+// I = max(I + alpha d, G) where alpha > 0; g_prev = g everywhere.
+void launch_cg_step(const DevData& d, double* I, const double* dir, const double* alpha, const double* g,
+                    double* g_prev, cudaStream_t st);
 void launch_clip_f32_to_f64(const DevData& d, const float* in, double* out, cudaStream_t st);
 void launch_f64_to_f32(int64_t n, const double* in, float* out, cudaStream_t st);
-
-enum DotKind { DOT_BETA = 0, DOT_SLOPE = 1, DOT_MAX = 2 };
 
 }  // namespace msk

@@ -421,7 +421,7 @@ struct RedArgs {
 // log(I/G) stays FP64: with an FP32 log the 50-iteration solve of the
 // 64x64 problem ended 1.4e-3 (relative L2) from the oracle's image in the
 // BF16X3 form, against 4.6e-4.
-// With sc.scal set, SCAL_SPLIT further blocks per image (the first ones in
+// With sc.scal set, sc.splits further blocks per image (the first ones in
 // x, so that they start with the first wave) run the objective's scalar
 // reduction (scalars_block): it needs only the forward's chi^2 partials and
 // the prep's entropy partials, so it shares this launch instead of taking one
@@ -433,11 +433,9 @@ __global__ void __launch_bounds__(RedGeo<WIDE>::THREADS) k_adj_fold_reduce(DevDa
     __shared__ float sh[2][SPLIT][ELEMS][2];
     const int N = d.N;
     const int64_t NN = (int64_t)N * N;
-    const int n_scal = OUT == RED_GRAD && a.sc.scal ? SCAL_SPLIT : 0;
+    const int n_scal = OUT == RED_GRAD && a.sc.scal ? a.sc.splits : 0;
     if (OUT == RED_GRAD && (int)blockIdx.x < n_scal) {
-        scalars_block<THREADS>(d, a.sc.tile_off, a.sc.chi_part, a.sc.ent_part, a.sc.with_entropy, a.sc.n_ent,
-                                   scalars_part(a.sc.img_tmp, d.n_images), a.sc.img_tmp, a.sc.scal,
-                                   scalars_counter(a.sc.img_tmp, d.n_images), blockIdx.y, blockIdx.x);
+        scalars_block<THREADS>(d, a.sc, blockIdx.y, blockIdx.x);
         return;
     }
     const int BLK = N < 256 ? N : 256, nbx = N / BLK;
@@ -540,7 +538,7 @@ void launch_adj_fold_reduce_grad(const DevData& d, const ImgSrc& src, const int*
                                const float* ymax, int projected, float* out32, double* full64, double* proj64,
                                const ScalarArgs& sc, cudaStream_t st) {
     const RedArgs a{cb_unit_off, partial, ymax, nullptr, projected, out32, full64, proj64, sc};
-    launch_red<RED_GRAD>(d, src, a, sc.scal ? SCAL_SPLIT : 0, st);
+    launch_red<RED_GRAD>(d, src, a, sc.scal ? sc.splits : 0, st);
 }
 
 }  // namespace msk

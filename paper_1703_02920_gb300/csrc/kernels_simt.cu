@@ -33,23 +33,6 @@ void launch_phase_prep(int64_t Z, const double* u, const double* v, double dx, d
     k_phase_prep<<<(unsigned)((Z + 255) / 256), 256, 0, st>>>(Z, u, v, dx, dy, pa, pb);
 }
 
-
-template <int BLOCK>
-__device__ __forceinline__ double block_max(double x, double* sh) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_down_sync(0xffffffffu, x, o));
-    int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0) sh[w] = x;
-    __syncthreads();
-    double r = 0.0;
-    if (threadIdx.x == 0) {
-        r = sh[0];
-        for (int i = 1; i < BLOCK / 32; ++i) r = fmax(r, sh[i]);
-    }
-    __syncthreads();
-    return r;
-}
-
 // ---------------------------------------------------------------------------
 // a2, BF16X3: attenuation, centring and splitting of the forward's operand
 // (FP16X3: kernels_fold_prep.cu).
@@ -414,125 +397,32 @@ void launch_finalize(const DevData& d, const ImgSrc& src, int fast_log, const do
 // Ordered FP64 reductions of tile partials into per-image and total scalars.
 // scal layout: [0..2] = Phi, chi^2, S totals; [3 + 3i ...] per image.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_scalars(DevData d, const int* __restrict__ tile_off,
-                                                 const double* __restrict__ chi_part,
-                                                 const double* __restrict__ ent_part, int with_entropy,
-                                                 int n_ent_blocks, double* part, double* img_tmp, double* scal,
-                                                 unsigned* counter) {
-    scalars_block<256>(d, tile_off, chi_part, ent_part, with_entropy, n_ent_blocks, part, img_tmp, scal, counter,
-                  blockIdx.x, blockIdx.y);
+__global__ void __launch_bounds__(256) k_scalars(DevData d, ScalarArgs sc) {
+    scalars_block<256>(d, sc, blockIdx.x, blockIdx.y);
 }
 
-void launch_scalars(const DevData& d, const int* tile_off, const double* chi_part,
-                    const double* ent_part, int with_entropy, int n_ent, double* scal, double* img_tmp,
-                    cudaStream_t st) {
-    double* part = scalars_part(img_tmp, d.n_images);
-    unsigned* counter = scalars_counter(img_tmp, d.n_images);
-    k_scalars<<<dim3(d.n_images, SCAL_SPLIT), 256, 0, st>>>(d, tile_off, chi_part, ent_part, with_entropy,
-                                                             n_ent, part, img_tmp, scal, counter);
+void launch_scalars(const DevData& d, const ScalarArgs& sc, cudaStream_t st) {
+    k_scalars<<<dim3(d.n_images, sc.splits), 256, 0, st>>>(d, sc);
 }
 
-int scalars_tmp_doubles(int n_images) { return 3 * n_images + 2 * SCAL_SPLIT * n_images + 1; }
+int scalars_tmp_doubles(int n_images) { return 2 * SCAL_SPLIT * n_images + 1; }
 
-// ---------------------------------------------------------------------------
-// a8: CG vector kernels (FP64), per image.
-// DOT_BETA : out[2i] = gprev.gprev, out[2i+1] = (g - gprev).g   (Polak-Ribiere)
-// DOT_SLOPE: out[2i] = gfull.d,     out[2i+1] = g.g
-// DOT_MAX  : out[2i] = max I,       out[2i+1] = max |d|
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_dots_part(DevData d, int which, const double* __restrict__ a,
-                                                   const double* __restrict__ b,
-                                                   const double* __restrict__ c, double* part) {
-    __shared__ double sh[8];
-    const int64_t NN = (int64_t)d.N * d.N;
-    const int i = blockIdx.y;
-    const int64_t p = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    double x0 = 0.0, x1 = 0.0;
-    if (p < NN) {
-        const int64_t q = (int64_t)i * NN + p;
-        if (which == DOT_BETA) {          // a = g, b = gprev
-            x0 = b[q] * b[q];
-            x1 = (a[q] - b[q]) * a[q];
-        } else if (which == DOT_SLOPE) {  // a = gfull, b = d, c = g
-            x0 = a[q] * b[q];
-            x1 = c[q] * c[q];
-        } else {                          // a = I, b = d
-            x0 = a[q];
-            x1 = fabs(b[q]);
-        }
-    }
-    double r0, r1;
-    if (which == DOT_MAX) {
-        r0 = block_max<256>(x0, sh);
-        r1 = block_max<256>(x1, sh);
-    } else {
-        r0 = block_sum<256>(x0, sh);
-        r1 = block_sum<256>(x1, sh);
-    }
-    if (threadIdx.x == 0) {
-        part[((int64_t)i * gridDim.x + blockIdx.x) * 2] = r0;
-        part[((int64_t)i * gridDim.x + blockIdx.x) * 2 + 1] = r1;
-    }
-}
-
-__global__ void __launch_bounds__(256) k_dots_final(int which, int nblk, const double* __restrict__ part,
-                                                    double* out) {
-    __shared__ double sh[8];
-    const int i = blockIdx.x;
-    double x0 = (which == DOT_MAX) ? 0.0 : 0.0, x1 = 0.0;
-    for (int b = threadIdx.x; b < nblk; b += 256) {
-        double p0 = part[((int64_t)i * nblk + b) * 2], p1 = part[((int64_t)i * nblk + b) * 2 + 1];
-        if (which == DOT_MAX) { x0 = fmax(x0, p0); x1 = fmax(x1, p1); }
-        else { x0 += p0; x1 += p1; }
-    }
-    double r0, r1;
-    if (which == DOT_MAX) { r0 = block_max<256>(x0, sh); r1 = block_max<256>(x1, sh); }
-    else { r0 = block_sum<256>(x0, sh); r1 = block_sum<256>(x1, sh); }
-    if (threadIdx.x == 0) { out[2 * i] = r0; out[2 * i + 1] = r1; }
-}
-
-void launch_dots(const DevData& d, int which, const double* a, const double* b, const double* c,
-                 double* part, double* out, cudaStream_t st) {
-    int nblk = prep_blocks(d.N);
-    k_dots_part<<<dim3(nblk, d.n_images), 256, 0, st>>>(d, which, a, b, c, part);
-    k_dots_final<<<d.n_images, 256, 0, st>>>(which, nblk, part, out);
-}
-
-// Search direction per image, mode_i: 0 keep, 1 d = -g + beta_i d, 2 d = -g;
-// then the bound projection: a pixel at I = G cannot move down.
-__global__ void __launch_bounds__(256) k_cg_direction(DevData d, const double* __restrict__ I,
-                                                      const double* __restrict__ g,
-                                                      const double* __restrict__ beta,
-                                                      const int* __restrict__ mode, double* dir) {
-    const int64_t NN = (int64_t)d.N * d.N;
-    const int i = blockIdx.y;
-    const int64_t p = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    if (p >= NN || mode[i] == 0) return;
-    const int64_t q = (int64_t)i * NN + p;
-    double nd = mode[i] == 2 ? -g[q] : -g[q] + beta[i] * dir[q];
-    if (I[q] <= d.G && nd < 0.0) nd = 0.0;
-    dir[q] = nd;
-}
-
-void launch_cg_direction(const DevData& d, const double* I, const double* g, const double* beta,
-                         const int* mode, double* dir, cudaStream_t st) {
-    k_cg_direction<<<dim3(prep_blocks(d.N), d.n_images), 256, 0, st>>>(d, I, g, beta, mode, dir);
-}
-
-// I = max(I + alpha_i d, G) for images with alpha_i > 0.
+// I = max(I + alpha_i d, G) for images with alpha_i > 0; g_prev = g.
 __global__ void __launch_bounds__(256) k_cg_step(DevData d, double* I, const double* __restrict__ dir,
-                                                 const double* __restrict__ alpha) {
+                                                 const double* __restrict__ alpha, const double* __restrict__ g,
+                                                 double* __restrict__ g_prev) {
     const int64_t NN = (int64_t)d.N * d.N;
     const int i = blockIdx.y;
     const int64_t p = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    if (p >= NN || !(alpha[i] > 0.0)) return;
+    if (p >= NN) return;
     const int64_t q = (int64_t)i * NN + p;
-    I[q] = fmax(I[q] + alpha[i] * dir[q], d.G);
+    g_prev[q] = g[q];
+    if (alpha[i] > 0.0) I[q] = fmax(I[q] + alpha[i] * dir[q], d.G);
 }
 
-void launch_cg_step(const DevData& d, double* I, const double* dir, const double* alpha,
-                    cudaStream_t st) {
-    k_cg_step<<<dim3(prep_blocks(d.N), d.n_images), 256, 0, st>>>(d, I, dir, alpha);
+void launch_cg_step(const DevData& d, double* I, const double* dir, const double* alpha, const double* g,
+                    double* g_prev, cudaStream_t st) {
+    k_cg_step<<<dim3(prep_blocks(d.N), d.n_images), 256, 0, st>>>(d, I, dir, alpha, g, g_prev);
 }
 
 __global__ void k_clip_f32_to_f64(int64_t n, const float* __restrict__ in, double* __restrict__ out,

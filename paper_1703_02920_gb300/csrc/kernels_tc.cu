@@ -508,7 +508,7 @@ void launch_adj_tc_reduce(const DevData& d, const int* cb_unit_off, const float*
 // log(I/G) stays FP64: with an FP32 log the 50-iteration solve of the
 // 64x64 problem ended 1.4e-3 (relative L2) from the oracle's image in the
 // BF16X3 form, against 4.6e-4.
-// With sc.scal set, SCAL_SPLIT further blocks per image (the first ones in
+// With sc.scal set, sc.splits further blocks per image (the first ones in
 // x, so that they start with the first wave) run the objective's scalar
 // reduction (scalars_block): it needs only the forward's chi^2 partials and
 // the prep's entropy partials, so it shares this launch instead of taking one
@@ -521,11 +521,9 @@ __global__ void __launch_bounds__(256) k_adj_tc_reduce_grad(DevData d, ImgSrc sr
     __shared__ float sh[4][RED_ELEMS][2];
     const int N = d.N;
     const int64_t NN = (int64_t)N * N;
-    const int n_scal = sc.scal ? SCAL_SPLIT : 0;
+    const int n_scal = sc.scal ? sc.splits : 0;
     if ((int)blockIdx.x < n_scal) {
-        scalars_block<256>(d, sc.tile_off, sc.chi_part, sc.ent_part, sc.with_entropy, sc.n_ent,
-                      scalars_part(sc.img_tmp, d.n_images), sc.img_tmp, sc.scal,
-                      scalars_counter(sc.img_tmp, d.n_images), blockIdx.y, blockIdx.x);
+        scalars_block<256>(d, sc, blockIdx.y, blockIdx.x);
         return;
     }
     const int BLK = N < 256 ? N : 256;
@@ -560,7 +558,7 @@ void launch_adj_tc_reduce_grad(const DevData& d, const ImgSrc& src, const int* c
                                const ScalarArgs& sc, cudaStream_t st) {
     const int64_t NN = (int64_t)d.N * d.N;
     const unsigned gb = (unsigned)((NN + RED_ELEMS - 1) / RED_ELEMS);
-    dim3 grid(gb + (sc.scal ? SCAL_SPLIT : 0), d.C);
+    dim3 grid(gb + (sc.scal ? sc.splits : 0), d.C);
     k_adj_tc_reduce_grad<<<grid, 256, 0, st>>>(d, src, cb_unit_off, partial, projected, out32, full64,
                                                 proj64, sc);
 }

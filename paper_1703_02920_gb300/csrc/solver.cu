@@ -1,8 +1,16 @@
 // Device-side control of the projected Polak-Ribiere CG (Eq. minproblem):
 // the conjugate-gradient bookkeeping, the line-search state machine and the
-// loop conditions run in single-block controller kernels, so that a whole
-// solve is one launch of a CUDA graph whose loops are conditional WHILE
-// nodes (the host reads the results once, at the end).
+// loop conditions run on the device, so that a whole solve is one launch of a
+// CUDA graph whose loops are conditional WHILE nodes (the host reads the results
+// once, at the end).
+//
+// A small problem's solve is a chain of kernels of a few microseconds each, so
+// its time is their number.  Every control step therefore runs in the last block
+// of the reduction that feeds it: the dot products and the vector update before
+// them are one launch with the decision per image (k_cg_beta, k_cg_direction),
+// the scalar reduction of a probe feeds the line search and, at its end, accepts
+// the step (k_scalars_ls).  64 x 64 with 10,260 visibilities, five iterations with 60
+// probes: 2.06 ms with a launch per step and per reduction stage, 1.67 ms so.
 //
 // Per iteration (every scalar in FP64):
 //   beta_i = max(0, (g - g_prev).g / g_prev.g_prev)  (0 on restarts: the first
@@ -20,7 +28,9 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "common.cuh"
 #include "internal.h"
+#include "reduce.cuh"
 #include "solver.h"
 
 namespace msk {
@@ -283,118 +293,146 @@ __global__ void __launch_bounds__(CTL_THREADS) k_cg_init(int NI, CgImage* st, Cg
     set_cond(ctl, 0, any && ctl->k < ctl->n_iter && ctl->status == 0, h_outer);
 }
 
-// Polak-Ribiere beta from dots = (g_prev.g_prev, (g - g_prev).g) per image;
-// direction mode 1 (d = -g + beta d) or 2 (d = -g) for active images, 0 keep.
-__global__ void __launch_bounds__(CTL_THREADS) k_cg_beta(int NI, CgImage* st, const CgControl* ctl,
-                                                         const double* dots, double* beta, int* mode) {
-    const int k = ctl->k;
-    for (int i = threadIdx.x; i < NI; i += CTL_THREADS) {
-        double b = 0.0;
-        if (k > 0 && k % RESTART != 0) {
-            const double gg = dots[2 * i], pr = dots[2 * i + 1];
-            if (gg > 0.0) b = fmax(0.0, pr / gg);
-        }
-        st[i].beta = b;
-        beta[i] = b;
-        mode[i] = st[i].active ? (b == 0.0 ? 2 : 1) : 0;
+// ---------------------------------------------------------------------------
+// Sums of x0, x1 and maxima of m0, m1 over an image's pixels: a block's result
+// goes to part, and the image's last block to finish (count[i], zero between
+// launches) combines the blocks' results in order.  True in the threads of that
+// block, which hold the totals in thread 0.
+// ---------------------------------------------------------------------------
+struct Totals {
+    double x0, x1, m0, m1;
+};
+
+__device__ __forceinline__ void block_max2(double& x, double& y, double (*sh)[2]) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        x = fmax(x, __shfl_down_sync(0xffffffffu, x, o));
+        y = fmax(y, __shfl_down_sync(0xffffffffu, y, o));
     }
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    if (l == 0) {
+        sh[w][0] = x;
+        sh[w][1] = y;
+    }
+    __syncthreads();
+    if (w == 0) {
+        x = sh[l % (CTL_THREADS / 32)][0];
+        y = sh[l % (CTL_THREADS / 32)][1];
+#pragma unroll
+        for (int o = CTL_THREADS / 64; o > 0; o >>= 1) {
+            x = fmax(x, __shfl_down_sync(0xffffffffu, x, o));
+            y = fmax(y, __shfl_down_sync(0xffffffffu, y, o));
+        }
+    }
+    __syncthreads();
 }
 
-// slope = grad Phi . d; an active image whose d is not a descent direction
-// restarts with d = -g (mode 2, beta 0); the others keep d (mode 0).
-__global__ void __launch_bounds__(CTL_THREADS) k_cg_slope(int NI, CgImage* st, const double* dots, double* beta,
-                                                          int* mode) {
-    for (int i = threadIdx.x; i < NI; i += CTL_THREADS) {
-        CgImage& s = st[i];
-        s.slope = dots[2 * i];
-        mode[i] = 0;
-        if (s.active && s.slope >= 0.0) {
-            mode[i] = 2;
+template <bool MAXIMA>
+__device__ bool image_totals(int i, double& x0, double& x1, double& m0, double& m1, Totals* part, unsigned* count) {
+    __shared__ double sh[CTL_THREADS / 32][2];
+    __shared__ bool last;
+    const int nblk = gridDim.x;
+    block_sum2<CTL_THREADS>(x0, x1, sh);
+    if (MAXIMA) block_max2(m0, m1, sh);
+    if (threadIdx.x == 0) {
+        part[(int64_t)i * nblk + blockIdx.x] = {x0, x1, m0, m1};
+        __threadfence();
+        last = atomicAdd(count + i, 1u) == (unsigned)nblk - 1;
+    }
+    __syncthreads();
+    if (!last) return false;
+    __threadfence();
+    x0 = x1 = m0 = m1 = 0.0;
+    for (int b = threadIdx.x; b < nblk; b += CTL_THREADS) {
+        const double* p = (const double*)(part + (int64_t)i * nblk + b);
+        x0 += __ldcg(p);
+        x1 += __ldcg(p + 1);
+        if (MAXIMA) {
+            m0 = fmax(m0, __ldcg(p + 2));
+            m1 = fmax(m1, __ldcg(p + 3));
+        }
+    }
+    block_sum2<CTL_THREADS>(x0, x1, sh);
+    if (MAXIMA) block_max2(m0, m1, sh);
+    if (threadIdx.x == 0) count[i] = 0;
+    return true;
+}
+
+// Polak-Ribiere beta from g_prev.g_prev and (g - g_prev).g; direction mode 1
+// (d = -g + beta d) or 2 (d = -g) for active images, 0 keep.
+__global__ void __launch_bounds__(CTL_THREADS) k_cg_beta(DevData d, const double* __restrict__ g,
+                                                         const double* __restrict__ g_prev, CgImage* st,
+                                                         const CgControl* ctl, double* beta, int* mode,
+                                                         Totals* part, unsigned* count) {
+    const int64_t NN = (int64_t)d.N * d.N;
+    const int i = blockIdx.y;
+    const int64_t p = (int64_t)blockIdx.x * CTL_THREADS + threadIdx.x;
+    double x0 = 0.0, x1 = 0.0, m0 = 0.0, m1 = 0.0;
+    if (p < NN) {
+        const double a = g[i * NN + p], b = g_prev[i * NN + p];
+        x0 = b * b;
+        x1 = (a - b) * a;
+    }
+    if (!image_totals<false>(i, x0, x1, m0, m1, part, count) || threadIdx.x != 0) return;
+    const int k = ctl->k;
+    double b = 0.0;
+    if (k > 0 && k % RESTART != 0 && x0 > 0.0) b = fmax(0.0, x1 / x0);
+    st[i].beta = b;
+    beta[i] = b;
+    mode[i] = st[i].active ? (b == 0.0 ? 2 : 1) : 0;
+}
+
+// Search direction per image (mode 0 keep, 1 d = -g + beta d, 2 d = -g; a pixel
+// at I = G cannot move down), its slope grad Phi . d, max I and max |d| (dots).
+// An active image whose d is not a descent direction gets mode 2 and beta 0, the
+// others mode 0; the second launch (again) takes the former only, and stops an
+// image still without descent.
+__global__ void __launch_bounds__(CTL_THREADS) k_cg_direction(DevData d, bool again, const double* __restrict__ I,
+                                                              const double* __restrict__ g,
+                                                              const double* __restrict__ gfull, CgImage* st,
+                                                              CgControl* ctl, double* beta, int* mode, double* dir,
+                                                              double* dots, Totals* part, unsigned* count) {
+    const int64_t NN = (int64_t)d.N * d.N;
+    const int i = blockIdx.y, md = mode[i];
+    if (again && md == 0) return;
+    const int64_t p = (int64_t)blockIdx.x * CTL_THREADS + threadIdx.x;
+    double x0 = 0.0, x1 = 0.0, m0 = 0.0, m1 = 0.0;
+    if (p < NN) {
+        const int64_t q = i * NN + p;
+        double nd;
+        if (md == 0) {
+            nd = dir[q];
+        } else {
+            nd = md == 2 ? -g[q] : -g[q] + beta[i] * dir[q];
+            if (I[q] <= d.G && nd < 0.0) nd = 0.0;
+            dir[q] = nd;
+        }
+        x0 = gfull[q] * nd;
+        m0 = I[q];
+        m1 = fabs(nd);
+    }
+    if (!image_totals<true>(i, x0, x1, m0, m1, part, count) || threadIdx.x != 0) return;
+    CgImage& s = st[i];
+    s.slope = x0;
+    dots[2 * i] = m0;
+    dots[2 * i + 1] = m1;
+    const bool uphill = s.active && s.slope >= 0.0;
+    if (again) {
+        if (uphill) {
+            s.active = 0;
+            ctl->stopped_early = 1;
+        }
+    } else {
+        mode[i] = uphill ? 2 : 0;
+        if (uphill) {
             s.beta = 0.0;
             beta[i] = 0.0;
         }
     }
 }
 
-// Slopes of the restarted directions; an image still without descent stops.
-__global__ void __launch_bounds__(CTL_THREADS) k_cg_slope2(int NI, CgImage* st, CgControl* ctl, const double* dots,
-                                                           const int* mode) {
-    int stopped = 0;
-    for (int i = threadIdx.x; i < NI; i += CTL_THREADS) {
-        CgImage& s = st[i];
-        if (mode[i] == 2) s.slope = dots[2 * i];
-        if (s.active && s.slope >= 0.0) {
-            s.active = 0;
-            stopped = 1;
-        }
-    }
-    stopped = block_any(stopped);
-    if (threadIdx.x == 0 && stopped) ctl->stopped_early = 1;
-}
-
-// First trial step and line-search start.  scal holds 1/2 sum w |F(A d)|^2 per
-// image in its chi^2 slot (curvature pass); dots = (max I, max |d|).
-__global__ void __launch_bounds__(CTL_THREADS) k_ls_start(int NI, CgImage* st, CgControl* ctl, const double* scal,
-                                                          const double* dots, double* alpha, const int* dstatus,
-                                                          unsigned long long h_inner) {
-    int run = 0, bad = 0;
-    for (int i = threadIdx.x; i < NI; i += CTL_THREADS) {
-        CgImage& s = st[i];
-        alpha[i] = 0.0;
-        s.ls.phase = LS_DONE;
-        if (!s.active) continue;
-        const double curv = 2.0 * scal[4 + 3 * i];
-        if (!finite(curv)) bad = 1;
-        double a0 = curv > 0.0 ? -s.slope / curv : 0.0;
-        if (!(a0 > 0.0)) a0 = dots[2 * i] / dots[2 * i + 1];
-        ls_start(s.ls, s.phi, a0);
-        alpha[i] = s.ls.req;
-        run = 1;
-    }
-    run = block_any(run);
-    bad = block_any(bad);
-    if (threadIdx.x == 0) {
-        ctl->rounds = 0;
-        if (bad) ctl->status |= CG_NONFINITE;
-        if (*dstatus) ctl->status |= CG_DEVICE;
-    }
-    __syncthreads();
-    set_cond(ctl, 1, run && ctl->status == 0, h_inner);
-}
-
-// One probe evaluated: scal holds Phi(max(I + alpha d, G)) - Phi(I) per image.
-__global__ void __launch_bounds__(CTL_THREADS) k_ls_feed(int NI, CgImage* st, CgControl* ctl, const double* scal,
-                                                         double* alpha, const int* dstatus,
-                                                         unsigned long long h_inner) {
-    int run = 0, bad = 0;
-    for (int i = threadIdx.x; i < NI; i += CTL_THREADS) {
-        CgImage& s = st[i];
-        if (s.active && s.ls.phase != LS_DONE) {
-            const double f = s.phi + scal[3 + 3 * i];
-            if (!finite(f)) bad = 1;
-            ls_feed(s.ls, f);
-        }
-        const bool r = s.active && s.ls.phase != LS_DONE;
-        alpha[i] = r ? s.ls.req : 0.0;
-        run |= r;
-    }
-    run = block_any(run);
-    bad = block_any(bad);
-    if (threadIdx.x == 0) {
-        ctl->rounds += 1;
-        ctl->probes += 1;
-        if (bad) ctl->status |= CG_NONFINITE;
-        if (*dstatus) ctl->status |= CG_DEVICE;
-        // every line search ends within LS_MAX_EVALS + 2 probes; the cap only
-        // guards the loop against a state that should not occur
-        if (ctl->rounds >= LS_MAX_EVALS + 8) ctl->status |= CG_LOOP;
-    }
-    __syncthreads();
-    set_cond(ctl, 1, run && ctl->status == 0, h_inner);
-}
-
 // Accepted steps: alpha per image (0 for images that stop: no decrease found).
-__global__ void __launch_bounds__(CTL_THREADS) k_cg_finish(int NI, CgImage* st, CgControl* ctl, double* alpha) {
+__device__ void accept_steps(int NI, CgImage* st, CgControl* ctl, double* alpha) {
     int stopped = 0;
     const int fail = ctl->status != 0;
     for (int i = threadIdx.x; i < NI; i += CTL_THREADS) {
@@ -413,6 +451,67 @@ __global__ void __launch_bounds__(CTL_THREADS) k_cg_finish(int NI, CgImage* st, 
     }
     stopped = block_any(stopped);
     if (threadIdx.x == 0 && stopped && !fail) ctl->stopped_early = 1;
+}
+
+// The scalar reduction, then in its last block one step of the line searches.
+// START: scal holds 1/2 sum w |F(A d)|^2 per image in its chi^2 slot (curvature
+// pass), dots = (max I, max |d|): first trial step and line-search start.
+// Otherwise one probe was evaluated: scal holds Phi(max(I + alpha d, G)) - Phi(I).
+// When no image asks for another probe, the steps are accepted.
+template <bool START>
+__global__ void __launch_bounds__(CTL_THREADS) k_scalars_ls(DevData d, ScalarArgs sc, CgImage* st, CgControl* ctl,
+                                                            const double* dots, double* alpha, const int* dstatus,
+                                                            unsigned long long h_inner) {
+    // The state machine runs on a copy whose loads are all in flight during the
+    // reduction: in place, every branch would wait for its own.
+    const int NI = d.n_images;
+    CgImage mine;
+    if ((int)threadIdx.x < NI) mine = st[threadIdx.x];
+    if (!scalars_block<CTL_THREADS>(d, sc, blockIdx.x, blockIdx.y)) return;
+    __syncthreads();
+    int run = 0, bad = 0;
+    for (int i = threadIdx.x; i < NI; i += CTL_THREADS) {
+        if (i != (int)threadIdx.x) mine = st[i];
+        bool r = false;
+        if (START) {
+            mine.ls.phase = LS_DONE;
+            if (mine.active) {
+                const double curv = 2.0 * __ldcg(sc.scal + 4 + 3 * i);
+                if (!finite(curv)) bad = 1;
+                double a0 = curv > 0.0 ? -mine.slope / curv : 0.0;
+                if (!(a0 > 0.0)) a0 = dots[2 * i] / dots[2 * i + 1];
+                ls_start(mine.ls, mine.phi, a0);
+                r = true;
+            }
+        } else if (mine.active && mine.ls.phase != LS_DONE) {
+            const double f = mine.phi + __ldcg(sc.scal + 3 + 3 * i);
+            if (!finite(f)) bad = 1;
+            ls_feed(mine.ls, f);
+            r = mine.ls.phase != LS_DONE;
+        }
+        st[i].ls = mine.ls;
+        alpha[i] = r ? mine.ls.req : 0.0;
+        run |= r;
+    }
+    run = block_any(run);
+    bad = block_any(bad);
+    if (threadIdx.x == 0) {
+        if (START) {
+            ctl->rounds = 0;
+        } else {
+            ctl->rounds += 1;
+            ctl->probes += 1;
+        }
+        if (bad) ctl->status |= CG_NONFINITE;
+        if (*dstatus) ctl->status |= CG_DEVICE;
+        // every line search ends within LS_MAX_EVALS + 2 probes; the cap only
+        // guards the loop against a state that should not occur
+        if (!START && ctl->rounds >= LS_MAX_EVALS + 8) ctl->status |= CG_LOOP;
+    }
+    __syncthreads();
+    const bool more = run && ctl->status == 0;
+    if (!more) accept_steps(NI, st, ctl, alpha);
+    set_cond(ctl, 1, more, h_inner);
 }
 
 // After the step's objective + gradient: history row k + 1, counters and the
@@ -455,26 +554,23 @@ void launch_cg_init(int NI, CgImage* st, CgControl* ctl, const double* scal, dou
                     unsigned long long h_outer, cudaStream_t s) {
     k_cg_init<<<1, CTL_THREADS, 0, s>>>(NI, st, ctl, scal, hist, dstatus, h_outer);
 }
-void launch_cg_beta(int NI, CgImage* st, const CgControl* ctl, const double* dots, double* beta, int* mode,
-                    cudaStream_t s) {
-    k_cg_beta<<<1, CTL_THREADS, 0, s>>>(NI, st, ctl, dots, beta, mode);
+void launch_cg_beta(const DevData& d, const double* g, const double* g_prev, CgImage* st, const CgControl* ctl,
+                    double* beta, int* mode, double* part, unsigned* count, cudaStream_t s) {
+    k_cg_beta<<<dim3(prep_blocks(d.N), d.n_images), CTL_THREADS, 0, s>>>(d, g, g_prev, st, ctl, beta, mode,
+                                                                        (Totals*)part, count);
 }
-void launch_cg_slope(int NI, CgImage* st, const double* dots, double* beta, int* mode, cudaStream_t s) {
-    k_cg_slope<<<1, CTL_THREADS, 0, s>>>(NI, st, dots, beta, mode);
+void launch_cg_direction(const DevData& d, bool again, const double* I, const double* g, const double* gfull,
+                         CgImage* st, CgControl* ctl, double* beta, int* mode, double* dir, double* dots,
+                         double* part, unsigned* count, cudaStream_t s) {
+    k_cg_direction<<<dim3(prep_blocks(d.N), d.n_images), CTL_THREADS, 0, s>>>(
+        d, again, I, g, gfull, st, ctl, beta, mode, dir, dots, (Totals*)part, count);
 }
-void launch_cg_slope2(int NI, CgImage* st, CgControl* ctl, const double* dots, const int* mode, cudaStream_t s) {
-    k_cg_slope2<<<1, CTL_THREADS, 0, s>>>(NI, st, ctl, dots, mode);
-}
-void launch_ls_start(int NI, CgImage* st, CgControl* ctl, const double* scal, const double* dots, double* alpha,
-                     const int* dstatus, unsigned long long h_inner, cudaStream_t s) {
-    k_ls_start<<<1, CTL_THREADS, 0, s>>>(NI, st, ctl, scal, dots, alpha, dstatus, h_inner);
-}
-void launch_ls_feed(int NI, CgImage* st, CgControl* ctl, const double* scal, double* alpha, const int* dstatus,
-                    unsigned long long h_inner, cudaStream_t s) {
-    k_ls_feed<<<1, CTL_THREADS, 0, s>>>(NI, st, ctl, scal, alpha, dstatus, h_inner);
-}
-void launch_cg_finish(int NI, CgImage* st, CgControl* ctl, double* alpha, cudaStream_t s) {
-    k_cg_finish<<<1, CTL_THREADS, 0, s>>>(NI, st, ctl, alpha);
+void launch_scalars_ls(const DevData& d, const ScalarArgs& sc, bool start, CgImage* st, CgControl* ctl,
+                       const double* dots, double* alpha, const int* dstatus, unsigned long long h_inner,
+                       cudaStream_t s) {
+    const dim3 grid(d.n_images, sc.splits);
+    if (start) k_scalars_ls<true><<<grid, CTL_THREADS, 0, s>>>(d, sc, st, ctl, dots, alpha, dstatus, h_inner);
+    else k_scalars_ls<false><<<grid, CTL_THREADS, 0, s>>>(d, sc, st, ctl, dots, alpha, dstatus, h_inner);
 }
 void launch_cg_record(int NI, CgImage* st, CgControl* ctl, const double* scal, double* hist, const int* dstatus,
                       unsigned long long h_outer, cudaStream_t s) {

@@ -42,19 +42,21 @@ struct CgControl {
     long long probes; // probes over the whole solve
 };
 
-// Controller kernels (one block each).  A non-zero handle is the conditional
-// node whose condition the kernel sets (outer: iterations; inner: probes).
+// Controller kernels.  A non-zero handle is the conditional node whose condition
+// the kernel sets (outer: iterations; inner: probes).  part: 4 doubles per block
+// of prep_blocks(N) and image; count: one counter per image, zero between launches.
+struct DevData;
+struct ScalarArgs;
 void launch_cg_init(int NI, CgImage* st, CgControl* ctl, const double* scal, double* hist, const int* dstatus,
                     unsigned long long h_outer, cudaStream_t s);
-void launch_cg_beta(int NI, CgImage* st, const CgControl* ctl, const double* dots, double* beta, int* mode,
-                    cudaStream_t s);
-void launch_cg_slope(int NI, CgImage* st, const double* dots, double* beta, int* mode, cudaStream_t s);
-void launch_cg_slope2(int NI, CgImage* st, CgControl* ctl, const double* dots, const int* mode, cudaStream_t s);
-void launch_ls_start(int NI, CgImage* st, CgControl* ctl, const double* scal, const double* dots, double* alpha,
-                     const int* dstatus, unsigned long long h_inner, cudaStream_t s);
-void launch_ls_feed(int NI, CgImage* st, CgControl* ctl, const double* scal, double* alpha, const int* dstatus,
-                    unsigned long long h_inner, cudaStream_t s);
-void launch_cg_finish(int NI, CgImage* st, CgControl* ctl, double* alpha, cudaStream_t s);
+void launch_cg_beta(const DevData& d, const double* g, const double* g_prev, CgImage* st, const CgControl* ctl,
+                    double* beta, int* mode, double* part, unsigned* count, cudaStream_t s);
+void launch_cg_direction(const DevData& d, bool again, const double* I, const double* g, const double* gfull,
+                         CgImage* st, CgControl* ctl, double* beta, int* mode, double* dir, double* dots,
+                         double* part, unsigned* count, cudaStream_t s);
+void launch_scalars_ls(const DevData& d, const ScalarArgs& sc, bool start, CgImage* st, CgControl* ctl,
+                       const double* dots, double* alpha, const int* dstatus, unsigned long long h_inner,
+                       cudaStream_t s);
 void launch_cg_record(int NI, CgImage* st, CgControl* ctl, const double* scal, double* hist, const int* dstatus,
                       unsigned long long h_outer, cudaStream_t s);
 
