@@ -83,19 +83,24 @@ struct mem_ctx {
     unsigned* col_count = nullptr;              // column-mean completion counters (zero between calls)
     float *ymax = nullptr, *ymax_part = nullptr;  // FP16X3: max |y| (adjoint operand scale), partials
     float* partial = nullptr;  // adjoint unit partials (FP32, one BLK x BLK block each)
-    int* dstatus = nullptr;
+    int* dstatus = nullptr;  // first word of the block that holds scal after it
     float* stage = nullptr;  // host-call staging (image, gradient)
     // pinned host words for the scalar and status readback (one copy pair and
     // one stream synchronisation per call; nullptr: pageable fallback)
     double* hscal = nullptr;
     size_t hscal_n = 0;
 
-    // CUDA graphs: each repeated launch sequence is captured once (on a private
-    // stream: the legacy default stream cannot be captured) and replayed on st
-    struct GraphSlot {
+    // CUDA graphs: a launch sequence that repeats with the same buffers is
+    // captured once (on a private stream: the legacy default stream cannot be
+    // captured) and replayed on st
+    struct GraphKey {
         const void* k1 = nullptr;
         const void* k2 = nullptr;
         int k3 = -1, prec = -1;
+        bool operator==(const GraphKey& o) const { return k1 == o.k1 && k2 == o.k2 && k3 == o.k3 && prec == o.prec; }
+    };
+    struct GraphSlot {
+        GraphKey key, last;  // of the captured graph; of the previous call
         int64_t nlaunch = 0;
         cudaGraphExec_t exec = nullptr;
     };
@@ -372,7 +377,7 @@ mem_status ensure_buffers(mem_ctx* c) {
     const size_t NN = (size_t)c->N * c->N;
     TRY(dalloc(c, &c->chi_part, (size_t)4 * std::max(std::max(c->n_tiles, c->n_tiles_tc), 1)));
     TRY(dalloc(c, &c->ent_part, (size_t)c->n_images * std::max(prep_blocks(c->N), std::max(tc_ent_blocks(c->N), fold_ent_blocks(c->N)))));
-    TRY(dalloc(c, &c->scal, (size_t)3 + 3 * c->n_images));
+    c->scal = (double*)c->dstatus + 1;
     if (!c->img_tmp) {  // holds the scalar reduction's completion counter, which starts at zero
         TRY(dalloc(c, &c->img_tmp, (size_t)scalars_tmp_doubles(c->n_images)));
         CK(cudaMemsetAsync(c->img_tmp, 0, scalars_tmp_doubles(c->n_images) * sizeof(double), c->st),
@@ -595,13 +600,26 @@ void drop_graphs(mem_ctx* c) {
 }
 
 // Run `body` (kernel launches on c->st only) through the graph slot: replay
-// when the slot was captured for the same keys, else capture and replay.
+// when the slot was captured for the same keys, capture and replay when the
+// previous call had them too, else launch directly.  A caller whose gradient
+// goes to a new buffer each time would otherwise pay for a capture per call:
+// 64 x 64, evaluation and readback, same buffers 38 us, two pairs of buffers in
+// turn 64 us captured and 45 us launched.
 // Buffers must already exist (no allocation inside a capture).
 mem_status graphed(mem_ctx* c, mem_ctx::GraphSlot& g, const void* k1, const void* k2, int k3,
                    const std::function<mem_status()>& body) {
     if (!c->graphs || c->profiling) return body();
-    if (!(g.exec && g.k1 == k1 && g.k2 == k2 && g.k3 == k3 && g.prec == c->prec)) {
+    mem_ctx::GraphKey key;
+    key.k1 = k1;
+    key.k2 = k2;
+    key.k3 = k3;
+    key.prec = c->prec;
+    const bool repeated = g.last == key;
+    g.last = key;
+    if (!(g.exec && g.key == key)) {
+        if (!repeated) return body();
         drop_graph(g);
+        g.last = key;
         if (!c->cap_st) CK(cudaStreamCreateWithFlags(&c->cap_st, cudaStreamNonBlocking), "capture stream");
         cudaStream_t user = c->st;
         c->st = c->cap_st;
@@ -628,10 +646,7 @@ mem_status graphed(mem_ctx* c, mem_ctx::GraphSlot& g, const void* k1, const void
             g.exec = nullptr;
             return cuda_fail(c, e, "graph instantiate");
         }
-        g.k1 = k1;
-        g.k2 = k2;
-        g.k3 = k3;
-        g.prec = c->prec;
+        g.key = key;
         g.nlaunch = n;
     }
     CK(cudaGraphLaunch(g.exec, c->st), "graph launch");
@@ -642,7 +657,7 @@ mem_status graphed(mem_ctx* c, mem_ctx::GraphSlot& g, const void* k1, const void
 mem_status read_scalars(mem_ctx* c, std::vector<double>& out) {
     out.resize(3 + 3 * (size_t)c->n_images);
     const size_t n = out.size();
-    if (c->hscal_n < n + 1) {  // the scalars, then the status word
+    if (c->hscal_n < n + 1) {  // the status word's slot, then the scalars
         if (c->hscal) cudaFreeHost(c->hscal);
         c->hscal = nullptr;
         c->hscal_n = 0;
@@ -650,13 +665,12 @@ mem_status read_scalars(mem_ctx* c, std::vector<double>& out) {
         else cudaGetLastError();  // pageable fallback below
     }
     if (c->hscal) {
-        // both words in pinned memory: two asynchronous copies, one synchronisation
-        int* hs = (int*)(c->hscal + n);
-        CK(cudaMemcpyAsync(c->hscal, c->scal, n * sizeof(double), cudaMemcpyDeviceToHost, c->st), "scalar readback");
-        CK(cudaMemcpyAsync(hs, c->dstatus, sizeof(int), cudaMemcpyDeviceToHost, c->st), "status readback");
+        // both in one copy to pinned memory
+        CK(cudaMemcpyAsync(c->hscal, c->dstatus, (n + 1) * sizeof(double), cudaMemcpyDeviceToHost, c->st),
+           "scalar readback");
         CK(cudaStreamSynchronize(c->st), "stream synchronize");
-        if (*hs & DEV_TIMEOUT) TRY(check_status(c));
-        std::copy(c->hscal, c->hscal + n, out.begin());
+        if (*(const int*)c->hscal & DEV_TIMEOUT) TRY(check_status(c));
+        std::copy(c->hscal + 1, c->hscal + 1 + n, out.begin());
     } else {
         CK(cudaMemcpyAsync(out.data(), c->scal, n * sizeof(double), cudaMemcpyDeviceToHost, c->st),
            "scalar readback");
@@ -1358,7 +1372,7 @@ mem_status mem_create(const mem_config* cfg, const double* u, const double* v, c
         (s = dalloc(c, &c->pb, std::max<int64_t>(Z, 1))) || (s = dalloc(c, &c->vo, std::max<int64_t>(Z, 1))) ||
         (s = dalloc(c, &c->vo32, std::max<int64_t>(Z, 1))) || (s = dalloc(c, &c->w32, std::max<int64_t>(Z, 1))) ||
         (s = dalloc(c, &c->beam, (size_t)C * NN)) || (s = dalloc(c, &c->doff, (size_t)C + 1)) ||
-        (s = dalloc(c, &c->dstatus, 1))) {
+        (s = dalloc(c, &c->dstatus, 2 * (size_t)(4 + 3 * c->n_images)))) {
         g_last_error = c->err;
         return bail(s);
     }
@@ -1386,7 +1400,7 @@ mem_status mem_create(const mem_config* cfg, const double* u, const double* v, c
     if (e == cudaSuccess) e = cpy(c->vo32, vo32h.data(), Z * sizeof(float4));
     if (e == cudaSuccess) e = cpy(c->beam, pb, C * NN * sizeof(float));
     if (e == cudaSuccess) e = cpy(c->doff, c->off.data(), (C + 1) * sizeof(int64_t));
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->dstatus, 0, sizeof(int), c->st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->dstatus, 0, (4 + 3 * c->n_images) * sizeof(double), c->st);
     if (e != cudaSuccess) {
         cuda_fail(c, e, "upload");
         g_last_error = c->err;
