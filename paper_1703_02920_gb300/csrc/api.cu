@@ -407,7 +407,8 @@ mem_status ensure_buffers(mem_ctx* c) {
         TRY(dalloc(c, &c->ymax_part, (size_t)256));
         const int BLK = tca_blk(c->N);
         TRY(dalloc(c, &c->partial, std::max<size_t>(c->units_h.size(), 1) * BLK * BLK));
-        if (c->fwd_kernel == MEM_FWD_RESIDENT && (c->prec == MEM_PREC_BF16X3 || fold_combines(c->N)))
+        if (c->fwd_kernel == MEM_FWD_RESIDENT &&
+            (c->prec == MEM_PREC_BF16X3 ? fwd_rs_ks(c->N) < c->N : fold_combines(c->N)))
             TRY(dalloc(c, &c->vpart, (size_t)2 * std::max<int64_t>(c->Z, 1)));
     }
     int ks = 1;
@@ -481,9 +482,9 @@ mem_status run_forward(mem_ctx* c, const ImgSrc& src, int mode, bool entropy, vo
                                            c->chi_part, ymax, c->vpart, c->Z, c->num_sms, c->spin,
                                            c->dstatus, c->st);
         } else if (resident) {
-            launch_fwd_rs(d, c->tiles_tc, c->n_tiles_tc, c->planes, c->cmean, mode, (float2*)yout, c->chi_part,
-                          (double2*)c->vpart, c->Z, c->num_sms, c->spin, c->dstatus, c->st);
-            if (c->n_tiles_tc > 0) c->launches += 2;  // and the slice combination
+            c->launches += launch_fwd_rs(d, c->tiles_tc, c->n_tiles_tc, c->planes, c->cmean, mode, (float2*)yout,
+                                         c->chi_part, (double2*)c->vpart, c->Z, c->num_sms, c->spin, c->dstatus,
+                                         c->st);
         } else {
             launch_fwd_tc(d, c->tiles_tc, c->n_tiles_tc, c->planes, c->cmean, mode, (float2*)yout, c->chi_part,
                           c->num_sms, c->spin, c->dstatus, c->st);

@@ -370,6 +370,24 @@ __device__ __forceinline__ void umma6_fold_elect(uint32_t dt, uint32_t ah, uint3
         "r"(ah), "r"(al), "r"(bh), "r"(bl), "r"(hia), "r"(hib), "r"(ka), "r"(kb), "r"(idesc), "r"(acc), "r"(1u));
 }
 
+// The stage's four correction products in the order hi x lo, lo x hi per K step.
+__device__ __forceinline__ void umma_cross_elect(uint32_t dt, uint32_t ah, uint32_t al, uint32_t bh, uint32_t bl,
+                                                 uint32_t hia, uint32_t hib, uint32_t ka, uint32_t kb,
+                                                 uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n .reg .pred p, one, e;\n .reg .b64 d0, d1, d2, d3, d4, d5, d6, d7;\n .reg .b32 t0, t1, t2, t3;\n"
+        " setp.ne.b32 p, %10, 0;\n setp.ne.b32 one, %11, 0;\n"
+        " elect.sync _|e, 0xffffffff;\n"
+        " mov.b64 d0, {%1, %5};\n mov.b64 d1, {%2, %5};\n mov.b64 d2, {%3, %6};\n mov.b64 d3, {%4, %6};\n"
+        " add.u32 t0, %1, %7;\n add.u32 t1, %2, %7;\n add.u32 t2, %3, %8;\n add.u32 t3, %4, %8;\n"
+        " mov.b64 d4, {t0, %5};\n mov.b64 d5, {t1, %5};\n mov.b64 d6, {t2, %6};\n mov.b64 d7, {t3, %6};\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], d0, d3, %9, p;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], d1, d2, %9, one;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], d4, d7, %9, one;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], d5, d6, %9, one;\n}\n" ::"r"(dt),
+        "r"(ah), "r"(al), "r"(bh), "r"(bl), "r"(hia), "r"(hib), "r"(ka), "r"(kb), "r"(idesc), "r"(acc), "r"(1u));
+}
+
 // The stage's four correction products only, and its two main products only
 // (for an accumulation that issues all of its corrections first).
 __device__ __forceinline__ void umma_corrections_elect(uint32_t dt, uint32_t ah, uint32_t al, uint32_t bh,

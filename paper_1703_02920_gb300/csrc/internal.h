@@ -159,11 +159,12 @@ void launch_fwd_tc(const DevData& d, const VisTile* tiles, int n_tiles, const vo
                    int mode, float2* yout, double* chi_part, int grid, uint64_t spin, int* status, cudaStream_t st);
 // BF16X3 forward, resident operand (N <= 256): the image rows are cut into
 // slices of fwd_rs_ks(N); each CTA keeps one slice of the operand planes in
-// shared memory; slice partials (FP64, [slice][visibility]) are combined by a
-// second kernel that also applies the forward mode.
+// shared memory; the partials of several slices (FP64, [slice][visibility]) are
+// combined by a second kernel, which then applies the forward mode.  Returns the
+// launches.
 __host__ __device__ inline int fwd_rs_ks(int N) { return N < 128 ? N : 128; }
 int fwd_rs_smem_bytes(int N, int stages);
-void launch_fwd_rs(const DevData& d, const VisTile* tiles, int n_tiles, const void* planes, const float* cmean,
+int launch_fwd_rs(const DevData& d, const VisTile* tiles, int n_tiles, const void* planes, const float* cmean,
                    int mode, float2* yout, double* chi_part, double2* vpart, int64_t z_total, int num_sms,
                    uint64_t spin, int* status, cudaStream_t st);
 // The paper's gridded forward: the 2-D real-to-complex transform of every
