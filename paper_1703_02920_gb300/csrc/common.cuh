@@ -560,11 +560,13 @@ __device__ __forceinline__ void split16x2p(float2 v, uint32_t& hi, uint32_t& lo)
         hi = *reinterpret_cast<const uint32_t*>(&h);
         lo = *reinterpret_cast<const uint32_t*>(&l);
     } else {
-        const __nv_bfloat162 h = __float22bfloat162_rn(v);
-        const float2 hf = __bfloat1622float2(h);
-        const __nv_bfloat162 l = __float22bfloat162_rn(__ffma2_rn(hf, make_float2(-1.f, -1.f), v));
-        hi = *reinterpret_cast<const uint32_t*>(&h);
-        lo = *reinterpret_cast<const uint32_t*>(&l);
+        // a - hi as one mixed-precision FMA (exact), without a conversion of hi
+        // back to FP32
+        asm("{\n .reg .b16 h0, h1, m1;\n .reg .f32 la, lb;\n mov.b16 m1, 0xBF80;\n cvt.rn.bf16x2.f32 %0, %3, %2;\n"
+            " mov.b32 {h0, h1}, %0;\n fma.rn.f32.bf16 la, h0, m1, %2;\n fma.rn.f32.bf16 lb, h1, m1, %3;\n"
+            " cvt.rn.bf16x2.f32 %1, lb, la;\n}\n"
+            : "=&r"(hi), "=r"(lo)
+            : "f"(v.x), "f"(v.y));
     }
 }
 

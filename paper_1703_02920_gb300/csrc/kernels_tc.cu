@@ -36,9 +36,18 @@ namespace msk {
 // FP32 two-sum).
 // Operands are MN-major (8 consecutive pixels of one visibility per 16-byte
 // core-matrix row), the layout the per-visibility phase recurrences produce.
-// Roles: warp 4 MMA + TMEM owner; the other 13 warps produce operand stages,
-// and warps 0-3 (TMEM lane quadrants 0-3) also drain the accumulator to the
-// split-K partials every ADJ_DRAIN stages and at the end of each unit.
+// Roles: warps 0-3 (TMEM lane quadrants 0-3) drain the accumulator to the split-K
+// partials every ADJ_DRAIN stages and at the end of each unit; warp 4 MMA + TMEM
+// owner; warps 8-23 produce operand stages, two groups of eight on alternate
+// stages, so that a stage's latencies (inputs, slot wait, stores, proxy fence)
+// overlap the other group's.
+//
+// What bounds it: the MMAs (N >= 256: 1,536 clocks a stage) and the issue slots of
+// the producers, which need nearly as many.  With all producer warps on the same
+// stage its chain of latencies, about 2,100 clocks whatever N, was the bound.
+// 1024 x 1024 with 100,000 visibilities: 743 -> 598 us (the MMAs alone 0.52 ms),
+// 256 x 256 with 300,000: 148 -> 121 us, 128 x 128 with 100,003: 51 -> 31 us (CUDA
+// events around the launch, about 5 us of which are theirs); the same bits.
 // ===========================================================================
 constexpr int ADJ_MAX_STAGES = 3;
 // Stages (of 16 visibilities) accumulated in TMEM before the accumulator is
@@ -48,8 +57,8 @@ constexpr int ADJ_MAX_STAGES = 3;
 // bias at ~2.5e-5 relative however many visibilities a unit spans.  The drains
 // add with round-to-nearest FP32 reductions, which have no such bias.
 constexpr int ADJ_DRAIN = 256;
-constexpr int ADJ_THREADS = 448;
-constexpr int ADJ_PRODUCER_WARPS = ADJ_THREADS / 32 - 1;  // every warp but the MMA warp
+constexpr int ADJ_PRODUCERS = 16;  // producer warps: two groups of eight, alternate stages
+constexpr int ADJ_THREADS = 32 * (8 + ADJ_PRODUCERS);
 
 __host__ __device__ inline int adj_rows(int BLK) { return BLK < 128 ? 128 : BLK; }
 __host__ __device__ inline int adj_stage_bytes(int BLK) {
@@ -86,9 +95,8 @@ __host__ __device__ inline void adj_partial_rc(int64_t i, int BLK, int& n, int& 
 }
 
 // Drain of the TMEM accumulator by warps 0-3 (TMEM lane quadrant = warp):
-// partial (one unit's block, layout above) = [partial +] accumulator.  Kept
-// out of line so that its registers do not add to the producers' loop.
-__device__ __noinline__ void adj_drain(uint32_t tmem, float* out, int BLK, int n_mt, int warp, int lane,
+// partial (one unit's block, layout above) = [partial +] accumulator.
+__device__ void adj_drain(uint32_t tmem, float* out, int BLK, int n_mt, int warp, int lane,
                                        bool first) {
     const int RB = BLK < 128 ? BLK : 128;
     for (int mt = 0; mt < n_mt; ++mt) {
@@ -153,7 +161,7 @@ __global__ void __launch_bounds__(ADJ_THREADS, 1)
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < ADJ_STAGES; ++s) {
-            mbar_init(&S.full[s], ADJ_PRODUCER_WARPS);
+            mbar_init(&S.full[s], ADJ_PRODUCERS / 2);
             mbar_init(&S.empty[s], 1);
         }
         mbar_init(&S.tfull, 1);
@@ -227,126 +235,101 @@ __global__ void __launch_bounds__(ADJ_THREADS, 1)
             mbar_wait(&S.drain, 0, drain_limit(spin), (volatile int*)&dummy, status);
         }
         __syncwarp();
-    } else {
-        // ------------------------------------------ producers (13 warps, 416 thr)
+    } else if (warp < 4) {
+        // -------------------------------------------------------------- drain
+        // after the last stage of each accumulation segment into the unit's
+        // partial
+        uint32_t dr = 0;
+        bool ok = true;
+        for (int u = u0; u < u1 && ok; ++u) {
+            const int nst = (int)((units[u].count + TCA_BK - 1) / TCA_BK);
+            for (int seg0 = 0; seg0 < nst; seg0 += ADJ_DRAIN, ++dr) {
+                ok = __all_sync(0xffffffffu, mbar_wait(&S.tfull, dr & 1, spin, abort, status, 1024));
+                if (!ok) break;
+                tc_fence_after();
+                adj_drain(tmem, partial + (int64_t)u * BLK * BLK, BLK, n_mt, warp, lane,
+                          seg0 == 0 /* the unit's first segment stores */);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&S.tempty);
+            }
+        }
+    } else if (warp >= 8) {
+        // ---------------------------------------- producers (two groups of 8)
         // A warp-iteration builds two items (8 pixels of 16 visibilities each,
         // one per half-warp).  Whole warps take one side, Ey items (A operand)
         // or P items (B operand), so each thread builds one step table per
-        // stage and the halves of a warp never diverge.  A stage has 16
-        // warp-iterations per side (N >= 256); the table gives each warp a
-        // contiguous run of them such that every SM sub-partition (warp % 4;
-        // their FMA pipes are the busy units) carries 8 per stage and no warp
-        // more than 3.  Smaller images use the runs' first entries.
-        const int pw = warp < 4 ? warp : warp - 1;  // producer warp 0..12
-        const int ey_side = (0x3F >> pw) & 1;       // warps 0-3, 5, 6
-        const int wi_start = (int)((0xA6EC8039E63C0ull >> (4 * pw)) & 15);
-        const int wi_cap = (int)((0x2222233323323ull >> (4 * pw)) & 15);
+        // stage and the halves of a warp never diverge.  Every SM sub-partition
+        // (warp % 4) has one warp of each side and group.
+        const uint32_t grp = (warp - 8) >> 3;
+        const bool ey_side = ((warp >> 2) & 1) == 0;
         const int half = lane >> 4;
         const int jj = lane & 15;           // visibility within the stage
         const int ngA = R / 8, ngB = BLK / 8;
-        const int wi_end = min(wi_start + wi_cap, (ey_side ? ngA : ngB) / 2);
-        uint32_t sc = 0, dr = 0;  // stages produced; accumulator drains (warps 0-3)
+        const int wi_end = (ey_side ? ngA : ngB) / 2;
+        const int ng = ey_side ? ngA : ngB, plane = ey_side ? a_plane : b_plane;
+        const int side = ey_side ? 0 : 4 * a_plane;  // offset within a stage
+        uint32_t sc = 0;  // stages so far, both groups'
         bool ok = true;
         for (int u = u0; u < u1 && ok; ++u) {
             const AdjUnit un = units[u];
-            const int blk_n0 = (un.block / nbx) * BLK, blk_m0 = (un.block % nbx) * BLK;
+            const int p0 = (ey_side ? un.block / nbx : un.block % nbx) * BLK - c0;  // first pixel
             const int nst = (int)((un.count + TCA_BK - 1) / TCA_BK);
-            // per-visibility inputs of the next stage are loaded one stage ahead
-            auto fetch = [&](int ks, uint64_t& fa, uint64_t& fb, float2& fy) {
+            // this group's inputs of its next stage are loaded one stage ahead
+            // (the phase of the side, and y on the P side)
+            uint64_t np = 0;
+            float2 ny = make_float2(0.f, 0.f);
+            auto fetch = [&](int ks) {
                 const int64_t kv = (int64_t)ks * TCA_BK + jj;
-                fa = 0;
-                fb = 0;
-                fy = make_float2(0.f, 0.f);
+                np = 0;
+                ny = make_float2(0.f, 0.f);
                 if (ks < nst && kv < un.count) {
-                    if (FROM_UV) {
-                        fa = to_fixed_turns(d.u[un.start + kv] * d.dx);
-                        fb = to_fixed_turns(d.v[un.start + kv] * d.dy);
-                    } else {
-                        fa = d.pa[un.start + kv];
-                        fb = d.pb[un.start + kv];
-                    }
-                    fy = y[un.start + kv];
+                    if (FROM_UV) np = ey_side ? to_fixed_turns(d.v[un.start + kv] * d.dy)
+                                              : to_fixed_turns(d.u[un.start + kv] * d.dx);
+                    else np = (ey_side ? d.pb : d.pa)[un.start + kv];
+                    if (!ey_side) ny = y[un.start + kv];
                 }
             };
-            uint64_t na, nb;
-            float2 ny;
-            fetch(0, na, nb, ny);
-          for (int seg0 = 0; seg0 < nst && ok; seg0 += ADJ_DRAIN) {
-            const int seg1 = min(nst, seg0 + ADJ_DRAIN);
-            for (int ks = seg0; ks < seg1; ++ks, ++sc) {
-                const int s = sc % ADJ_STAGES;
-                const uint64_t pa = na, pb = nb;
+            const int k0 = (int)((sc ^ grp) & 1);
+            fetch(k0);
+            for (int ks = k0; ks < nst; ks += 2) {
+                const uint32_t q = sc + ks;
+                const int s = q % ADJ_STAGES;
+                const uint64_t ph = np;
                 const cf2 yv = {ny.x, ny.y};
                 const bool valid = (int64_t)ks * TCA_BK + jj < un.count;
-                fetch(ks + 1, na, nb, ny);
+                fetch(ks + 2);
                 // rotation steps exp(-i 2 pi q c), q = 0..7, by powers of one SFU
                 // value: c = b for the Ey side, a for the P side (computed before
                 // the wait for the ring slot, which they do not need)
                 cf2 st[8];
                 st[0] = {1.f, 0.f};
-                st[1] = cis_neg(ey_side ? pb : pa);
+                st[1] = cis_neg(ph);
                 st[2] = cmul(st[1], st[1]);
                 st[4] = cmul(st[2], st[2]);
                 st[3] = cmul(st[2], st[1]);
                 st[5] = cmul(st[4], st[1]);
                 st[6] = cmul(st[4], st[2]);
                 st[7] = cmul(st[4], st[3]);
-                ok = __all_sync(0xffffffffu, mbar_wait(&S.empty[s], ((sc / ADJ_STAGES) & 1) ^ 1, spin,
+                if (!ey_side) {
+                    // P = y conj(Ex): conj(base) times conj(steps)
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) st[k].y = -st[k].y;
+                }
+                const Rot8 w = rot8_of(st);
+                ok = __all_sync(0xffffffffu, mbar_wait(&S.empty[s], ((q / ADJ_STAGES) & 1) ^ 1, spin,
                                                        abort, status, 64));
                 if (!ok) break;
-                unsigned char* A = smem + s * stage_bytes;
-                unsigned char* B = A + 4 * a_plane;
-                // at most 3 warp-iterations (the table): unrolled so that the
-                // items' independent arithmetic interleaves
-#pragma unroll
-                for (int r = 0; r < 3; ++r) {
-                    const int wi = wi_start + r;
-                    if (wi >= wi_end) break;
-                    const int item = ey_side ? 2 * wi + half : ngA + 2 * wi + half;
+                unsigned char* dst0 = smem + s * stage_bytes + side + (jj >> 3) * ng * 128 + (jj & 7) * 16;
+#pragma unroll 2
+                for (int wi = warp & 3; wi < wi_end; wi += 4) {
+                    const int g = 2 * wi + half;
                     uint4 rh = {0, 0, 0, 0}, rl = {0, 0, 0, 0}, ih = {0, 0, 0, 0}, il = {0, 0, 0, 0};
-                    unsigned char* dst;
-                    int plane;
-                    if (item < ngA) {
-                        const int g = item;
-                        const int n0 = blk_n0 + g * 8;
-                        if (valid && g * 8 < BLK) {
-                            const cf2 base = cis_neg(phase_mul(n0 - c0, pb));
-                            cf2 z[8];
-#pragma unroll
-                            for (int q = 0; q < 8; ++q) z[q] = cmul(base, st[q]);
-                            split_bf16x2(z[0].x, z[1].x, rh.x, rl.x);
-                            split_bf16x2(z[2].x, z[3].x, rh.y, rl.y);
-                            split_bf16x2(z[4].x, z[5].x, rh.z, rl.z);
-                            split_bf16x2(z[6].x, z[7].x, rh.w, rl.w);
-                            split_bf16x2(z[0].y, z[1].y, ih.x, il.x);
-                            split_bf16x2(z[2].y, z[3].y, ih.y, il.y);
-                            split_bf16x2(z[4].y, z[5].y, ih.z, il.z);
-                            split_bf16x2(z[6].y, z[7].y, ih.w, il.w);
-                        }
-                        dst = A + ((jj >> 3) * ngA + g) * 128 + (jj & 7) * 16;
-                        plane = a_plane;
-                    } else {
-                        const int g = item - ngA;
-                        const int m0 = blk_m0 + g * 8;
-                        if (valid) {
-                            // P = y conj(Ex): conj(base) times conj(steps)
-                            const cf2 e = cis_neg(phase_mul(m0 - c0, pa));
-                            const cf2 base = cmul(yv, cf2{e.x, -e.y});
-                            cf2 z[8];
-#pragma unroll
-                            for (int q = 0; q < 8; ++q) z[q] = cmul(base, cf2{st[q].x, -st[q].y});
-                            split_bf16x2(z[0].x, z[1].x, rh.x, rl.x);
-                            split_bf16x2(z[2].x, z[3].x, rh.y, rl.y);
-                            split_bf16x2(z[4].x, z[5].x, rh.z, rl.z);
-                            split_bf16x2(z[6].x, z[7].x, rh.w, rl.w);
-                            split_bf16x2(z[0].y, z[1].y, ih.x, il.x);
-                            split_bf16x2(z[2].y, z[3].y, ih.y, il.y);
-                            split_bf16x2(z[4].y, z[5].y, ih.z, il.z);
-                            split_bf16x2(z[6].y, z[7].y, ih.w, il.w);
-                        }
-                        dst = B + ((jj >> 3) * ngB + g) * 128 + (jj & 7) * 16;
-                        plane = b_plane;
+                    if (valid && g * 8 < BLK) {
+                        const cf2 e = cis_neg(phase_mul(p0 + g * 8, ph));
+                        table8_split<false>(ey_side ? e : cmul(yv, cf2{e.x, -e.y}), w, rh, rl, ih, il);
                     }
+                    unsigned char* dst = dst0 + g * 128;
                     *(uint4*)(dst + 0 * plane) = rh;
                     *(uint4*)(dst + 1 * plane) = rl;
                     *(uint4*)(dst + 2 * plane) = ih;
@@ -356,19 +339,7 @@ __global__ void __launch_bounds__(ADJ_THREADS, 1)
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&S.full[s]);
             }
-            // warps 0-3 drain the accumulator after the last stage of each
-            // accumulation segment into the unit's partial
-            if (!ok || warp >= 4) continue;
-            ok = __all_sync(0xffffffffu, mbar_wait(&S.tfull, dr & 1, spin, abort, status, 1024));
-            if (!ok) break;
-            tc_fence_after();
-            adj_drain(tmem, partial + (int64_t)u * BLK * BLK, BLK, n_mt, warp, lane,
-                      seg0 == 0 /* the unit's first segment stores */);
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&S.tempty);
-            ++dr;
-          }
+            sc += nst;
         }
     }
 
