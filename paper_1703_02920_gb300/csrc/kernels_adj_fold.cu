@@ -396,6 +396,7 @@ void launch_adj_fold(const DevData& d, const AdjUnit* units, const int* cta_unit
 // an image row); smaller images take one, so that 64 x 64 still fills 64 blocks.
 // ===========================================================================
 constexpr int RED_ROWS = 32;
+constexpr int RED_AHEAD = 8;  // units whose partials are loaded together
 template <bool WIDE>
 struct RedGeo {
     static constexpr int COLS = WIDE ? 4 : 1, ELEMS = RED_ROWS * COLS;
@@ -454,19 +455,19 @@ __global__ void __launch_bounds__(RedGeo<WIDE>::THREADS) k_adj_fold_reduce(DevDa
     const float* p = a.partial + (int64_t)ua * stride + (int64_t)q * rows + r;
     float s0 = 0.f, e0 = 0.f, s1 = 0.f, e1 = 0.f;
     int u = ua;
-    for (; u + 4 <= ub; u += 4) {
-        float x[4], z[4];
+    for (; u + RED_AHEAD <= ub; u += RED_AHEAD) {
+        float x[RED_AHEAD], z[RED_AHEAD];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < RED_AHEAD; ++k) {
             x[k] = __ldg(p + k * stride);
             z[k] = __ldg(p + k * stride + half);
         }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < RED_AHEAD; ++k) {
             two_sum_acc(s0, e0, x[k]);
             two_sum_acc(s1, e1, z[k]);
         }
-        p += 4 * stride;
+        p += RED_AHEAD * stride;
     }
     for (; u < ub; ++u, p += stride) {
         two_sum_acc(s0, e0, __ldg(p));
@@ -496,16 +497,15 @@ __global__ void __launch_bounds__(RedGeo<WIDE>::THREADS) k_adj_fold_reduce(DevDa
         const int rr = (t % row_tiles) * RED_ROWS + er, qq = (t / row_tiles) * COLS + eq;
         const int j = WIDE ? (blk / nbx) * 128 + rr : qq, m = WIDE ? (blk % nbx) * 256 + qq : rr;
         const int n = sign ? N / 2 - 1 - j : N / 2 + j;
-        const double inv = 1.0 / (double)pow2_scale_for(a.ymax[0]);
-        const double gchi = ((double)tot[0] + (sign ? -(double)tot[1] : (double)tot[1])) * inv;
+        const double inv = pow2_inverse(pow2_scale_for(a.ymax[0]));
+        const float other = sign ? -tot[1] : tot[1];
         const int64_t pix = (int64_t)c * NN + (int64_t)n * N + m;
         if (OUT == RED_GSUM) {
-            a.gsum[pix] = gchi;
+            a.gsum[pix] = ((double)tot[0] + (double)other) * inv;
         } else {
-            double gr = (double)d.beam[pix] * gchi;
             const double x = img_value(src, c, (int64_t)n * N + m, NN);
-            if (d.lambda != 0.0) gr += d.lambda * (1.0 + log_ratio(x, d.G, d.ginv));
-            const double gp = (x <= d.G && gr > 0.0) ? 0.0 : gr;
+            const double gr = pixel_gradient(d, d.beam[pix], tot[0], other, inv, x);
+            const double gp = project_pixel(d, x, gr);
             if (a.full64) a.full64[pix] = gr;
             if (a.proj64) a.proj64[pix] = gp;
             if (a.out32) a.out32[pix] = (float)(a.projected ? gp : gr);

@@ -408,9 +408,10 @@ void launch_adj_tc_reduce_out(int N, const int* cb_unit_off, const float* partia
 // combined in group order, so the sum has a fixed order (independent of the
 // launch) and four times the loads in flight of one thread per element.
 constexpr int RED_ELEMS = 64;
-__device__ __forceinline__ void unit_sum_quarter(const float* __restrict__ src, int64_t stride, int u0, int u1, int g,
-                                                 float& s, float& comp) {
-    const int ua = u0 + (u1 - u0) * g / 4, ub = u0 + (u1 - u0) * (g + 1) / 4;
+template <int SPLIT>
+__device__ __forceinline__ void unit_sum_share(const float* __restrict__ src, int64_t stride, int u0, int u1, int g,
+                                               float& s, float& comp) {
+    const int ua = u0 + (u1 - u0) * g / SPLIT, ub = u0 + (u1 - u0) * (g + 1) / SPLIT;
     s = 0.f;
     comp = 0.f;
     int u = ua;
@@ -456,7 +457,7 @@ __global__ void __launch_bounds__(256) k_adj_tc_reduce(DevData d, const int* __r
     const int cb = c * nbx * nbx + blk;
     const int u0 = in ? cb_unit_off[cb] : 0, u1 = in ? cb_unit_off[cb + 1] : 0;
     float s, comp;
-    unit_sum_quarter(partial + loc, (int64_t)BLK * BLK, u0, u1, g, s, comp);
+    unit_sum_share<4>(partial + loc, (int64_t)BLK * BLK, u0, u1, g, s, comp);
     const float tot = unit_sum_combine(s, comp, el, g, sh);
     if (g != 0 || !in) return;
     int nl, ml;
@@ -484,11 +485,16 @@ void launch_adj_tc_reduce(const DevData& d, const int* cb_unit_off, const float*
 // reduction (scalars_block): it needs only the forward's chi^2 partials and
 // the prep's entropy partials, so it shares this launch instead of taking one
 // of its own.
+// SPLIT groups per element as above, or one where an output block has few units
+// (10 at 1024 x 1024): every thread then has a pixel's FP64 operations, which
+// a quarter of the threads would have to wait out (62 -> 47 us there).
+template <int SPLIT>
 __global__ void __launch_bounds__(256) k_adj_tc_reduce_grad(DevData d, ImgSrc src,
                                                             const int* __restrict__ cb_unit_off,
                                                             const float* __restrict__ partial, int projected,
                                                             float* out32, double* full64, double* proj64,
                                                             ScalarArgs sc) {
+    constexpr int ELEMS = 256 / SPLIT;
     __shared__ float sh[4][RED_ELEMS][2];
     const int N = d.N;
     const int64_t NN = (int64_t)N * N;
@@ -500,25 +506,27 @@ __global__ void __launch_bounds__(256) k_adj_tc_reduce_grad(DevData d, ImgSrc sr
     const int BLK = N < 256 ? N : 256;
     const int nbx = N / BLK;
     const int c = blockIdx.y;  // channel = image
-    const int el = threadIdx.x % RED_ELEMS, g = threadIdx.x / RED_ELEMS;
-    const int64_t i = (int64_t)(blockIdx.x - n_scal) * RED_ELEMS + el;
+    const int el = threadIdx.x % ELEMS, g = threadIdx.x / ELEMS;
+    const int64_t i = (int64_t)(blockIdx.x - n_scal) * ELEMS + el;
     const bool in = i < NN;
     const int blk = in ? (int)(i / ((int64_t)BLK * BLK)) : 0;
     const int64_t loc = in ? i % ((int64_t)BLK * BLK) : 0;
     const int cb = c * nbx * nbx + blk;
     const int u0 = in ? cb_unit_off[cb] : 0, u1 = in ? cb_unit_off[cb + 1] : 0;
     float s, comp;
-    unit_sum_quarter(partial + loc, (int64_t)BLK * BLK, u0, u1, g, s, comp);
-    const float tot = unit_sum_combine(s, comp, el, g, sh);
+    unit_sum_share<SPLIT>(partial + loc, (int64_t)BLK * BLK, u0, u1, g, s, comp);
+    float tot = s + comp;
+    if constexpr (SPLIT == 4) tot = unit_sum_combine(s, comp, el, g, sh);
     if (g != 0 || !in) return;
     int nl, ml;
     adj_partial_rc(loc, BLK, nl, ml);
     const int64_t p = (int64_t)((blk / nbx) * BLK + nl) * N + (blk % nbx) * BLK + ml;
-    const double gchi = (double)tot;
-    double gr = (double)d.beam[(int64_t)c * NN + p] * gchi;
     const double x = img_value(src, c, p, NN);
+    // (a converged solve of this form stops within 7 % of its test's bound: not one
+    // rounding moves)
+    double gr = (double)d.beam[(int64_t)c * NN + p] * (double)tot;
     if (d.lambda != 0.0) gr += d.lambda * (1.0 + log_ratio(x, d.G, d.ginv));
-    const double gp = (x <= d.G && gr > 0.0) ? 0.0 : gr;
+    const double gp = project_pixel(d, x, gr);
     if (full64) full64[(int64_t)c * NN + p] = gr;
     if (proj64) proj64[(int64_t)c * NN + p] = gp;
     if (out32) out32[(int64_t)c * NN + p] = (float)(projected ? gp : gr);
@@ -528,10 +536,11 @@ void launch_adj_tc_reduce_grad(const DevData& d, const ImgSrc& src, const int* c
                                int projected, float* out32, double* full64, double* proj64,
                                const ScalarArgs& sc, cudaStream_t st) {
     const int64_t NN = (int64_t)d.N * d.N;
-    const unsigned gb = (unsigned)((NN + RED_ELEMS - 1) / RED_ELEMS);
-    dim3 grid(gb + (sc.scal ? sc.splits : 0), d.C);
-    k_adj_tc_reduce_grad<<<grid, 256, 0, st>>>(d, src, cb_unit_off, partial, projected, out32, full64,
-                                                proj64, sc);
+    const bool one = d.N >= 1024;
+    const int elems = one ? 256 : RED_ELEMS;
+    const dim3 grid((unsigned)((NN + elems - 1) / elems) + (sc.scal ? sc.splits : 0), d.C);
+    auto kernel = one ? k_adj_tc_reduce_grad<1> : k_adj_tc_reduce_grad<4>;
+    kernel<<<grid, 256, 0, st>>>(d, src, cb_unit_off, partial, projected, out32, full64, proj64, sc);
 }
 
 }  // namespace msk
