@@ -81,7 +81,8 @@ struct mem_ctx {
     float4* cmean4 = nullptr;                   // FP16X3: means and inverse scale per strip
     double* col_psum = nullptr;                 // column-mean partial sums
     unsigned* col_count = nullptr;              // column-mean completion counters (zero between calls)
-    float *ymax = nullptr, *ymax_part = nullptr;  // FP16X3: max |y| (adjoint operand scale), partials
+    float* ymax = nullptr;           // FP16X3: max |y| (adjoint operand scale)
+    unsigned* ymax_count = nullptr;  // its running maximum and completion counter, zero between launches
     float* partial = nullptr;  // adjoint unit partials (FP32, one BLK x BLK block each)
     int* dstatus = nullptr;  // first word of the block that holds scal after it
     float* stage = nullptr;  // host-call staging (image, gradient)
@@ -404,7 +405,10 @@ mem_status ensure_buffers(mem_ctx* c) {
             TRY(dalloc(c, &c->col_psum, (size_t)colmean_tmp_count(c->N, c->C)));
         }
         TRY(dalloc(c, &c->ymax, (size_t)1));
-        TRY(dalloc(c, &c->ymax_part, (size_t)256));
+        if (!c->ymax_count) {
+            TRY(dalloc(c, &c->ymax_count, (size_t)2));
+            CK(cudaMemsetAsync(c->ymax_count, 0, 2 * sizeof(unsigned), c->st), "counters");
+        }
         const int BLK = tca_blk(c->N);
         TRY(dalloc(c, &c->partial, std::max<size_t>(c->units_h.size(), 1) * BLK * BLK));
         if (c->fwd_kernel == MEM_FWD_RESIDENT &&
@@ -519,44 +523,49 @@ mem_status run_forward(mem_ctx* c, const ImgSrc& src, int mode, bool entropy, vo
     return MEM_OK;
 }
 
-// adjoint of y (already in y32 / y64) into gsum; returns ks used.
-// ymax_ready: the FP16X3 operand scale's maximum was written by the RESID
-// forward that produced y32.
-mem_status run_adjoint(mem_ctx* c, int* ks_out, bool ymax_ready = false, bool reduce = true) {
+// What run_adjoint leaves: gsum (ks shares of it), for the tensor-core forms
+// alternatively the units' partials only or the sums as FP32 in out32.
+struct AdjointOut {
+    int ks = 1;
+    bool reduce = true;
+    float* out32 = nullptr;
+};
+
+// adjoint of y (y64 in the FP64 form).  ymax_ready: the FP16X3 operand scale's
+// maximum was written by the kernel that produced y.
+mem_status run_adjoint(mem_ctx* c, const float2* y, bool ymax_ready, AdjointOut& out) {
     DevData d = c->dd();
     if (is_tc(c->prec)) {
         const int f16 = c->prec == MEM_PREC_FP16X3;
         if (f16 && !ymax_ready) {
             KTimer t(c, "ymax");
-            launch_absmax(2 * c->Z, (const float*)c->y32, c->ymax_part, c->ymax, c->st);
-            c->launches += 2;
+            launch_absmax(c->Z, y, c->num_sms, c->ymax_count, c->ymax, c->st);
+            c->launches++;
         }
         if (c->adj_ctas > 0) {
             KTimer t(c, "adj_tc");
             if (f16)
-                launch_adj_fold(d, c->units, c->cta_off, c->adj_ctas, c->y32, c->ymax, c->partial, c->spin, c->dstatus,
+                launch_adj_fold(d, c->units, c->cta_off, c->adj_ctas, y, c->ymax, c->partial, c->spin, c->dstatus,
                                 c->st);
             else
-                launch_adj_tc(d, c->units, c->cta_off, c->adj_ctas, c->y32, c->partial, c->spin, c->dstatus, c->st);
+                launch_adj_tc(d, c->units, c->cta_off, c->adj_ctas, y, c->partial, c->spin, c->dstatus, c->st);
             c->launches++;
             TRY(after_launch(c, "adjoint kernel"));
         }
-        *ks_out = 1;
-        if (!reduce) return MEM_OK;
+        if (!out.reduce) return MEM_OK;
         KTimer t(c, "adj_tc_reduce");
-        if (f16) launch_adj_fold_reduce(d, c->cb_off, c->partial, c->ymax, c->gsum, c->st);
-        else launch_adj_tc_reduce(d, c->cb_off, c->partial, c->gsum, c->st);
+        if (f16) launch_adj_fold_reduce(d, c->cb_off, c->partial, c->ymax, c->gsum, out.out32, c->st);
+        else launch_adj_tc_reduce(d, c->cb_off, c->partial, c->gsum, out.out32, c->st);
         c->launches++;
         TRY(after_launch(c, "adjoint reduction"));
-        *ks_out = 1;
     } else {
         int ks = adj_splits(c);
         KTimer t(c, c->prec == MEM_PREC_FP64_DIRECT ? "adj_direct_f64" : "adj_direct_f32");
         if (c->prec == MEM_PREC_FP64_DIRECT) launch_adj_f64(d, c->y64, c->gsum, ks, c->st);
-        else launch_adj_direct(d, c->y32, c->gsum, ks, c->st);
+        else launch_adj_direct(d, y, c->gsum, ks, c->st);
         c->launches++;
         TRY(after_launch(c, "adjoint kernel"));
-        *ks_out = ks;
+        out.ks = ks;
     }
     return MEM_OK;
 }
@@ -570,8 +579,9 @@ mem_status run_objgrad(mem_ctx* c, const ImgSrc& src, int projected, float* out3
     // gradient assembly and the objective's scalar reduction are one launch
     const bool fused = is_tc(c->prec) && !c->shared;
     TRY(run_forward(c, src, FWD_RESID, true, yout, fused));
-    int ks = 1;
-    TRY(run_adjoint(c, &ks, true, !fused));
+    AdjointOut adj;
+    adj.reduce = !fused;
+    TRY(run_adjoint(c, c->y32, true, adj));
     if (fused) {
         KTimer t(c, "adj_reduce_grad");
         const ScalarArgs sc = scalar_args(c, true);
@@ -583,7 +593,7 @@ mem_status run_objgrad(mem_ctx* c, const ImgSrc& src, int projected, float* out3
                                       c->st);
     } else {
         KTimer t(c, "finalize");
-        launch_finalize(c->dd(), src, is_tc(c->prec), c->gsum, ks, projected, out32, full64, proj64, c->st);
+        launch_finalize(c->dd(), src, is_tc(c->prec), c->gsum, adj.ks, projected, out32, full64, proj64, c->st);
     }
     c->launches++;
     return after_launch(c, "gradient assembly");
@@ -1161,12 +1171,15 @@ mem_status dirty_from(mem_ctx* c, int what, float* out_dev) {
            "weight sums");
     }
     DevData d = c->dd();
-    launch_dirty_y(d, c->wsum, what, c->Z, c->y32, c->prec == MEM_PREC_FP64_DIRECT ? c->y64 : nullptr, c->st);
-    if (c->Z > 0) c->launches++;
+    launch_dirty_y(d, c->wsum, what, c->Z, c->y32, c->prec == MEM_PREC_FP64_DIRECT ? c->y64 : nullptr, c->num_sms,
+                   c->ymax_count, c->prec == MEM_PREC_FP16X3 ? c->ymax : nullptr, c->st);
+    c->launches++;
     TRY(after_launch(c, "dirty image weights"));
-    int ks = 1;
-    TRY(run_adjoint(c, &ks));
-    launch_dirty_out(d, c->gsum, ks, out_dev, c->st);
+    AdjointOut adj;
+    if (is_tc(c->prec)) adj.out32 = out_dev;
+    TRY(run_adjoint(c, c->y32, true, adj));
+    if (is_tc(c->prec)) return MEM_OK;
+    launch_dirty_out(d, c->gsum, adj.ks, out_dev, c->st);
     c->launches++;
     return after_launch(c, "dirty image");
 }
@@ -1480,17 +1493,15 @@ mem_status mem_adjoint(mem_ctx* c, const float* y_dev, float* img_dev) {
     if (!c || !img_dev || (!y_dev && c->Z > 0)) return fail(c, MEM_EINVAL, "null argument");
     if (!aligned(y_dev, 8)) return fail(c, MEM_EINVAL, "y_dev must be 8-byte aligned");
     TRY(ensure_buffers(c));
-    if (c->Z > 0) {
-        if (c->prec == MEM_PREC_FP64_DIRECT) {
-            k_f32_to_f64<<<(unsigned)((2 * c->Z + 255) / 256), 256, 0, c->st>>>(2 * c->Z, y_dev, (double*)c->y64);
-        } else {
-            CK(cudaMemcpyAsync(c->y32, y_dev, (size_t)c->Z * sizeof(float2), cudaMemcpyDeviceToDevice, c->st),
-               "copy y");
-        }
-        c->launches += (c->prec == MEM_PREC_FP64_DIRECT);
+    if (c->Z > 0 && c->prec == MEM_PREC_FP64_DIRECT) {
+        k_f32_to_f64<<<(unsigned)((2 * c->Z + 255) / 256), 256, 0, c->st>>>(2 * c->Z, y_dev, (double*)c->y64);
+        c->launches++;
     }
-    int ks = 1;
-    TRY(run_adjoint(c, &ks));
+    // images of one channel each: sum and assembly in one launch, as in run_objgrad
+    const bool fused = is_tc(c->prec) && !c->shared;
+    AdjointOut adj;
+    adj.reduce = !fused;
+    TRY(run_adjoint(c, (const float2*)y_dev, false, adj));
     // beam factor and channel sum only: lambda = 0 view of the assembly
     DevData d = c->dd();
     d.lambda = 0.0;
@@ -1498,7 +1509,13 @@ mem_status mem_adjoint(mem_ctx* c, const float* y_dev, float* img_dev) {
     // the assembly reads pixel values only for the entropy term and projection;
     // give it the output buffer as a harmless source (lambda = 0, no projection)
     src.f32 = img_dev;
-    launch_finalize(d, src, is_tc(c->prec), c->gsum, ks, 0, img_dev, nullptr, nullptr, c->st);
+    if (fused && c->prec == MEM_PREC_FP16X3)
+        launch_adj_fold_reduce_grad(d, src, c->cb_off, c->partial, c->ymax, 0, img_dev, nullptr, nullptr, ScalarArgs{},
+                                    c->st);
+    else if (fused)
+        launch_adj_tc_reduce_grad(d, src, c->cb_off, c->partial, 0, img_dev, nullptr, nullptr, ScalarArgs{}, c->st);
+    else
+        launch_finalize(d, src, is_tc(c->prec), c->gsum, adj.ks, 0, img_dev, nullptr, nullptr, c->st);
     c->launches++;
     return after_launch(c, "adjoint assembly");
 }

@@ -116,10 +116,11 @@ void launch_prep_fold(const DevData& d, const ImgSrc& src, void* planes, float4*
 // pixels per entropy partial of launch_prep_fold, partials per image
 __host__ __device__ inline int fold_ent_pixels(int N) { return N <= 256 ? 256 : 1024; }
 __host__ __device__ inline int fold_ent_blocks(int N) { return (N * N + fold_ent_pixels(N) - 1) / fold_ent_pixels(N); }
-// max |component| of n floats into ymax[0]; the FP16X3 adjoint scales y by
+// max |component| of Z visibilities into ymax[0]; the FP16X3 adjoint scales y by
 // pow2_scale_for(ymax[0]).  The forward writes the same maximum of the y it
-// produces (RESID mode) when given ymax (zeroed before).
-void launch_absmax(int64_t n, const float* y, float* part, float* ymax, cudaStream_t st);
+// produces (RESID mode) when given ymax (zeroed before), and so does
+// launch_dirty_y.  count: two words, zero between launches.
+void launch_absmax(int64_t Z, const float2* y, int num_sms, unsigned* count, float* ymax, cudaStream_t st);
 __host__ __device__ inline int prep_blocks(int N) { return (int)(((int64_t)N * N + 255) / 256); }
 
 void launch_fwd_direct(const DevData& d, const VisTile* tiles, int n_tiles, const float* B, int mode, float2* yout,
@@ -178,7 +179,7 @@ void launch_grid_fft(const DevData& d, const float* img, int M, float2* R, float
 // 1 PSF, 2 residuals against the model in y32 / y64), and the per-channel
 // image from the adjoint's FP64 sums (no primary-beam factor).
 void launch_dirty_y(const DevData& d, const double* wsum, int what, int64_t z_total, float2* y32, double2* y64,
-                    cudaStream_t st);
+                    int num_sms, unsigned* count, float* ymax, cudaStream_t st);
 void launch_dirty_out(const DevData& d, const double* gsum, int ks, float* out, cudaStream_t st);
 void launch_grid_interp(const DevData& d, int M, const float2* F, int64_t z_total, float2* vis, cudaStream_t st);
 // Adjoint: units sorted by CTA: CTA b runs units [cta_unit_off[b],
@@ -192,13 +193,13 @@ void launch_adj_fold(const DevData& d, const AdjUnit* units, const int* cta_unit
                      const float* ymax, float* partial, uint64_t spin, int* status, cudaStream_t st);
 // into gsum[C][N*N], without the beam factor
 void launch_adj_fold_reduce(const DevData& d, const int* cb_unit_off, const float* partial, const float* ymax,
-                            double* gsum, cudaStream_t st);
+                            double* gsum, float* out32, cudaStream_t st);
 // BF16X3.
 int adj_tc_smem_bytes(int N, int stages);
 void launch_adj_tc(const DevData& d, const AdjUnit* units, const int* cta_unit_off, int n_ctas, const float2* y,
                    float* partial, uint64_t spin, int* status, cudaStream_t st);
 void launch_adj_tc_reduce(const DevData& d, const int* cb_unit_off, const float* partial, double* gsum,
-                          cudaStream_t st);
+                          float* out32, cudaStream_t st);
 // Variant reading u, v (FP64, wavelengths) instead of the prepared phase
 // increments: the caller passes d.u, d.v, d.dx, d.dy; d.pa / d.pb are unused.
 void launch_adj_tc_uv(const DevData& d, const AdjUnit* units, const int* cta_unit_off, int n_ctas,

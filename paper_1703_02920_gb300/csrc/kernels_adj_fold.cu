@@ -408,9 +408,9 @@ struct RedArgs {
     const int* cb_unit_off;
     const float* partial;
     const float* ymax;   // partials are divided by pow2_scale_for(ymax[0])
-    double* gsum;        // RED_GSUM: [C][N*N], without the beam factor
+    double* gsum;        // RED_GSUM: [C][N*N], without the beam factor (or as FP32 in out32)
     int projected;       // RED_GRAD
-    float* out32;        // RED_GRAD (each output nullable)
+    float* out32;        // (each output nullable)
     double *full64, *proj64;
     ScalarArgs sc;       // RED_GRAD: objective scalars, see below
 };
@@ -501,7 +501,9 @@ __global__ void __launch_bounds__(RedGeo<WIDE>::THREADS) k_adj_fold_reduce(DevDa
         const float other = sign ? -tot[1] : tot[1];
         const int64_t pix = (int64_t)c * NN + (int64_t)n * N + m;
         if (OUT == RED_GSUM) {
-            a.gsum[pix] = ((double)tot[0] + (double)other) * inv;
+            const double g = ((double)tot[0] + (double)other) * inv;
+            if (a.out32) a.out32[pix] = (float)g;
+            else a.gsum[pix] = g;
         } else {
             const double x = img_value(src, c, (int64_t)n * N + m, NN);
             const double gr = pixel_gradient(d, d.beam[pix], tot[0], other, inv, x);
@@ -525,8 +527,9 @@ static void launch_red(const DevData& d, const ImgSrc& src, const RedArgs& a, in
 }
 
 void launch_adj_fold_reduce(const DevData& d, const int* cb_unit_off, const float* partial, const float* ymax,
-                          double* gsum, cudaStream_t st) {
+                            double* gsum, float* out32, cudaStream_t st) {
     RedArgs a{};
+    a.out32 = out32;
     a.cb_unit_off = cb_unit_off;
     a.partial = partial;
     a.ymax = ymax;

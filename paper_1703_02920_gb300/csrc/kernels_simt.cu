@@ -3,6 +3,7 @@
 // FP32 (one exponential per visibility-pixel pair, the comparator of the
 // tensor-core form), gradient assembly with the entropy term and positivity
 // projection, ordered FP64 reductions and the CG vector updates.
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 
@@ -140,34 +141,43 @@ void launch_planes(const DevData& d, const ImgSrc& src, void* planes, const floa
     k_planes<<<dim3(prep_blocks(d.N), d.C), 256, 0, st>>>(d, src, (__nv_bfloat16*)planes, cmean);
 }
 
-// max |y| over n floats: 256 block maxima, then one block forms the scale.
-__global__ void __launch_bounds__(256) k_absmax_part(int64_t n, const float* __restrict__ y,
-                                                     float* __restrict__ part) {
-    float mx = 0.f;
-    for (int64_t k = (int64_t)blockIdx.x * 256 + threadIdx.x; k < n; k += (int64_t)gridDim.x * 256)
-        mx = fmaxf(mx, fabsf(y[k]));
+// The maximum of every block's mx (of 256 threads) into ymax[0]: count[0] holds
+// the running maximum (non-negative floats order as their bits), count[1] the
+// blocks that have added theirs; the last one hands over and leaves both zero.
+__device__ __forceinline__ void max_over_blocks(float mx, unsigned* count, float* ymax) {
+    __shared__ float sh[8];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_down_sync(0xffffffffu, mx, o));
-    __shared__ float sh[8];
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = mx;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = sh[0];
-        for (int k = 1; k < 8; ++k) t = fmaxf(t, sh[k]);
-        part[blockIdx.x] = t;
-    }
-}
-
-__global__ void k_absmax_final(const float* __restrict__ part, float* ymax) {
     if (threadIdx.x != 0) return;
-    float t = 0.f;
-    for (int k = 0; k < 256; ++k) t = fmaxf(t, part[k]);
-    ymax[0] = t;
+    for (int k = 0; k < 8; ++k) mx = fmaxf(mx, sh[k]);
+    atomicMax(count, __float_as_uint(mx));
+    __threadfence();
+    if (atomicAdd(count + 1, 1u) != gridDim.x - 1) return;
+    __threadfence();
+    ymax[0] = __uint_as_float(atomicExch(count, 0u));
+    count[1] = 0;
 }
 
-void launch_absmax(int64_t n, const float* y, float* part, float* ymax, cudaStream_t st) {
-    k_absmax_part<<<256, 256, 0, st>>>(n, y, part);
-    k_absmax_final<<<1, 32, 0, st>>>(part, ymax);
+// max |y| over n floats.
+__global__ void __launch_bounds__(256) k_absmax(int64_t n, const float2* __restrict__ y, unsigned* count,
+                                                float* ymax) {
+    float mx = 0.f;
+    for (int64_t k = (int64_t)blockIdx.x * 256 + threadIdx.x; k < n; k += (int64_t)gridDim.x * 256) {
+        const float2 v = y[k];
+        mx = fmaxf(mx, fmaxf(fabsf(v.x), fabsf(v.y)));
+    }
+    max_over_blocks(mx, count, ymax);
+}
+
+// blocks of a pass over Z visibilities: one wave of four per SM at most
+static unsigned vis_blocks(int64_t Z, int num_sms) {
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>((Z + 255) / 256, 4 * num_sms));
+}
+
+void launch_absmax(int64_t Z, const float2* y, int num_sms, unsigned* count, float* ymax, cudaStream_t st) {
+    k_absmax<<<vis_blocks(Z, num_sms), 256, 0, st>>>(Z, y, count, ymax);
 }
 
 // a2, FP32 direct form: B_c = A_c I.
@@ -457,26 +467,33 @@ namespace msk {
 // ---------------------------------------------------------------------------
 // what: 0 measured visibilities, 1 PSF (V = 1), 2 residuals V° - V, with the
 // model V read from y64 (FP64 form) or y32 at the same index it overwrites.
+// ymax (nullable): receives the result's maximum |component|, which the FP16X3
+// adjoint scales by; here it costs no pass of its own (100,003
+// visibilities: three launches of 16 us together, now one of 7).
 __global__ void __launch_bounds__(256) k_dirty_y(DevData d, const double* __restrict__ wsum, int what,
                                                  int64_t z_total, float2* __restrict__ y32,
-                                                 double2* __restrict__ y64) {
-    const int64_t j = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    if (j >= z_total) return;
-    int lo = 0, hi = d.C;
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) / 2;
-        if (d.off[mid] <= j) lo = mid;
-        else hi = mid;
+                                                 double2* __restrict__ y64, unsigned* count, float* ymax) {
+    float mx = 0.f;
+    for (int64_t j = (int64_t)blockIdx.x * 256 + threadIdx.x; j < z_total; j += (int64_t)gridDim.x * 256) {
+        int lo = 0, hi = d.C;
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) / 2;
+            if (d.off[mid] <= j) lo = mid;
+            else hi = mid;
+        }
+        const double om = d.w[j] / wsum[lo];
+        double2 v = what == 1 ? make_double2(1.0, 0.0) : d.vo[j];
+        if (what == 2) {
+            const double2 m = y64 ? y64[j] : make_double2((double)y32[j].x, (double)y32[j].y);
+            v.x -= m.x;
+            v.y -= m.y;
+        }
+        const float2 o = make_float2((float)(om * v.x), (float)(om * v.y));
+        y32[j] = o;
+        if (y64) y64[j] = make_double2(om * v.x, om * v.y);
+        mx = fmaxf(mx, fmaxf(fabsf(o.x), fabsf(o.y)));
     }
-    const double om = d.w[j] / wsum[lo];
-    double2 v = what == 1 ? make_double2(1.0, 0.0) : d.vo[j];
-    if (what == 2) {
-        const double2 m = y64 ? y64[j] : make_double2((double)y32[j].x, (double)y32[j].y);
-        v.x -= m.x;
-        v.y -= m.y;
-    }
-    y32[j] = make_float2((float)(om * v.x), (float)(om * v.y));
-    if (y64) y64[j] = make_double2(om * v.x, om * v.y);
+    if (ymax) max_over_blocks(mx, count, ymax);
 }
 
 __global__ void __launch_bounds__(256) k_dirty_out(DevData d, const double* __restrict__ gsum, int ks,
@@ -491,9 +508,8 @@ __global__ void __launch_bounds__(256) k_dirty_out(DevData d, const double* __re
 }
 
 void launch_dirty_y(const DevData& d, const double* wsum, int what, int64_t z_total, float2* y32, double2* y64,
-                    cudaStream_t st) {
-    if (z_total <= 0) return;
-    k_dirty_y<<<(unsigned)((z_total + 255) / 256), 256, 0, st>>>(d, wsum, what, z_total, y32, y64);
+                    int num_sms, unsigned* count, float* ymax, cudaStream_t st) {
+    k_dirty_y<<<vis_blocks(z_total, num_sms), 256, 0, st>>>(d, wsum, what, z_total, y32, y64, count, ymax);
 }
 
 void launch_dirty_out(const DevData& d, const double* gsum, int ks, float* out, cudaStream_t st) {

@@ -441,7 +441,7 @@ __device__ __forceinline__ float unit_sum_combine(float s, float comp, int el, i
 
 __global__ void __launch_bounds__(256) k_adj_tc_reduce(DevData d, const int* __restrict__ cb_unit_off,
                                                        const float* __restrict__ partial,
-                                                       double* __restrict__ gsum) {
+                                                       double* __restrict__ gsum, float* __restrict__ out32) {
     __shared__ float sh[4][RED_ELEMS][2];
     const int N = d.N;
     const int64_t NN = (int64_t)N * N;
@@ -463,14 +463,15 @@ __global__ void __launch_bounds__(256) k_adj_tc_reduce(DevData d, const int* __r
     int nl, ml;
     adj_partial_rc(loc, BLK, nl, ml);
     const int64_t p = (int64_t)((blk / nbx) * BLK + nl) * N + (blk % nbx) * BLK + ml;
-    gsum[(int64_t)c * NN + p] = (double)tot;
+    if (out32) out32[(int64_t)c * NN + p] = tot;
+    else gsum[(int64_t)c * NN + p] = (double)tot;
 }
 
-void launch_adj_tc_reduce(const DevData& d, const int* cb_unit_off, const float* partial, double* gsum,
+void launch_adj_tc_reduce(const DevData& d, const int* cb_unit_off, const float* partial, double* gsum, float* out32,
                           cudaStream_t st) {
     const int64_t NN = (int64_t)d.N * d.N;
     dim3 grid((unsigned)((NN + RED_ELEMS - 1) / RED_ELEMS), d.C);
-    k_adj_tc_reduce<<<grid, 256, 0, st>>>(d, cb_unit_off, partial, gsum);
+    k_adj_tc_reduce<<<grid, 256, 0, st>>>(d, cb_unit_off, partial, gsum, out32);
 }
 
 // The unit-partial sum of k_adj_tc_reduce followed directly by the gradient
