@@ -172,7 +172,7 @@ int launch_fwd_rs(const DevData& d, const VisTile* tiles, int n_tiles, const voi
 // channel's A_c * I zero-padded to M x M (image centred), as this library's
 // own FFT kernels (rows into R[C][M/2+1][N], columns into F[C][M][M/2+1]),
 // then the modulated bilinear interpolation of the half spectra.
-constexpr int GRID_FFT_MAX = 8192;  // M <= 8192: two M-point buffers per CTA in shared memory
+constexpr int GRID_FFT_MAX = 8192;  // M <= 8192: two M-point buffers and the roots per CTA in shared memory (196 KB)
 bool grid_fft_size_ok(int N, int M);  // N even, M = 2^a q with q in {1, 3, 5, 7}, M <= GRID_FFT_MAX
 void launch_grid_fft(const DevData& d, const float* img, int M, float2* R, float2* F, cudaStream_t st);
 // Dirty image / PSF / residual map: weighted adjoint inputs (what: 0 data,
