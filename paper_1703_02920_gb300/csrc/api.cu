@@ -89,7 +89,6 @@ struct mem_ctx {
     // pinned host words for the scalar and status readback (one copy pair and
     // one stream synchronisation per call; nullptr: pageable fallback)
     double* hscal = nullptr;
-    size_t hscal_n = 0;
 
     // CUDA graphs: a launch sequence that repeats with the same buffers is
     // captured once (on a private stream: the legacy default stream cannot be
@@ -571,20 +570,26 @@ mem_status run_adjoint(mem_ctx* c, const float2* y, bool ymax_ready, AdjointOut&
 }
 
 // Objective + gradient at `src`; gradient outputs optional.
+// images of one channel each: the objective's scalars are formed in the gradient's
+// launch, and host (nullable) receives them there
+bool fused_objgrad(const mem_ctx* c) { return is_tc(c->prec) && !c->shared; }
+
 mem_status run_objgrad(mem_ctx* c, const ImgSrc& src, int projected, float* out32, double* full64,
-                       double* proj64) {
+                       double* proj64, double* host = nullptr) {
     TRY(ensure_buffers(c));
     void* yout = c->prec == MEM_PREC_FP64_DIRECT ? (void*)c->y64 : (void*)c->y32;
     // images of one channel each: the adjoint's unit-partial sum, the
     // gradient assembly and the objective's scalar reduction are one launch
-    const bool fused = is_tc(c->prec) && !c->shared;
+    const bool fused = fused_objgrad(c);
     TRY(run_forward(c, src, FWD_RESID, true, yout, fused));
     AdjointOut adj;
     adj.reduce = !fused;
     TRY(run_adjoint(c, c->y32, true, adj));
     if (fused) {
         KTimer t(c, "adj_reduce_grad");
-        const ScalarArgs sc = scalar_args(c, true);
+        ScalarArgs sc = scalar_args(c, true);
+        sc.host = host;
+        sc.status = c->dstatus;
         if (c->prec == MEM_PREC_FP16X3)
             launch_adj_fold_reduce_grad(c->dd(), src, c->cb_off, c->partial, c->ymax, projected, out32, full64, proj64,
                                         sc, c->st);
@@ -665,23 +670,27 @@ mem_status graphed(mem_ctx* c, mem_ctx::GraphSlot& g, const void* k1, const void
     return MEM_OK;
 }
 
-mem_status read_scalars(mem_ctx* c, std::vector<double>& out) {
+// Pinned host words for the status word's slot and the scalars (nullptr: none to be had).
+double* host_words(mem_ctx* c) {
+    const size_t n = 4 + 3 * (size_t)c->n_images;
+    if (!c->hscal && cudaMallocHost((void**)&c->hscal, n * sizeof(double)) != cudaSuccess) {
+        c->hscal = nullptr;
+        cudaGetLastError();
+    }
+    return c->hscal;
+}
+
+// on_host: the evaluation's last kernel writes host_words itself.
+mem_status read_scalars(mem_ctx* c, std::vector<double>& out, bool on_host) {
     out.resize(3 + 3 * (size_t)c->n_images);
     const size_t n = out.size();
-    if (c->hscal_n < n + 1) {  // the status word's slot, then the scalars
-        if (c->hscal) cudaFreeHost(c->hscal);
-        c->hscal = nullptr;
-        c->hscal_n = 0;
-        if (cudaMallocHost((void**)&c->hscal, (n + 1) * sizeof(double)) == cudaSuccess) c->hscal_n = n + 1;
-        else cudaGetLastError();  // pageable fallback below
-    }
-    if (c->hscal) {
-        // both in one copy to pinned memory
-        CK(cudaMemcpyAsync(c->hscal, c->dstatus, (n + 1) * sizeof(double), cudaMemcpyDeviceToHost, c->st),
-           "scalar readback");
+    if (double* h = host_words(c)) {
+        if (!on_host)
+            CK(cudaMemcpyAsync(h, c->dstatus, (n + 1) * sizeof(double), cudaMemcpyDeviceToHost, c->st),
+               "scalar readback");
         CK(cudaStreamSynchronize(c->st), "stream synchronize");
-        if (*(const int*)c->hscal & DEV_TIMEOUT) TRY(check_status(c));
-        std::copy(c->hscal + 1, c->hscal + 1 + n, out.begin());
+        if (*(const int*)h & DEV_TIMEOUT) TRY(check_status(c));
+        std::copy(h + 1, h + 1 + n, out.begin());
     } else {
         CK(cudaMemcpyAsync(out.data(), c->scal, n * sizeof(double), cudaMemcpyDeviceToHost, c->st),
            "scalar readback");
@@ -1525,11 +1534,12 @@ mem_status mem_objective_grad(mem_ctx* c, const float* image_dev, float* grad_de
     if (!c || !image_dev) return fail(c, MEM_EINVAL, "null argument");
     ImgSrc src{image_dev, nullptr, nullptr, nullptr, c->G, 0};
     TRY(ensure_buffers(c));
+    double* host = fused_objgrad(c) ? host_words(c) : nullptr;
     TRY(graphed(c, c->g_objgrad, image_dev, grad_dev, projected ? 1 : 0,
-                [&]() { return run_objgrad(c, src, projected, grad_dev, nullptr, nullptr); }));
+                [&]() { return run_objgrad(c, src, projected, grad_dev, nullptr, nullptr, host); }));
     if (out3_host) {
         std::vector<double> sc;
-        TRY(read_scalars(c, sc));
+        TRY(read_scalars(c, sc, host != nullptr));
         out3_host[0] = sc[0];
         out3_host[1] = sc[1];
         out3_host[2] = sc[2];
@@ -1549,7 +1559,7 @@ mem_status mem_objective_grad_host(mem_ctx* c, const float* image_host, float* g
     if (grad_host)
         CK(cudaMemcpyAsync(grad_host, dgrad, n * sizeof(float), cudaMemcpyDeviceToHost, c->st), "gradient download");
     std::vector<double> sc;
-    TRY(read_scalars(c, sc));
+    TRY(read_scalars(c, sc, fused_objgrad(c) && host_words(c)));
     if (out3_host) {
         out3_host[0] = sc[0];
         out3_host[1] = sc[1];

@@ -114,6 +114,14 @@ __device__ __host__ inline unsigned* scalars_counter(double* img_tmp, int n_imag
     return (unsigned*)(img_tmp + 2 * SCAL_SPLIT * n_images);
 }
 
+// The finished scalars (and the status word) to the host.  Whole block.
+__device__ __forceinline__ void scalars_to_host(const ScalarArgs& sc, int n_images) {
+    if (!sc.host) return;
+    __syncthreads();
+    for (int k = threadIdx.x; k < 3 + 3 * n_images; k += blockDim.x) sc.host[1 + k] = __ldcg(sc.scal + k);
+    if (threadIdx.x == 0) *(int*)sc.host = *sc.status;
+}
+
 // Every thread of the block (THREADS) calls this (block-wide barriers inside).
 // Returns true in every thread of the one block that has all scalars in scal
 // (__ldcg reads them).
@@ -167,7 +175,10 @@ __device__ __forceinline__ bool scalars_block(const DevData& d, const ScalarArgs
         }
     }
     __syncthreads();
-    if (alone) return true;
+    if (alone) {
+        scalars_to_host(sc, d.n_images);
+        return true;
+    }
     if (!last) return false;
     __threadfence();
     // Stage 2 (last block): one warp per image adds its partials (read through
@@ -198,6 +209,7 @@ __device__ __forceinline__ bool scalars_block(const DevData& d, const ScalarArgs
         sc.scal[2] = tc;
         *scalars_counter(sc.img_tmp, d.n_images) = 0;  // ready for the next evaluation
     }
+    scalars_to_host(sc, d.n_images);
     return true;
 }
 
