@@ -105,6 +105,7 @@ struct mem_ctx {
         cudaGraphExec_t exec = nullptr;
     };
     bool graphs = true;
+    bool capturing = false;  // launches go into a graph: see launch_chained
     cudaStream_t cap_st = nullptr;
     GraphSlot g_objgrad;
     // the whole solve (evaluations, CG and line-search control) as one graph
@@ -175,6 +176,7 @@ struct mem_ctx {
         d.fwd_bn = fwd_kernel == MEM_FWD_RESIDENT ? N : fwd_bn;
         d.fwd_stages = fwd_stages;
         d.adj_stages = adj_stages;
+        d.chain = !capturing;
         return d;
     }
 };
@@ -645,7 +647,9 @@ mem_status graphed(mem_ctx* c, mem_ctx::GraphSlot& g, const void* k1, const void
             c->st = user;
             return cuda_fail(c, e, "begin capture");
         }
+        c->capturing = true;
         mem_status s = body();
+        c->capturing = false;
         cudaGraph_t graph = nullptr;
         e = cudaStreamEndCapture(c->cap_st, &graph);
         c->st = user;
@@ -907,7 +911,9 @@ mem_status capture_into(mem_ctx* c, cudaGraph_t g, const std::function<mem_statu
         c->st = user;
         return cuda_fail(c, e, "begin capture");
     }
+    c->capturing = true;
     mem_status s = body();
+    c->capturing = false;
     cudaGraph_t out = nullptr;
     e = cudaStreamEndCapture(c->cap_st, &out);
     c->st = user;

@@ -81,6 +81,12 @@ __device__ __forceinline__ cf2 cmul(cf2 a, cf2 b) {
     return {fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x)};
 }
 
+// A chained launch (launch_chained): the next grid may start from here on; it
+// waits, where it calls chain_wait, until every grid before it has completed and
+// its writes are visible.  Without the launch attribute both do nothing.
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---------------------------------------------------------------------------
 // Shared-memory addresses, mbarriers
 // ---------------------------------------------------------------------------

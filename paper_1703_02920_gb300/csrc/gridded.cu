@@ -129,6 +129,8 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_rows(DevData d, const float
     extern __shared__ float2 sh[];
     float2 *a = sh, *b = sh + M, *w = sh + 2 * M;
     root_table(w, M);
+    chain_next();
+    chain_wait();
     const int N = d.N, o = (M - N) / 2, H = M / 2 + 1;
     const int c = blockIdx.y, n0 = 2 * blockIdx.x;
     const int i = d.shared ? 0 : c;
@@ -165,6 +167,8 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_cols(int N, int M, const fl
     extern __shared__ float2 sh[];
     float2 *a = sh, *b = sh + M, *w = sh + 2 * M;
     root_table(w, M);
+    chain_next();
+    chain_wait();
     const int o = (M - N) / 2, H = M / 2 + 1;
     const int k = blockIdx.x, c = blockIdx.y;
     const float2* Rk = R + ((int64_t)c * H + k) * N;
@@ -198,6 +202,8 @@ __device__ __forceinline__ float2 grid_value(const float2* __restrict__ F, int M
 // FP64 units; 10 us now, bound by the gathers.)
 __global__ void __launch_bounds__(256) k_grid_interp(DevData d, int M, const float2* __restrict__ F,
                                                      int64_t z_total, float2* __restrict__ vis) {
+    chain_next();
+    chain_wait();
     const int64_t j = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (j >= z_total) return;
     const uint64_t pa = d.pa[j], pb = d.pb[j];
@@ -235,13 +241,13 @@ void launch_grid_fft(const DevData& d, const float* img, int M, float2* R, float
     const int smem = 3 * M * (int)sizeof(float2);
     cudaFuncSetAttribute(k_fft_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     cudaFuncSetAttribute(k_fft_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    k_fft_rows<<<dim3(d.N / 2, d.C), FFT_THREADS, smem, st>>>(d, img, M, R);
-    k_fft_cols<<<dim3(H, d.C), FFT_THREADS, smem, st>>>(d.N, M, R, F);
+    launch_chained(k_fft_rows, dim3(d.N / 2, d.C), FFT_THREADS, smem, st, d.chain, 1, d, img, M, R);
+    launch_chained(k_fft_cols, dim3(H, d.C), FFT_THREADS, smem, st, d.chain, 1, d.N, M, (const float2*)R, F);
 }
 
 void launch_grid_interp(const DevData& d, int M, const float2* F, int64_t z_total, float2* vis, cudaStream_t st) {
     if (z_total <= 0) return;
-    k_grid_interp<<<(unsigned)((z_total + 255) / 256), 256, 0, st>>>(d, M, F, z_total, vis);
+    launch_chained(k_grid_interp, dim3((unsigned)((z_total + 255) / 256)), 256, 0, st, d.chain, 1, d, M, F, z_total, vis);
 }
 
 }  // namespace msk

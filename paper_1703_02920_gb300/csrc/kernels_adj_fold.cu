@@ -183,6 +183,8 @@ __global__ void __launch_bounds__(ADJ_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = S.tmem_base;
+    chain_next();
+    chain_wait();
 
     if (warp == ADJ_PRODUCER_WARPS) {
         // The whole warp runs the issue loop, converged (every wait's outcome is
@@ -365,8 +367,8 @@ template <int SHAPE, int VB, int STAGES>
 static void launch_adj_variant(const AdjArgs& a) {
     const int smem = STAGES * AdjGeo<SHAPE>::stage_bytes(VB) + 1024;
     cudaFuncSetAttribute(k_adj_fold<SHAPE, VB, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    k_adj_fold<SHAPE, VB, STAGES><<<a.n_ctas, ADJ_THREADS, smem, a.st>>>(
-        a.d, a.units, a.cta_unit_off, a.y, a.ymax, a.partial, a.spin, a.status);
+    launch_chained(k_adj_fold<SHAPE, VB, STAGES>, dim3(a.n_ctas), ADJ_THREADS, smem, a.st, a.d.chain, 1, a.d, a.units,
+                   a.cta_unit_off, a.y, a.ymax, a.partial, a.spin, a.status);
 }
 
 void launch_adj_fold(const DevData& d, const AdjUnit* units, const int* cta_unit_off, int n_ctas, const float2* y,
@@ -434,6 +436,8 @@ __global__ void __launch_bounds__(RedGeo<WIDE>::THREADS) k_adj_fold_reduce(DevDa
     __shared__ float sh[2][SPLIT][ELEMS][2];
     const int N = d.N;
     const int64_t NN = (int64_t)N * N;
+    chain_next();
+    chain_wait();
     const int n_scal = OUT == RED_GRAD && a.sc.scal ? a.sc.splits : 0;
     if (OUT == RED_GRAD && (int)blockIdx.x < n_scal) {
         scalars_block<THREADS>(d, a.sc, blockIdx.y, blockIdx.x);
@@ -519,11 +523,11 @@ template <int OUT>
 static void launch_red(const DevData& d, const ImgSrc& src, const RedArgs& a, int extra, cudaStream_t st) {
     const int64_t half = (int64_t)d.N * d.N / 2;
     if (d.N >= 256)
-        k_adj_fold_reduce<OUT, true><<<dim3((unsigned)(half / RedGeo<true>::ELEMS) + extra, d.C), RedGeo<true>::THREADS, 0,
-                                  st>>>(d, src, a);
+        launch_chained(k_adj_fold_reduce<OUT, true>, dim3((unsigned)(half / RedGeo<true>::ELEMS) + extra, d.C),
+                       RedGeo<true>::THREADS, 0, st, d.chain, 1, d, src, a);
     else
-        k_adj_fold_reduce<OUT, false><<<dim3((unsigned)(half / RedGeo<false>::ELEMS) + extra, d.C),
-                                   RedGeo<false>::THREADS, 0, st>>>(d, src, a);
+        launch_chained(k_adj_fold_reduce<OUT, false>, dim3((unsigned)(half / RedGeo<false>::ELEMS) + extra, d.C),
+                       RedGeo<false>::THREADS, 0, st, d.chain, 1, d, src, a);
 }
 
 void launch_adj_fold_reduce(const DevData& d, const int* cb_unit_off, const float* partial, const float* ymax,

@@ -269,6 +269,8 @@ __global__ void __launch_bounds__(FW_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = S.tmem_base;
+    chain_next();
+    chain_wait();
 
     if (warp >= 8 && warp < 12) regs_dec<FW_REGS_MISC>();
     if (warp == 8) {
@@ -717,6 +719,8 @@ __global__ void __launch_bounds__(FW_THREADS, 1)
 __global__ void __launch_bounds__(128) k_fold_combine(DevData d, const VisTile* __restrict__ tiles,
                                                      const float4* __restrict__ vpart, int64_t z_total, int mode,
                                                      float2* yout, double* chi_part, unsigned* ymax_bits) {
+    chain_next();
+    chain_wait();
     const VisTile tl = tiles[blockIdx.x];
     float chi = 0.f, ym = 0.f;
     if ((int)threadIdx.x < tl.count) {
@@ -759,9 +763,8 @@ void launch_variant(const FwdArgs& a, int grid) {
         return;
     }
     cudaFuncSetAttribute(k_fwd_fold<STAGES, RES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    k_fwd_fold<STAGES, RES><<<grid, FW_THREADS, smem, a.st>>>(a.d, a.tiles, a.n_tiles, a.planes, a.cmean,
-                                                                 a.mode, a.yout, a.chi_part, a.ymax_bits,
-                                                                 a.vpart, a.z_total, a.spin, a.status);
+    launch_chained(k_fwd_fold<STAGES, RES>, dim3(grid), FW_THREADS, smem, a.st, a.d.chain, 1, a.d, a.tiles, a.n_tiles,
+                   a.planes, a.cmean, a.mode, a.yout, a.chi_part, a.ymax_bits, a.vpart, a.z_total, a.spin, a.status);
 }
 
 void launch_stages(const FwdArgs& a, int res, int grid) {
@@ -801,7 +804,8 @@ int launch_fwd_fold(const DevData& d, int resident, const VisTile* tiles, int n_
     const int grid = res == RES_PART ? 2 * std::max(1, std::min(num_sms / 2, n_tiles)) : std::min(num_sms, n_tiles);
     launch_stages(a, res, grid);
     if (res != RES_PART) return 1;
-    k_fold_combine<<<n_tiles, 128, 0, st>>>(d, tiles, vpart, z_total, mode, yout, chi_part, (unsigned*)ymax);
+    launch_chained(k_fold_combine, dim3(n_tiles), 128, 0, st, d.chain, 1, d, tiles, (const float4*)vpart, z_total, mode, yout,
+                   chi_part, (unsigned*)ymax);
     return 2;
 }
 

@@ -77,6 +77,8 @@ __global__ void __launch_bounds__(FP_THREADS) k_prep_fold(DevData d, ImgSrc src,
     __shared__ double shd[FP_THREADS / 32];
     const int N = d.N, M = N / 2;
     const int64_t NN = (int64_t)N * N;
+    chain_next();
+    chain_wait();
     if ((int)blockIdx.x >= n_strip_ctas) {
         // ------------------------------------------------------ entropy
         const int n_ent = fold_ent_blocks(N), b = (int)blockIdx.x - n_strip_ctas;
@@ -209,19 +211,10 @@ void launch_prep_fold(const DevData& d, const ImgSrc& src, void* planes, float4*
                       double* ent_part, cudaStream_t st) {
     const int cluster = strip_cluster(d.N), strips = d.N / 32 * d.C * cluster;
     const int ent = ent_part ? fold_ent_blocks(d.N) * d.n_images : 0;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(strips + (ent + cluster - 1) / cluster * cluster));
-    cfg.blockDim = dim3(FP_THREADS);
-    cfg.stream = st;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = cluster;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
     const bool keep = d.N / 2 / cluster <= 16 * FP_KEEP;
-    cudaLaunchKernelEx(&cfg, keep ? k_prep_fold<true> : k_prep_fold<false>, d, src, strips, cluster,
-                       (uint16_t*)planes, cmean, ymax_clear, ent_part);
+    launch_chained(keep ? k_prep_fold<true> : k_prep_fold<false>,
+                   dim3((unsigned)(strips + (ent + cluster - 1) / cluster * cluster)), FP_THREADS, 0, st, d.chain,
+                   cluster, d, src, strips, cluster, (uint16_t*)planes, cmean, ymax_clear, ent_part);
 }
 
 }  // namespace msk

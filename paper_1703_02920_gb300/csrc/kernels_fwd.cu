@@ -114,6 +114,8 @@ __global__ void __launch_bounds__(F2_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = S.tmem_base;
+    chain_next();
+    chain_wait();
 
     if (warp == 4) {
         // ---------------------------------------------------------------- MMA
@@ -453,8 +455,8 @@ static void launch_fwd_variant(const DevData& d, const VisTile* tiles, int n_til
                                uint64_t spin, int* status, cudaStream_t st) {
     const int smem = fwd_tc_smem_bytes(d.N, d.fwd_bn, STAGES);
     cudaFuncSetAttribute(k_fwd_tc<STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    k_fwd_tc<STAGES><<<grid, F2_THREADS, smem, st>>>(d, tiles, n_tiles, (const uint16_t*)planes, cmean, mode, yout,
-                                                     chi_part, spin, status);
+    launch_chained(k_fwd_tc<STAGES>, dim3(grid), F2_THREADS, smem, st, d.chain, 1, d, tiles, n_tiles,
+                   (const uint16_t*)planes, cmean, mode, yout, chi_part, spin, status);
 }
 
 void launch_fwd_tc(const DevData& d, const VisTile* tiles, int n_tiles, const void* planes, const float* cmean,

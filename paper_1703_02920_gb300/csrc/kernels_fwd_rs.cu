@@ -169,6 +169,8 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = S.tmem_base;
+    chain_next();
+    chain_wait();
 
     if (warp >= 8 && warp < 12) regs_dec<RS_REGS_MISC>();
     if (warp == 8) {
@@ -444,6 +446,8 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
 __global__ void __launch_bounds__(64) k_fwd_combine(DevData d, const VisTile* __restrict__ tiles,
                                                     const double2* __restrict__ vpart, int n_slices,
                                                     int64_t z_total, int mode, float2* yout, double* chi_part) {
+    chain_next();
+    chain_wait();
     const int t = blockIdx.x;
     const VisTile tl = tiles[t];
     const int jv = threadIdx.x;
@@ -473,8 +477,8 @@ void launch_rs_variant(const DevData& d, const VisTile* tiles, int n_tiles, cons
     }();
     if (!regs_ok) grid = 0;  // a launch with no blocks leaves an error for the caller's check
     cudaFuncSetAttribute(k_fwd_rs<STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    k_fwd_rs<STAGES><<<grid, RS_THREADS, smem, st>>>(d, tiles, n_tiles, (const uint16_t*)planes, cmean, vpart,
-                                                     z_total, mode, yout, chi_part, spin, status);
+    launch_chained(k_fwd_rs<STAGES>, dim3(grid), RS_THREADS, smem, st, d.chain, 1, d, tiles, n_tiles,
+                   (const uint16_t*)planes, cmean, vpart, z_total, mode, yout, chi_part, spin, status);
 }
 
 }  // namespace
@@ -495,7 +499,8 @@ int launch_fwd_rs(const DevData& d, const VisTile* tiles, int n_tiles, const voi
     auto launch = stages <= 4 ? launch_rs_variant<4> : stages == 5 ? launch_rs_variant<5> : launch_rs_variant<6>;
     launch(d, tiles, n_tiles, planes, cmean, vpart, z_total, mode, yout, chi_part, grid, spin, status, st);
     if (n_slices == 1) return 1;
-    k_fwd_combine<<<n_tiles, 64, 0, st>>>(d, tiles, vpart, n_slices, z_total, mode, yout, chi_part);
+    launch_chained(k_fwd_combine, dim3(n_tiles), 64, 0, st, d.chain, 1, d, tiles, (const double2*)vpart, n_slices, z_total,
+                   mode, yout, chi_part);
     return 2;
 }
 

@@ -50,6 +50,8 @@ __global__ void __launch_bounds__(256) k_colsum(DevData d, ImgSrc src, double* _
                                                 double* __restrict__ ent_part) {
     __shared__ double sh[8][33];
     __shared__ bool last;
+    chain_next();
+    chain_wait();
     const int N = d.N;
     const int64_t NN = (int64_t)N * N;
     const int c = blockIdx.z, rb = blockIdx.y;
@@ -101,7 +103,8 @@ __global__ void __launch_bounds__(256) k_colsum(DevData d, ImgSrc src, double* _
 
 void launch_colmean(const DevData& d, const ImgSrc& src, float* cmean, double* psum, unsigned* count,
                     double* ent_part, cudaStream_t st) {
-    k_colsum<<<dim3((d.N + 31) / 32, COL_RB, d.C), 256, 0, st>>>(d, src, psum, count, cmean, ent_part);
+    launch_chained(k_colsum, dim3((d.N + 31) / 32, COL_RB, d.C), 256, 0, st, d.chain, 1, d, src, psum, count, cmean,
+                   ent_part);
 }
 
 int colmean_tmp_count(int N, int C) { return COL_RB * N * C; }
@@ -120,6 +123,8 @@ __device__ __forceinline__ int64_t tc_plane_index(int n, int m, int N, int BN) {
 
 __global__ void __launch_bounds__(256) k_planes(DevData d, ImgSrc src, __nv_bfloat16* __restrict__ planes,
                                                 const float* __restrict__ cmean) {
+    chain_next();
+    chain_wait();
     const int N = d.N, BN = d.fwd_bn;
     const int64_t NN = (int64_t)N * N;
     const int c = blockIdx.y;
@@ -138,7 +143,7 @@ __global__ void __launch_bounds__(256) k_planes(DevData d, ImgSrc src, __nv_bflo
 }
 
 void launch_planes(const DevData& d, const ImgSrc& src, void* planes, const float* cmean, cudaStream_t st) {
-    k_planes<<<dim3(prep_blocks(d.N), d.C), 256, 0, st>>>(d, src, (__nv_bfloat16*)planes, cmean);
+    launch_chained(k_planes, dim3(prep_blocks(d.N), d.C), 256, 0, st, d.chain, 1, d, src, (__nv_bfloat16*)planes, cmean);
 }
 
 // The maximum of every block's mx (of 256 threads) into ymax[0]: count[0] holds
@@ -163,6 +168,8 @@ __device__ __forceinline__ void max_over_blocks(float mx, unsigned* count, float
 // max |y| over n floats.
 __global__ void __launch_bounds__(256) k_absmax(int64_t n, const float2* __restrict__ y, unsigned* count,
                                                 float* ymax) {
+    chain_next();
+    chain_wait();
     float mx = 0.f;
     for (int64_t k = (int64_t)blockIdx.x * 256 + threadIdx.x; k < n; k += (int64_t)gridDim.x * 256) {
         const float2 v = y[k];
@@ -177,7 +184,7 @@ static unsigned vis_blocks(int64_t Z, int num_sms) {
 }
 
 void launch_absmax(int64_t Z, const float2* y, int num_sms, unsigned* count, float* ymax, cudaStream_t st) {
-    k_absmax<<<vis_blocks(Z, num_sms), 256, 0, st>>>(Z, y, count, ymax);
+    launch_chained(k_absmax, dim3(vis_blocks(Z, num_sms)), 256, 0, st, 1, 1, Z, y, count, ymax);
 }
 
 // a2, FP32 direct form: B_c = A_c I.
@@ -376,6 +383,8 @@ __global__ void __launch_bounds__(256) k_finalize(DevData d, ImgSrc src,
                                                   const double* __restrict__ gsum, int ks,
                                                   int projected, float* out32, double* full64,
                                                   double* proj64) {
+    chain_next();
+    chain_wait();
     const int N = d.N;
     const int64_t NN = (int64_t)N * N;
     const int i = blockIdx.y;
@@ -399,8 +408,8 @@ __global__ void __launch_bounds__(256) k_finalize(DevData d, ImgSrc src,
 void launch_finalize(const DevData& d, const ImgSrc& src, int fast_log, const double* gsum, int ks, int projected,
                      float* out32, double* full64, double* proj64, cudaStream_t st) {
     dim3 grid(prep_blocks(d.N), d.n_images);
-    if (fast_log) k_finalize<true><<<grid, 256, 0, st>>>(d, src, gsum, ks, projected, out32, full64, proj64);
-    else k_finalize<false><<<grid, 256, 0, st>>>(d, src, gsum, ks, projected, out32, full64, proj64);
+    launch_chained(fast_log ? k_finalize<true> : k_finalize<false>, grid, 256, 0, st, d.chain, 1, d, src, gsum, ks,
+                   projected, out32, full64, proj64);
 }
 
 // ---------------------------------------------------------------------------
@@ -408,11 +417,13 @@ void launch_finalize(const DevData& d, const ImgSrc& src, int fast_log, const do
 // scal layout: [0..2] = Phi, chi^2, S totals; [3 + 3i ...] per image.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_scalars(DevData d, ScalarArgs sc) {
+    chain_next();
+    chain_wait();
     scalars_block<256>(d, sc, blockIdx.x, blockIdx.y);
 }
 
 void launch_scalars(const DevData& d, const ScalarArgs& sc, cudaStream_t st) {
-    k_scalars<<<dim3(d.n_images, sc.splits), 256, 0, st>>>(d, sc);
+    launch_chained(k_scalars, dim3(d.n_images, sc.splits), 256, 0, st, d.chain, 1, d, sc);
 }
 
 int scalars_tmp_doubles(int n_images) { return 2 * SCAL_SPLIT * n_images + 1; }
@@ -473,6 +484,8 @@ namespace msk {
 __global__ void __launch_bounds__(256) k_dirty_y(DevData d, const double* __restrict__ wsum, int what,
                                                  int64_t z_total, float2* __restrict__ y32,
                                                  double2* __restrict__ y64, unsigned* count, float* ymax) {
+    chain_next();
+    chain_wait();
     float mx = 0.f;
     for (int64_t j = (int64_t)blockIdx.x * 256 + threadIdx.x; j < z_total; j += (int64_t)gridDim.x * 256) {
         int lo = 0, hi = d.C;
@@ -509,7 +522,8 @@ __global__ void __launch_bounds__(256) k_dirty_out(DevData d, const double* __re
 
 void launch_dirty_y(const DevData& d, const double* wsum, int what, int64_t z_total, float2* y32, double2* y64,
                     int num_sms, unsigned* count, float* ymax, cudaStream_t st) {
-    k_dirty_y<<<vis_blocks(z_total, num_sms), 256, 0, st>>>(d, wsum, what, z_total, y32, y64, count, ymax);
+    launch_chained(k_dirty_y, dim3(vis_blocks(z_total, num_sms)), 256, 0, st, d.chain, 1, d, wsum, what, z_total, y32, y64,
+                   count, ymax);
 }
 
 void launch_dirty_out(const DevData& d, const double* gsum, int ks, float* out, cudaStream_t st) {

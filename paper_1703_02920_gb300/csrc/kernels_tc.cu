@@ -178,6 +178,8 @@ __global__ void __launch_bounds__(ADJ_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = S.tmem_base;
+    chain_next();
+    chain_wait();
 
     if (warp == 4) {
         // The whole warp runs the issue loop, converged (every wait's outcome is
@@ -356,7 +358,8 @@ static void launch_adj_variant(const DevData& d, const AdjUnit* units, const int
                                const float2* y, float* partial, uint64_t spin, int* status, cudaStream_t st) {
     const int smem = adj_tc_smem_bytes(d.N, STAGES);
     cudaFuncSetAttribute(k_adj_tc<FROM_UV, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    k_adj_tc<FROM_UV, STAGES><<<n_ctas, ADJ_THREADS, smem, st>>>(d, units, cta_unit_off, y, partial, spin, status);
+    launch_chained(k_adj_tc<FROM_UV, STAGES>, dim3(n_ctas), ADJ_THREADS, smem, st, d.chain, 1, d, units, cta_unit_off, y,
+                   partial, spin, status);
 }
 
 void launch_adj_tc(const DevData& d, const AdjUnit* units, const int* cta_unit_off, int n_ctas, const float2* y,
@@ -443,6 +446,8 @@ __global__ void __launch_bounds__(256) k_adj_tc_reduce(DevData d, const int* __r
                                                        const float* __restrict__ partial,
                                                        double* __restrict__ gsum, float* __restrict__ out32) {
     __shared__ float sh[4][RED_ELEMS][2];
+    chain_next();
+    chain_wait();
     const int N = d.N;
     const int64_t NN = (int64_t)N * N;
     const int BLK = N < 256 ? N : 256;
@@ -471,7 +476,7 @@ void launch_adj_tc_reduce(const DevData& d, const int* cb_unit_off, const float*
                           cudaStream_t st) {
     const int64_t NN = (int64_t)d.N * d.N;
     dim3 grid((unsigned)((NN + RED_ELEMS - 1) / RED_ELEMS), d.C);
-    k_adj_tc_reduce<<<grid, 256, 0, st>>>(d, cb_unit_off, partial, gsum, out32);
+    launch_chained(k_adj_tc_reduce, grid, 256, 0, st, d.chain, 1, d, cb_unit_off, partial, gsum, out32);
 }
 
 // The unit-partial sum of k_adj_tc_reduce followed directly by the gradient
@@ -497,6 +502,8 @@ __global__ void __launch_bounds__(256) k_adj_tc_reduce_grad(DevData d, ImgSrc sr
                                                             ScalarArgs sc) {
     constexpr int ELEMS = 256 / SPLIT;
     __shared__ float sh[4][RED_ELEMS][2];
+    chain_next();
+    chain_wait();
     const int N = d.N;
     const int64_t NN = (int64_t)N * N;
     const int n_scal = sc.scal ? sc.splits : 0;
@@ -541,7 +548,7 @@ void launch_adj_tc_reduce_grad(const DevData& d, const ImgSrc& src, const int* c
     const int elems = one ? 256 : RED_ELEMS;
     const dim3 grid((unsigned)((NN + elems - 1) / elems) + (sc.scal ? sc.splits : 0), d.C);
     auto kernel = one ? k_adj_tc_reduce_grad<1> : k_adj_tc_reduce_grad<4>;
-    kernel<<<grid, 256, 0, st>>>(d, src, cb_unit_off, partial, projected, out32, full64, proj64, sc);
+    launch_chained(kernel, grid, 256, 0, st, d.chain, 1, d, src, cb_unit_off, partial, projected, out32, full64, proj64, sc);
 }
 
 }  // namespace msk

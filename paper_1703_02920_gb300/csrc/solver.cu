@@ -465,6 +465,8 @@ __global__ void __launch_bounds__(CTL_THREADS) k_scalars_ls(DevData d, ScalarArg
     // The state machine runs on a copy whose loads are all in flight during the
     // reduction: in place, every branch would wait for its own.
     const int NI = d.n_images;
+    chain_next();
+    chain_wait();
     CgImage mine;
     if ((int)threadIdx.x < NI) mine = st[threadIdx.x];
     if (!scalars_block<CTL_THREADS>(d, sc, blockIdx.x, blockIdx.y)) return;
@@ -569,8 +571,8 @@ void launch_scalars_ls(const DevData& d, const ScalarArgs& sc, bool start, CgIma
                        const double* dots, double* alpha, const int* dstatus, unsigned long long h_inner,
                        cudaStream_t s) {
     const dim3 grid(d.n_images, sc.splits);
-    if (start) k_scalars_ls<true><<<grid, CTL_THREADS, 0, s>>>(d, sc, st, ctl, dots, alpha, dstatus, h_inner);
-    else k_scalars_ls<false><<<grid, CTL_THREADS, 0, s>>>(d, sc, st, ctl, dots, alpha, dstatus, h_inner);
+    launch_chained(start ? k_scalars_ls<true> : k_scalars_ls<false>, grid, CTL_THREADS, 0, s, d.chain, 1, d, sc, st, ctl,
+                   dots, alpha, dstatus, h_inner);
 }
 void launch_cg_record(int NI, CgImage* st, CgControl* ctl, const double* scal, double* hist, const int* dstatus,
                       unsigned long long h_outer, cudaStream_t s) {
