@@ -276,10 +276,18 @@ def run_reference(args, rank, world):
     return 0
 
 
-def roofline(kprof: dict, units: int, config: int) -> dict:
+def executed_per_algorithmic(precision: str) -> float:
+    """Tensor-core flops executed per algorithmic flop: three products per
+    product in the split forms, half of them on FP16x3's folded image (mirror
+    pixels share theirs)."""
+    return 1.5 if precision == "fp16x3" else 3.0
+
+
+def roofline(kprof: dict, units: int, config: int, executed: float = 3.0) -> dict:
     """Roofline object of the dominant kernel from per-launch CUDA-event times.
     Each launch is timed alone (events around it), so the split forms are held
-    against the burst bf16 peak; the fp16 dense rate is the same."""
+    against the burst bf16 peak; the fp16 dense rate is the same.  executed: see
+    executed_per_algorithmic."""
     peaks, src = _peaks()
     dom = max(kprof.items(), key=lambda kv: kv[1][0]) if kprof else ("none", (0.0, 1))
     name, (tot_ms, cnt) = dom
@@ -293,11 +301,12 @@ def roofline(kprof: dict, units: int, config: int) -> dict:
             sus = peaks.get("bf16_tflops_sustained", peak)
             return {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                     "frac": achieved / peak, "traffic": _traffic(name) if config == 2 else None,
-                    "executed_frac": 3 * achieved / peak, "algorithmic_cap": 1.0 / 3.0,
+                    "executed_frac": executed * achieved / peak, "algorithmic_cap": 1.0 / executed,
                     "note": f"{name}{' (+ slice combination)' if name == 'fwd_rs' else ''}: "
                             f"{avg_ms:.3f} ms/launch, 4 algorithmic flops per vis*pixel "
-                            f"(12 executed in the 3-term split, so the algorithmic fraction is capped at 1/3: "
-                            f"executed {3 * achieved:.0f} TFLOP/s); peak = {src} burst bf16 "
+                            f"({4 * executed:.0f} executed in the 3-term split"
+                            f"{' on the folded image' if executed < 3 else ''}, so the algorithmic fraction is "
+                            f"capped at {1 / executed:.2f}: executed {executed * achieved:.0f} TFLOP/s); peak = {src} burst bf16 "
                             f"(of sustained: {achieved / sus:.3f})"}
         if name.endswith("direct_f32"):
             # one SFU sine and one SFU cosine per (visibility, pixel) pair; peak
@@ -350,7 +359,7 @@ def large_block(precision: str, steps: int, warmup: int = 3, config: int = 5) ->
     ctx.close()
     return {"workload": WORKLOADS[config], "precision": precision, "steps": steps, "warmup": warmup,
             "ms_per_step": ms, "value": units / (ms * 1e-3), "unit": UNIT, "gpu_launches": launches,
-            "tiles": tiles, "roofline": roofline(kprof, units, config),
+            "tiles": tiles, "roofline": roofline(kprof, units, config, executed_per_algorithmic(precision)),
             "kernels": {k: {"ms_per_launch": v[0] / max(v[1], 1), "launches": v[1]} for k, v in kprof.items()}}
 
 
@@ -520,7 +529,7 @@ def main():
     e2e_val = job_value(units, world, max_over_ranks(statistics.mean(e2e_ms), dist, "cuda"))
 
     # ---- roofline of the dominant kernel (algorithmic flops per launch / event time)
-    roof = roofline(kprof, units, args.config)
+    roof = roofline(kprof, units, args.config, executed_per_algorithmic(args.precision))
     kernels = {k: {"ms_per_launch": v[0] / max(v[1], 1), "launches": v[1],
                    "share": v[0] / max(sum(x[0] for x in kprof.values()), 1e-30)} for k, v in kprof.items()}
 
@@ -553,10 +562,10 @@ def main():
     if not args.no_solve and args.solve_iters > 0:
         I0 = torch.full_like(img, float(ds.G))
         solve = {}
-        # the FP64 form takes about a minute per iteration at 256 x 256 and 1e6
+        # the FP64 form takes seconds per iteration at 256 x 256 and 1e6
         # visibilities: one timed iteration, no warm-up (its set-up is negligible)
         legs = [("form", args.precision, args.solve_iters, True)]
-        if units <= 2e11:  # the FP64 iteration is about a minute at 6.5e10 vis*pixel
+        if units <= 2e11:
             legs.append(("fp64", "fp64_direct", 1, False))
         for key, prec, iters, warm in legs:
             sctx = ctx if prec == args.precision else memsynth.Context(ds, precision=prec)
