@@ -378,7 +378,8 @@ int adj_splits(const mem_ctx* c) {
 mem_status ensure_buffers(mem_ctx* c) {
     const size_t NN = (size_t)c->N * c->N;
     TRY(dalloc(c, &c->chi_part, (size_t)4 * std::max(std::max(c->n_tiles, c->n_tiles_tc), 1)));
-    TRY(dalloc(c, &c->ent_part, (size_t)c->n_images * std::max(prep_blocks(c->N), std::max(tc_ent_blocks(c->N), fold_ent_blocks(c->N)))));
+    TRY(dalloc(c, &c->ent_part, (size_t)c->n_images * std::max({prep_blocks(c->N), tc_ent_blocks(c->N),
+                                                                fold_ent_blocks(c->N), f64_ent_blocks(c->N)})));
     c->scal = (double*)c->dstatus + 1;
     if (!c->img_tmp) {  // holds the scalar reduction's completion counter, which starts at zero
         TRY(dalloc(c, &c->img_tmp, (size_t)scalars_tmp_doubles(c->n_images)));

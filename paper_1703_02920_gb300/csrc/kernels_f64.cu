@@ -8,7 +8,7 @@
 // (visibility, pixel) pair takes about fifty operations a pair.  The FP64 units
 // (1.7 operations a clock and SM) bound both kernels; everything else hides
 // behind them.  64 x 64 with 10,260 visibilities, objective and gradient: 8.0 ms
-// with an exponential per pair, 0.40 ms now (CUDA events).
+// with an exponential per pair, 0.31 ms now.
 #include <algorithm>
 #include <cstdint>
 
@@ -45,7 +45,7 @@ __device__ __forceinline__ uint64_t half_phase(int k, uint64_t p) {
 
 // ---------------------------------------------------------------------------
 // Operand: the four mirror sums per (j, l), [channel][l / F_LB][j][l % F_LB][4],
-// columns beyond N/2 zero; entropy partials per 256 quadruples.
+// columns beyond N/2 zero; an entropy partial per block.
 // ---------------------------------------------------------------------------
 constexpr int F_LB = 16;  // columns l per block of the forward
 constexpr int F_JC = 16;  // rows j per work unit
@@ -53,13 +53,18 @@ constexpr int F_TH = 128; // visibilities per tile
 
 __host__ __device__ inline int f64_lblocks(int N) { return (N / 2 + F_LB - 1) / F_LB; }
 
-__global__ void __launch_bounds__(256) k_prep_f64(DevData d, ImgSrc src, double* __restrict__ B,
+// A block takes f64_prep_threads(N) quadruples: a pixel's FP64 operations, about
+// fifty with the entropy's logarithm, bound the kernel, so a small image spreads
+// over the SMs (64 x 64: four blocks of 256 took 21 us, 32 of 32 take 18, CUDA events).
+__host__ __device__ inline int f64_prep_threads(int N) { return N <= 160 ? 32 : 256; }
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) k_prep_f64(DevData d, ImgSrc src, double* __restrict__ B,
                                                   double* __restrict__ ent_part) {
-    __shared__ double sh[8];
+    __shared__ double sh[THREADS / 32];
     const int N = d.N, M = N / 2, LP = f64_lblocks(N) * F_LB;
     const int64_t NN = (int64_t)N * N;
     const int c = blockIdx.y, i = image_of(d, c);
-    const int64_t q = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    const int64_t q = (int64_t)blockIdx.x * THREADS + threadIdx.x;
     const bool ent = ent_part && !(d.shared && c != 0);
     double e = 0.0;
     if (q < (int64_t)M * LP) {
@@ -94,7 +99,7 @@ __global__ void __launch_bounds__(256) k_prep_f64(DevData d, ImgSrc src, double*
         out[1] = make_double2(f[2], f[3]);
     }
     if (ent) {
-        const double s = block_sum<256>(e, sh);
+        const double s = block_sum<THREADS>(e, sh);
         if (threadIdx.x == 0) ent_part[(int64_t)i * gridDim.x + blockIdx.x] = -s;
     }
 }
@@ -299,7 +304,10 @@ __global__ void __launch_bounds__(A_TH) k_adj_f64(DevData d, const double2* __re
 }  // namespace
 
 int64_t f64_operand_doubles(int N) { return (int64_t)f64_lblocks(N) * F_LB * (N / 2) * 4; }
-int f64_ent_blocks(int N) { return (int)(((int64_t)(N / 2) * f64_lblocks(N) * F_LB + 255) / 256); }
+int f64_ent_blocks(int N) {
+    const int t = f64_prep_threads(N);
+    return (int)(((int64_t)(N / 2) * f64_lblocks(N) * F_LB + t - 1) / t);
+}
 
 // shares of a tile's work units: eight warps per SM, four per tile
 int f64_shares(int N, int n_tiles, int num_sms) {
@@ -315,7 +323,9 @@ int f64_adj_splits(const DevData& d, int num_sms) {
 }
 
 void launch_prep_f64(const DevData& d, const ImgSrc& src, double* B, double* ent_part, cudaStream_t st) {
-    k_prep_f64<<<dim3(f64_ent_blocks(d.N), d.C), 256, 0, st>>>(d, src, B, ent_part);
+    const dim3 grid(f64_ent_blocks(d.N), d.C);
+    if (f64_prep_threads(d.N) == 32) k_prep_f64<32><<<grid, 32, 0, st>>>(d, src, B, ent_part);
+    else k_prep_f64<256><<<grid, 256, 0, st>>>(d, src, B, ent_part);
 }
 
 int launch_fwd_f64(const DevData& d, const VisTile* tiles, int n_tiles, const double* B, int mode, double2* yout,

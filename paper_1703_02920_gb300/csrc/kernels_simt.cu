@@ -378,25 +378,42 @@ void launch_adj_direct(const DevData& d, const float2* y, double* gsum, int ks, 
 // factor; Eq. chi2-multi for a shared image), plus lambda (1 + log(I/G))
 // (Eq. Sgradient), then the positive projection at the bound I = G.
 // ---------------------------------------------------------------------------
-template <bool FAST_LOG>
+// SPLIT threads per pixel: group g sums the g-th part of the ks shares, and the
+// groups' sums are added in order.  One thread per pixel would wait for its 152
+// loads and additions in turn (64 x 64, FP64 form: 28.7 -> 12.3 us, CUDA events).
+constexpr int FIN_SPLIT = 8;
+template <bool FAST_LOG, int SPLIT>
 __global__ void __launch_bounds__(256) k_finalize(DevData d, ImgSrc src,
                                                   const double* __restrict__ gsum, int ks,
                                                   int projected, float* out32, double* full64,
                                                   double* proj64) {
+    constexpr int PIX = 256 / SPLIT;
+    __shared__ double sh[SPLIT][PIX];
     chain_next();
     chain_wait();
     const int N = d.N;
     const int64_t NN = (int64_t)N * N;
     const int i = blockIdx.y;
-    const int64_t p = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    if (p >= NN) return;
+    const int el = threadIdx.x % PIX, grp = threadIdx.x / PIX;
+    const int64_t p = (int64_t)blockIdx.x * PIX + el;
     int c_lo = d.shared ? 0 : i, c_hi = d.shared ? d.C : i + 1;
     double g = 0.0;
-    for (int c = c_lo; c < c_hi; ++c) {
-        double s = 0.0;
-        for (int k = 0; k < ks; ++k) s += gsum[((int64_t)k * d.C + c) * NN + p];
-        g += (double)d.beam[(int64_t)c * NN + p] * s;
+    if (p < NN) {
+        const int ka = ks * grp / SPLIT, kb = ks * (grp + 1) / SPLIT;
+        for (int c = c_lo; c < c_hi; ++c) {
+            double s = 0.0;
+#pragma unroll 4
+            for (int k = ka; k < kb; ++k) s += gsum[((int64_t)k * d.C + c) * NN + p];
+            g += (double)d.beam[(int64_t)c * NN + p] * s;
+        }
     }
+    if (SPLIT > 1) {
+        sh[grp][el] = g;
+        __syncthreads();
+        if (grp != 0) return;
+        for (int k = 1; k < SPLIT; ++k) g += sh[k][el];
+    }
+    if (p >= NN) return;
     double x = img_value(src, i, p, NN);
     if (d.lambda != 0.0) g += d.lambda * (1.0 + (FAST_LOG ? log_ratio(x, d.G, d.ginv) : log(x / d.G)));
     double gp = (x <= d.G && g > 0.0) ? 0.0 : g;
@@ -407,9 +424,11 @@ __global__ void __launch_bounds__(256) k_finalize(DevData d, ImgSrc src,
 
 void launch_finalize(const DevData& d, const ImgSrc& src, int fast_log, const double* gsum, int ks, int projected,
                      float* out32, double* full64, double* proj64, cudaStream_t st) {
-    dim3 grid(prep_blocks(d.N), d.n_images);
-    launch_chained(fast_log ? k_finalize<true> : k_finalize<false>, grid, 256, 0, st, d.chain, 1, d, src, gsum, ks,
-                   projected, out32, full64, proj64);
+    const bool split = ks >= FIN_SPLIT;
+    const int pix = split ? 256 / FIN_SPLIT : 256;
+    auto kernel = fast_log ? k_finalize<true, 1> : split ? k_finalize<false, FIN_SPLIT> : k_finalize<false, 1>;
+    launch_chained(kernel, dim3((unsigned)(((int64_t)d.N * d.N + pix - 1) / pix), d.n_images), 256, 0, st, d.chain, 1, d,
+                   src, gsum, ks, projected, out32, full64, proj64);
 }
 
 // ---------------------------------------------------------------------------
