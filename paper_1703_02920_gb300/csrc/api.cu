@@ -577,13 +577,17 @@ mem_status run_adjoint(mem_ctx* c, const float2* y, bool ymax_ready, AdjointOut&
 // launch, and host (nullable) receives them there
 bool fused_objgrad(const mem_ctx* c) { return is_tc(c->prec) && !c->shared; }
 
-mem_status run_objgrad(mem_ctx* c, const ImgSrc& src, int projected, float* out32, double* full64,
+mem_status run_objgrad(mem_ctx* c, const ImgSrc& image, int projected, float* out32, double* full64,
                        double* proj64, double* host = nullptr) {
     TRY(ensure_buffers(c));
     void* yout = c->prec == MEM_PREC_FP64_DIRECT ? (void*)c->y64 : (void*)c->y32;
     // images of one channel each: the adjoint's unit-partial sum, the
-    // gradient assembly and the objective's scalar reduction are one launch
+    // gradient assembly and the objective's scalar reduction are one launch, and
+    // gsum, which then holds no sums, carries the pixels' log(I / G) from the
+    // entropy to the gradient (12 FP64 operations a pixel)
     const bool fused = fused_objgrad(c);
+    ImgSrc src = image;
+    if (fused) src.lg = c->gsum;
     TRY(run_forward(c, src, FWD_RESID, true, yout, fused));
     AdjointOut adj;
     adj.reduce = !fused;

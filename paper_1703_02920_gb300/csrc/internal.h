@@ -95,6 +95,8 @@ struct ImgSrc {
     const double* alpha;  // per image (device)
     double G;
     int diff;             // operand is max(I + alpha d, G) - I, entropy as a difference
+    double* lg = nullptr; // log(I / G) per image and pixel (nullable): the entropy's pass writes
+                          // it, the gradient's reads it instead of forming it again
 };
 
 // FWD_VIS: write V.  FWD_RESID: write y = w (V - V^o), chi^2 partials.

@@ -510,7 +510,8 @@ __global__ void __launch_bounds__(RedGeo<WIDE>::THREADS) k_adj_fold_reduce(DevDa
             else a.gsum[pix] = g;
         } else {
             const double x = img_value(src, c, (int64_t)n * N + m, NN);
-            const double gr = pixel_gradient(d, d.beam[pix], tot[0], other, inv, x);
+            // (an image per channel: pix is the image's pixel too)
+            const double gr = pixel_gradient(d, d.beam[pix], tot[0], other, inv, x, src.lg ? src.lg + pix : nullptr);
             const double gp = project_pixel(d, x, gr);
             if (a.full64) a.full64[pix] = gr;
             if (a.proj64) a.proj64[pix] = gp;

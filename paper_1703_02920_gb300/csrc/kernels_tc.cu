@@ -533,7 +533,8 @@ __global__ void __launch_bounds__(256) k_adj_tc_reduce_grad(DevData d, ImgSrc sr
     // (a converged solve of this form stops within 7 % of its test's bound: not one
     // rounding moves)
     double gr = (double)d.beam[(int64_t)c * NN + p] * (double)tot;
-    if (d.lambda != 0.0) gr += d.lambda * (1.0 + log_ratio(x, d.G, d.ginv));
+    if (d.lambda != 0.0)
+        gr += d.lambda * (1.0 + (src.lg ? src.lg[(int64_t)c * NN + p] : log_ratio(x, d.G, d.ginv)));
     const double gp = project_pixel(d, x, gr);
     if (full64) full64[(int64_t)c * NN + p] = gr;
     if (proj64) proj64[(int64_t)c * NN + p] = gp;

@@ -35,15 +35,16 @@ __device__ __forceinline__ int image_of(const DevData& d, int c) { return d.shar
 // of two, and the entropy's part.  Sum and product are FP32 pairs (good to 2^-46 of
 // FP32 inputs), the rest FP64: the pixel's FP64 operations bound this step on
 // large images, 20 of them where converting first and dividing by the scale took
-// 34 (1024 x 1024, gradient reduction: 70 -> 49 us; a cube of six 256 x 256 34 -> 29
-// us, CUDA events around the launch).
+// 34, and 8 with the logarithm that the entropy has left in lg (1024 x 1024,
+// gradient reduction: 70 -> 49 -> 37 us; a cube of six 256 x 256 34 -> 29 -> 24 us,
+// CUDA events around the launch).
 __device__ __forceinline__ double pixel_gradient(const DevData& d, float beam, float t0, float t1, double scale,
-                                                 double x) {
+                                                 double x, const double* lg) {
     const float s = t0 + t1, v = s - t0, e = (t0 - (s - v)) + (t1 - v);
     const float p = beam * s, q = fmaf(beam, e, fmaf(beam, s, -p));
     const double g = (double)p + (double)q;
     if (d.lambda == 0.0) return g * scale;
-    return fma(g, scale, fma(d.lambda, log_ratio(x, d.G, d.ginv), d.lambda));
+    return fma(g, scale, fma(d.lambda, lg ? *lg : log_ratio(x, d.G, d.ginv), d.lambda));
 }
 
 // 1 / f of a power of two f, exactly, without a division.
@@ -61,7 +62,9 @@ __device__ __forceinline__ double project_pixel(const DevData& d, double x, doub
 // whose operand is the difference max(I + alpha d, G) - I, the change against
 // the base image.
 __device__ __forceinline__ double entropy_term(const DevData& d, const ImgSrc& src, double x, int64_t q) {
-    double e = x * log_ratio(x, d.G, d.ginv);
+    const double l = log_ratio(x, d.G, d.ginv);
+    if (src.lg) src.lg[q] = l;
+    double e = x * l;
     if (src.diff) {
         const double x0 = src.f64[q];
         e -= x0 * log_ratio(x0, d.G, d.ginv);
