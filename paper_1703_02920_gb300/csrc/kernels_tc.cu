@@ -31,7 +31,7 @@ namespace msk {
 // ===========================================================================
 // Adjoint: split-K over visibilities.  A CTA owns a contiguous run of
 // (channel, output block, visibility range) units, accumulates each unit's
-// BLK x BLK block of G in TMEM over 16-visibility stages and drains it to an
+// BLK x BLK block of G in TMEM over stages of 16 or 32 visibilities and drains it to an
 // FP32 partial buffer; partials are summed in unit order afterwards (compensated
 // FP32 two-sum).
 // Operands are MN-major (8 consecutive pixels of one visibility per 16-byte
@@ -61,8 +61,12 @@ constexpr int ADJ_PRODUCERS = 16;  // producer warps: two groups of eight, alter
 constexpr int ADJ_THREADS = 32 * (8 + ADJ_PRODUCERS);
 
 __host__ __device__ inline int adj_rows(int BLK) { return BLK < 128 ? 128 : BLK; }
+// Visibilities per stage: 32 where three stages of them fit, one per lane of a
+// producer warp, so that no two lanes form the same step table (128 x 128 with
+// 100,003 visibilities 31 -> 27 us, 400,000 94 -> 79); else 16, and a warp's halves take different pixels.
+__host__ __device__ inline int adj_vb(int BLK) { return BLK <= 128 ? 32 : 16; }
 __host__ __device__ inline int adj_stage_bytes(int BLK) {
-    return 4 * adj_rows(BLK) * TCA_BK * 2 + 4 * BLK * TCA_BK * 2;
+    return 4 * adj_rows(BLK) * adj_vb(BLK) * 2 + 4 * BLK * adj_vb(BLK) * 2;
 }
 int adj_tc_smem_bytes(int N, int stages) { return stages * adj_stage_bytes(tca_blk(N)) + 1024; }
 __host__ __device__ inline uint32_t adj_tmem_cols(int BLK) {
@@ -141,18 +145,19 @@ struct AdjShared {
 // FROM_UV: phase increments reduced from u, v inside the producers instead of
 // read from the prepared arrays.
 // ADJ_STAGES: depth of the shared-memory pipeline (autotuned).
-template <bool FROM_UV, int ADJ_STAGES>
+template <bool FROM_UV, int ADJ_STAGES, int VB>
 __global__ void __launch_bounds__(ADJ_THREADS, 1)
     k_adj_tc(DevData d, const AdjUnit* __restrict__ units, const int* __restrict__ cta_unit_off,
              const float2* __restrict__ y, float* __restrict__ partial, uint64_t spin, int* status) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ AdjShared S;
+    constexpr int DRAIN = ADJ_DRAIN * 16 / VB;  // stages per accumulation
     const int N = d.N, c0 = N / 2;
     const int BLK = N < 256 ? N : 256;
     const int R = adj_rows(BLK);           // A rows (image rows n, padded to 128)
     const int n_mt = R / 128;
     const int nbx = N / BLK;
-    const int a_plane = R * TCA_BK * 2, b_plane = BLK * TCA_BK * 2;
+    const int a_plane = R * VB * 2, b_plane = BLK * VB * 2;
     const int stage_bytes = 4 * a_plane + 4 * b_plane;
     const uint32_t tcols = adj_tmem_cols(BLK);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -200,12 +205,12 @@ __global__ void __launch_bounds__(ADJ_THREADS, 1)
             bool ok = true;
             uint32_t it = 0;  // accumulation segments so far (tfull / tempty phases)
             for (int u = u0; u < u1 && ok; ++u) {
-              const int nst = (int)((units[u].count + TCA_BK - 1) / TCA_BK);
-              for (int seg0 = 0; seg0 < nst && ok; seg0 += ADJ_DRAIN, ++it) {
+              const int nst = (int)((units[u].count + VB - 1) / VB);
+              for (int seg0 = 0; seg0 < nst && ok; seg0 += DRAIN, ++it) {
                 ok = __all_sync(~0u, mbar_wait(&S.tempty, (it & 1) ^ 1, spin, abort, status));
                 if (!ok) break;
                 tc_fence_after();
-                const int seg1 = min(nst, seg0 + ADJ_DRAIN);
+                const int seg1 = min(nst, seg0 + DRAIN);
                 for (int ks = seg0; ks < seg1; ++ks, ++sc) {
                     const int s = sc % ADJ_STAGES;
                     ok = __all_sync(~0u, mbar_wait(&S.full[s], (sc / ADJ_STAGES) & 1, spin, abort, status));
@@ -214,18 +219,22 @@ __global__ void __launch_bounds__(ADJ_THREADS, 1)
                     const uint64_t so = (uint64_t)((uint32_t)(s * stage_bytes) >> 4);
                     const uint64_t bre_h = d_b + so, bre_l = bre_h + pb16;
                     const uint64_t bim_h = bre_h + 2 * pb16, bim_l = bre_h + 3 * pb16;
-                    for (int mt = 0; mt < n_mt; ++mt) {
-                        const uint64_t are_h = d_a + so + (uint64_t)(mt * 2048 >> 4);  // 16 groups of 8 rows
-                        const uint64_t are_l = are_h + pa16, aim_h = are_h + 2 * pa16, aim_l = are_h + 3 * pa16;
-                        const uint32_t dt = tmem + (uint32_t)(mt * BLK);
-                        const uint32_t acc = ks > seg0 ? 1u : 0u;
-                        // products sharing an A tile read it once (collector buffer)
-                        umma_f16_elect<MMA_FILL>(dt, are_h, bre_h, idesc, acc);
-                        umma_f16_elect<MMA_LASTUSE>(dt, are_h, bre_l, idesc, 1u);
-                        umma_f16_elect<MMA_PLAIN>(dt, are_l, bre_h, idesc, 1u);
-                        umma_f16_elect<MMA_FILL>(dt, aim_h, bim_h, idesc, 1u);
-                        umma_f16_elect<MMA_LASTUSE>(dt, aim_h, bim_l, idesc, 1u);
-                        umma_f16_elect<MMA_PLAIN>(dt, aim_l, bim_h, idesc, 1u);
+#pragma unroll
+                    for (int kk = 0; kk < VB / 16; ++kk) {
+                        for (int mt = 0; mt < n_mt; ++mt) {
+                            const uint64_t ka = (uint64_t)(kk * 2 * lboA >> 4), kb = (uint64_t)(kk * 2 * lboB >> 4);
+                            const uint64_t are_h = d_a + so + ka + (uint64_t)(mt * 2048 >> 4);  // 16 groups of 8 rows
+                            const uint64_t are_l = are_h + pa16, aim_h = are_h + 2 * pa16, aim_l = are_h + 3 * pa16;
+                            const uint32_t dt = tmem + (uint32_t)(mt * BLK);
+                            const uint32_t acc = ks > seg0 || kk > 0 ? 1u : 0u;
+                            // products sharing an A tile read it once (collector buffer)
+                            umma_f16_elect<MMA_FILL>(dt, are_h, bre_h + kb, idesc, acc);
+                            umma_f16_elect<MMA_LASTUSE>(dt, are_h, bre_l + kb, idesc, 1u);
+                            umma_f16_elect<MMA_PLAIN>(dt, are_l, bre_h + kb, idesc, 1u);
+                            umma_f16_elect<MMA_FILL>(dt, aim_h, bim_h + kb, idesc, 1u);
+                            umma_f16_elect<MMA_LASTUSE>(dt, aim_h, bim_l + kb, idesc, 1u);
+                            umma_f16_elect<MMA_PLAIN>(dt, aim_l, bim_h + kb, idesc, 1u);
+                        }
                     }
                     umma_commit_elect(&S.empty[s]);
                 }
@@ -244,8 +253,8 @@ __global__ void __launch_bounds__(ADJ_THREADS, 1)
         uint32_t dr = 0;
         bool ok = true;
         for (int u = u0; u < u1 && ok; ++u) {
-            const int nst = (int)((units[u].count + TCA_BK - 1) / TCA_BK);
-            for (int seg0 = 0; seg0 < nst; seg0 += ADJ_DRAIN, ++dr) {
+            const int nst = (int)((units[u].count + VB - 1) / VB);
+            for (int seg0 = 0; seg0 < nst; seg0 += DRAIN, ++dr) {
                 ok = __all_sync(0xffffffffu, mbar_wait(&S.tfull, dr & 1, spin, abort, status, 1024));
                 if (!ok) break;
                 tc_fence_after();
@@ -258,17 +267,18 @@ __global__ void __launch_bounds__(ADJ_THREADS, 1)
         }
     } else if (warp >= 8) {
         // ---------------------------------------- producers (two groups of 8)
-        // A warp-iteration builds two items (8 pixels of 16 visibilities each,
-        // one per half-warp).  Whole warps take one side, Ey items (A operand)
+        // A warp-iteration builds an item (8 pixels of 32 visibilities), or two of
+        // 16 visibilities, one per half-warp.  Whole warps take one side, Ey items (A operand)
         // or P items (B operand), so each thread builds one step table per
         // stage and the halves of a warp never diverge.  Every SM sub-partition
         // (warp % 4) has one warp of each side and group.
         const uint32_t grp = (warp - 8) >> 3;
         const bool ey_side = ((warp >> 2) & 1) == 0;
-        const int half = lane >> 4;
-        const int jj = lane & 15;           // visibility within the stage
+        constexpr int IPW = 32 / VB;          // items per warp-iteration
+        const int half = VB == 16 ? lane >> 4 : 0;
+        const int jj = lane & (VB - 1);       // visibility within the stage
         const int ngA = R / 8, ngB = BLK / 8;
-        const int wi_end = (ey_side ? ngA : ngB) / 2;
+        const int wi_end = (ey_side ? ngA : ngB) / IPW;
         const int ng = ey_side ? ngA : ngB, plane = ey_side ? a_plane : b_plane;
         const int side = ey_side ? 0 : 4 * a_plane;  // offset within a stage
         uint32_t sc = 0;  // stages so far, both groups'
@@ -276,13 +286,13 @@ __global__ void __launch_bounds__(ADJ_THREADS, 1)
         for (int u = u0; u < u1 && ok; ++u) {
             const AdjUnit un = units[u];
             const int p0 = (ey_side ? un.block / nbx : un.block % nbx) * BLK - c0;  // first pixel
-            const int nst = (int)((un.count + TCA_BK - 1) / TCA_BK);
+            const int nst = (int)((un.count + VB - 1) / VB);
             // this group's inputs of its next stage are loaded one stage ahead
             // (the phase of the side, and y on the P side)
             uint64_t np = 0;
             float2 ny = make_float2(0.f, 0.f);
             auto fetch = [&](int ks) {
-                const int64_t kv = (int64_t)ks * TCA_BK + jj;
+                const int64_t kv = (int64_t)ks * VB + jj;
                 np = 0;
                 ny = make_float2(0.f, 0.f);
                 if (ks < nst && kv < un.count) {
@@ -299,7 +309,7 @@ __global__ void __launch_bounds__(ADJ_THREADS, 1)
                 const int s = q % ADJ_STAGES;
                 const uint64_t ph = np;
                 const cf2 yv = {ny.x, ny.y};
-                const bool valid = (int64_t)ks * TCA_BK + jj < un.count;
+                const bool valid = (int64_t)ks * VB + jj < un.count;
                 fetch(ks + 2);
                 // rotation steps exp(-i 2 pi q c), q = 0..7, by powers of one SFU
                 // value: c = b for the Ey side, a for the P side (computed before
@@ -325,7 +335,7 @@ __global__ void __launch_bounds__(ADJ_THREADS, 1)
                 unsigned char* dst0 = smem + s * stage_bytes + side + (jj >> 3) * ng * 128 + (jj & 7) * 16;
 #pragma unroll 2
                 for (int wi = warp & 3; wi < wi_end; wi += 4) {
-                    const int g = 2 * wi + half;
+                    const int g = IPW * wi + half;
                     uint4 rh = {0, 0, 0, 0}, rl = {0, 0, 0, 0}, ih = {0, 0, 0, 0}, il = {0, 0, 0, 0};
                     if (valid && g * 8 < BLK) {
                         const cf2 e = cis_neg(phase_mul(p0 + g * 8, ph));
@@ -357,9 +367,10 @@ template <bool FROM_UV, int STAGES>
 static void launch_adj_variant(const DevData& d, const AdjUnit* units, const int* cta_unit_off, int n_ctas,
                                const float2* y, float* partial, uint64_t spin, int* status, cudaStream_t st) {
     const int smem = adj_tc_smem_bytes(d.N, STAGES);
-    cudaFuncSetAttribute(k_adj_tc<FROM_UV, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    launch_chained(k_adj_tc<FROM_UV, STAGES>, dim3(n_ctas), ADJ_THREADS, smem, st, d.chain, 1, d, units, cta_unit_off, y,
-                   partial, spin, status);
+    auto kernel = adj_vb(tca_blk(d.N)) == 32 ? k_adj_tc<FROM_UV, STAGES, 32> : k_adj_tc<FROM_UV, STAGES, 16>;
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    launch_chained(kernel, dim3(n_ctas), ADJ_THREADS, smem, st, d.chain, 1, d, units, cta_unit_off, y, partial, spin,
+                   status);
 }
 
 void launch_adj_tc(const DevData& d, const AdjUnit* units, const int* cta_unit_off, int n_ctas, const float2* y,
