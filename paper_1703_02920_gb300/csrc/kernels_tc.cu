@@ -46,15 +46,16 @@ namespace msk {
 // the producers, which need nearly as many.  With all producer warps on the same
 // stage its chain of latencies, about 2,100 clocks whatever N, was the bound.
 // 1024 x 1024 with 100,000 visibilities: 743 -> 598 us (the MMAs alone 0.52 ms),
-// 256 x 256 with 300,000: 148 -> 121 us, 128 x 128 with 100,003: 51 -> 31 us (CUDA
-// events around the launch, about 5 us of which are theirs); the same bits.
+// 256 x 256 with 300,000: 148 -> 121 us, 128 x 128 with 100,003: 51 -> 31 us, and
+// 28 with stages of 32 (CUDA events around the launch, about 5 us of which are
+// theirs); the same bits.
 // ===========================================================================
 constexpr int ADJ_MAX_STAGES = 3;
-// Stages (of 16 visibilities) accumulated in TMEM before the accumulator is
-// added into the unit's FP32 partial.  The tensor core rounds each MMA's
-// addition into its FP32 accumulator toward zero, so an accumulation of K
-// MMAs shrinks by up to ~K ulp; bounding K (6 MMAs per stage) bounds that
-// bias at ~2.5e-5 relative however many visibilities a unit spans.  The drains
+// Stages of 16 visibilities (half as many of 32) accumulated in TMEM before the
+// accumulator is added into the unit's FP32 partial.  The tensor core rounds each
+// MMA's addition into its FP32 accumulator toward zero, so an accumulation of K
+// MMAs shrinks by up to ~K ulp; bounding K (6 MMAs per 16 visibilities) bounds
+// that bias at ~2.5e-5 relative however many visibilities a unit spans.  The drains
 // add with round-to-nearest FP32 reductions, which have no such bias.
 constexpr int ADJ_DRAIN = 256;
 constexpr int ADJ_PRODUCERS = 16;  // producer warps: two groups of eight, alternate stages
@@ -63,7 +64,8 @@ constexpr int ADJ_THREADS = 32 * (8 + ADJ_PRODUCERS);
 __host__ __device__ inline int adj_rows(int BLK) { return BLK < 128 ? 128 : BLK; }
 // Visibilities per stage: 32 where three stages of them fit, one per lane of a
 // producer warp, so that no two lanes form the same step table (128 x 128 with
-// 100,003 visibilities 31 -> 27 us, 400,000 94 -> 79); else 16, and a warp's halves take different pixels.
+// 100,003 visibilities 31 -> 28 us, 400,000 94 -> 80); else 16, and a warp's
+// halves take different pixels.
 __host__ __device__ inline int adj_vb(int BLK) { return BLK <= 128 ? 32 : 16; }
 __host__ __device__ inline int adj_stage_bytes(int BLK) {
     return 4 * adj_rows(BLK) * adj_vb(BLK) * 2 + 4 * BLK * adj_vb(BLK) * 2;
