@@ -18,6 +18,7 @@ CASES = [
     (256, [65, 0, 127], False, ("resident", 256, 4, 3)), (256, [20001], False, ("resident", 256, 6, 2)),
     (256, [1, 200], True, None), (256, [129], False, ("stream", 128, 4, 2)), (512, [127], False, None),
     (512, [65], False, ("stream", 32, 3, 3)), (768, [70], False, None),
+    (64, [700001], False, None),  # over 4,096 visibilities a block: the adjoint's accumulator is drained within a unit
 ]
 
 
