@@ -84,6 +84,12 @@ __device__ __forceinline__ cf2 cmul(cf2 a, cf2 b) {
 // A chained launch (launch_chained): the next grid may start from here on; it
 // waits, where it calls chain_wait, until every grid before it has completed and
 // its writes are visible.  Without the launch attribute both do nothing.
+//
+// A grid of a chain is resident while the ones before it still write, so what an
+// earlier grid writes (and what the caller's kernels write: images, y) is not
+// read-only during its life.  Such buffers come as plain pointers and plain
+// loads; const __restrict__ and __ldg, which promise read-only data and which
+// nothing keeps behind the wait, are for what a context uploads once.
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

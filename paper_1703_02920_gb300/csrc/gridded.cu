@@ -124,7 +124,7 @@ __device__ float2* fft_shared(float2* a, float2* b, const float2* w, int M) {
 // Row pass: CTA (pair q, channel c) transforms rows 2q and 2q + 1 of the N x N
 // window of A_c * I (centred in the M x M padded image) and writes their half
 // spectra to R[c][k][n], k = 0..M/2.
-__global__ void __launch_bounds__(FFT_THREADS) k_fft_rows(DevData d, const float* __restrict__ img, int M,
+__global__ void __launch_bounds__(FFT_THREADS) k_fft_rows(DevData d, const float* img, int M,
                                                           float2* __restrict__ R) {
     extern __shared__ float2 sh[];
     float2 *a = sh, *b = sh + M, *w = sh + 2 * M;
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_rows(DevData d, const float
 
 // Column pass: CTA (column k, channel c) transforms R[c][k][.] placed at the
 // window rows of a length-M column and writes F[c][l][k], modulated.
-__global__ void __launch_bounds__(FFT_THREADS) k_fft_cols(int N, int M, const float2* __restrict__ R,
+__global__ void __launch_bounds__(FFT_THREADS) k_fft_cols(int N, int M, const float2* R,
                                                           float2* __restrict__ F) {
     extern __shared__ float2 sh[];
     float2 *a = sh, *b = sh + M, *w = sh + 2 * M;
@@ -189,10 +189,10 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_cols(int N, int M, const fl
 // Value of the modulated transform at grid frequency (k, l), 0 <= k, l < M, from
 // the half spectrum (columns 0..M/2; the rest by Hermitian symmetry of a real
 // image's transform; M is even, so the modulation survives the reduction mod M).
-__device__ __forceinline__ float2 grid_value(const float2* __restrict__ F, int M, int k, int l) {
+__device__ __forceinline__ float2 grid_value(const float2* F, int M, int k, int l) {
     const int H = M / 2 + 1;
-    if (k < H) return __ldg(F + (int64_t)l * H + k);
-    const float2 f = __ldg(F + (int64_t)(l ? M - l : 0) * H + (M - k));
+    if (k < H) return F[(int64_t)l * H + k];
+    const float2 f = F[(int64_t)(l ? M - l : 0) * H + (M - k)];
     return make_float2(f.x, -f.y);
 }
 
@@ -200,7 +200,7 @@ __device__ __forceinline__ float2 grid_value(const float2* __restrict__ F, int M
 // fraction of the 64-bit fixed-point phases times M.  (In FP64, products, floors
 // and 64-bit remainders took 44 us for 999,600 samples at M = 768, bound by the
 // FP64 units; 10 us now, bound by the gathers.)
-__global__ void __launch_bounds__(256) k_grid_interp(DevData d, int M, const float2* __restrict__ F,
+__global__ void __launch_bounds__(256) k_grid_interp(DevData d, int M, const float2* F,
                                                      int64_t z_total, float2* __restrict__ vis) {
     chain_next();
     chain_wait();

@@ -148,7 +148,7 @@ struct AdjShared {
 template <int SHAPE, int VB, int STAGES>
 __global__ void __launch_bounds__(ADJ_THREADS, 1)
     k_adj_fold(DevData d, const AdjUnit* __restrict__ units, const int* __restrict__ cta_unit_off,
-             const float2* __restrict__ y, const float* __restrict__ ymax, float* __restrict__ partial,
+             const float2* y, const float* ymax, float* __restrict__ partial,
              uint64_t spin, int* status) {
     using Geo = AdjGeo<SHAPE>;
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -463,8 +463,8 @@ __global__ void __launch_bounds__(RedGeo<WIDE>::THREADS) k_adj_fold_reduce(DevDa
         float x[RED_AHEAD], z[RED_AHEAD];
 #pragma unroll
         for (int k = 0; k < RED_AHEAD; ++k) {
-            x[k] = __ldg(p + k * stride);
-            z[k] = __ldg(p + k * stride + half);
+            x[k] = p[k * stride];
+            z[k] = p[k * stride + half];
         }
 #pragma unroll
         for (int k = 0; k < RED_AHEAD; ++k) {
@@ -474,8 +474,8 @@ __global__ void __launch_bounds__(RedGeo<WIDE>::THREADS) k_adj_fold_reduce(DevDa
         p += RED_AHEAD * stride;
     }
     for (; u < ub; ++u, p += stride) {
-        two_sum_acc(s0, e0, __ldg(p));
-        two_sum_acc(s1, e1, __ldg(p + half));
+        two_sum_acc(s0, e0, p[0]);
+        two_sum_acc(s1, e1, p[half]);
     }
     sh[0][g][el][0] = s0;
     sh[0][g][el][1] = e0;

@@ -206,9 +206,8 @@ __device__ __forceinline__ void finish_warp(float chi, float ym, int mode, doubl
 // STAGES: depth of the shared-memory pipeline (autotuned).
 template <int STAGES, int RES>
 __global__ void __launch_bounds__(FW_THREADS, 1)
-    k_fwd_fold(DevData d, const VisTile* __restrict__ tiles, int n_tiles, const uint16_t* __restrict__ planes,
-             const float4* __restrict__ cmean, int mode,
-             float2* __restrict__ yout, double* __restrict__ chi_part, unsigned* __restrict__ ymax_bits,
+    k_fwd_fold(DevData d, const VisTile* __restrict__ tiles, int n_tiles, const uint16_t* planes,
+             const float4* cmean, int mode, float2* yout, double* __restrict__ chi_part, unsigned* __restrict__ ymax_bits,
              float4* __restrict__ vpart, int64_t z_total, uint64_t spin, int* status) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ F2Shared S;
@@ -619,7 +618,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1)
                     // mean's term cm S enters once per column: with the block's
                     // first segment only.
                     float4 cm = {0.f, 0.f, 0.f, 0.f};
-                    if (lane < BN / (2 * MEAN_L)) cm = __ldg(cm_part + mb * (BN / (2 * MEAN_L)) + lane);
+                    if (lane < BN / (2 * MEAN_L)) cm = cm_part[mb * (BN / (2 * MEAN_L)) + lane];
                     if (seg != 0) cm.x = cm.y = 0.f;
                     ok = __all_sync(0xffffffffu, mbar_wait(&S.tfull[b], it & 1, spin, abort, status, 32));
                     if (!ok) break;
@@ -717,7 +716,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1)
 // RES_PART: one block of 128 threads per tile adds the two parts' sums and
 // applies the mode.
 __global__ void __launch_bounds__(128) k_fold_combine(DevData d, const VisTile* __restrict__ tiles,
-                                                     const float4* __restrict__ vpart, int64_t z_total, int mode,
+                                                     const float4* vpart, int64_t z_total, int mode,
                                                      float2* yout, double* chi_part, unsigned* ymax_bits) {
     chain_next();
     chain_wait();

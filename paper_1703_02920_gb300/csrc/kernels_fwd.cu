@@ -76,8 +76,7 @@ struct F2Shared {
 template <int F2_STAGES>
 __global__ void __launch_bounds__(F2_THREADS, 1)
     k_fwd_tc(DevData d, const VisTile* __restrict__ tiles, int n_tiles,
-             const uint16_t* __restrict__ planes, const float* __restrict__ cmean,
-             int mode, float2* __restrict__ yout, double* __restrict__ chi_part, uint64_t spin, int* status) {
+             const uint16_t* planes, const float* cmean, int mode, float2* yout, double* __restrict__ chi_part, uint64_t spin, int* status) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ F2Shared S;
     const int N = d.N, c0 = N / 2;
@@ -303,7 +302,7 @@ __global__ void __launch_bounds__(F2_THREADS, 1)
             if (tl.chan != cm_chan) {
                 __syncwarp();
                 const float4* src = (const float4*)(cmean + (int64_t)tl.chan * N);
-                for (int i = lane; i < N / 4; i += 32) ((float4*)cmw)[i] = __ldg(src + i);
+                for (int i = lane; i < N / 4; i += 32) ((float4*)cmw)[i] = src[i];
                 __syncwarp();
                 cm_chan = tl.chan;
             }

@@ -122,9 +122,9 @@ __device__ __forceinline__ void rs_finish_chi(double chi, int mode, int jv, doub
 
 template <int STAGES>
 __global__ void __launch_bounds__(RS_THREADS, 1)
-    k_fwd_rs(DevData d, const VisTile* __restrict__ tiles, int n_tiles, const uint16_t* __restrict__ planes,
-             const float* __restrict__ cmean, double2* __restrict__ vpart,
-             int64_t z_total, int mode, float2* __restrict__ yout, double* __restrict__ chi_part, uint64_t spin,
+    k_fwd_rs(DevData d, const VisTile* __restrict__ tiles, int n_tiles, const uint16_t* planes,
+             const float* cmean, double2* __restrict__ vpart,
+             int64_t z_total, int mode, float2* yout, double* __restrict__ chi_part, uint64_t spin,
              int* status) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ RsShared S;
@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
                 const int m0 = q * 16;
                 float4 cq4[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) cq4[k] = __ldg((const float4*)(cm + m0) + k);
+                for (int k = 0; k < 4; ++k) cq4[k] = ((const float4*)(cm + m0))[k];
                 const cf2 base = cis_neg(phase_mul(m0 - c0, pa));
                 const cf2 base8 = cmul(base, step8);
                 const float* cq = (const float*)cq4;
@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
 // One block of 64 threads per tile: V = sum of the slice partials (fixed
 // order), then the forward mode.
 __global__ void __launch_bounds__(64) k_fwd_combine(DevData d, const VisTile* __restrict__ tiles,
-                                                    const double2* __restrict__ vpart, int n_slices,
+                                                    const double2* vpart, int n_slices,
                                                     int64_t z_total, int mode, float2* yout, double* chi_part) {
     chain_next();
     chain_wait();

@@ -122,7 +122,7 @@ __device__ __forceinline__ int64_t tc_plane_index(int n, int m, int N, int BN) {
 }
 
 __global__ void __launch_bounds__(256) k_planes(DevData d, ImgSrc src, __nv_bfloat16* __restrict__ planes,
-                                                const float* __restrict__ cmean) {
+                                                const float* cmean) {
     chain_next();
     chain_wait();
     const int N = d.N, BN = d.fwd_bn;
@@ -166,7 +166,7 @@ __device__ __forceinline__ void max_over_blocks(float mx, unsigned* count, float
 }
 
 // max |y| over n floats.
-__global__ void __launch_bounds__(256) k_absmax(int64_t n, const float2* __restrict__ y, unsigned* count,
+__global__ void __launch_bounds__(256) k_absmax(int64_t n, const float2* y, unsigned* count,
                                                 float* ymax) {
     chain_next();
     chain_wait();
@@ -383,8 +383,7 @@ void launch_adj_direct(const DevData& d, const float2* y, double* gsum, int ks, 
 // loads and additions in turn (64 x 64, FP64 form: 28.7 -> 12.3 us, CUDA events).
 constexpr int FIN_SPLIT = 8;
 template <bool FAST_LOG, int SPLIT>
-__global__ void __launch_bounds__(256) k_finalize(DevData d, ImgSrc src,
-                                                  const double* __restrict__ gsum, int ks,
+__global__ void __launch_bounds__(256) k_finalize(DevData d, ImgSrc src, const double* gsum, int ks,
                                                   int projected, float* out32, double* full64,
                                                   double* proj64) {
     constexpr int PIX = 256 / SPLIT;
@@ -501,8 +500,7 @@ namespace msk {
 // adjoint scales by; here it costs no pass of its own (100,003
 // visibilities: three launches of 16 us together, now one of 7).
 __global__ void __launch_bounds__(256) k_dirty_y(DevData d, const double* __restrict__ wsum, int what,
-                                                 int64_t z_total, float2* __restrict__ y32,
-                                                 double2* __restrict__ y64, unsigned* count, float* ymax) {
+                                                 int64_t z_total, float2* y32, double2* y64, unsigned* count, float* ymax) {
     chain_next();
     chain_wait();
     float mx = 0.f;

@@ -150,7 +150,7 @@ struct AdjShared {
 template <bool FROM_UV, int ADJ_STAGES, int VB>
 __global__ void __launch_bounds__(ADJ_THREADS, 1)
     k_adj_tc(DevData d, const AdjUnit* __restrict__ units, const int* __restrict__ cta_unit_off,
-             const float2* __restrict__ y, float* __restrict__ partial, uint64_t spin, int* status) {
+             const float2* y, float* __restrict__ partial, uint64_t spin, int* status) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ AdjShared S;
     constexpr int DRAIN = ADJ_DRAIN * 16 / VB;  // stages per accumulation
@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(256) k_adj_tc_reduce_out(int N, const int* __r
     const int64_t p = (int64_t)((blk / nbx) * BLK + nl) * N + (blk % nbx) * BLK + ml;
     float s = 0.f, comp = 0.f;
     for (int u = cb_unit_off[blk]; u < cb_unit_off[blk + 1]; ++u)
-        two_sum_acc(s, comp, __ldg(partial + (int64_t)u * BLK * BLK + loc));
+        two_sum_acc(s, comp, partial[(int64_t)u * BLK * BLK + loc]);
     out[p] = beam[p] * (s + comp);
 }
 
@@ -425,7 +425,7 @@ void launch_adj_tc_reduce_out(int N, const int* cb_unit_off, const float* partia
 // launch) and four times the loads in flight of one thread per element.
 constexpr int RED_ELEMS = 64;
 template <int SPLIT>
-__device__ __forceinline__ void unit_sum_share(const float* __restrict__ src, int64_t stride, int u0, int u1, int g,
+__device__ __forceinline__ void unit_sum_share(const float* src, int64_t stride, int u0, int u1, int g,
                                                float& s, float& comp) {
     const int ua = u0 + (u1 - u0) * g / SPLIT, ub = u0 + (u1 - u0) * (g + 1) / SPLIT;
     s = 0.f;
@@ -434,11 +434,11 @@ __device__ __forceinline__ void unit_sum_share(const float* __restrict__ src, in
     for (; u + 8 <= ub; u += 8) {
         float q[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) q[k] = __ldg(src + (int64_t)(u + k) * stride);
+        for (int k = 0; k < 8; ++k) q[k] = src[(int64_t)(u + k) * stride];
 #pragma unroll
         for (int k = 0; k < 8; ++k) two_sum_acc(s, comp, q[k]);
     }
-    for (; u < ub; ++u) two_sum_acc(s, comp, __ldg(src + (int64_t)u * stride));
+    for (; u < ub; ++u) two_sum_acc(s, comp, src[(int64_t)u * stride]);
 }
 
 // Combine the four groups' (sum, compensation) pairs through shared memory;
@@ -456,7 +456,7 @@ __device__ __forceinline__ float unit_sum_combine(float s, float comp, int el, i
 }
 
 __global__ void __launch_bounds__(256) k_adj_tc_reduce(DevData d, const int* __restrict__ cb_unit_off,
-                                                       const float* __restrict__ partial,
+                                                       const float* partial,
                                                        double* __restrict__ gsum, float* __restrict__ out32) {
     __shared__ float sh[4][RED_ELEMS][2];
     chain_next();
@@ -510,7 +510,7 @@ void launch_adj_tc_reduce(const DevData& d, const int* cb_unit_off, const float*
 template <int SPLIT>
 __global__ void __launch_bounds__(256) k_adj_tc_reduce_grad(DevData d, ImgSrc src,
                                                             const int* __restrict__ cb_unit_off,
-                                                            const float* __restrict__ partial, int projected,
+                                                            const float* partial, int projected,
                                                             float* out32, double* full64, double* proj64,
                                                             ScalarArgs sc) {
     constexpr int ELEMS = 256 / SPLIT;
