@@ -87,8 +87,10 @@ struct mem_ctx {
     int* dstatus = nullptr;  // first word of the block that holds scal after it
     float* stage = nullptr;  // host-call staging (image, gradient)
     // pinned host words for the scalar and status readback (one copy pair and
-    // one stream synchronisation per call; nullptr: pageable fallback)
+    // one stream synchronisation per call; nullptr: pageable fallback).  Asked for
+    // once: captured graphs and readbacks both go by whether they exist.
     double* hscal = nullptr;
+    bool hscal_asked = false;
 
     // CUDA graphs: a launch sequence that repeats with the same buffers is
     // captured once (on a private stream: the legacy default stream cannot be
@@ -381,6 +383,13 @@ mem_status ensure_buffers(mem_ctx* c) {
     TRY(dalloc(c, &c->ent_part, (size_t)c->n_images * std::max({prep_blocks(c->N), tc_ent_blocks(c->N),
                                                                 fold_ent_blocks(c->N), f64_ent_blocks(c->N)})));
     c->scal = (double*)c->dstatus + 1;
+    if (!c->hscal_asked) {
+        c->hscal_asked = true;
+        if (cudaMallocHost((void**)&c->hscal, (4 + 3 * (size_t)c->n_images) * sizeof(double)) != cudaSuccess) {
+            c->hscal = nullptr;
+            cudaGetLastError();
+        }
+    }
     if (!c->img_tmp) {  // holds the scalar reduction's completion counter, which starts at zero
         TRY(dalloc(c, &c->img_tmp, (size_t)scalars_tmp_doubles(c->n_images)));
         CK(cudaMemsetAsync(c->img_tmp, 0, scalars_tmp_doubles(c->n_images) * sizeof(double), c->st),
@@ -679,22 +688,15 @@ mem_status graphed(mem_ctx* c, mem_ctx::GraphSlot& g, const void* k1, const void
     return MEM_OK;
 }
 
-// Pinned host words for the status word's slot and the scalars (nullptr: none to be had).
-double* host_words(mem_ctx* c) {
-    const size_t n = 4 + 3 * (size_t)c->n_images;
-    if (!c->hscal && cudaMallocHost((void**)&c->hscal, n * sizeof(double)) != cudaSuccess) {
-        c->hscal = nullptr;
-        cudaGetLastError();
-    }
-    return c->hscal;
-}
+// Where the evaluation's last kernel writes the status word's slot and the
+// scalars itself (nullptr: they are copied after it).
+double* kernel_host_words(const mem_ctx* c) { return fused_objgrad(c) ? c->hscal : nullptr; }
 
-// on_host: the evaluation's last kernel writes host_words itself.
-mem_status read_scalars(mem_ctx* c, std::vector<double>& out, bool on_host) {
+mem_status read_scalars(mem_ctx* c, std::vector<double>& out) {
     out.resize(3 + 3 * (size_t)c->n_images);
     const size_t n = out.size();
-    if (double* h = host_words(c)) {
-        if (!on_host)
+    if (double* h = c->hscal) {
+        if (!kernel_host_words(c))
             CK(cudaMemcpyAsync(h, c->dstatus, (n + 1) * sizeof(double), cudaMemcpyDeviceToHost, c->st),
                "scalar readback");
         CK(cudaStreamSynchronize(c->st), "stream synchronize");
@@ -1545,12 +1547,12 @@ mem_status mem_objective_grad(mem_ctx* c, const float* image_dev, float* grad_de
     if (!c || !image_dev) return fail(c, MEM_EINVAL, "null argument");
     ImgSrc src{image_dev, nullptr, nullptr, nullptr, c->G, 0};
     TRY(ensure_buffers(c));
-    double* host = fused_objgrad(c) ? host_words(c) : nullptr;
+    double* host = kernel_host_words(c);
     TRY(graphed(c, c->g_objgrad, image_dev, grad_dev, projected ? 1 : 0,
                 [&]() { return run_objgrad(c, src, projected, grad_dev, nullptr, nullptr, host); }));
     if (out3_host) {
         std::vector<double> sc;
-        TRY(read_scalars(c, sc, host != nullptr));
+        TRY(read_scalars(c, sc));
         out3_host[0] = sc[0];
         out3_host[1] = sc[1];
         out3_host[2] = sc[2];
@@ -1570,7 +1572,7 @@ mem_status mem_objective_grad_host(mem_ctx* c, const float* image_host, float* g
     if (grad_host)
         CK(cudaMemcpyAsync(grad_host, dgrad, n * sizeof(float), cudaMemcpyDeviceToHost, c->st), "gradient download");
     std::vector<double> sc;
-    TRY(read_scalars(c, sc, fused_objgrad(c) && host_words(c)));
+    TRY(read_scalars(c, sc));
     if (out3_host) {
         out3_host[0] = sc[0];
         out3_host[1] = sc[1];
