@@ -156,8 +156,9 @@ __global__ void __launch_bounds__(FP_THREADS) k_prep_fold(DevData d, ImgSrc src,
         mean[k] = red[0][k] / (float)(M * MEAN_L);
         top = fmaxf(top, fabsf(mean[k]));
     }
-    // (a strip of zeros, or of values below 2^-80, keeps a finite scale)
-    const float sc = pow2_scale_for(fmaxf(red[0][4] + top, 8.27180613e-25f));
+    // The scale follows the strip down to 2^-113, where it is 2^127, the largest
+    // power of two: fluxes in W/m^2/Hz (1 mJy = 1e-29) keep their 22 bits.
+    const float sc = pow2_scale_for(fmaxf(red[0][4] + top, 9.62964972e-35f));
     if (rank == 0 && threadIdx.x < 2) {
         // (P mean, Q mean, 1 / scale) of the cosine and of the sine part
         cmean[((int64_t)c * 2 + threadIdx.x) * (N / 32) + strip] =
