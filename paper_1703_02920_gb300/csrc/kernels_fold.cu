@@ -54,8 +54,8 @@
 //
 // Roles (five warpgroups): warps 0-3 and 4-7 epilogue groups; warp 8 MMA issue
 // (converged, one elected lane) + TMEM owner + resident copies, warp 9 copies
-// of the streamed operand, warps 10 and 11 finish the tiles (both parts' sums
-// -> V -> mode); warps 12-19 table producers.  Every SM sub-partition holds two
+// of the streamed operand, warps 10 and 11 (RES_BOTH: 9 too) finish the tiles (both
+// parts' sums -> V -> mode); warps 12-19 table producers.  Every SM sub-partition holds two
 // epilogue warps, two producers and one of the others; the register split
 // gives the epilogue 128 registers.  Every mbarrier wait is bounded.
 //
@@ -70,6 +70,7 @@
 // MMA work.
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "common.cuh"
 #include "internal.h"
@@ -109,7 +110,7 @@ struct F2Shared {
     uint64_t tfull[2];
     uint64_t tempty[2];   // 4 epilogue warps
     uint64_t xfull[2];    // both parts' sums of a tile (8 epilogue warps)
-    uint64_t xempty[2];   // read by the two finishing warps
+    uint64_t xempty[2];   // both halves of a tile read by finishing warps
     uint64_t bres;        // resident operand copy (transaction bytes)
     uint64_t bfree;       // MMAs reading the resident operand done
     uint64_t drain;
@@ -130,40 +131,102 @@ __host__ inline int f2_smem_bytes(int N, int BN, int stages, int res) {
            (res == RES_PART ? 0 : 2 * 2 * 128 * 16) + 1024;
 }
 
-// What a visibility's last steps read besides its sums, loaded ahead of them.
-struct FinishIn {
-    uint64_t half;  // (a + b) / 2
-    float4 o;       // V° as FP32 pairs (Re hi, Im hi, Re lo, Im lo)
-    float2 y;       // FWD_DCHI: the base image's weighted residual
+// A visibility's last steps: from both parts' sums, compensated pairs
+//   c = (sum c_l Tss, sum y_l Tsa),  s = (sum c_l Tas, sum y_l Taa),
+// V = exp(i pi (a + b)) W, then the forward mode.  finish_vis returns the
+// visibility's chi^2 term (twice that, but for FWD_DCHI); ym receives max
+// |component| of the weighted residual.  Finish holds what they read besides the
+// sums, loaded ahead of them.
+//
+// RES_STREAM: FP32 pairs.  The residual V - V° is an exact pair difference, and
+// chi^2 per visibility needs only FP32 relative accuracy (the partials are summed
+// in FP64).  The resident forms take residual, weight and chi^2 in FP64: any weight
+// and residual that FP64 holds (sigma below 5e-20 overflows an FP32 weight).  A
+// thread then waits out a chain of a dozen FP64 operations and five more per sum,
+// so RES_BOTH has three finishing warps instead of two, and loads a job ahead: with
+// two and without, 128 x 128 with 400,000 visibilities took 71 us, now 60.6, with
+// FP32 pairs 57.4 (64 x 64 with 10,260: 10.9, 10.4, 9.9; CUDA events).
+template <typename T>
+struct Finish;
+
+template <>
+struct Finish<float> {
+    uint64_t a, b;
+    float4 o;  // V° as FP32 pairs (Re hi, Im hi, Re lo, Im lo)
+    float2 y;  // FWD_DCHI: the base image's weighted residual
     float w;
 };
-__device__ __forceinline__ FinishIn finish_load(const DevData& d, int64_t j, int mode, const float2* yout) {
-    FinishIn f;
-    f.half = (uint64_t)((int64_t)d.pa[j] >> 1) + (uint64_t)((int64_t)d.pb[j] >> 1);
-    f.o = make_float4(0.f, 0.f, 0.f, 0.f);
-    f.y = make_float2(0.f, 0.f);
-    f.w = 0.f;
-    if (mode != FWD_VIS) f.w = d.w32[j];
+template <>
+struct Finish<double> {
+    uint64_t a, b;
+    double2 o;
+    double w;
+    float2 y;
+};
+template <typename T>
+__device__ __forceinline__ Finish<T> finish_load(const DevData& d, int64_t j, int mode, const float2* yout) {
+    Finish<T> f{};
+    f.a = d.pa[j];
+    f.b = d.pb[j];
     if (mode == FWD_DCHI) f.y = yout[j];
-    if (mode == FWD_RESID || mode == FWD_CHI) f.o = d.vo32[j];
+    if constexpr (sizeof(T) == 8) {
+        if (mode != FWD_VIS) f.w = d.w[j];
+        if (mode == FWD_RESID || mode == FWD_CHI) f.o = d.vo[j];
+    } else {
+        if (mode != FWD_VIS) f.w = d.w32[j];
+        if (mode == FWD_RESID || mode == FWD_CHI) f.o = d.vo32[j];
+    }
     return f;
 }
 
-// The rest of one visibility: W (the folded sum, compensated pairs) turned to
-// V = exp(i pi (a + b)) W, then the forward mode.  Returns the visibility's
-// chi^2 term; ym receives max |component| of the weighted residual.
-// FP32 pair arithmetic: the residual V - V° is an exact pair difference, and
-// chi^2 per visibility needs only FP32 relative accuracy (the partials are
-// summed in FP64).
-__device__ __forceinline__ float finish_vis(const FinishIn& f, int64_t j, float2 wre, float2 wim, int mode,
-                                            float2* yout, float& ym) {
-    const cf2 e = cis_neg_accurate((uint32_t)((0 - f.half) >> 32));
+// W turned to V = exp(i pi (a + b)) W, as pairs.
+__device__ __forceinline__ void turn_sums(uint64_t a_, uint64_t b_, float4 c, float4 s, float2& vre, float2& vim) {
+    const uint64_t half = (uint64_t)((int64_t)a_ >> 1) + (uint64_t)((int64_t)b_ >> 1);
+    const cf2 e = cis_neg_accurate((uint32_t)((0 - half) >> 32));
+    const float2 wre = df_add(c.x, c.y, -s.z, -s.w);  // c Tss - y Taa
+    const float2 wim = df_add(c.z, c.w, s.x, s.y);    // y Tsa + c Tas
     auto prod = [](float c, float2 w) {  // c * (w.x + w.y) as a pair
         const float p = c * w.x;
         return make_float2(p, fmaf(c, w.y, fmaf(c, w.x, -p)));
     };
     const float2 a = prod(e.x, wre), b = prod(-e.y, wim), g = prod(e.x, wim), h = prod(e.y, wre);
-    const float2 vre = df_add(a.x, a.y, b.x, b.y), vim = df_add(g.x, g.y, h.x, h.y);
+    vre = df_add(a.x, a.y, b.x, b.y);
+    vim = df_add(g.x, g.y, h.x, h.y);
+}
+
+// Only a valid visibility writes and counts; the arithmetic has no branch on it,
+// so that two of a thread's visibilities share the FP64 units' latency.
+__device__ __forceinline__ double finish_vis(const Finish<double>& f, int64_t j, bool valid, float4 c, float4 s,
+                                             int mode, float2* yout, float& ym) {
+    float2 vre, vim;
+    turn_sums(f.a, f.b, c, s, vre, vim);
+    if (mode == FWD_VIS) {
+        if (valid) yout[j] = make_float2(vre.x + vre.y, vim.x + vim.y);
+        return 0.0;
+    }
+    // V° is zero here in FWD_CURV and FWD_DCHI
+    const double rr = ((double)vre.x - f.o.x) + (double)vre.y, ri = ((double)vim.x - f.o.y) + (double)vim.y;
+    double chi;
+    if (mode == FWD_DCHI) {
+        const double h = 0.5 * f.w;
+        chi = fma(fma(h, rr, (double)f.y.x), rr, fma(h, ri, (double)f.y.y) * ri);
+    } else {
+        const double yr = f.w * rr, yi = f.w * ri;
+        chi = fma(yr, rr, yi * ri);
+        if (mode == FWD_RESID && valid) {
+            const float2 yv = make_float2((float)yr, (float)yi);
+            yout[j] = yv;
+            ym = fmaxf(fabsf(yv.x), fabsf(yv.y));
+        }
+    }
+    return valid ? chi : 0.0;
+}
+
+__device__ __forceinline__ float finish_vis(const Finish<float>& f, int64_t j, bool valid, float4 c, float4 s,
+                                            int mode, float2* yout, float& ym) {
+    if (!valid) return 0.f;
+    float2 vre, vim;
+    turn_sums(f.a, f.b, c, s, vre, vim);
     if (mode == FWD_VIS) {
         yout[j] = make_float2(vre.x + vre.y, vim.x + vim.y);
         return 0.f;
@@ -181,24 +244,30 @@ __device__ __forceinline__ float finish_vis(const FinishIn& f, int64_t j, float2
         yout[j] = yv;
         ym = fmaxf(fabsf(yv.x), fabsf(yv.y));
     }
-    return 0.5f * f.w * (rr * rr + ri * ri);
+    return f.w * (rr * rr + ri * ri);
 }
 
-// One warp's (32 visibilities') contribution to the tile partials.
-__device__ __forceinline__ void finish_warp(float chi, float ym, int mode, double* chi_slot, unsigned* ymax_bits,
-                                            int lane) {
-    if (mode == FWD_RESID && ymax_bits) {
-        // order-independent maximum (non-negative floats order as their bits)
+// Order-independent maximum (non-negative floats order as their bits).
+__device__ __forceinline__ void finish_max(float ym, int mode, unsigned* ymax_bits, int lane) {
+    if (mode != FWD_RESID || !ymax_bits) return;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ym = fmaxf(ym, __shfl_down_sync(0xffffffffu, ym, o));
-        if (lane == 0) atomicMax(ymax_bits, __float_as_uint(ym));
-    }
-    if (mode != FWD_VIS) {
-        // one partial per warp, summed later in a fixed order
+    for (int o = 16; o > 0; o >>= 1) ym = fmaxf(ym, __shfl_down_sync(0xffffffffu, ym, o));
+    if (lane == 0) atomicMax(ymax_bits, __float_as_uint(ym));
+}
+
+// The tile partials of two groups of 32 visibilities, one of each per lane, summed
+// later in a fixed order.  After the first step the warp's halves hold one group
+// each, so that both take five additions together.  finish_vis leaves the factor
+// 1/2 of FWD_RESID, FWD_CHI and FWD_CURV to the sum.
+template <typename T>
+__device__ __forceinline__ void finish_chi(T chi0, T chi1, int mode, double* chi_slots, int lane) {
+    if (mode == FWD_VIS) return;
+    const bool up = lane >= 16;
+    const T other = __shfl_xor_sync(0xffffffffu, up ? chi0 : chi1, 16);
+    T x = (up ? chi1 : chi0) + other;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) chi += __shfl_down_sync(0xffffffffu, chi, o);
-        if (lane == 0) *chi_slot = (double)chi;
-    }
+    for (int o = 8; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o, 16);
+    if ((lane & 15) == 0) chi_slots[lane >> 4] = mode == FWD_DCHI ? (double)x : 0.5 * (double)x;
 }
 
 // The operand's strips of MEAN_L columns l are scaled by powers of two, undone in
@@ -376,7 +445,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1)
         mbar_wait(&S.drain, 0, drain_limit(spin), (volatile int*)&dummy, status);
         if (!ok && nres > 0) mbar_wait(&S.bres, (nres - 1) & 1, drain_limit(spin), (volatile int*)&dummy, status);
         __syncwarp();
-    } else if (warp == 9) {
+    } else if (warp == 9 && RES != RES_BOTH) {
         // --------------------------------------------- streamed operand copies
         if (RES == RES_STREAM && lane == 0) {
             uint32_t sc = 0;
@@ -429,37 +498,66 @@ __global__ void __launch_bounds__(FW_THREADS, 1)
             }
         }
         __syncwarp();
-    } else if (warp < 12 && warp >= 10) {
+    } else if (warp < 12 && warp >= 9) {
         // ------------------------------------------------- finishing warps
-        // Warp 10 takes visibilities 0 .. 63 of a tile, warp 11 the others.
+        // A job is half a tile, two visibilities per thread; the finishing warps
+        // (10 and 11, with RES_BOTH 9 too) take them in turn.
         if (RES != RES_PART) {
+            using T = std::conditional_t<RES == RES_STREAM, float, double>;
+            constexpr int N_FIN = RES == RES_BOTH ? 3 : 2;
+            constexpr bool AHEAD = RES == RES_BOTH;
             const float4* xsum = (const float4*)(ring + STAGES * stage_bytes);
-            bool ok = true;
-            uint32_t ti = 0;
-            for (int t = t_begin; t < t_end && ok; t += t_step, ++ti) {
-                const VisTile tl = tiles[t];
-                const int q0 = 2 * (warp - 10);
-                FinishIn in[2];
+            const int jobs = t_begin < t_end ? 2 * ((t_end - t_begin + t_step - 1) / t_step) : 0;
+            auto tile_of = [&](int job) { return tiles[t_begin + (job >> 1) * t_step]; };
+            auto load = [&](const VisTile& tl, int job, Finish<T>(&f)[2]) {
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    const int jv = 32 * (q0 + h) + lane;
-                    in[h] = finish_load(d, tl.start + (jv < tl.count ? jv : 0), mode, yout);
+                    const int jv = 64 * (job & 1) + 32 * h + lane;
+                    f[h] = finish_load<T>(d, tl.start + (jv < tl.count ? jv : 0), mode, yout);
+                }
+            };
+            // AHEAD: a job's inputs arrive while the one before it is finished, its
+            // tile's descriptor another job ahead
+            const int job0 = warp - (12 - N_FIN);
+            VisTile tl_next = {}, tl_after = {};
+            Finish<T> next[2];
+            if (AHEAD && job0 < jobs) {
+                tl_next = tile_of(job0);
+                if (job0 + N_FIN < jobs) tl_after = tile_of(job0 + N_FIN);
+                load(tl_next, job0, next);
+            }
+            bool ok = true;
+            for (int job = job0; job < jobs && ok; job += N_FIN) {
+                const uint32_t ti = (uint32_t)job >> 1;
+                VisTile tl;
+                Finish<T> in[2];
+                if (AHEAD) {
+                    tl = tl_next;
+                    in[0] = next[0];
+                    in[1] = next[1];
+                    if (job + N_FIN < jobs) {
+                        tl_next = tl_after;
+                        if (job + 2 * N_FIN < jobs) tl_after = tile_of(job + 2 * N_FIN);
+                        load(tl_next, job + N_FIN, next);
+                    }
+                } else {
+                    tl = tile_of(job);
+                    load(tl, job, in);
                 }
                 ok = __all_sync(0xffffffffu, mbar_wait(&S.xfull[ti & 1], (ti >> 1) & 1, spin, abort, status, 250));
                 if (!ok) break;
                 const float4* slot = xsum + (ti & 1) * 256;
+                T chi[2];
+                float ym[2] = {0.f, 0.f};
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    const int jv = 32 * (q0 + h) + lane;
-                    const float4 xc = slot[jv], xs = slot[128 + jv];
-                    float chi = 0.f, ym = 0.f;
-                    if (jv < tl.count) {
-                        const float2 wre = df_add(xc.x, xc.y, -xs.z, -xs.w);  // c Tss - y Taa
-                        const float2 wim = df_add(xc.z, xc.w, xs.x, xs.y);    // y Tsa + c Tas
-                        chi = finish_vis(in[h], tl.start + jv, wre, wim, mode, yout, ym);
-                    }
-                    finish_warp(chi, ym, mode, chi_part + (int64_t)t * 4 + q0 + h, ymax_bits, lane);
+                    const int jv = 64 * (job & 1) + 32 * h + lane;
+                    chi[h] = finish_vis(in[h], tl.start + jv, jv < tl.count, slot[jv], slot[128 + jv], mode, yout,
+                                        ym[h]);
                 }
+                finish_max(fmaxf(ym[0], ym[1]), mode, ymax_bits, lane);
+                finish_chi(chi[0], chi[1], mode, chi_part + ((int64_t)(t_begin + (int)ti * t_step) * 2 + (job & 1)) * 2,
+                           lane);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&S.xempty[ti & 1]);
             }
@@ -549,7 +647,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1)
                 }
             }
         }
-    } else {
+    } else if (warp < 8) {
         // ------------------------ epilogue (two groups of four warps)
         // TMEM lane = visibility: warp q of a group holds visibilities
         // 32q .. 32q+31.  Group 0 drains accumulator 0 (the cosine part),
@@ -713,21 +811,27 @@ __global__ void __launch_bounds__(FW_THREADS, 1)
     }
 }
 
-// RES_PART: one block of 128 threads per tile adds the two parts' sums and
+// RES_PART: one block of 64 threads per tile adds the two parts' sums and
 // applies the mode.
-__global__ void __launch_bounds__(128) k_fold_combine(DevData d, const VisTile* __restrict__ tiles,
+__global__ void __launch_bounds__(64) k_fold_combine(DevData d, const VisTile* __restrict__ tiles,
                                                      const float4* vpart, int64_t z_total, int mode,
                                                      float2* yout, double* chi_part, unsigned* ymax_bits) {
     chain_next();
     chain_wait();
     const VisTile tl = tiles[blockIdx.x];
-    float chi = 0.f, ym = 0.f;
-    if ((int)threadIdx.x < tl.count) {
-        const int64_t j = tl.start + threadIdx.x;
-        const float4 c = vpart[j], s = vpart[z_total + j];
-        chi = finish_vis(finish_load(d, j, mode, yout), j, df_add(c.x, c.y, -s.z, -s.w), df_add(c.z, c.w, s.x, s.y), mode, yout, ym);
+    // two visibilities per thread, one of each half of the tile's groups
+    double chi[2];
+    float ym[2] = {0.f, 0.f};
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int jv = 32 * (2 * warp + h) + lane;
+        const int64_t j = tl.start + (jv < tl.count ? jv : 0);
+        chi[h] = finish_vis(finish_load<double>(d, j, mode, yout), j, jv < tl.count, vpart[j], vpart[z_total + j], mode,
+                            yout, ym[h]);
     }
-    finish_warp(chi, ym, mode, chi_part + (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5), ymax_bits, threadIdx.x & 31);
+    finish_max(fmaxf(ym[0], ym[1]), mode, ymax_bits, lane);
+    finish_chi(chi[0], chi[1], mode, chi_part + (int64_t)blockIdx.x * 4 + 2 * warp, lane);
 }
 
 struct FwdArgs {
@@ -803,7 +907,7 @@ int launch_fwd_fold(const DevData& d, int resident, const VisTile* tiles, int n_
     const int grid = res == RES_PART ? 2 * std::max(1, std::min(num_sms / 2, n_tiles)) : std::min(num_sms, n_tiles);
     launch_stages(a, res, grid);
     if (res != RES_PART) return 1;
-    launch_chained(k_fold_combine, dim3(n_tiles), 128, 0, st, d.chain, 1, d, tiles, (const float4*)vpart, z_total, mode, yout,
+    launch_chained(k_fold_combine, dim3(n_tiles), 64, 0, st, d.chain, 1, d, tiles, (const float4*)vpart, z_total, mode, yout,
                    chi_part, (unsigned*)ymax);
     return 2;
 }
