@@ -161,7 +161,7 @@ struct mem_ctx {
         d.n_images = n_images;
         d.shared = shared;
         d.G = G;
-        d.ginv = 1.0 / G;
+        d.ginv = ratio_inverse(G);
         d.lambda = lambda;
         d.pa = pa;
         d.pb = pb;

@@ -1,6 +1,7 @@
 // Internal interfaces of libmemsynth: device data views and kernel launchers.
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -26,13 +27,17 @@ struct AdjUnit {
     int64_t count;
 };
 
+// 1 / G for log_ratio; infinite, which takes the library's logarithm, where G times
+// a number near 1 might leave the normal range.
+inline double ratio_inverse(double G) { return G < 1e-300 || G > 1e300 ? HUGE_VAL : 1.0 / G; }
+
 // Read-only problem data resident on the device.
 struct DevData {
     int N;
     int C;
     int n_images;
     int shared;          // 1: one image for all channels
-    double G, ginv;      // ginv = 1 / G
+    double G, ginv;      // ginv = ratio_inverse(G)
     double lambda;
     const uint64_t* pa;  // frac(u dx) as 64-bit fixed-point turns
     const uint64_t* pb;  // frac(v dy)
