@@ -32,17 +32,14 @@ __device__ __forceinline__ double block_sum(double x, double* sh) {
 __device__ __forceinline__ int image_of(const DevData& d, int c) { return d.shared ? 0 : c; }
 
 // A pixel's gradient from its chi^2 part, beam (t0 + t1) scale with scale a power
-// of two, and the entropy's part.  Sum and product are FP32 pairs (good to 2^-46 of
-// FP32 inputs), the rest FP64: the pixel's FP64 operations bound this step on
-// large images, 20 of them where converting first and dividing by the scale took
-// 34, and 8 with the logarithm that the entropy has left in lg (1024 x 1024,
-// gradient reduction: 70 -> 49 -> 37 us; a cube of six 256 x 256 34 -> 29 -> 24 us,
-// CUDA events around the launch).
+// of two, and the entropy's part, in FP64: any beam and sum that FP32 holds.  The
+// pixel's FP64 operations bound this step on large images: with the scale divided
+// out and the logarithm formed again the gradient reduction took 70 us at 1024 x
+// 1024, with the inverse scale and the logarithm that the entropy left in lg 41 us
+// (CUDA events around the launch).
 __device__ __forceinline__ double pixel_gradient(const DevData& d, float beam, float t0, float t1, double scale,
                                                  double x, const double* lg) {
-    const float s = t0 + t1, v = s - t0, e = (t0 - (s - v)) + (t1 - v);
-    const float p = beam * s, q = fmaf(beam, e, fmaf(beam, s, -p));
-    const double g = (double)p + (double)q;
+    const double g = (double)beam * ((double)t0 + (double)t1);
     if (d.lambda == 0.0) return g * scale;
     return fma(g, scale, fma(d.lambda, lg ? *lg : log_ratio(x, d.G, d.ginv), d.lambda));
 }
