@@ -216,9 +216,9 @@ __global__ void __launch_bounds__(256) k_grid_interp(DevData d, int M, const flo
     }
     const float2* Fc = F + (int64_t)lo * M * (M / 2 + 1);
     const int k = (int)__umul64hi(pa, (uint64_t)M), l = (int)__umul64hi(pb, (uint64_t)M);
-    // (the top 32 bits of the fractions: 2^-33 off at most, then FP32)
-    const float fx = (float)(uint32_t)((pa * (uint64_t)M) >> 32) * 2.3283064365386963e-10f;
-    const float fy = (float)(uint32_t)((pb * (uint64_t)M) >> 32) * 2.3283064365386963e-10f;
+    // (all 64 bits of the fractions, rounded to FP32: small ones keep their digits)
+    const float fx = __ull2float_rn(pa * (uint64_t)M) * 5.421010862427522e-20f;
+    const float fy = __ull2float_rn(pb * (uint64_t)M) * 5.421010862427522e-20f;
     const int k1 = k + 1 == M ? 0 : k + 1, l1 = l + 1 == M ? 0 : l + 1;
     const float2 a = grid_value(Fc, M, k, l), b = grid_value(Fc, M, k1, l);
     const float2 e = grid_value(Fc, M, k, l1), f = grid_value(Fc, M, k1, l1);
