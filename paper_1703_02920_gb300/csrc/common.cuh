@@ -38,11 +38,6 @@ __device__ __forceinline__ float phase_to_angle_f32(uint64_t p) {
     return (float)(int32_t)(uint32_t)(p >> 32) * k2pi_2m32;
 }
 
-// Turns in [-0.5, 0.5) as FP64 from all 64 bits.
-__device__ __forceinline__ double phase_to_turns_f64(uint64_t p) {
-    return (double)(int64_t)p * 5.421010862427522e-20;  // 2^-64
-}
-
 // Compensated accumulation (Neumaier): s + c carries the sum of the added
 // terms to about twice FP32 precision, in a fixed order.
 __device__ __forceinline__ void two_sum_acc(float& s, float& c, float x) {
@@ -273,23 +268,6 @@ __device__ __forceinline__ void tc_fence_after() {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// D[tmem] (+)= A[smem] * B[smem]^T, kind::f16 (bf16 inputs, fp32 accumulate).
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
-                                          uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
-}
-
-// Arrive on an mbarrier once all previously issued tcgen05 ops of this thread complete.
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-            smem_u32(bar))
-        : "memory");
-}
-
 // Whole-warp forms of the MMA issue and commit.  Every lane of the warp
 // executes them, converged, and elect.sync picks the issuing lane.  For a
 // full member mask the election is deterministic (the same lane on every
@@ -488,25 +466,9 @@ __host__ __device__ __forceinline__ float pow2_scale_for(float x) {
     return ldexpf(1.f, 15 - e);
 }
 
-// Split x into bf16 hi + lo with x ~= hi + lo (|x - hi - lo| <~ 2^-16 |x|).
-__device__ __forceinline__ void split_bf16x2(float a, float b, uint32_t& hi, uint32_t& lo) {
-    __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-    float2 hf = __bfloat1622float2(h);
-    __nv_bfloat162 l = __floats2bfloat162_rn(a - hf.x, b - hf.y);
-    hi = *reinterpret_cast<uint32_t*>(&h);
-    lo = *reinterpret_cast<uint32_t*>(&l);
-}
-
-// Split into the 16-bit format of the tensor-core form (F16: f16, else bf16).
-template <bool F16>
-__device__ __forceinline__ void split16x2(float a, float b, uint32_t& hi, uint32_t& lo) {
-    if (F16) split_f16x2(a, b, hi, lo);
-    else split_bf16x2(a, b, hi, lo);
-}
-
 // ---------------------------------------------------------------------------
 // Packed FP32x2 forms (sm_100 and later) of the table arithmetic above.
-// Every component sees the roundings of cmul / split16x2 in the same order,
+// Every component sees the roundings of cmul and of the split in the same order,
 // two lanes per instruction.
 // ---------------------------------------------------------------------------
 
@@ -561,42 +523,31 @@ __device__ __forceinline__ Rot8 rot8_steps(uint64_t p, cf2& step8) {
     return r;
 }
 
-// split16x2 of the pair v = (a, b): the residual a - hi, b - hi in one
-// packed subtraction.
-template <bool F16>
-__device__ __forceinline__ void split16x2p(float2 v, uint32_t& hi, uint32_t& lo) {
-    if (F16) {
-        const __half2 h = __float22half2_rn(v);
-        const float2 hf = __half22float2(h);
-        const __half2 l = __float22half2_rn(__ffma2_rn(hf, make_float2(-1.f, -1.f), v));
-        hi = *reinterpret_cast<const uint32_t*>(&h);
-        lo = *reinterpret_cast<const uint32_t*>(&l);
-    } else {
-        // a - hi as one mixed-precision FMA (exact), without a conversion of hi
-        // back to FP32
-        asm("{\n .reg .b16 h0, h1, m1;\n .reg .f32 la, lb;\n mov.b16 m1, 0xBF80;\n cvt.rn.bf16x2.f32 %0, %3, %2;\n"
-            " mov.b32 {h0, h1}, %0;\n fma.rn.f32.bf16 la, h0, m1, %2;\n fma.rn.f32.bf16 lb, h1, m1, %3;\n"
-            " cvt.rn.bf16x2.f32 %1, lb, la;\n}\n"
-            : "=&r"(hi), "=r"(lo)
-            : "f"(v.x), "f"(v.y));
-    }
+// Split the pair (a, b) into bf16 hi + lo with x ~= hi + lo (|x - hi - lo| <~ 2^-16
+// |x|).  x - hi is one mixed-precision FMA (exact), without a conversion of hi back
+// to FP32.
+__device__ __forceinline__ void split_pair_bf16(float2 v, uint32_t& hi, uint32_t& lo) {
+    asm("{\n .reg .b16 h0, h1, m1;\n .reg .f32 la, lb;\n mov.b16 m1, 0xBF80;\n cvt.rn.bf16x2.f32 %0, %3, %2;\n"
+        " mov.b32 {h0, h1}, %0;\n fma.rn.f32.bf16 la, h0, m1, %2;\n fma.rn.f32.bf16 lb, h1, m1, %3;\n"
+        " cvt.rn.bf16x2.f32 %1, lb, la;\n}\n"
+        : "=&r"(hi), "=r"(lo)
+        : "f"(v.x), "f"(v.y));
 }
 
 // Eight rotated entries split into the four 16-byte operand rows of one
 // 8-element group: Re hi/lo and Im hi/lo.
-template <bool F16>
 __device__ __forceinline__ void table8_split(cf2 base, const Rot8& w, uint4& rh, uint4& rl, uint4& ih,
                                              uint4& il) {
     float2 re[4], im[4];
     rotate8(base, w, re, im);
-    split16x2p<F16>(re[0], rh.x, rl.x);
-    split16x2p<F16>(re[1], rh.y, rl.y);
-    split16x2p<F16>(re[2], rh.z, rl.z);
-    split16x2p<F16>(re[3], rh.w, rl.w);
-    split16x2p<F16>(im[0], ih.x, il.x);
-    split16x2p<F16>(im[1], ih.y, il.y);
-    split16x2p<F16>(im[2], ih.z, il.z);
-    split16x2p<F16>(im[3], ih.w, il.w);
+    split_pair_bf16(re[0], rh.x, rl.x);
+    split_pair_bf16(re[1], rh.y, rl.y);
+    split_pair_bf16(re[2], rh.z, rl.z);
+    split_pair_bf16(re[3], rh.w, rl.w);
+    split_pair_bf16(im[0], ih.x, il.x);
+    split_pair_bf16(im[1], ih.y, il.y);
+    split_pair_bf16(im[2], ih.z, il.z);
+    split_pair_bf16(im[3], ih.w, il.w);
 }
 
 // ---------------------------------------------------------------------------

@@ -8,7 +8,7 @@
 namespace msk {
 
 // Device status word bits (the host maps them to mem_status).
-enum : int { DEV_OK = 0, DEV_TIMEOUT = 1, DEV_BADARG = 2 };
+enum : int { DEV_OK = 0, DEV_TIMEOUT = 1 };
 
 // Consecutive visibilities of one channel (the forward kernels' unit: at most
 // VIS_TILE, or TC_TILE).

@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(F2_THREADS, 1)
                     if (valid) {
                         const int n0 = ks * TC_BK + g * 8;
                         base = (ks % PHASE_REFRESH) ? cmul(base, step_bk) : cis_neg(phase_mul(n0 - c0, pb));
-                        table8_split<false>(base, w, rh, rl, ih, il);
+                        table8_split(base, w, rh, rl, ih, il);
                     }
                     ok = __all_sync(0xffffffffu, mbar_wait(&S.empty[s], ((sc / F2_STAGES) & 1) ^ 1, spin,
                                                            abort, status, 64));

@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(RS_THREADS, 1)
                 uint4 rh = {0, 0, 0, 0}, rl = {0, 0, 0, 0}, ih = {0, 0, 0, 0}, il = {0, 0, 0, 0};
                 if (valid) {
                     const int n0 = slice * KS + ks * TC_BK + g * 8;
-                    table8_split<false>(cis_neg(phase_mul(n0 - c0, pb)), w, rh, rl, ih, il);
+                    table8_split(cis_neg(phase_mul(n0 - c0, pb)), w, rh, rl, ih, il);
                 }
                 ok = __all_sync(0xffffffffu,
                                 mbar_wait(&S.empty[s], ((sc / STAGES) & 1) ^ 1, spin, abort, status, 64));

@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(ADJ_THREADS, 1)
                     uint4 rh = {0, 0, 0, 0}, rl = {0, 0, 0, 0}, ih = {0, 0, 0, 0}, il = {0, 0, 0, 0};
                     if (valid && g * 8 < BLK) {
                         const cf2 e = cis_neg(phase_mul(p0 + g * 8, ph));
-                        table8_split<false>(ey_side ? e : cmul(yv, cf2{e.x, -e.y}), w, rh, rl, ih, il);
+                        table8_split(ey_side ? e : cmul(yv, cf2{e.x, -e.y}), w, rh, rl, ih, il);
                     }
                     unsigned char* dst = dst0 + g * 128;
                     *(uint4*)(dst + 0 * plane) = rh;
