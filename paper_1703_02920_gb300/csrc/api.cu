@@ -47,7 +47,7 @@ struct mem_ctx {
     std::vector<void*> allocs;
 
     // resident data
-    double *u = nullptr, *v = nullptr, *w = nullptr;
+    double* w = nullptr;
     uint64_t *pa = nullptr, *pb = nullptr;
     double2* vo = nullptr;
     float4* vo32 = nullptr;  // V° as FP32 (hi, lo) pairs, for the tensor-core epilogues
@@ -155,7 +155,7 @@ struct mem_ctx {
     size_t cg_hist_cap = 0;
 
     DevData dd() const {
-        DevData d;
+        DevData d{};
         d.N = N;
         d.C = C;
         d.n_images = n_images;
@@ -165,8 +165,6 @@ struct mem_ctx {
         d.lambda = lambda;
         d.pa = pa;
         d.pb = pb;
-        d.u = u;
-        d.v = v;
         d.vo = vo;
         d.w = w;
         d.vo32 = vo32;
@@ -1403,8 +1401,7 @@ mem_status mem_create(const mem_config* cfg, const double* u, const double* v, c
 
     const size_t NN = (size_t)N * N;
     mem_status s;
-    if ((s = dalloc(c, &c->u, std::max<int64_t>(Z, 1))) || (s = dalloc(c, &c->v, std::max<int64_t>(Z, 1))) ||
-        (s = dalloc(c, &c->w, std::max<int64_t>(Z, 1))) || (s = dalloc(c, &c->pa, std::max<int64_t>(Z, 1))) ||
+    if ((s = dalloc(c, &c->w, std::max<int64_t>(Z, 1))) || (s = dalloc(c, &c->pa, std::max<int64_t>(Z, 1))) ||
         (s = dalloc(c, &c->pb, std::max<int64_t>(Z, 1))) || (s = dalloc(c, &c->vo, std::max<int64_t>(Z, 1))) ||
         (s = dalloc(c, &c->vo32, std::max<int64_t>(Z, 1))) || (s = dalloc(c, &c->w32, std::max<int64_t>(Z, 1))) ||
         (s = dalloc(c, &c->beam, (size_t)C * NN)) || (s = dalloc(c, &c->doff, (size_t)C + 1)) ||
@@ -1428,8 +1425,15 @@ mem_status mem_create(const mem_config* cfg, const double* u, const double* v, c
     auto cpy = [&](void* dst, const void* src, size_t bytes) {
         return bytes ? cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, c->st) : cudaSuccess;
     };
-    e = cpy(c->u, u, Z * sizeof(double));
-    if (e == cudaSuccess) e = cpy(c->v, v, Z * sizeof(double));
+    // u and v only form the phases: they pass through vo's space
+    double* uv = (double*)c->vo;
+    e = cpy(uv, u, Z * sizeof(double));
+    if (e == cudaSuccess) e = cpy(uv + Z, v, Z * sizeof(double));
+    if (e == cudaSuccess) {
+        launch_phase_prep(Z, uv, uv + Z, c->dx, c->dy, c->pa, c->pb, c->st);
+        c->launches++;
+        e = cudaGetLastError();
+    }
     if (e == cudaSuccess) e = cpy(c->w, wh.data(), Z * sizeof(double));
     if (e == cudaSuccess) e = cpy(c->vo, vis_obs, Z * 2 * sizeof(double));
     if (e == cudaSuccess) e = cpy(c->w32, w32h.data(), Z * sizeof(float));
@@ -1442,9 +1446,6 @@ mem_status mem_create(const mem_config* cfg, const double* u, const double* v, c
         g_last_error = c->err;
         return bail(MEM_ECUDA);
     }
-    launch_phase_prep(Z, c->u, c->v, c->dx, c->dy, c->pa, c->pb, c->st);
-    c->launches++;
-
     build_tiles(c, VIS_TILE, c->tiles_h, c->tile_off_h);
     build_tiles(c, TC_TILE, c->tiles_tc_h, c->tile_off_tc_h);
     c->n_tiles = (int)c->tiles_h.size();

@@ -41,7 +41,7 @@ struct DevData {
     double lambda;
     const uint64_t* pa;  // frac(u dx) as 64-bit fixed-point turns
     const uint64_t* pb;  // frac(v dy)
-    const double* u;
+    const double* u;     // wavelengths: launch_adj_tc_uv only (a context keeps their phases)
     const double* v;
     const double2* vo;   // observed visibilities
     const double* w;     // 1/sigma^2
