@@ -72,10 +72,12 @@ struct mem_ctx {
     float2* y32 = nullptr;
     double2* y64 = nullptr;
     double *chi_part = nullptr, *ent_part = nullptr, *gsum = nullptr, *scal = nullptr, *img_tmp = nullptr;
-    int gsum_ks = 0;
+    int gsum_ks = 0;                   // shares that it holds
+    int gsum_asked = 0;                // FP64: shares asked for
     float* bf32 = nullptr;
     double* bf64 = nullptr;
     double2* wpart64 = nullptr;  // FP64 forward: sums per share of the work
+    bool wpart64_asked = false;
     uint16_t* planes = nullptr;
     float* cmean = nullptr;  // means of the centred tensor-core operand
     float4* cmean4 = nullptr;                   // FP16X3: means and inverse scale per strip
@@ -368,11 +370,14 @@ mem_status after_launch(mem_ctx* c, const char* what) {
     return MEM_OK;
 }
 
-// Visibility shares of the adjoint in the forms whose sums go through gsum.
+// Visibility shares of the adjoint in the forms whose sums go through gsum, and of
+// the FP64 forward.  The FP64 form takes fewer where its buffers for them could not be
+// had (ensure_buffers).
 int adj_splits(const mem_ctx* c) {
-    return c->prec == MEM_PREC_FP64_DIRECT ? f64_adj_splits(c->dd(), c->num_sms)
+    return c->prec == MEM_PREC_FP64_DIRECT ? std::min(f64_adj_splits(c->dd(), c->num_sms), c->gsum_ks)
                                            : adj_direct_splits(c->dd(), c->num_sms);
 }
+int fwd64_shares(const mem_ctx* c) { return c->wpart64 ? f64_shares(c->N, c->n_tiles, c->num_sms) : 1; }
 
 // Buffers needed by the current precision.
 mem_status ensure_buffers(mem_ctx* c) {
@@ -397,8 +402,6 @@ mem_status ensure_buffers(mem_ctx* c) {
     if (c->prec == MEM_PREC_FP64_DIRECT) {
         TRY(dalloc(c, &c->y64, (size_t)std::max<int64_t>(c->Z, 1)));
         TRY(dalloc(c, &c->bf64, (size_t)c->C * f64_operand_doubles(c->N)));
-        const int shares = f64_shares(c->N, c->n_tiles, c->num_sms);
-        if (shares > 1) TRY(dalloc(c, &c->wpart64, (size_t)shares * std::max<int64_t>(c->Z, 1)));
     } else if (c->prec == MEM_PREC_FP32_DIRECT) {
         TRY(dalloc(c, &c->bf32, (size_t)c->C * NN));
     } else {
@@ -424,13 +427,31 @@ mem_status ensure_buffers(mem_ctx* c) {
             (c->prec == MEM_PREC_BF16X3 ? fwd_rs_ks(c->N) < c->N : fold_combines(c->N)))
             TRY(dalloc(c, &c->vpart, (size_t)2 * std::max<int64_t>(c->Z, 1)));
     }
-    int ks = 1;
-    if (!is_tc(c->prec)) ks = adj_splits(c);
-    if (ks > c->gsum_ks) {
-        // grow: the old block stays allocated until destroy (rare)
-        c->gsum = nullptr;
-        TRY(dalloc(c, &c->gsum, (size_t)ks * c->C * NN));
-        c->gsum_ks = ks;
+    const bool f64 = c->prec == MEM_PREC_FP64_DIRECT;
+    const int ks = f64 ? f64_adj_splits(c->dd(), c->num_sms) : is_tc(c->prec) ? 1 : adj_splits(c);
+    if (ks > c->gsum_ks && !(f64 && ks <= c->gsum_asked)) {
+        // the FP64 form's shares only spread the work: under a memory limit it takes
+        // as many as fit (and keeps what it has); the old block stays allocated until
+        // destroy (rare)
+        double* grown = nullptr;
+        int k = ks;
+        mem_status st = dalloc(c, &grown, (size_t)k * c->C * NN);
+        while (st != MEM_OK && f64 && k > c->gsum_ks + 1) {
+            k = std::max(k / 2, c->gsum_ks + 1);
+            st = dalloc(c, &grown, (size_t)k * c->C * NN);
+        }
+        if (st == MEM_OK) {
+            c->gsum = grown;
+            c->gsum_ks = k;
+        } else if (!f64 || !c->gsum) {
+            return st;
+        }
+        if (f64) c->gsum_asked = ks;
+    }
+    if (f64 && !c->wpart64_asked) {
+        c->wpart64_asked = true;
+        const int shares = f64_shares(c->N, c->n_tiles, c->num_sms);
+        if (shares > 1) dalloc(c, &c->wpart64, (size_t)shares * std::max<int64_t>(c->Z, 1));
     }
     return MEM_OK;
 }
@@ -516,7 +537,7 @@ mem_status run_forward(mem_ctx* c, const ImgSrc& src, int mode, bool entropy, vo
         KTimer t(c, f64 ? "fwd_direct_f64" : "fwd_direct_f32");
         if (f64) {
             c->launches += launch_fwd_f64(d, c->tiles, c->n_tiles, c->bf64, mode, (double2*)yout, c->chi_part,
-                                          c->wpart64, f64_shares(c->N, c->n_tiles, c->num_sms), c->Z, c->st);
+                                          c->wpart64, fwd64_shares(c), c->Z, c->st);
         } else {
             launch_fwd_direct(d, c->tiles, c->n_tiles, c->bf32, mode, (float2*)yout, c->chi_part, c->st);
             if (c->n_tiles > 0) c->launches++;

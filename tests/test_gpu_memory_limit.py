@@ -1,0 +1,83 @@
+"""Contexts at a device memory limit (MEMSYNTH_MAX_BYTES, a failure made on the host):
+what fits is taken, what does not is refused, and a refused call leaves the context
+usable."""
+import numpy as np
+import pytest
+
+from paper_1703_02920_gb300 import synth as S
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ms():
+    from paper_1703_02920_gb300 import memsynth
+    memsynth.load()
+    return memsynth
+
+
+def _least(ms, monkeypatch, ds, form):
+    """The smallest limit (to 256 bytes) that lets a context be created."""
+    lo, hi = 0, 1 << 28
+    while hi - lo > 256:
+        mid = (lo + hi) // 2
+        monkeypatch.setenv("MEMSYNTH_MAX_BYTES", str(mid))
+        try:
+            ms.Context(ds, precision=form).close()
+            hi = mid
+        except ms.MemError as e:
+            assert e.status == 2
+            lo = mid
+    return hi
+
+
+@pytest.mark.parametrize("N", [64, 80])
+def test_fp64_form_shares_its_work_by_what_fits(ms, monkeypatch, N):
+    """The FP64 form needs no more than the FP32 form, whose shares are fewer, and its
+    own FP64 operand and residual; with fewer shares its sums are the same to the
+    order of FP64 additions."""
+    import torch
+    ds = S.random_problem(N, 900, 37, lam=1.0)
+    img = torch.from_numpy(ds.truth).cuda()
+    monkeypatch.delenv("MEMSYNTH_MAX_BYTES", raising=False)
+    ctx = ms.Context(ds, precision="fp64_direct")
+    want = ctx.objective_grad(img)
+    ctx.close()
+    limit = _least(ms, monkeypatch, ds, "fp32_direct") + 16 * ds.Z + 8 * N * (N + 16) + 4096
+    for cap in (limit, _least(ms, monkeypatch, ds, "fp64_direct")):
+        monkeypatch.setenv("MEMSYNTH_MAX_BYTES", str(cap))
+        ctx = ms.Context(ds, precision="fp64_direct")
+        for _ in range(3):
+            got = ctx.objective_grad(img)
+            for a, b in zip(got[:3], want[:3]):
+                assert abs(a - b) <= 1e-11 * abs(b)
+            assert torch.linalg.norm(got[3] - want[3]) <= 2e-7 * torch.linalg.norm(want[3])
+        ctx.close()
+
+
+def test_other_forms_keep_their_shares_after_a_limited_fp64(ms, monkeypatch):
+    """An FP64 context with few shares switched to the FP32 form: either its own shares
+    fit, or it is refused; never the FP64 form's smaller block."""
+    import torch
+    ds = S.random_problem(64, 900, 41, lam=1.0)
+    img = torch.from_numpy(ds.truth).cuda()
+    monkeypatch.delenv("MEMSYNTH_MAX_BYTES", raising=False)
+    ctx = ms.Context(ds, precision="fp32_direct")
+    want = ctx.objective_grad(img)
+    ctx.close()
+    least = _least(ms, monkeypatch, ds, "fp64_direct")
+    for cap in (least, least + (1 << 20), least + (3 << 20), least + (8 << 20)):
+        monkeypatch.setenv("MEMSYNTH_MAX_BYTES", str(cap))
+        ctx = ms.Context(ds, precision="fp64_direct")
+        first = ctx.objective_grad(img)
+        try:
+            ctx.set_precision("fp32_direct")
+        except ms.MemError as e:
+            assert e.status == 2
+        else:
+            got = ctx.objective_grad(img)
+            assert got[:3] == want[:3] and torch.equal(got[3], want[3])
+        ctx.set_precision("fp64_direct")
+        again = ctx.objective_grad(img)
+        assert again[0] == first[0] and torch.equal(again[3], first[3])
+        ctx.close()
