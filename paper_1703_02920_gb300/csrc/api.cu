@@ -1183,7 +1183,11 @@ mem_status mem_forward_gridded(mem_ctx* c, const float* image_dev, int32_t pad, 
         }
         c->grid_pad = 0;
         TRY(dalloc(c, &c->grid_R, (size_t)c->C * H * c->N));
-        TRY(dalloc(c, &c->grid_F, (size_t)c->C * M * H));
+        const mem_status st = dalloc(c, &c->grid_F, (size_t)c->C * M * H);
+        if (st != MEM_OK) {  // (not left for another pad, whose size it is not)
+            dfree(c, &c->grid_R, (size_t)c->C * H * c->N);
+            return st;
+        }
         c->grid_pad = pad;
     }
     DevData d = c->dd();

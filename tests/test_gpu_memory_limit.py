@@ -81,3 +81,27 @@ def test_other_forms_keep_their_shares_after_a_limited_fp64(ms, monkeypatch):
         again = ctx.objective_grad(img)
         assert again[0] == first[0] and torch.equal(again[3], first[3])
         ctx.close()
+
+
+def test_gridded_buffers_that_do_not_fit_are_given_back(ms, monkeypatch, oracle_mod):
+    """Row spectra of a padding whose 2-D spectra do not fit are not kept: the next
+    padding has its own."""
+    import torch
+    N = 64
+    ds = S.random_problem(N, 100, 43, lam=1.0)
+    least = _least(ms, monkeypatch, ds, "fp32_direct")
+    rows = lambda pad: (pad * N // 2 + 1) * N * 8  # noqa: E731
+    whole = lambda pad: (pad * N // 2 + 1) * pad * N * 8  # noqa: E731
+    cap = least + rows(1) + whole(1) + 2048
+    assert rows(2) < cap - least < rows(2) + whole(1)
+    monkeypatch.setenv("MEMSYNTH_MAX_BYTES", str(cap))
+    ctx = ms.Context(ds, precision="fp32_direct")
+    img = torch.from_numpy(ds.truth).cuda()
+    for _ in range(2):
+        with pytest.raises(ms.MemError) as e:
+            ctx.forward_gridded(img, 2)
+        assert e.value.status == 2
+        got = ctx.forward_gridded(img, 1).cpu().numpy().astype(np.float64)
+        ref = oracle_mod.forward_gridded(N, ds.dx, ds.dy, ds.u, ds.v, ds.pb[0].astype(np.float64) * ds.truth[0], 1)
+        assert np.max(np.abs(got[:, 0] + 1j * got[:, 1] - ref)) <= 2e-5 * np.max(np.abs(ref))
+    ctx.close()
