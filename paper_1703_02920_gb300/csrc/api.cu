@@ -1634,6 +1634,7 @@ mem_status mem_solve(mem_ctx* c, float* image_dev_inout, int32_t n_iter, mem_sol
         // grow: the old block stays allocated until destroy; the solve graph
         // refers to the history buffer and is rebuilt
         c->cg_hist = nullptr;
+        c->cg_hist_cap = 0;
         TRY(dalloc(c, &c->cg_hist, std::max(hist_n, (size_t)NI * 51 * 6)));
         c->cg_hist_cap = std::max(hist_n, (size_t)NI * 51 * 6);
     }

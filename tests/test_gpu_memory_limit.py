@@ -105,3 +105,22 @@ def test_gridded_buffers_that_do_not_fit_are_given_back(ms, monkeypatch, oracle_
         ref = oracle_mod.forward_gridded(N, ds.dx, ds.dy, ds.u, ds.v, ds.pb[0].astype(np.float64) * ds.truth[0], 1)
         assert np.max(np.abs(got[:, 0] + 1j * got[:, 1] - ref)) <= 2e-5 * np.max(np.abs(ref))
     ctx.close()
+
+
+def test_solve_after_a_history_that_did_not_fit(ms, monkeypatch):
+    import torch
+    ds = S.random_problem(64, 900, 47, lam=1.0)
+    start = torch.full((1, 64, 64), ds.G, dtype=torch.float32, device="cuda")
+    monkeypatch.delenv("MEMSYNTH_MAX_BYTES", raising=False)
+    ctx = ms.Context(ds, precision="fp16x3")
+    want = ctx.solve(start, 3)
+    ctx.close()
+    monkeypatch.setenv("MEMSYNTH_MAX_BYTES", str(_least(ms, monkeypatch, ds, "fp16x3") + (4 << 20)))
+    ctx = ms.Context(ds, precision="fp16x3")
+    for _ in range(2):
+        got = ctx.solve(start, 3)
+        assert torch.equal(got[0], want[0]) and np.array_equal(got[2], want[2])
+        with pytest.raises(ms.MemError) as e:
+            ctx.solve(start, 200000)  # a history of 9.6 MB
+        assert e.value.status == 2
+    ctx.close()
