@@ -1155,9 +1155,13 @@ mem_status mem_set_tiling(mem_ctx* c, const mem_tiling_t* t) {
                     "stages; resident kernel N <= 256 and 4..%d stages; adjoint 2|3 stages",
                     c->N <= 256 ? resident_stages(c) : 0);
     TRY(mem_sync(c));
+    const mem_tiling_t old = tiling_of(c);
     apply_tiling(c, x);
     drop_graphs(c);
-    return MEM_OK;
+    // (a call that is captured into the caller's graph cannot allocate)
+    const mem_status st = ensure_buffers(c);
+    if (st != MEM_OK) apply_tiling(c, old);
+    return st;
 }
 
 mem_status mem_tiling(const mem_ctx* c, mem_tiling_t* out) {
