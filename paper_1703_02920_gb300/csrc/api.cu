@@ -748,11 +748,14 @@ namespace {
 // (MEMSYNTH_TUNE_CACHE, default $HOME/.cache/libmemsynth_tune.txt) keyed by
 // device name, N, log2 of the visibility count, channel count and form.
 // ---------------------------------------------------------------------------
+constexpr const char* FOLDED = "|folded";
 std::string tune_key(const mem_ctx* c) {
     int zb = 0;
     while (((int64_t)1 << (zb + 1)) <= std::max<int64_t>(c->Z, 1)) ++zb;
     char buf[256];
-    std::snprintf(buf, sizeof buf, "%s|N=%d|z=%d|C=%d|prec=%d|folded", c->gpu_name.c_str(), c->N, zb, c->C, c->prec);
+    // (the FP16X3 kernels of entries without the suffix contracted the unfolded image)
+    std::snprintf(buf, sizeof buf, "%s|N=%d|z=%d|C=%d|prec=%d%s", c->gpu_name.c_str(), c->N, zb, c->C, c->prec,
+                  c->prec == MEM_PREC_FP16X3 ? FOLDED : "");
     std::string k = buf;
     for (char& ch : k)
         if (ch == ' ') ch = '_';
@@ -845,7 +848,8 @@ void tune_load(mem_ctx* c) {
     char k[256];
     mem_tiling_t t;
     while (std::fscanf(f, "%255s %d %d %d %d", k, &t.fwd_kernel, &t.fwd_cols, &t.fwd_stages, &t.adj_stages) == 5)
-        if (key == k && tune_valid(c, t)) apply_tiling(c, t);
+        // (BF16X3 entries carry the suffix or not, from either side of that change)
+        if ((key == k || (c->prec == MEM_PREC_BF16X3 && key + FOLDED == k)) && tune_valid(c, t)) apply_tiling(c, t);
     std::fclose(f);
 }
 
