@@ -111,12 +111,13 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
-def _traffic(kernel: str):
-    """DRAM bytes per launch from the committed ncu record, or None when the
-    kernel's sources changed since the capture (or there is no record)."""
+def _traffic(kernel: str, precision: str = "fp16x3"):
+    """DRAM bytes per launch from the committed ncu record of the form's kernel
+    (the forms share timer names), or None when the kernel's sources changed
+    since the capture (or there is no record)."""
     import hashlib
     try:
-        rec = json.load(open(os.path.join(ROOT, "profiles", "traffic.json")))[kernel]
+        rec = json.load(open(os.path.join(ROOT, "profiles", "traffic.json")))[precision][kernel]
         h = hashlib.sha256()
         for f in rec["sources"]:
             h.update(open(os.path.join(ROOT, f), "rb").read())
@@ -283,7 +284,7 @@ def executed_per_algorithmic(precision: str) -> float:
     return 1.5 if precision == "fp16x3" else 3.0
 
 
-def roofline(kprof: dict, units: int, config: int, executed: float = 3.0) -> dict:
+def roofline(kprof: dict, units: int, config: int, executed: float = 3.0, precision: str = "fp16x3") -> dict:
     """Roofline object of the dominant kernel from per-launch CUDA-event times.
     Each launch is timed alone (events around it), so the split forms are held
     against the burst bf16 peak; the fp16 dense rate is the same.  executed: see
@@ -300,7 +301,7 @@ def roofline(kprof: dict, units: int, config: int, executed: float = 3.0) -> dic
             peak = peaks.get("bf16_tflops")
             sus = peaks.get("bf16_tflops_sustained", peak)
             return {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                    "frac": achieved / peak, "traffic": _traffic(name) if config == 2 else None,
+                    "frac": achieved / peak, "traffic": _traffic(name, precision) if config == 2 else None,
                     "executed_frac": executed * achieved / peak, "algorithmic_cap": 1.0 / executed,
                     "note": f"{name}{' (+ slice combination)' if name == 'fwd_rs' else ''}: "
                             f"{avg_ms:.3f} ms/launch, 4 algorithmic flops per vis*pixel "
@@ -359,7 +360,7 @@ def large_block(precision: str, steps: int, warmup: int = 3, config: int = 5) ->
     ctx.close()
     return {"workload": WORKLOADS[config], "precision": precision, "steps": steps, "warmup": warmup,
             "ms_per_step": ms, "value": units / (ms * 1e-3), "unit": UNIT, "gpu_launches": launches,
-            "tiles": tiles, "roofline": roofline(kprof, units, config, executed_per_algorithmic(precision)),
+            "tiles": tiles, "roofline": roofline(kprof, units, config, executed_per_algorithmic(precision), precision),
             "kernels": {k: {"ms_per_launch": v[0] / max(v[1], 1), "launches": v[1]} for k, v in kprof.items()}}
 
 
@@ -529,7 +530,7 @@ def main():
     e2e_val = job_value(units, world, max_over_ranks(statistics.mean(e2e_ms), dist, "cuda"))
 
     # ---- roofline of the dominant kernel (algorithmic flops per launch / event time)
-    roof = roofline(kprof, units, args.config, executed_per_algorithmic(args.precision))
+    roof = roofline(kprof, units, args.config, executed_per_algorithmic(args.precision), args.precision)
     kernels = {k: {"ms_per_launch": v[0] / max(v[1], 1), "launches": v[1],
                    "share": v[0] / max(sum(x[0] for x in kprof.values()), 1e-30)} for k, v in kprof.items()}
 
