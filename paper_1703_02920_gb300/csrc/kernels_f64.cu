@@ -54,9 +54,12 @@ constexpr int F_TH = 128; // visibilities per tile
 __host__ __device__ inline int f64_lblocks(int N) { return (N / 2 + F_LB - 1) / F_LB; }
 
 // A block takes f64_prep_threads(N) quadruples: a pixel's FP64 operations, about
-// fifty with the entropy's logarithm, bound the kernel, so a small image spreads
-// over the SMs (64 x 64: four blocks of 256 took 21 us, 32 of 32 take 18, CUDA events).
-__host__ __device__ inline int f64_prep_threads(int N) { return N <= 160 ? 32 : 256; }
+// fifty with the entropy's logarithm, bound the kernel, so an image whose blocks of
+// 256 would not fill the SMs several times over spreads in blocks of 32: 64 x 64 13.4
+// us against 19.6, 256 x 256 14.2 against 19.9, 512 x 512 (256 blocks of 256) 30.1
+// against 33.8; 1024 x 1024 98.9 against 98.6, where more partials cost the scalar
+// reduction 2 us (CUDA events).
+__host__ __device__ inline int f64_prep_threads(int N) { return N <= 512 ? 32 : 256; }
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS) k_prep_f64(DevData d, ImgSrc src, double* __restrict__ B,
                                                   double* __restrict__ ent_part) {
