@@ -630,7 +630,7 @@ mem_status run_objgrad(mem_ctx* c, const ImgSrc& image, int projected, float* ou
                                         sc, c->st);
         else
             launch_adj_tc_reduce_grad(c->dd(), src, c->cb_off, c->partial, projected, out32, full64, proj64, sc,
-                                      c->st);
+                                      (int)c->units_h.size(), c->st);
     } else {
         KTimer t(c, "finalize");
         launch_finalize(c->dd(), src, is_tc(c->prec), c->gsum, adj.ks, projected, out32, full64, proj64, c->st);
@@ -1569,7 +1569,8 @@ mem_status mem_adjoint(mem_ctx* c, const float* y_dev, float* img_dev) {
         launch_adj_fold_reduce_grad(d, src, c->cb_off, c->partial, c->ymax, 0, img_dev, nullptr, nullptr, ScalarArgs{},
                                     c->st);
     else if (fused)
-        launch_adj_tc_reduce_grad(d, src, c->cb_off, c->partial, 0, img_dev, nullptr, nullptr, ScalarArgs{}, c->st);
+        launch_adj_tc_reduce_grad(d, src, c->cb_off, c->partial, 0, img_dev, nullptr, nullptr, ScalarArgs{},
+                                  (int)c->units_h.size(), c->st);
     else
         launch_finalize(d, src, is_tc(c->prec), c->gsum, adj.ks, 0, img_dev, nullptr, nullptr, c->st);
     c->launches++;

@@ -280,7 +280,7 @@ void launch_adj_fold_reduce_grad(const DevData& d, const ImgSrc& src, const int*
                                  const ScalarArgs& sc, cudaStream_t st);
 void launch_adj_tc_reduce_grad(const DevData& d, const ImgSrc& src, const int* cb_unit_off, const float* partial,
                                int projected, float* out32, double* full64, double* proj64, const ScalarArgs& sc,
-                               cudaStream_t st);
+                               int n_units, cudaStream_t st);
 
 // grad_i = sum_{c in image i} A_c * sum_k gsum[k][c] + lambda (1 + log(I/G)); optional projection.
 // fast_log: log_ratio instead of the library's logarithm (tensor-core forms).

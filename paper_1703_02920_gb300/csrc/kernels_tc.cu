@@ -504,9 +504,13 @@ void launch_adj_tc_reduce(const DevData& d, const int* cb_unit_off, const float*
 // reduction (scalars_block): it needs only the forward's chi^2 partials and
 // the prep's entropy partials, so it shares this launch instead of taking one
 // of its own.
-// SPLIT groups per element as above, or one where an output block has few units
-// (10 at 1024 x 1024): every thread then has a pixel's FP64 operations, which
-// a quarter of the threads would have to wait out (62 -> 47 us there).
+// SPLIT groups per element as above, or one where an output block has few units and
+// the images fill the SMs with a thread per pixel: every thread then has a pixel's
+// FP64 operations, which a quarter of the threads would have to wait out.  One against
+// four groups, us by CUDA events: 1024 x 1024 (10 units a block) 31 and 58, 512 x 512
+// (38) 18 and 21, 256 x 256 with 64 channels (3) 99 and 214, 6 (26) 22 and 33, 3 (51) 19
+// and 22, 2 (76) 22 and 19, 1 (152) 31 and 16; 128 x 128 with 4 channels (38) 14 and
+// 14; 64 x 64 with 4 (38, 64 blocks of a thread per pixel) 14 and 12.
 template <int SPLIT>
 __global__ void __launch_bounds__(256) k_adj_tc_reduce_grad(DevData d, ImgSrc src,
                                                             const int* __restrict__ cb_unit_off,
@@ -556,9 +560,10 @@ __global__ void __launch_bounds__(256) k_adj_tc_reduce_grad(DevData d, ImgSrc sr
 
 void launch_adj_tc_reduce_grad(const DevData& d, const ImgSrc& src, const int* cb_unit_off, const float* partial,
                                int projected, float* out32, double* full64, double* proj64,
-                               const ScalarArgs& sc, cudaStream_t st) {
+                               const ScalarArgs& sc, int n_units, cudaStream_t st) {
     const int64_t NN = (int64_t)d.N * d.N;
-    const bool one = d.N >= 1024;
+    const int nbx = d.N / tca_blk(d.N);
+    const bool one = n_units <= 40ll * d.C * nbx * nbx && d.C * NN >= 256 * 256;
     const int elems = one ? 256 : RED_ELEMS;
     const dim3 grid((unsigned)((NN + elems - 1) / elems) + (sc.scal ? sc.splits : 0), d.C);
     auto kernel = one ? k_adj_tc_reduce_grad<1> : k_adj_tc_reduce_grad<4>;
