@@ -82,8 +82,8 @@ __device__ __forceinline__ cf2 cmul(cf2 a, cf2 b) {
 //
 // A grid of a chain is resident while the ones before it still write, so what an
 // earlier grid writes (and what the caller's kernels write: images, y) is not
-// read-only during its life.  Such buffers come as plain pointers and plain
-// loads; const __restrict__ and __ldg, which promise read-only data and which
+// read-only during its life.  Such buffers come as plain pointers and plain loads
+// or __ldcg; const __restrict__ and __ldg, which promise read-only data and which
 // nothing keeps behind the wait, are for what a context uploads once.
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
