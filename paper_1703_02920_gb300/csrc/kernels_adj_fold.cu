@@ -55,18 +55,20 @@ namespace msk {
 // What bounds it: at 256 x 256 with 999,600 visibilities 0.22 ms, against 0.45 ms
 // for the unfolded kernel it replaces (CUDA events); a stage of 32 visibilities
 // holds 1,536 clocks of MMA work (0.16 ms) and takes about 2,000.  The producers
-// issue 96 % of the clocks: what counts is their instructions, about 600 per warp
-// and stage.  Stages of 16 visibilities repeat the step factors twice as often
+// set that: issue slots are 66 % active, about 440 instructions per producer warp and
+// stage, and a warp can only fill a slot while the ring's other one is in the MMAs.
+// Stages of 16 visibilities repeat the step factors twice as often
 // (0.28 ms); rotating every entry instead of sharing products about a group's
 // centre, and converting hi back to FP32, took 0.245 ms; packed FP32 pairs 0.258.
 // ===========================================================================
 constexpr int ADJ_MAX_STAGES = 3;
 // Visibilities accumulated in TMEM before the accumulators are added into the
 // unit's FP32 partials.  The tensor core rounds each MMA's addition into its
-// FP32 accumulator toward zero, so an accumulation of K MMAs shrinks by up to
-// ~K ulp; bounding K (3 MMAs per 16 visibilities) bounds that bias at ~2.5e-5
-// relative however many visibilities a unit spans.  The drains add with
-// round-to-nearest FP32 reductions, which have no such bias.
+// FP32 accumulator toward zero, so an accumulation of K MMAs (3 per 16
+// visibilities, K = 1,536) shrinks by up to K ulp, 1e-4 to 2e-4 at worst; sums of
+// one sign, which shrink most, measured 8.6e-6 low however many visibilities a unit
+// spans.  The drains add with round-to-nearest FP32 reductions, which have no such
+// bias.
 constexpr int ADJ_DRAIN = 8192;
 constexpr int ADJ_PRODUCER_WARPS = 12;
 constexpr int ADJ_THREADS = 32 * (ADJ_PRODUCER_WARPS + 1);

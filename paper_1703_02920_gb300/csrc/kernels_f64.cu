@@ -222,9 +222,9 @@ __global__ void __launch_bounds__(F_TH) k_fwd_f64_finish(DevData d, const VisTil
 //   cc = sum Re y' cos a cos b,  ss = sum Re y' sin a sin b,
 //   sc = sum Im y' sin a cos b,  cs = sum Im y' cos a sin b.
 // A block owns 32 x 32 quadruples (2 x 2 per thread) over a share of the
-// channel's visibilities; per 32 visibilities half of its threads write the row
-// factors (times y') and column factors to shared memory, 16 per thread from one
-// sincospi and a complex recurrence.
+// channel's visibilities; per 16 visibilities half of its threads write the row
+// factors (times y') and column factors to shared memory, eight per thread from
+// one sincospi and a complex recurrence.
 // ---------------------------------------------------------------------------
 constexpr int A_T = 32;   // quadruples per block side
 constexpr int A_V = 16;   // visibilities per shared-memory batch

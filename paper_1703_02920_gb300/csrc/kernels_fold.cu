@@ -568,7 +568,7 @@ __global__ void __launch_bounds__(FW_THREADS, 1)
         // (slot wait, stores, proxy fence) then overlap the other group's.
         // thread -> visibility jv = A row: 32 entries c_j (cosine part) or y_j
         // (sine part), as four groups of 8 rows.  A warp's 16-byte stores fill
-        // whole 128-byte core matrices (no bank conflicts).
+        // whole 128-byte core matrices, four wavefronts each.
         regs_dec<FW_REGS_PROD>();
         const int ptid = threadIdx.x - 384;
         const int jv = ptid & 127;

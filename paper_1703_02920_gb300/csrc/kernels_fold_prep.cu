@@ -9,8 +9,12 @@
 // them through distributed shared memory and no second launch has to wait for a
 // whole image.  (Column means over the image with one scale per channel took a
 // second launch and a completion counter: 23 + 8 us at 256 x 256 where this one
-// takes 12 us, CUDA events around the launches.)  Products and mirror sums are FP32 pairs, good to 2^-45; the
-// means only centre the operand, so plain FP32 sums in a fixed order serve.
+// takes 12 us, CUDA events around the launches.)
+// Products and mirror sums are FP32 pairs, good to 2^-45: the 22 bits of the split are
+// the same as from FP64 sums (error against 64-bit products on four kinds of images,
+// 256 x 256: equal to the seven digits printed, 6.1e-9 rms of the strip's scale on
+// random pixels).  The means only centre the operand, so plain FP32 sums in a fixed
+// order serve.
 //
 // The entropy sum is independent of the strips: further CTAs of the same launch
 // take 256 pixels per pass each, FP64 throughout.

@@ -54,9 +54,10 @@ constexpr int ADJ_MAX_STAGES = 3;
 // Stages of 16 visibilities (half as many of 32) accumulated in TMEM before the
 // accumulator is added into the unit's FP32 partial.  The tensor core rounds each
 // MMA's addition into its FP32 accumulator toward zero, so an accumulation of K
-// MMAs shrinks by up to ~K ulp; bounding K (6 MMAs per 16 visibilities) bounds
-// that bias at ~2.5e-5 relative however many visibilities a unit spans.  The drains
-// add with round-to-nearest FP32 reductions, which have no such bias.
+// MMAs (6 per 16 visibilities, K = 1,536) shrinks by up to K ulp, 1e-4 to 2e-4 at
+// worst; sums of one sign, which shrink most, measured 4.3e-6 low however many
+// visibilities a unit spans.  The drains add with round-to-nearest FP32 reductions,
+// which have no such bias.
 constexpr int ADJ_DRAIN = 256;
 constexpr int ADJ_PRODUCERS = 16;  // producer warps: two groups of eight, alternate stages
 constexpr int ADJ_THREADS = 32 * (8 + ADJ_PRODUCERS);
